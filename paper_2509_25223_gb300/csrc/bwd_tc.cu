@@ -1758,7 +1758,7 @@ __global__ void __launch_bounds__(po::NTP, 1) bwd_post_kernel(TcBwdParams P) {
 size_t bwd_tc_extra_bytes(long long nrec, bool deriv) {
   const size_t nct = (size_t)nrec;
   return nct * (4 * 64 * D * sizeof(float) + 2 * (size_t)D * D * sizeof(float) +
-                mask_bytes_per_chunk(D, deriv));
+                mask_bytes_per_chunk(D, deriv, true));
 }
 
 cudaError_t launch_bwd_tc(const FwdParams &f, const void *dO, const float *dST, const float *dRT,

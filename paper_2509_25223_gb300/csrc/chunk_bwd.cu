@@ -763,19 +763,13 @@ struct BwdLayout {
 // identity T matrices in its records), the variants the fp32 one
 bool use_tc_bwd(const rdn_fwd_args &f, int variant) {
   (void)variant;
-  return f.dtype == RDN_BF16 && f.Dk == 128 && !(f.flags & RDN_FLAG_VARIANTS & ~kTcVariants);
+  return fwd_uses_tc(f.Dk, f.dtype == RDN_BF16);
 }
 
 // The forward's per-chunk records are valid input when the caller passes the
-// forward's workspace with its chunk-start states and they are in the format
-// this backward reads: shared-memory images where the forward ran the
-// tensor-core scan, read by the tensor-core backward; fp32 otherwise (the
-// two choices agree for every argument set, so the check only guards them).
-bool reuse_fwd_records(const rdn_fwd_args &f, int variant) {
-  const FwdParams fp = make_fwd_params(f);
-  return f.workspace && f.S_chunks &&
-         fwd_uses_tc(fp, f.Dk, f.dtype == RDN_BF16) == use_tc_bwd(f, variant);
-}
+// forward's workspace with its chunk-start states (the forward wrote them in
+// the format this backward reads: both choose their kernels by fwd_uses_tc).
+bool reuse_fwd_records(const rdn_fwd_args &f) { return f.workspace && f.S_chunks; }
 
 BwdLayout layout(const rdn_bwd_args &a, int variant) {
   const rdn_fwd_args &f = a.fwd;
@@ -784,7 +778,7 @@ BwdLayout layout(const rdn_bwd_args &a, int variant) {
   const size_t accf = f.Dk == 128 ? Acc<128>::FLOATS : Acc<64>::FLOATS;
   BwdLayout l;
   // the forward's records are read from its workspace when it is passed
-  l.prep = reuse_fwd_records(f, variant) ? 0 : align256(sizeof(float) * nrec * kRecFloats);
+  l.prep = reuse_fwd_records(f) ? 0 : align256(sizeof(float) * nrec * kRecFloats);
   // (the tensor-core kernels keep their per-chunk sums in shared memory)
   l.acc = tc ? 0 : align256(sizeof(float) * nrec * accf);
   const bool need_states = f.S_chunks == nullptr;
@@ -793,7 +787,7 @@ BwdLayout layout(const rdn_bwd_args &a, int variant) {
   l.o = need_states ? align256(esz * (size_t)f.B * f.T * f.H * f.Dv) : 0;
   l.tc = tc ? align256(bwd_tc_extra_bytes(nrec, f.flags & RDN_FLAG_TANH_RESIDUAL)) : 0;
   // normalised q, k (RDN_FLAG_QK_NORM), unless the forward's workspace has them
-  l.qk = reuse_fwd_records(f, variant) ? 0 : align256(qk_norm_bytes(f));
+  l.qk = reuse_fwd_records(f) ? 0 : align256(qk_norm_bytes(f));
   // and, with bf16 inputs, dq, dk (w.r.t. the normalised q, k) in fp32 for
   // the normalisation's backward: its projection (dy - y <y, dy>) would
   // otherwise start from bf16-rounded dy
@@ -863,7 +857,7 @@ static cudaError_t launch_bwd_impl(const rdn_bwd_args &a, int variant, cudaStrea
   const bool grad_f32 = p.f.f32out != 0;
   p.f.f32out = 0;
   p.f.inject = fault_injection() == 4 ? 2 : 0;
-  const bool reuse = reuse_fwd_records(f, variant);
+  const bool reuse = reuse_fwd_records(f);
   p.f.ws = reuse ? (float *)f.workspace : (float *)ws;
   p.f.err = status_word();
   if (f.cu_seqlens) {  // this call's own copy of the packed-sequence table
@@ -876,7 +870,7 @@ static cudaError_t launch_bwd_impl(const rdn_bwd_args &a, int variant, cudaStrea
     set_qk_norm_copies(p.f, f, reuse ? (char *)f.workspace + qk_norm_offset(f)
                                      : ws + l.prep + l.acc + 2 * l.states + l.o + l.tc);
   if (reuse && (f.flags & RDN_FLAG_SAVE_FOR_BWD)) {  // E, E2 and the mask kept by the forward
-    const SavedLayout sl = saved_layout((size_t)p.f.nrec, f.Dv, f.flags & RDN_FLAG_TANH_RESIDUAL);
+    const SavedLayout sl = saved_layout(f);
     p.f.sv_E = (uint8_t *)f.workspace + sl.e;
     p.f.sv_E2 = (uint8_t *)f.workspace + sl.e2;
     p.f.sv_mask = (unsigned long long *)((char *)f.workspace + sl.mask);
@@ -890,13 +884,9 @@ static cudaError_t launch_bwd_impl(const rdn_bwd_args &a, int variant, cudaStrea
     p.f.S_chunks = (float *)(ws + l.prep + l.acc);
     p.f.R_chunks = (float *)(ws + l.prep + l.acc + l.states);
     p.f.o = ws + l.prep + l.acc + 2 * l.states;
-    e = launch_fwd_parts(p.f, f.Dk, rdnv, bf, true, true, s);
-    // the tensor-core forward leaves its records as shared-memory images,
-    // which the tensor-core backward reads too; the SIMT backward needs fp32
-    if (e == cudaSuccess && fwd_uses_tc(p.f, f.Dk, bf) && !tc)
-      e = launch_prep(p.f, f.Dk, rdnv, bf, false, s);
+    e = launch_fwd_parts(p.f, f.Dk, rdnv, bf, s);
   } else if (!reuse) {
-    e = launch_prep(p.f, f.Dk, rdnv, bf, tc, s);
+    e = launch_prep(p.f, f.Dk, rdnv, bf, s);
   }
   if (e != cudaSuccess) return e;
   p.Sc = p.f.S_chunks;

@@ -7,7 +7,6 @@ namespace rdn {
 
 constexpr int C = kChunk;
 constexpr int kThreads = 256;
-constexpr int kDVS = 32;  // value columns per scan CTA
 
 // Per-chunk workspace record written by chunk_prep (floats).
 constexpr int kCC = C * C;
@@ -53,52 +52,92 @@ struct BlockMM {
   __device__ static __forceinline__ int col() { return threadIdx.x % N; }
 };
 
-// (I + A)^-1 for a 64 x 64 strictly lower A (row stride ld), by 16 x 16
-// blocks, with 128 threads (g = thread index within the group):
-//   diagonal blocks  T_ii = (I + A_ii)^-1 by forward substitution (one thread
-//                    per block column, the column kept in registers);
-//   block row i      W_j = sum_{k=j}^{i-1} A_ik T_kj,  T_ij = -T_ii W_j.
-// W is scratch of 3 x 256 floats.  The caller synchronises the block between
-// the calls of the 4 stages (stage 0: diagonal; stage i: block row i).
-__device__ __forceinline__ void inv_diag_blocks(const float *A, float *Tm, int ld, int g) {
-  if (g < 64) {
-    const int blk = g >> 4, col = g & 15, b0 = blk * 16;
-    float x[16];
+// T = (I + A)^-1 for a strictly lower 64 x 64 A, by 128 threads (g = thread
+// index in the group); W is 32 x 32 scratch (row stride LDW; the block of Tm
+// at rows 0..31, columns 32..63 will do, which no stage touches).  The caller synchronises the
+// block between the stages (0: diagonal blocks; 1, 2: the 16-row blocks; 3, 4:
+// the 32-row block), all groups of the block running the same stage.  The
+// 16 x 16 blocks above the diagonal are never written: the caller zeroes them
+// once.
+template <int LDA, int LDT, int LDW>
+__device__ __forceinline__ void inv64_stage(int stage, const float *A, float *Tm, float *W, int g) {
+  if (stage == 0) {
+    // diagonal 16 x 16 blocks: thread (block, column) forward-substitutes its
+    // column, x[r] = delta(r, col) - sum_{m < r} A[r][m] x[m], the terms added
+    // in the order of m; the updates of the rows below m are independent, so
+    // they are made as soon as x[m] is final (a 16-step chain instead of 120)
+    if (g < 64) {
+      const int b0 = (g >> 4) * 16, col = g & 15;
+      float x[16];
 #pragma unroll
-    for (int r = 0; r < 16; ++r) {
-      float s = (r == col) ? 1.f : 0.f;
+      for (int r = 0; r < 16; ++r) x[r] = (r == col) ? 1.f : 0.f;
 #pragma unroll
-      for (int m = 0; m < r; ++m) s = fmaf(-A[(b0 + r) * ld + b0 + m], x[m], s);
-      x[r] = (r < col) ? 0.f : s;
+      for (int m = 0; m < 16; ++m) {
+        if (m < col) x[m] = 0.f;  // (above the diagonal)
+#pragma unroll
+        for (int r = m + 1; r < 16; ++r) x[r] = fmaf(-A[(b0 + r) * LDA + b0 + m], x[m], x[r]);
+      }
+#pragma unroll
+      for (int r = 0; r < 16; ++r) Tm[(b0 + r) * LDT + b0 + col] = x[r];
     }
+  } else if (stage <= 2) {
+    // 16-row blocks (i, j) = (1, 0) and (3, 2): W = A_ij T_jj, then
+    // T_ij = -T_ii W; thread (block, row r, columns 4q .. 4q + 3)
+    const int bi = 2 * (g >> 6) + 1, bj = bi - 1, r = (g >> 2) & 15, q = g & 3;
+    float *w = W + (g >> 6) * 16 * LDW;
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    if (stage == 1) {
 #pragma unroll
-    for (int r = 0; r < 16; ++r) Tm[(b0 + r) * ld + b0 + col] = x[r];
-  }
-  // zero the strictly upper blocks once
-  for (int e = g; e < 64 * 64; e += 128) {
-    const int r = e >> 6, c = e & 63;
-    if ((c >> 4) > (r >> 4)) Tm[r * ld + c] = 0.f;
-  }
-}
-__device__ __forceinline__ void inv_block_row_w(const float *A, const float *Tm, float *W, int ld,
-                                                int i, int g) {
-  for (int e = g; e < i * 256; e += 128) {
-    const int j = e >> 8, r = (e >> 4) & 15, cc = e & 15;
-    float s = 0.f;
-    for (int k = j; k < i; ++k)
+      for (int k = 0; k < 16; ++k) {
+        const float a = A[(16 * bi + r) * LDA + 16 * bj + k];
+        const float4 t = *reinterpret_cast<const float4 *>(Tm + (16 * bj + k) * LDT + 16 * bj + 4 * q);
+        acc[0] = fmaf(a, t.x, acc[0]); acc[1] = fmaf(a, t.y, acc[1]);
+        acc[2] = fmaf(a, t.z, acc[2]); acc[3] = fmaf(a, t.w, acc[3]);
+      }
+      *reinterpret_cast<float4 *>(w + r * LDW + 4 * q) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+    } else {
 #pragma unroll
-      for (int m = 0; m < 16; ++m)
-        s = fmaf(A[(16 * i + r) * ld + 16 * k + m], Tm[(16 * k + m) * ld + 16 * j + cc], s);
-    W[e] = s;
-  }
-}
-__device__ __forceinline__ void inv_block_row_t(float *Tm, const float *W, int ld, int i, int g) {
-  for (int e = g; e < i * 256; e += 128) {
-    const int j = e >> 8, r = (e >> 4) & 15, cc = e & 15;
-    float s = 0.f;
-#pragma unroll
-    for (int m = 0; m < 16; ++m) s = fmaf(Tm[(16 * i + r) * ld + 16 * i + m], W[j * 256 + m * 16 + cc], s);
-    Tm[(16 * i + r) * ld + 16 * j + cc] = -s;
+      for (int k = 0; k < 16; ++k) {
+        const float a = Tm[(16 * bi + r) * LDT + 16 * bi + k];
+        const float4 t = *reinterpret_cast<const float4 *>(w + k * LDW + 4 * q);
+        acc[0] = fmaf(a, t.x, acc[0]); acc[1] = fmaf(a, t.y, acc[1]);
+        acc[2] = fmaf(a, t.z, acc[2]); acc[3] = fmaf(a, t.w, acc[3]);
+      }
+      *reinterpret_cast<float4 *>(Tm + (16 * bi + r) * LDT + 16 * bj + 4 * q) =
+          make_float4(-acc[0], -acc[1], -acc[2], -acc[3]);
+    }
+  } else {
+    // the 32-row block: W = A[32:64, 0:32] T[0:32, 0:32], then
+    // T[32:64, 0:32] = -T[32:64, 32:64] W; thread (rows rp, rp + 16, columns 4q .. 4q + 3)
+    const int q = g & 7, rp = g >> 3;
+    float a0[4] = {0.f, 0.f, 0.f, 0.f}, a1[4] = {0.f, 0.f, 0.f, 0.f};
+    if (stage == 3) {
+#pragma unroll 8
+      for (int k = 0; k < 32; ++k) {
+        const float x0 = A[(32 + rp) * LDA + k], x1 = A[(48 + rp) * LDA + k];
+        const float4 t = *reinterpret_cast<const float4 *>(Tm + k * LDT + 4 * q);
+        a0[0] = fmaf(x0, t.x, a0[0]); a0[1] = fmaf(x0, t.y, a0[1]);
+        a0[2] = fmaf(x0, t.z, a0[2]); a0[3] = fmaf(x0, t.w, a0[3]);
+        a1[0] = fmaf(x1, t.x, a1[0]); a1[1] = fmaf(x1, t.y, a1[1]);
+        a1[2] = fmaf(x1, t.z, a1[2]); a1[3] = fmaf(x1, t.w, a1[3]);
+      }
+      *reinterpret_cast<float4 *>(W + rp * LDW + 4 * q) = make_float4(a0[0], a0[1], a0[2], a0[3]);
+      *reinterpret_cast<float4 *>(W + (rp + 16) * LDW + 4 * q) = make_float4(a1[0], a1[1], a1[2], a1[3]);
+    } else {
+#pragma unroll 8
+      for (int k = 0; k < 32; ++k) {
+        const float x0 = Tm[(32 + rp) * LDT + 32 + k], x1 = Tm[(48 + rp) * LDT + 32 + k];
+        const float4 t = *reinterpret_cast<const float4 *>(W + k * LDW + 4 * q);
+        a0[0] = fmaf(x0, t.x, a0[0]); a0[1] = fmaf(x0, t.y, a0[1]);
+        a0[2] = fmaf(x0, t.z, a0[2]); a0[3] = fmaf(x0, t.w, a0[3]);
+        a1[0] = fmaf(x1, t.x, a1[0]); a1[1] = fmaf(x1, t.y, a1[1]);
+        a1[2] = fmaf(x1, t.z, a1[2]); a1[3] = fmaf(x1, t.w, a1[3]);
+      }
+      *reinterpret_cast<float4 *>(Tm + (32 + rp) * LDT + 4 * q) =
+          make_float4(-a0[0], -a0[1], -a0[2], -a0[3]);
+      *reinterpret_cast<float4 *>(Tm + (48 + rp) * LDT + 4 * q) =
+          make_float4(-a1[0], -a1[1], -a1[2], -a1[3]);
+    }
   }
 }
 
@@ -195,19 +234,28 @@ __device__ __forceinline__ void rec_decode(const FwdParams &p, long long r, int 
 
 // Where the forward keeps those intermediates: after the nrec record slots.
 // With the tanh residual (deriv) the clip mask's place holds the residual
-// map's derivative instead, [chunk][j][t] as 16-bit fixed point (grad_q16).
+// map's derivative instead: [chunk][j][t] as 16-bit fixed point (grad_q16) on
+// the tensor-core path, [chunk][t][j] fp32 on the fp32 path, which keeps every
+// intermediate in 32 bits (its E and E2 are [chunk][t][j] fp32, its clip mask
+// [chunk][t] rows of Dv bits).
 struct SavedLayout {
   size_t e, e2, mask, bytes;  // byte offsets from the workspace base; region size
 };
-inline size_t mask_bytes_per_chunk(int Dv, bool deriv) {
-  return deriv ? (size_t)Dv * C * 2 : (size_t)Dv * sizeof(unsigned long long);
+inline size_t mask_bytes_per_chunk(int Dv, bool deriv, bool tc) {
+  return deriv ? (size_t)Dv * C * (tc ? 2 : 4) : (size_t)Dv * sizeof(unsigned long long);
 }
-inline SavedLayout saved_layout(size_t nct, int Dv, bool deriv) {
+// Whether a call runs the tensor-core kernels (and its records are
+// shared-memory images): bf16 inputs, d = 128, every variant flag, RDN and RLA
+// alike.
+inline bool fwd_uses_tc(int DK, bool bf16) { return bf16 && DK == 128; }
+inline SavedLayout saved_layout(const rdn_fwd_args &a) {
+  const size_t nct = (size_t)call_records(a);
   SavedLayout l;
   l.e = nct * sizeof(float) * (size_t)kRecFloats;
-  l.e2 = l.e + nct * sizeof(float) * C * Dv;
-  l.mask = l.e2 + nct * sizeof(float) * C * Dv;
-  l.bytes = l.mask + nct * mask_bytes_per_chunk(Dv, deriv) - l.e;
+  l.e2 = l.e + nct * sizeof(float) * C * a.Dv;
+  l.mask = l.e2 + nct * sizeof(float) * C * a.Dv;
+  l.bytes = l.mask - l.e + nct * mask_bytes_per_chunk(a.Dv, a.flags & RDN_FLAG_TANH_RESIDUAL,
+                                                      fwd_uses_tc(a.Dk, a.dtype == RDN_BF16));
   return l;
 }
 
@@ -251,7 +299,7 @@ inline size_t qk_norm_offset(const rdn_fwd_args &a) {
   const size_t nrec = (size_t)call_records(a);
   size_t off = sizeof(float) * (size_t)kRecFloats * nrec;
   if (a.flags & RDN_FLAG_SAVE_FOR_BWD)
-    off += saved_layout(nrec, a.Dv, a.flags & RDN_FLAG_TANH_RESIDUAL).bytes;
+    off += saved_layout(a).bytes;
   return off;
 }
 // Points p.q, p.k at the normalised copies starting at `base`.
@@ -261,23 +309,12 @@ inline void set_qk_norm_copies(FwdParams &p, const rdn_fwd_args &a, char *base) 
   p.k = base + half;
 }
 
-// The variant flags the tensor-core kernels implement: all four (the decayed
-// residual, the plain combine, the tanh residual, the stateless correction).
-constexpr unsigned kTcVariants = RDN_FLAG_DECAYED_RESIDUAL | RDN_FLAG_PLAIN_COMBINE |
-                                 RDN_FLAG_TANH_RESIDUAL | RDN_FLAG_STATELESS_AUX;
-// Whether the forward runs the tensor-core scan (and its records are
-// shared-memory images): bf16 inputs, d = 128, no variant flag outside
-// kTcVariants, for RDN and RLA alike.
-inline bool fwd_uses_tc(const FwdParams &p, int DK, bool bf16) {
-  return bf16 && DK == 128 && (p.mods & ~kTcVariants) == 0;
-}
-
 // Tensor-core scan (fwd_tc.cu): bf16 inputs with d_k = d_v = 128.
 cudaError_t launch_fwd_tc(const FwdParams &p, bool rdnv, cudaStream_t s);
 
-// Prep kernel alone; img selects the shared-memory-image record format read
-// by the tensor-core kernels (else the fp32 format of the SIMT kernels).
-cudaError_t launch_prep(const FwdParams &p, int DK, bool rdnv, bool bf16, bool img, cudaStream_t s);
+// The forward's prep kernel alone (per-chunk records into p.ws, in the format
+// that this call's kernels read).
+cudaError_t launch_prep(const FwdParams &p, int DK, bool rdnv, bool bf16, cudaStream_t s);
 
 // Tensor-core backward (bwd_tc.cu): recompute, chain and post kernels.
 cudaError_t launch_prep_tc(const FwdParams &p, bool rla, cudaStream_t s);
@@ -287,9 +324,19 @@ cudaError_t launch_bwd_tc(const FwdParams &f, const void *dO, const float *dST, 
                           float *dbeta, float *dgamma, float *dS0, float *dR0, char *extra,
                           bool rla, bool grad_f32, bool dqk_f32, cudaStream_t s);
 
-// Launch the forward's prep kernel (per-chunk records into p.ws) and/or its
-// scan kernel (outputs, optional chunk-start states).
-cudaError_t launch_fwd_parts(const FwdParams &p, int DK, bool rdnv, bool bf16, bool do_prep,
-                             bool do_scan, cudaStream_t s);
+// Launch the forward: prep (per-chunk records into p.ws), then the scan
+// (outputs, optional chunk-start states).
+cudaError_t launch_fwd_parts(const FwdParams &p, int DK, bool rdnv, bool bf16, cudaStream_t s);
+
+// E, E2 and the residual's mask of every chunk (p.sv_*) from the chunk-start
+// states p.S_chunks, p.R_chunks (fp32 path).
+cudaError_t launch_recompute(const FwdParams &p, int DK, bool rdnv, bool bf16, cudaStream_t s);
+
+// The current device's SM count.
+inline cudaError_t sm_count(int *n) {
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  return e != cudaSuccess ? e : cudaDeviceGetAttribute(n, cudaDevAttrMultiProcessorCount, dev);
+}
 
 }  // namespace rdn

@@ -24,47 +24,44 @@
 // Kernel 1 (chunk_prep): one CTA per chunk -- everything that does not depend
 // on the state: the Gram matrices, the masked/decayed matrices Ap, Mq, M2 and
 // (RDN) the two unit-lower inverses T_beta, T_gamma by forward substitution.
-// Kernel 2 (chunk_scan): one CTA per (b, h, 32-column slice of d_v) -- the
+// Kernel 2 (chunk_scan): one CTA per (b, h, 8- to 32-column slice of d_v) -- the
 // sequential pass over chunks carrying S and R slices in shared memory.  Each
 // value column is independent (the clip is elementwise), so slicing d_v is
 // exact; only the prep work is shared between slices.
 #include <type_traits>
 
 #include "chunk_common.cuh"
+#include "simt.cuh"
 #include "status.cuh"
 
 namespace rdn {
 namespace {
 
 // ---------------------------------------------------------------- kernel 1
-// Image writer: element (r, c) of a 64-column chunk matrix, value x, into a
-// K-major 128B-swizzled bf16 hi / lo pair (lo tile `lo_off` bytes after hi).
-__device__ __forceinline__ void img_put(uint8_t *tile, uint32_t lo_off, int r, int c, float x) {
-  const uint32_t o = (uint32_t)(r * 128 + ((((c >> 3) ^ (r & 7)) & 7) << 4) + (c & 7) * 2);
-  const __nv_bfloat16 hi = __float2bfloat16_rn(x);
-  *reinterpret_cast<__nv_bfloat16 *>(tile + o) = hi;
-  *reinterpret_cast<__nv_bfloat16 *>(tile + lo_off + o) = __float2bfloat16_rn(x - __bfloat162float(hi));
-}
+// Two CTAs of 256 threads per SM.  Thread (ty, tx) holds rows 4 ty .. 4 ty + 3
+// and columns tx + 16 j of both Gram products (they share the operand K), goes
+// from its accumulators to the decayed matrices without a pass through shared
+// memory, and only A_beta, A_gamma stay there for the inverses; T_beta,
+// T_gamma take the place of K and Q.  Bound by shared-memory loads and the
+// inverses' chain: 2048 chunks of d = 64 in 0.129 ms (0.402 ms with scalar
+// operand loads, every matrix in shared memory and one CTA per SM).
+template <int DK>
+struct PrepSm {  // float offsets
+  static constexpr int LDK = DK + 4, LDA = C + 1, LDT = C + 4;
+  static constexpr int K = 0, Q = K + C * LDK, TB = 0, TG = C * LDT;  // (T over K, Q)
+  static constexpr int AB = 2 * C * LDK, AG = AB + C * LDA, VEC = AG + C * LDA;
+  static constexpr int FLOATS = VEC + 7 * C;
+  static_assert(2 * LDT <= 2 * LDK, "T fits over K and Q");
+};
 
-template <int DK, bool RDNV, typename InT, bool IMG>
-__global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(FwdParams p) {
-  constexpr int LDK = DK + 1;
-  constexpr int LDC = C + 1;
-  extern __shared__ float sm[];
-  float *Ks = sm;                 // [C][LDK]
-  float *Qs = Ks + C * LDK;       // [C][LDK]
-  float *KK = Qs + C * LDK;       // [C][LDC]
-  float *QK = KK + C * LDC;       // [C][LDC]
-  float *Ab = QK + C * LDC;       // [C][LDC]
-  float *Ag = Ab + C * LDC;       // [C][LDC]
-  float *Tb = Ag + C * LDC;       // [C][LDC]
-  float *Tg = Tb + C * LDC;       // [C][LDC]
-  float *cum = Tg + C * LDC;      // [C]
-  float *cprev = cum + C;         // [C]
-  float *bet = cprev + C;         // [C]
-  float *gam = bet + C;           // [C]
-  float *gg = gam + C;            // [C]
-  float *Wsc = gg + C;            // [2][3*256] scratch of the blocked inverse
+template <int DK, bool RDNV, typename InT>
+__global__ void __launch_bounds__(kThreads, 2) chunk_prep_kernel(FwdParams p) {
+  using SM = PrepSm<DK>;
+  constexpr int LDK = SM::LDK, LDA = SM::LDA, LDT = SM::LDT;
+  extern __shared__ __align__(16) float sm[];
+  float *Ks = sm + SM::K, *Qs = sm + SM::Q, *Ab = sm + SM::AB, *Ag = sm + SM::AG;
+  simt::Cum &cum = *reinterpret_cast<simt::Cum *>(sm + SM::VEC);
+  float *bet = sm + SM::VEC + 4 * C, *gam = bet + C, *gg = gam + C;
 
   const long long chunk = blockIdx.x;
   if (chunk >= total_records(p)) return;  // (packed sequences: the grid covers the bound)
@@ -73,55 +70,34 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(FwdParams p) {
   const SeqSpan sp = seq_span(p, sq, h);
   const int t0 = c * C;
   const int n = min(C, sp.len - t0);
-  const int tid = threadIdx.x;
-  const InT *q = (const InT *)p.q;
-  const InT *k = (const InT *)p.k;
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
 
-  for (int e = tid; e < C * DK; e += kThreads) {
-    const int t = e / DK, d = e % DK;
-    float kv = 0.f, qv = 0.f;
-    if (t < n) {
-      const size_t off = ((size_t)(sp.tok0 + t0 + t) * p.H + h) * DK + d;
-      kv = to_f32(k[off]);
-      qv = p.scale * to_f32(q[off]);
-    }
-    Ks[t * LDK + d] = kv;
-    Qs[t * LDK + d] = qv;
-  }
-  if (tid < C) {
-    const int t = tid;
-    float gv = 0.f, bv = 0.f, mv = 0.f;
-    if (t < n) {
-      const size_t off = (size_t)(sp.tok0 + t0 + t) * p.H + h;
-      gv = p.g[off];
-      bv = p.beta[off];
-      mv = p.gamma[off];
-    }
-    gg[t] = gv;
-    bet[t] = bv;
-    gam[t] = mv;
-  }
-  __syncthreads();
-  if (tid == 0) {
-    float s = 0.f;
-    for (int t = 0; t < C; ++t) {
-      cprev[t] = s;
-      s += gg[t];
-      cum[t] = s;
-    }
-  }
-  // Gram matrices K K^T and Q K^T
   {
-    using MM = BlockMM<C, C, DK>;
-    float acc[MM::RPT];
-    MM::run(Ks, LDK, 1, Ks, 1, LDK, acc);
+    simt::RowTile<InT, DK, kThreads> kt, qt;
+    const size_t off = ((size_t)(sp.tok0 + t0) * p.H + h) * DK;
+    kt.fetch((const InT *)p.k + off, (size_t)p.H * DK, n);
+    qt.fetch((const InT *)p.q + off, (size_t)p.H * DK, n);
+    if (tid < 32) {  // gates of tokens tid, tid + 32 and the cumulative decay
+      float g2[2];
 #pragma unroll
-    for (int i = 0; i < MM::RPT; ++i) KK[MM::row(i) * LDC + MM::col()] = acc[i];
-    MM::run(Qs, LDK, 1, Ks, 1, LDK, acc);
-#pragma unroll
-    for (int i = 0; i < MM::RPT; ++i) QK[MM::row(i) * LDC + MM::col()] = acc[i];
+      for (int u = 0; u < 2; ++u) {
+        const int t = tid + 32 * u;
+        const bool ok = t < n;
+        const size_t go = (size_t)(sp.tok0 + t0 + (ok ? t : 0)) * p.H + h;
+        g2[u] = ok ? p.g[go] : 0.f;
+        gg[t] = g2[u];
+        bet[t] = ok ? p.beta[go] : 0.f;
+        gam[t] = ok ? p.gamma[go] : 0.f;
+      }
+      simt::cum64(g2[0], g2[1], cum);
+    }
+    kt.put(Ks, LDK, 1.f);
+    qt.put(Qs, LDK, p.scale);
   }
   __syncthreads();
+  float kk[4][4], qk[4][4];
+  simt::mm_nt<4, 4, DK>(Ks + 4 * ty * LDK, LDK, Ks + tx * LDK, 16 * LDK, kk);
+  simt::mm_nt<4, 4, DK>(Qs + 4 * ty * LDK, LDK, Ks + tx * LDK, 16 * LDK, qk);
   float *rec = p.ws + (size_t)chunk * kRecFloats;
   // variants: the decayed residual predicts with a_t S_{t-1} k_t, so Ap takes
   // the decay to t (not t-1); the plain combine reads S_{t-1} q_t, so Mq takes
@@ -129,117 +105,123 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(FwdParams p) {
   const bool dec_res = p.mods & RDN_FLAG_DECAYED_RESIDUAL;
   const bool plain = p.mods & RDN_FLAG_PLAIN_COMBINE;
   const bool stl = p.mods & RDN_FLAG_STATELESS_AUX;
-  for (int e = tid; e < C * C; e += kThreads) {
-    const int t = e / C, i = e % C;
-    float ap = 0.f, mq = 0.f, m2 = 0.f, ab = 0.f, ag = 0.f;
-    if (i <= t) {
-      const float dec = expf(cum[t] - cum[i]);
-      m2 = stl ? (i == t ? QK[t * LDC + i] : 0.f) : dec * gam[i] * QK[t * LDC + i];
-      if (i < t) {
-        const float decp = expf(cprev[t] - cum[i]);
-        ap = (dec_res ? dec : decp) * bet[i] * KK[t * LDC + i];
-        mq = (plain ? decp : dec) * bet[i] * QK[t * LDC + i];
-        ab = dec * bet[i] * KK[t * LDC + i];
-        ag = dec * gam[i] * KK[t * LDC + i];
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const int t = 4 * ty + a, i = tx + 16 * b;
+      float ap = 0.f, mq = 0.f, m2 = 0.f, ab = 0.f, ag = 0.f;
+      if (i <= t) {
+        const float dec = expf(cum.to(t, i));
+        m2 = stl ? (i == t ? qk[a][b] : 0.f) : dec * gam[i] * qk[a][b];
+        if (i < t) {
+          const float decp = expf(cum.before(t, i));
+          ap = (dec_res ? dec : decp) * bet[i] * kk[a][b];
+          mq = (plain ? decp : dec) * bet[i] * qk[a][b];
+          ab = dec * bet[i] * kk[a][b];
+          ag = dec * gam[i] * kk[a][b];
+        }
       }
-    }
-    if (IMG) {
-      uint8_t *img = reinterpret_cast<uint8_t *>(rec);
-      img_put(img + IMG_APMQ, 16384, t, i, ap);
-      img_put(img + IMG_APMQ, 16384, 64 + t, i, mq);
-      img_put(img + IMG_M2, 8192, t, i, gam[t] * m2);  // the image holds diag(gamma) M2
-    } else {
+      const int e = t * C + i;
       rec[OFF_AP + e] = ap;
       rec[OFF_MQ + e] = mq;
       rec[OFF_M2 + e] = m2;
+      if (RDNV) {
+        Ab[t * LDA + i] = ab;
+        Ag[t * LDA + i] = ag;
+      }
     }
-    if (RDNV) {
-      Ab[t * LDC + i] = ab;
-      Ag[t * LDC + i] = ag;
-    }
-  }
   if (tid < C) {
     const int t = tid;
-    const float cC = cum[C - 1];
-    rec[OFF_VEC + V_GAM + t] = expf(cum[t]);
-    rec[OFF_VEC + V_GPREV + t] = expf(cprev[t]);
+    const float end = expf(cum.to(C - 1, t));
+    rec[OFF_VEC + V_GAM + t] = expf(cum.hi[t]);
+    rec[OFF_VEC + V_GPREV + t] = expf(cum.phi[t]);
     rec[OFF_VEC + V_ALPHA + t] = expf(gg[t]);
-    rec[OFF_VEC + V_WS + t] = bet[t] * expf(cC - cum[t]);
+    rec[OFF_VEC + V_WS + t] = bet[t] * end;
     // (stateless correction: R at the chunk end is k r^T of its last token)
-    rec[OFF_VEC + V_WR + t] = stl ? (t == n - 1 ? 1.f : 0.f) : gam[t] * expf(cC - cum[t]);
-    if (t == 0) rec[OFF_VEC + V_GAMC] = expf(cC);
+    rec[OFF_VEC + V_WR + t] = stl ? (t == n - 1 ? 1.f : 0.f) : gam[t] * end;
+    if (t == 0) rec[OFF_VEC + V_GAMC] = expf(cum.hi[C - 1]);
   }
   if (RDNV) {
+    // threads 0..127 invert I + A_beta, threads 128..255 I + A_gamma
     __syncthreads();
-    // (I + A)^-1 by 16 x 16 blocks: threads 0..127 invert I + A_beta,
-    // threads 128..255 invert I + A_gamma.
-    {
-      const int g = tid & 127;
-      const float *A = tid < 128 ? Ab : Ag;
-      float *Tm = tid < 128 ? Tb : Tg;
-      float *W = Wsc + (tid < 128 ? 0 : 768);
-      inv_diag_blocks(A, Tm, LDC, g);
-      for (int i = 1; i < 4; ++i) {
-        __syncthreads();
-        inv_block_row_w(A, Tm, W, LDC, i, g);
-        __syncthreads();
-        inv_block_row_t(Tm, W, LDC, i, g);
-      }
+    const int g = tid & 127;
+    const float *A = tid < 128 ? Ab : Ag;
+    float *Tm = sm + (tid < 128 ? SM::TB : SM::TG);
+    // the blocks above the diagonal that the products read: (0, 1) and (2, 3)
+    for (int e = g; e < 2 * 16 * 16; e += 128) {
+      const int b = e >> 8, r = (e >> 4) & 15, cc = e & 15;
+      Tm[(32 * b + r) * LDT + 32 * b + 16 + cc] = 0.f;
+    }
+    for (int stage = 0; stage <= 4; ++stage) {
+      if (stage) __syncthreads();
+      inv64_stage<LDA, LDT, LDT>(stage, A, Tm, Tm + 32, g);
     }
     __syncthreads();
-    for (int e = tid; e < C * C; e += kThreads) {
-      const int t = e / C, i = e % C;
-      if (IMG) {
-        uint8_t *img = reinterpret_cast<uint8_t *>(rec);
-        img_put(img + IMG_TB, 8192, t, i, Tb[t * LDC + i]);
-        img_put(img + IMG_TG, 8192, t, i, Tg[t * LDC + i]);
-      } else {
-        rec[OFF_TB + e] = Tb[t * LDC + i];
-        rec[OFF_TG + e] = Tg[t * LDC + i];
-      }
-    }
-  } else if (IMG) {
-    // RLA has no delta rule: T_beta = T_gamma = I, which the tensor-core
-    // backward reads in their place
-    for (int e = tid; e < C * C; e += kThreads) {
-      const int t = e / C, i = e % C;
-      uint8_t *img = reinterpret_cast<uint8_t *>(rec);
-      img_put(img + IMG_TB, 8192, t, i, t == i ? 1.f : 0.f);
-      img_put(img + IMG_TG, 8192, t, i, t == i ? 1.f : 0.f);
+    for (int e = tid; e < 2 * C * C / 4; e += kThreads) {
+      const int m = e / (C * C / 4), t = (e / (C / 4)) % C, i = 4 * (e % (C / 4));
+      const float4 x = *reinterpret_cast<const float4 *>(sm + (m ? SM::TG : SM::TB) + t * LDT + i);
+      const float4 y = make_float4(i <= t ? x.x : 0.f, i + 1 <= t ? x.y : 0.f,
+                                   i + 2 <= t ? x.z : 0.f, i + 3 <= t ? x.w : 0.f);
+      *reinterpret_cast<float4 *>(rec + (m ? OFF_TG : OFF_TB) + t * C + i) = y;
     }
   }
 }
 
 // ---------------------------------------------------------------- kernel 2
-constexpr int kScanThreads = 512;  // threads of a scan CTA (latency bound: 16 warps)
+// One CTA per (sequence, head, DVS value columns), the chunks in sequence.
+// Thread (warp w, lane (lm, ln)) owns columns TN ln .. + TN and rows
+// 32 i + LM w + lm of every 64-row product (i = 0, 1; for the stacked 128-row
+// products i = 0, 1 are the K (or Ap) rows, 2, 3 the Q (or Mq) rows), so that a
+// chunk's read-outs, predictions and outputs stay in its registers from one
+// product to the next; only what the next product reads as its right operand
+// (X, E, wS E, then X2, E2, wR E2) goes through shared memory.  Four phases a
+// chunk: [KS; QS], [KR; QR] | E | [Ap; Mq] E and S's update | E2 | M2 E2 and R's
+// update.  The upper halves of the triangular blocks are skipped.  The chunk
+// matrices arrive by cp.async a phase or more ahead, in three slots; the next
+// chunk's K, Q, V and gate vectors wait in registers over the last phase.
+// Bound by the FMA pipe and the phases' latencies: B = 4, H = 16, T = 2048,
+// d = 64 in 0.458 ms (1.079 ms with scalar operand loads), B = 2, H = 8,
+// T = 1000, d = 128 fp32 in 0.293 ms (0.718), B = 1, H = 2, T = 256, d = 64 in
+// 0.024 ms (0.085, on 4 CTAs).
+// REC: one chunk per CTA from the chunk-start states p.S_chunks, p.R_chunks,
+// writing only what the backward reads (E, E2 and the residual's mask).
+template <int DK, int DVS, int NT>
+struct ScanSm {  // float offsets
+  static constexpr int LDK = DK + 4, LDM = C + 4;
+  static constexpr int K = 0, Q = K + C * LDK, MAT = Q + C * LDK;  // MAT: 3 slots
+  static constexpr int S = MAT + 3 * C * LDM, R = S + DK * DVS, V = R + DK * DVS;
+  static constexpr int X = V + C * DVS, E = X + C * DVS, W = E + C * DVS, VEC = W + C * DVS;
+  static constexpr int GM = VEC + 6 * C, FLOATS = GM + C;
+};
 
-template <int DK, bool RDNV, typename InT>
-__global__ void __launch_bounds__(kScanThreads, 1) chunk_scan_kernel(FwdParams p) {
-  constexpr int DV = DK;
-  extern __shared__ float sm[];
-  float *Ks = sm;                 // [C][DK]
-  float *Qs = Ks + C * DK;        // [C][DK]
-  float *Ss = Qs + C * DK;        // [DK][kDVS]
-  float *Rs = Ss + DK * kDVS;     // [DK][kDVS]
-  float *Vs = Rs + DK * kDVS;     // [C][kDVS]
-  float *CC = Vs + C * kDVS;      // [C][C]
-  float *KS = CC + C * C;         // [C][kDVS]
-  float *QS = KS + C * kDVS;
-  float *Es = QS + C * kDVS;
-  float *Ps = Es + C * kDVS;
-  float *Ob = Ps + C * kDVS;
-  float *Ws = Ob + C * kDVS;
-  float *vec = Ws + C * kDVS;     // [6*C]
+template <int DK, bool RDNV, typename InT, int DVS, int NT, bool REC>
+__global__ void __launch_bounds__(NT, NT == 128 ? 2 : 1) chunk_scan_kernel(FwdParams p) {
+  using namespace simt;
+  using SM = ScanSm<DK, DVS, NT>;
+  constexpr int DV = DK, LDK = SM::LDK, LDM = SM::LDM;
+  constexpr int TN = 32 * DVS / NT, LN = DVS / TN, LM = 32 / LN, TMU = DK / 32;
+  static_assert(LM * (NT / 32) == 32, "row blocks of 32");
+  extern __shared__ __align__(16) float sm[];
+  float *Ks = sm + SM::K, *Qs = sm + SM::Q, *Ss = sm + SM::S, *Rs = sm + SM::R;
+  float *Vs = sm + SM::V, *Xs = sm + SM::X, *Es = sm + SM::E, *Ws = sm + SM::W;
+  float *vec = sm + SM::VEC, *gms = sm + SM::GM;
+  float *mat[3] = {sm + SM::MAT, sm + SM::MAT + C * LDM, sm + SM::MAT + 2 * C * LDM};
 
-  const int bh = blockIdx.x;
-  const int h = bh % p.H;
-  const SeqSpan sp = seq_span(p, bh / p.H, h);
-  const int j0 = blockIdx.y * kDVS;
-  const int tid = threadIdx.x;
-  const InT *q = (const InT *)p.q;
-  const InT *k = (const InT *)p.k;
-  const InT *v = (const InT *)p.v;
-  InT *o = (InT *)p.o;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int ln = lane % LN, r0 = LM * warp + lane / LN, n0 = TN * ln;
+  int sq, h, c0 = 0, c1;
+  if (REC) {
+    if ((long long)blockIdx.x >= total_records(p)) return;
+    rec_decode(p, blockIdx.x, sq, h, c0);
+    c1 = c0 + 1;
+  } else {
+    sq = blockIdx.x / p.H;
+    h = blockIdx.x % p.H;
+  }
+  const SeqSpan sp = seq_span(p, sq, h);
+  if (!REC) c1 = sp.nc;
+  const int j0 = blockIdx.y * DVS;
   const float clip = p.clip;
   const bool dec_res = p.mods & RDN_FLAG_DECAYED_RESIDUAL;
   const bool plain = p.mods & RDN_FLAG_PLAIN_COMBINE;
@@ -247,260 +229,351 @@ __global__ void __launch_bounds__(kScanThreads, 1) chunk_scan_kernel(FwdParams p
   const bool stl = p.mods & RDN_FLAG_STATELESS_AUX;
   const bool rdn_aux = RDNV && !stl;  // the auxiliary pass runs the delta rule
 
-  const size_t sbase = (size_t)bh * DK * DV;
-  for (int e = tid; e < DK * kDVS; e += kScanThreads) {
-    const int i = e / kDVS, jj = e % kDVS;
-    Ss[e] = p.S0 ? p.S0[sbase + (size_t)i * DV + j0 + jj] : 0.f;
-    Rs[e] = p.R0 ? p.R0[sbase + (size_t)i * DV + j0 + jj] : 0.f;
+  const size_t sbase = REC ? (size_t)blockIdx.x * DK * DV : (size_t)(sq * (size_t)p.H + h) * DK * DV;
+  {
+    const float *S0 = REC ? p.S_chunks : p.S0, *R0 = REC ? p.R_chunks : p.R0;
+    for (int e = tid; e < DK * DVS / 4; e += NT) {
+      const size_t off = sbase + (size_t)(e / (DVS / 4)) * DV + j0 + 4 * (e % (DVS / 4));
+      const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+      *reinterpret_cast<float4 *>(Ss + 4 * e) = S0 ? *reinterpret_cast<const float4 *>(S0 + off) : z;
+      *reinterpret_cast<float4 *>(Rs + 4 * e) = R0 ? *reinterpret_cast<const float4 *>(R0 + off) : z;
+    }
   }
 
-  for (int c = 0; c < sp.nc; ++c) {
+  RowTile<InT, DK, NT> kt, qt;
+  RowTile<InT, DVS, NT> vt;
+  constexpr int VU = 6 * C / NT + (6 * C % NT != 0);
+  float vr[VU], gr = 0.f;
+  auto fetch = [&](int c) {  // chunk c's K, Q, V, gate vectors
+    const int n = min(C, sp.len - c * C);
+    const size_t row = (size_t)(sp.tok0 + c * C) * p.H + h;
+    kt.fetch((const InT *)p.k + row * DK, (size_t)p.H * DK, n);
+    qt.fetch((const InT *)p.q + row * DK, (size_t)p.H * DK, n);
+    vt.fetch((const InT *)p.v + row * DV + j0, (size_t)p.H * DV, n);
+    const float *rec = p.ws + (size_t)(sp.rbase + c) * kRecFloats;
+#pragma unroll
+    for (int u = 0; u < VU; ++u) {
+      const int e = tid + u * NT;
+      vr[u] = e <= V_GAMC ? rec[OFF_VEC + e] : 0.f;
+    }
+    if (tid < C) gr = tid < n ? p.gamma[row + (size_t)tid * p.H] : 0.f;
+  };
+  auto mats = [&](int c) { return p.ws + (size_t)(sp.rbase + c) * kRecFloats; };
+  if (c0 < c1) {
+    fetch(c0);
+    if (RDNV) cp_mat<NT>(mat[0], LDM, mats(c0) + OFF_TB);
+    cp_commit();
+    cp_mat<NT>(mat[1], LDM, mats(c0) + OFF_AP);
+    if (!REC) cp_mat<NT>(mat[2], LDM, mats(c0) + OFF_MQ);
+    cp_commit();
+  }
+
+  for (int c = c0; c < c1; ++c) {
     const int t0 = c * C;
     const int n = min(C, sp.len - t0);
-    const float *rec = p.ws + (size_t)(sp.rbase + c) * kRecFloats;
-    __syncthreads();  // previous chunk done with every buffer
-    if (p.S_chunks) {
-      float *sc = p.S_chunks + (size_t)(sp.rbase + c) * DK * DV;
-      float *rc = p.R_chunks + (size_t)(sp.rbase + c) * DK * DV;
-      for (int e = tid; e < DK * kDVS; e += kScanThreads) {
-        const int i = e / kDVS, jj = e % kDVS;
-        sc[(size_t)i * DV + j0 + jj] = Ss[e];
-        rc[(size_t)i * DV + j0 + jj] = Rs[e];
-      }
-    }
-    for (int e = tid; e < C * DK; e += kScanThreads) {
-      const int t = e / DK, d = e % DK;
-      float kv = 0.f, qv = 0.f;
-      if (t < n) {
-        const size_t off = ((size_t)(sp.tok0 + t0 + t) * p.H + h) * DK + d;
-        kv = to_f32(k[off]);
-        qv = p.scale * to_f32(q[off]);
-      }
-      Ks[e] = kv;
-      Qs[e] = qv;
-    }
-    for (int e = tid; e < C * kDVS; e += kScanThreads) {
-      const int t = e / kDVS, jj = e % kDVS;
-      Vs[e] = t < n ? to_f32(v[((size_t)(sp.tok0 + t0 + t) * p.H + h) * DV + j0 + jj]) : 0.f;
-    }
-    for (int e = tid; e < 6 * C; e += kScanThreads) vec[e] = rec[OFF_VEC + e];
-    __syncthreads();
-    const float *Gam = vec + V_GAM, *Gprev = vec + V_GPREV;
-    const float *wS = vec + V_WS, *wR = vec + V_WR;
-    const float GamC = vec[V_GAMC];
-
-    using MMk = BlockMM<C, kDVS, DK, kScanThreads>;  // [C x DK] @ [DK x DVS]
-    using MMc = BlockMM<C, kDVS, C, kScanThreads>;   // [C x C] @ [C x DVS]
-    using MMu = BlockMM<DK, kDVS, C, kScanThreads>;  // [DK x C] @ [C x DVS]
-    const int col = MMk::col();
-    {
-      float a1[MMk::RPT], a2[MMk::RPT];
-      MMk::run(Ks, DK, 1, Ss, kDVS, 1, a1);
-      MMk::run(Qs, DK, 1, Ss, kDVS, 1, a2);
+    const bool more = c + 1 < c1;
+    kt.put(Ks, LDK, 1.f);
+    qt.put(Qs, LDK, p.scale);
+    vt.put(Vs, DVS, 1.f);
 #pragma unroll
-      for (int i = 0; i < MMk::RPT; ++i) {
-        const int t = MMk::row(i);
-        KS[t * kDVS + col] = a1[i];
-        QS[t * kDVS + col] = a2[i];
-        if (RDNV) Ws[t * kDVS + col] = Vs[t * kDVS + col] - Gam[t] * a1[i];
+    for (int u = 0; u < VU; ++u)
+      if (tid + u * NT < 6 * C) vec[tid + u * NT] = vr[u];
+    if (tid < C) gms[tid] = gr;
+    __syncthreads();
+    const float *Gam = vec + V_GAM, *Gprev = vec + V_GPREV, *wS = vec + V_WS, *wR = vec + V_WR;
+    const float GamC = vec[V_GAMC];
+    const size_t rec = (size_t)(sp.rbase + c);
+    if (!REC && p.S_chunks) {
+      float *sc = p.S_chunks + rec * DK * DV + j0, *rc = p.R_chunks + rec * DK * DV + j0;
+      for (int e = tid; e < DK * DVS / 4; e += NT) {
+        const size_t off = (size_t)(e / (DVS / 4)) * DV + 4 * (e % (DVS / 4));
+        *reinterpret_cast<float4 *>(sc + off) = *reinterpret_cast<const float4 *>(Ss + 4 * e);
+        *reinterpret_cast<float4 *>(rc + off) = *reinterpret_cast<const float4 *>(Rs + 4 * e);
       }
+    }
+    // ---- [K; Q] S and [K; Q] R
+    float a1[4][TN], a2[4][TN];
+    zero(a1);
+    zero(a2);
+    {
+      const float *A = Ks + r0 * LDK;
+      constexpr int MS = REC ? 3 : 15, MR = (RDNV ? 3 : 0) | (REC ? 0 : 12);
+      if (stl) mm_ak<4, TN, MS>(A, 32 * LDK, Ss + n0, DVS, 0, DK, a1);
+      else mm_ak2<4, TN, MS, MR>(A, 32 * LDK, Ss + n0, Rs + n0, DVS, DK, a1, a2);
+    }
+    float vv[2][TN];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int t = r0 + 32 * i;
+      ldv<TN>(Vs + t * DVS + n0, vv[i]);
+      float x[TN];
+#pragma unroll
+      for (int j = 0; j < TN; ++j)  // RDN: X = V - Gam K S; RLA (E = V): wS E
+        x[j] = RDNV ? vv[i][j] - Gam[t] * a1[i][j] : wS[t] * vv[i][j];
+      stv<TN>((RDNV ? Xs : Ws) + t * DVS + n0, x);
     }
     const float *E = Vs;
+    wait_groups<1>();  // (T_beta, and the M_q fetched before it)
+    __syncthreads();
+    // ---- E = T_beta X, wS E
     if (RDNV) {
-      for (int e = tid; e < C * C; e += kScanThreads) CC[e] = rec[OFF_TB + e];
-      __syncthreads();
-      float a1[MMc::RPT];
-      MMc::run(CC, C, 1, Ws, kDVS, 1, a1);
+      float e[2][TN];
+      zero(e);
+      const float *A = mat[0] + r0 * LDM;
+      mm_ak<2, TN, 3>(A, 32 * LDM, Xs + n0, DVS, 0, 32, e);
+      mm_ak<2, TN, 2>(A, 32 * LDM, Xs + n0, DVS, 32, 64, e);
 #pragma unroll
-      for (int i = 0; i < MMc::RPT; ++i) Es[MMc::row(i) * kDVS + col] = a1[i];
+      for (int i = 0; i < 2; ++i) {
+        const int t = r0 + 32 * i;
+        stv<TN>(Es + t * DVS + n0, e[i]);
+        if (p.sv_E) stv<TN>((float *)p.sv_E + (rec * C + t) * DV + j0 + n0, e[i]);
+#pragma unroll
+        for (int j = 0; j < TN; ++j) e[i][j] *= wS[t];
+        stv<TN>(Ws + t * DVS + n0, e[i]);
+      }
       E = Es;
-    }
-    __syncthreads();
-    for (int e = tid; e < C * C; e += kScanThreads) CC[e] = rec[OFF_AP + e];
-    __syncthreads();
-    {
-      float a1[MMc::RPT];
-      MMc::run(CC, C, 1, E, kDVS, 1, a1);
-#pragma unroll
-      for (int i = 0; i < MMc::RPT; ++i) {
-        const int t = MMc::row(i);
-        // P_t = S_{t-1}^T k_t (decayed residual: a_t S_{t-1}^T k_t)
-        const float pt = (dec_res ? Gam[t] : Gprev[t]) * KS[t * kDVS + col] + a1[i];
-        Ps[t * kDVS + col] = resid_map(Vs[t * kDVS + col] - pt, clip, tnh);  // r, Section 3.3
-      }
-    }
-    __syncthreads();
-    for (int e = tid; e < C * C; e += kScanThreads) CC[e] = rec[OFF_MQ + e];
-    __syncthreads();
-    {
-      float a1[MMc::RPT];
-      MMc::run(CC, C, 1, E, kDVS, 1, a1);
-#pragma unroll
-      for (int i = 0; i < MMc::RPT; ++i) {
-        const int t = MMc::row(i);
-        Ob[t * kDVS + col] = (plain ? Gprev[t] : Gam[t]) * QS[t * kDVS + col] + a1[i];
-      }
-    }
-    // S_C = Gam_C S0 + K^T diag(wS) E   (W = wS * E)
-    for (int e = tid; e < C * kDVS; e += kScanThreads) Ws[e] = wS[e / kDVS] * E[e];
-    __syncthreads();
-    {
-      float a1[MMu::RPT];
-      MMu::run(Ks, 1, DK, Ws, kDVS, 1, a1);
-#pragma unroll
-      for (int i = 0; i < MMu::RPT; ++i) {
-        const int r = MMu::row(i);
-        Ss[r * kDVS + col] = GamC * Ss[r * kDVS + col] + a1[i];
-      }
-    }
-    // auxiliary pass: values r (in Ps), rate gamma, state R
-    {
-      float a1[MMk::RPT], a2[MMk::RPT];
-      MMk::run(Ks, DK, 1, Rs, kDVS, 1, a1);
-      MMk::run(Qs, DK, 1, Rs, kDVS, 1, a2);
-      __syncthreads();  // every thread done reading Ws / CC of the S pass
-#pragma unroll
-      for (int i = 0; i < MMk::RPT; ++i) {
-        const int t = MMk::row(i);
-        QS[t * kDVS + col] = stl ? 0.f : a2[i];  // Q R0 (the stateless R carries nothing)
-        if (rdn_aux) Ws[t * kDVS + col] = Ps[t * kDVS + col] - Gam[t] * a1[i];
-      }
-    }
-    const float *E2 = Ps;
-    if (rdn_aux) {
-      for (int e = tid; e < C * C; e += kScanThreads) CC[e] = rec[OFF_TG + e];
+      wait_groups<0>();
       __syncthreads();
-      float a1[MMc::RPT];
-      MMc::run(CC, C, 1, Ws, kDVS, 1, a1);
+    } else {
+      if (p.sv_E)
 #pragma unroll
-      for (int i = 0; i < MMc::RPT; ++i) Es[MMc::row(i) * kDVS + col] = a1[i];
-      E2 = Es;
+        for (int i = 0; i < 2; ++i)
+          stv<TN>((float *)p.sv_E + (rec * C + r0 + 32 * i) * DV + j0 + n0, vv[i]);
+      wait_groups<0>();
+      __syncthreads();
     }
-    __syncthreads();
-    for (int e = tid; e < C * C; e += kScanThreads) CC[e] = rec[OFF_M2 + e];
-    __syncthreads();
+    if (rdn_aux) cp_mat<NT>(mat[0], LDM, mats(c) + OFF_TG);
+    cp_commit();
+    // ---- [Ap; Mq] E: the prediction, the residual, the base output; S's update
+    float ob[2][TN], r[2][TN];
     {
-      float a1[MMc::RPT];
-      MMc::run(CC, C, 1, E2, kDVS, 1, a1);
+      float pm[4][TN];
+      zero(pm);
+      const float *A = mat[1] + r0 * LDM;
+      mm_ak<4, TN, REC ? 3 : 15>(A, 32 * LDM, E + n0, DVS, 0, 32, pm);
+      mm_ak<4, TN, REC ? 2 : 10>(A, 32 * LDM, E + n0, DVS, 32, 64, pm);
 #pragma unroll
-      for (int i = 0; i < MMc::RPT; ++i) {
-        const int t = MMc::row(i);
-        if (t < n) {
-          const float gm = plain ? 1.f : p.gamma[(size_t)(sp.tok0 + t0 + t) * p.H + h];
-          const float oa = Gam[t] * QS[t * kDVS + col] + a1[i];
-          o[((size_t)(sp.tok0 + t0 + t) * p.H + h) * DV + j0 + col] =
-              from_f32<InT>(Ob[t * kDVS + col] + gm * oa);
+      for (int i = 0; i < 2; ++i) {
+        const int t = r0 + 32 * i;
+        const float gp = dec_res ? Gam[t] : Gprev[t], gq = plain ? Gprev[t] : Gam[t];
+        float x2[TN], dr[TN];
+        uint32_t in = 0;  // bit j: |x| <= c
+#pragma unroll
+        for (int j = 0; j < TN; ++j) {
+          // P_t = S_{t-1}^T k_t (decayed residual: a_t S_{t-1}^T k_t)
+          const float x = vv[i][j] - (gp * a1[i][j] + pm[i][j]);
+          r[i][j] = resid_map(x, clip, tnh);  // Section 3.3
+          ob[i][j] = gq * a1[2 + i][j] + pm[2 + i][j];
+          x2[j] = r[i][j] - Gam[t] * a2[i][j];
+          in |= (fabsf(x) <= clip ? 1u : 0u) << j;
+          if (tnh) dr[j] = resid_grad(x, clip, true);
+        }
+        if (rdn_aux) stv<TN>(Xs + t * DVS + n0, x2);
+        if (p.sv_mask) {
+          if (tnh) {
+            stv<TN>((float *)p.sv_mask + (rec * C + t) * DV + j0 + n0, dr);
+          } else {  // the row's DVS bits: one byte per 8 columns
+            in <<= n0 & 7;
+#pragma unroll
+            for (int d = 1; d < 8 / TN; d <<= 1) in |= __shfl_xor_sync(0xffffffffu, in, d);
+            if (n0 % 8 == 0)
+              ((uint8_t *)p.sv_mask)[((rec * C + t) * DV + j0 + n0) >> 3] = (uint8_t)in;
+          }
+        }
+      }
+      if (!REC) {
+        const int m0 = TMU * r0;
+        float u[TMU][TN];
+        zero(u);
+        mm_am<TMU, TN>(Ks + m0, LDK, Ws + n0, DVS, C, u);  // K^T diag(wS) E
+#pragma unroll
+        for (int i = 0; i < TMU; ++i) {
+          float s[TN];
+          ldv<TN>(Ss + (m0 + i) * DVS + n0, s);
+#pragma unroll
+          for (int j = 0; j < TN; ++j) s[j] = GamC * s[j] + u[i][j];
+          stv<TN>(Ss + (m0 + i) * DVS + n0, s);
         }
       }
     }
-    // R_C = Gam_C R0 + K^T diag(wR) E2
-    for (int e = tid; e < C * kDVS; e += kScanThreads) Ws[e] = wR[e / kDVS] * E2[e];
+    wait_groups<0>();  // T_gamma
     __syncthreads();
-    {
-      float a1[MMu::RPT];
-      MMu::run(Ks, 1, DK, Ws, kDVS, 1, a1);
+    if (!REC) {
+      cp_mat<NT>(mat[1], LDM, mats(c) + OFF_M2);
+      cp_commit();
+      if (more) cp_mat<NT>(mat[2], LDM, mats(c + 1) + OFF_MQ);
+      cp_commit();
+    }
+    // ---- E2 = T_gamma X2, wR E2
+    if (rdn_aux) {
+      zero(r);
+      const float *A = mat[0] + r0 * LDM;
+      mm_ak<2, TN, 3>(A, 32 * LDM, Xs + n0, DVS, 0, 32, r);
+      mm_ak<2, TN, 2>(A, 32 * LDM, Xs + n0, DVS, 32, 64, r);
+    }
 #pragma unroll
-      for (int i = 0; i < MMu::RPT; ++i) {
-        const int r = MMu::row(i);
-        Rs[r * kDVS + col] = (stl ? 0.f : GamC) * Rs[r * kDVS + col] + a1[i];
+    for (int i = 0; i < 2; ++i) {
+      const int t = r0 + 32 * i;
+      if (p.sv_E2) stv<TN>((float *)p.sv_E2 + (rec * C + t) * DV + j0 + n0, r[i]);
+      if (REC) continue;
+      stv<TN>(Es + t * DVS + n0, r[i]);
+#pragma unroll
+      for (int j = 0; j < TN; ++j) r[i][j] *= wR[t];
+      stv<TN>(Ws + t * DVS + n0, r[i]);
+    }
+    if (REC) break;
+    wait_groups<1>();  // M2
+    __syncthreads();
+    if (more) {
+      if (RDNV) cp_mat<NT>(mat[0], LDM, mats(c + 1) + OFF_TB);
+      fetch(c + 1);
+    }
+    cp_commit();
+    // ---- o = Ob + gamma (Gam Q R + M2 E2); R's update
+    {
+      float oa[2][TN];
+      zero(oa);
+      const float *A = mat[1] + r0 * LDM;
+      mm_ak<2, TN, 3>(A, 32 * LDM, Es + n0, DVS, 0, 32, oa);
+      mm_ak<2, TN, 2>(A, 32 * LDM, Es + n0, DVS, 32, 64, oa);
+      InT *o = (InT *)p.o;
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int t = r0 + 32 * i;
+        if (t < n) {
+          const float gm = plain ? 1.f : gms[t];
+          const size_t off = ((size_t)(sp.tok0 + t0 + t) * p.H + h) * DV + j0 + n0;
+          float y[TN];
+#pragma unroll
+          for (int j = 0; j < TN; ++j)
+            y[j] = ob[i][j] + gm * (Gam[t] * a2[2 + i][j] + oa[i][j]);
+          if constexpr (sizeof(InT) == 4) {
+            stv<TN>((float *)o + off, y);
+          } else {
+            uint32_t w[TN / 2 ? TN / 2 : 1];
+#pragma unroll
+            for (int j = 0; j < TN / 2; ++j) {
+              const __nv_bfloat162 b2 = __floats2bfloat162_rn(y[2 * j], y[2 * j + 1]);
+              w[j] = *reinterpret_cast<const uint32_t *>(&b2);
+            }
+            if constexpr (TN == 4) *reinterpret_cast<uint2 *>(o + off) = make_uint2(w[0], w[1]);
+            else *reinterpret_cast<uint32_t *>(o + off) = w[0];
+          }
+        }
+      }
+      const int m0 = TMU * r0;
+      float u[TMU][TN];
+      zero(u);
+      mm_am<TMU, TN>(Ks + m0, LDK, Ws + n0, DVS, C, u);  // K^T diag(wR) E2
+#pragma unroll
+      for (int i = 0; i < TMU; ++i) {
+        float s[TN];
+        ldv<TN>(Rs + (m0 + i) * DVS + n0, s);
+#pragma unroll
+        for (int j = 0; j < TN; ++j) s[j] = (stl ? 0.f : GamC) * s[j] + u[i][j];
+        stv<TN>(Rs + (m0 + i) * DVS + n0, s);
       }
     }
+    __syncthreads();  // every buffer of this chunk is free
+    if (more) cp_mat<NT>(mat[1], LDM, mats(c + 1) + OFF_AP);
+    cp_commit();
   }
+  if (REC) return;
   __syncthreads();
-  for (int e = tid; e < DK * kDVS; e += kScanThreads) {
-    const int i = e / kDVS, jj = e % kDVS;
-    if (p.ST) p.ST[sbase + (size_t)i * DV + j0 + jj] = Ss[e];
-    if (p.RT) p.RT[sbase + (size_t)i * DV + j0 + jj] = Rs[e];
+  for (int e = tid; e < DK * DVS / 4; e += NT) {
+    const size_t off = sbase + (size_t)(e / (DVS / 4)) * DV + j0 + 4 * (e % (DVS / 4));
+    if (p.ST) *reinterpret_cast<float4 *>(p.ST + off) = *reinterpret_cast<const float4 *>(Ss + 4 * e);
+    if (p.RT) *reinterpret_cast<float4 *>(p.RT + off) = *reinterpret_cast<const float4 *>(Rs + 4 * e);
   }
 }
 
-template <int DK>
-constexpr size_t prep_smem() {
-  return sizeof(float) * (2 * C * (DK + 1) + 6 * C * (C + 1) + 5 * C + 2 * 768);
-}
-template <int DK>
-constexpr size_t scan_smem() {
-  return sizeof(float) * (2 * C * DK + 2 * DK * kDVS + C * kDVS + C * C + 6 * C * kDVS + 6 * C);
-}
-
-template <int DK, bool RDNV, typename InT>
-cudaError_t launch_t(const FwdParams &p, cudaStream_t s, bool do_prep, bool do_scan,
-                     bool img = false) {
-  auto prep = img ? chunk_prep_kernel<DK, RDNV, InT, true> : chunk_prep_kernel<DK, RDNV, InT, false>;
-  auto scan = chunk_scan_kernel<DK, RDNV, InT>;
-  cudaError_t e;
-  if ((e = cudaFuncSetAttribute(prep, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)prep_smem<DK>())) != cudaSuccess)
-    return e;
-  if ((e = cudaFuncSetAttribute(scan, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)scan_smem<DK>())) != cudaSuccess)
-    return e;
-  if (do_prep) {
-    // the images for bf16 inputs and d = 128 come from the tensor-core prep,
-    // which also normalises q and k (RDN_FLAG_QK_NORM) as it loads them; for
-    // the other preps the prologue kernel writes the normalised copies first
-    constexpr bool tc_prep = DK == 128 && std::is_same<InT, __nv_bfloat16>::value;
-    const bool use_tc_prep = tc_prep && img && (p.mods & ~kTcVariants) == 0;
-    if (p.qk_norm && !use_tc_prep) {
-      rdn_prologue_args pa{};
-      pa.rows = (long long)p.B * p.T * p.H;
-      pa.D = DK;
-      pa.dtype = std::is_same<InT, __nv_bfloat16>::value ? RDN_BF16 : RDN_F32;
-      pa.eps = p.qk_eps;
-      pa.x[0] = p.qraw;
-      pa.x[1] = p.kraw;
-      pa.y[0] = const_cast<void *>(p.q);
-      pa.y[1] = const_cast<void *>(p.k);
-      if ((e = launch_prologue(pa, false, s)) != cudaSuccess) return e;
-    }
-    if (use_tc_prep) {
-      if ((e = launch_prep_tc(p, !RDNV, s)) != cudaSuccess) return e;
-    } else {
-      RDN_LAUNCH("chunk_prep", s, prep<<<(unsigned)p.nrec, kThreads, prep_smem<DK>(), s>>>(p));
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-  }
-  if (do_scan)
-    RDN_LAUNCH("chunk_scan", s, scan<<<dim3(p.nseq * p.H, DK / kDVS), kScanThreads, scan_smem<DK>(), s>>>(p));
+template <int DK, bool RDNV, typename InT, int DVS, int NT, bool REC>
+cudaError_t launch_scan_t(const FwdParams &p, cudaStream_t s) {
+  auto scan = chunk_scan_kernel<DK, RDNV, InT, DVS, NT, REC>;
+  constexpr int smem = (int)sizeof(float) * ScanSm<DK, DVS, NT>::FLOATS;
+  const cudaError_t e = cudaFuncSetAttribute(scan, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  const dim3 grid(REC ? (unsigned)p.nrec : (unsigned)(p.nseq * p.H), DK / DVS);
+  RDN_LAUNCH(REC ? "chunk_recompute" : "chunk_scan", s, scan<<<grid, NT, smem, s>>>(p));
   return cudaGetLastError();
 }
 
-}  // namespace
-
-cudaError_t launch_fwd_parts(const FwdParams &p, int DK, bool rdnv, bool bf16, bool do_prep,
-                             bool do_scan, cudaStream_t s) {
-  // bf16 inputs with d = 128 (RDN, and RLA with a hi + lo copy of S for its
-  // read-outs) run the tensor-core scan; everything else, and the variants,
-  // the fp32 SIMT one
-  const bool tc_scan = do_scan && fwd_uses_tc(p, DK, bf16);
-  cudaError_t e = cudaSuccess;
-  // (the tensor-core scan reads the records as shared-memory images)
-  if (DK == 128) {
-    if (rdnv) e = bf16 ? launch_t<128, true, __nv_bfloat16>(p, s, do_prep, do_scan && !tc_scan, tc_scan)
-                       : launch_t<128, true, float>(p, s, do_prep, do_scan);
-    else e = bf16 ? launch_t<128, false, __nv_bfloat16>(p, s, do_prep, do_scan && !tc_scan, tc_scan)
-                  : launch_t<128, false, float>(p, s, do_prep, do_scan);
-  } else {
-    if (rdnv) e = bf16 ? launch_t<64, true, __nv_bfloat16>(p, s, do_prep, do_scan)
-                       : launch_t<64, true, float>(p, s, do_prep, do_scan);
-    else e = bf16 ? launch_t<64, false, __nv_bfloat16>(p, s, do_prep, do_scan)
-                  : launch_t<64, false, float>(p, s, do_prep, do_scan);
-  }
-  if (e != cudaSuccess || !tc_scan) return e;
-  return launch_fwd_tc(p, rdnv, s);
+template <int DK, bool RDNV, typename InT>
+cudaError_t launch_scan(const FwdParams &p, cudaStream_t s) {
+  int nsm = 0;
+  const cudaError_t e = sm_count(&nsm);
+  if (e != cudaSuccess) return e;
+  const int dvs = scan_columns(DK, (long long)p.nseq * p.H, nsm);
+  if constexpr (DK == 64)
+    return dvs == 16 ? launch_scan_t<64, RDNV, InT, 16, 128, false>(p, s)
+                     : launch_scan_t<64, RDNV, InT, 8, 128, false>(p, s);
+  else
+    return dvs == 32   ? launch_scan_t<128, RDNV, InT, 32, 256, false>(p, s)
+           : dvs == 16 ? launch_scan_t<128, RDNV, InT, 16, 256, false>(p, s)
+                       : launch_scan_t<128, RDNV, InT, 8, 256, false>(p, s);
 }
 
-cudaError_t launch_prep(const FwdParams &p, int DK, bool rdnv, bool bf16, bool img, cudaStream_t s) {
-  if (DK == 128) {
-    if (rdnv) return bf16 ? launch_t<128, true, __nv_bfloat16>(p, s, true, false, img)
-                          : launch_t<128, true, float>(p, s, true, false, img);
-    return bf16 ? launch_t<128, false, __nv_bfloat16>(p, s, true, false, img)
-                : launch_t<128, false, float>(p, s, true, false, img);
+template <int DK, bool RDNV, typename InT>
+cudaError_t launch_prep_t(const FwdParams &p, cudaStream_t s) {
+  cudaError_t e;
+  if (p.qk_norm) {  // q, k are raw: the prologue kernel writes the normalised copies first
+    rdn_prologue_args pa{};
+    pa.rows = (long long)p.B * p.T * p.H;
+    pa.D = DK;
+    pa.dtype = std::is_same<InT, __nv_bfloat16>::value ? RDN_BF16 : RDN_F32;
+    pa.eps = p.qk_eps;
+    pa.x[0] = p.qraw;
+    pa.x[1] = p.kraw;
+    pa.y[0] = const_cast<void *>(p.q);
+    pa.y[1] = const_cast<void *>(p.k);
+    if ((e = launch_prologue(pa, false, s)) != cudaSuccess) return e;
   }
-  if (rdnv) return bf16 ? launch_t<64, true, __nv_bfloat16>(p, s, true, false, img)
-                        : launch_t<64, true, float>(p, s, true, false, img);
-  return bf16 ? launch_t<64, false, __nv_bfloat16>(p, s, true, false, img)
-              : launch_t<64, false, float>(p, s, true, false, img);
+  auto prep = chunk_prep_kernel<DK, RDNV, InT>;
+  constexpr int smem = (int)sizeof(float) * PrepSm<DK>::FLOATS;
+  if ((e = cudaFuncSetAttribute(prep, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
+    return e;
+  RDN_LAUNCH("chunk_prep", s, prep<<<(unsigned)p.nrec, kThreads, smem, s>>>(p));
+  return cudaGetLastError();
+}
+
+struct RunPrep {
+  const FwdParams &p;
+  cudaStream_t s;
+  template <int DK, bool RDNV, typename InT>
+  cudaError_t run() const { return launch_prep_t<DK, RDNV, InT>(p, s); }
+};
+struct RunScan {
+  const FwdParams &p;
+  cudaStream_t s;
+  template <int DK, bool RDNV, typename InT>
+  cudaError_t run() const { return launch_scan<DK, RDNV, InT>(p, s); }
+};
+
+struct RunRecompute {
+  const FwdParams &p;
+  cudaStream_t s;
+  template <int DK, bool RDNV, typename InT>
+  cudaError_t run() const {
+    return launch_scan_t<DK, RDNV, InT, DK == 64 ? 16 : 32, DK == 64 ? 128 : 256, true>(p, s);
+  }
+};
+
+}  // namespace
+
+cudaError_t launch_recompute(const FwdParams &p, int DK, bool rdnv, bool bf16, cudaStream_t s) {
+  return simt_dispatch(DK, rdnv, bf16, RunRecompute{p, s});
+}
+
+cudaError_t launch_prep(const FwdParams &p, int DK, bool rdnv, bool bf16, cudaStream_t s) {
+  if (fwd_uses_tc(DK, bf16)) return launch_prep_tc(p, !rdnv, s);
+  return simt_dispatch(DK, rdnv, bf16, RunPrep{p, s});
+}
+
+cudaError_t launch_fwd_parts(const FwdParams &p, int DK, bool rdnv, bool bf16, cudaStream_t s) {
+  const cudaError_t e = launch_prep(p, DK, rdnv, bf16, s);
+  if (e != cudaSuccess) return e;
+  if (fwd_uses_tc(DK, bf16)) return launch_fwd_tc(p, rdnv, s);
+  return simt_dispatch(DK, rdnv, bf16, RunScan{p, s});
 }
 
 // Block-wide inclusive scan of one value per thread (blockDim.x = 1024).
@@ -577,7 +650,7 @@ FwdPlan plan_fwd(const rdn_fwd_args &a, int variant) {
   // q, k (RDN_FLAG_QK_NORM), the packed-sequence table, then a 256-byte tail
   pl.total_bytes = pl.prep_bytes * nrec + seq_table_bytes(a) + 256;
   if (a.flags & RDN_FLAG_SAVE_FOR_BWD)
-    pl.total_bytes += saved_layout(nrec, a.Dv, a.flags & RDN_FLAG_TANH_RESIDUAL).bytes;
+    pl.total_bytes += saved_layout(a).bytes;
   pl.total_bytes += qk_norm_bytes(a);  // (after those: qk_norm_offset)
   return pl;
 }
@@ -605,13 +678,13 @@ cudaError_t launch_fwd(const rdn_fwd_args &a, int variant, cudaStream_t s) {
     p.seq = seq;
   }
   if (a.flags & RDN_FLAG_SAVE_FOR_BWD) {
-    const SavedLayout l = saved_layout((size_t)p.nrec, a.Dv, a.flags & RDN_FLAG_TANH_RESIDUAL);
+    const SavedLayout l = saved_layout(a);
     p.sv_E = (uint8_t *)a.workspace + l.e;
     p.sv_E2 = (uint8_t *)a.workspace + l.e2;
     p.sv_mask = (unsigned long long *)((char *)a.workspace + l.mask);
   }
   if (p.qk_norm) set_qk_norm_copies(p, a, (char *)a.workspace + qk_norm_offset(a));
-  return launch_fwd_parts(p, a.Dk, variant == 1, a.dtype == RDN_BF16, true, true, s);
+  return launch_fwd_parts(p, a.Dk, variant == 1, a.dtype == RDN_BF16, s);
 }
 
 }  // namespace rdn

@@ -64,93 +64,6 @@ __device__ __forceinline__ void img_row16(uint8_t *hi, uint32_t lo_off, int r, i
   }
 }
 
-// T = (I + A)^-1 for a strictly lower 64 x 64 A, by 128 threads (g = thread
-// index in the group); W is 32 x LDW scratch.  The caller synchronises the
-// block between the stages (0: diagonal blocks; 1, 2: the 16-row blocks; 3, 4:
-// the 32-row block), all groups of the block running the same stage.  The
-// 16 x 16 blocks above the diagonal are never written: the caller zeroes them
-// once.
-__device__ __forceinline__ void inv64_stage(int stage, const float *A, float *Tm, float *W, int g) {
-  if (stage == 0) {
-    // diagonal 16 x 16 blocks: thread (block, column) forward-substitutes its
-    // column, x[r] = delta(r, col) - sum_{m < r} A[r][m] x[m], the terms added
-    // in the order of m; the updates of the rows below m are independent, so
-    // they are made as soon as x[m] is final (a 16-step chain instead of 120)
-    if (g < 64) {
-      const int b0 = (g >> 4) * 16, col = g & 15;
-      float x[16];
-#pragma unroll
-      for (int r = 0; r < 16; ++r) x[r] = (r == col) ? 1.f : 0.f;
-#pragma unroll
-      for (int m = 0; m < 16; ++m) {
-        if (m < col) x[m] = 0.f;  // (above the diagonal)
-#pragma unroll
-        for (int r = m + 1; r < 16; ++r) x[r] = fmaf(-A[(b0 + r) * LDA + b0 + m], x[m], x[r]);
-      }
-#pragma unroll
-      for (int r = 0; r < 16; ++r) Tm[(b0 + r) * LDT + b0 + col] = x[r];
-    }
-  } else if (stage <= 2) {
-    // 16-row blocks (i, j) = (1, 0) and (3, 2): W = A_ij T_jj, then
-    // T_ij = -T_ii W; thread (block, row r, columns 4q .. 4q + 3)
-    const int bi = 2 * (g >> 6) + 1, bj = bi - 1, r = (g >> 2) & 15, q = g & 3;
-    float *w = W + (g >> 6) * 16 * LDW;
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    if (stage == 1) {
-#pragma unroll
-      for (int k = 0; k < 16; ++k) {
-        const float a = A[(16 * bi + r) * LDA + 16 * bj + k];
-        const float4 t = *reinterpret_cast<const float4 *>(Tm + (16 * bj + k) * LDT + 16 * bj + 4 * q);
-        acc[0] = fmaf(a, t.x, acc[0]); acc[1] = fmaf(a, t.y, acc[1]);
-        acc[2] = fmaf(a, t.z, acc[2]); acc[3] = fmaf(a, t.w, acc[3]);
-      }
-      *reinterpret_cast<float4 *>(w + r * LDW + 4 * q) = make_float4(acc[0], acc[1], acc[2], acc[3]);
-    } else {
-#pragma unroll
-      for (int k = 0; k < 16; ++k) {
-        const float a = Tm[(16 * bi + r) * LDT + 16 * bi + k];
-        const float4 t = *reinterpret_cast<const float4 *>(w + k * LDW + 4 * q);
-        acc[0] = fmaf(a, t.x, acc[0]); acc[1] = fmaf(a, t.y, acc[1]);
-        acc[2] = fmaf(a, t.z, acc[2]); acc[3] = fmaf(a, t.w, acc[3]);
-      }
-      *reinterpret_cast<float4 *>(Tm + (16 * bi + r) * LDT + 16 * bj + 4 * q) =
-          make_float4(-acc[0], -acc[1], -acc[2], -acc[3]);
-    }
-  } else {
-    // the 32-row block: W = A[32:64, 0:32] T[0:32, 0:32], then
-    // T[32:64, 0:32] = -T[32:64, 32:64] W; thread (rows rp, rp + 16, columns 4q .. 4q + 3)
-    const int q = g & 7, rp = g >> 3;
-    float a0[4] = {0.f, 0.f, 0.f, 0.f}, a1[4] = {0.f, 0.f, 0.f, 0.f};
-    if (stage == 3) {
-#pragma unroll 8
-      for (int k = 0; k < 32; ++k) {
-        const float x0 = A[(32 + rp) * LDA + k], x1 = A[(48 + rp) * LDA + k];
-        const float4 t = *reinterpret_cast<const float4 *>(Tm + k * LDT + 4 * q);
-        a0[0] = fmaf(x0, t.x, a0[0]); a0[1] = fmaf(x0, t.y, a0[1]);
-        a0[2] = fmaf(x0, t.z, a0[2]); a0[3] = fmaf(x0, t.w, a0[3]);
-        a1[0] = fmaf(x1, t.x, a1[0]); a1[1] = fmaf(x1, t.y, a1[1]);
-        a1[2] = fmaf(x1, t.z, a1[2]); a1[3] = fmaf(x1, t.w, a1[3]);
-      }
-      *reinterpret_cast<float4 *>(W + rp * LDW + 4 * q) = make_float4(a0[0], a0[1], a0[2], a0[3]);
-      *reinterpret_cast<float4 *>(W + (rp + 16) * LDW + 4 * q) = make_float4(a1[0], a1[1], a1[2], a1[3]);
-    } else {
-#pragma unroll 8
-      for (int k = 0; k < 32; ++k) {
-        const float x0 = Tm[(32 + rp) * LDT + 32 + k], x1 = Tm[(48 + rp) * LDT + 32 + k];
-        const float4 t = *reinterpret_cast<const float4 *>(W + k * LDW + 4 * q);
-        a0[0] = fmaf(x0, t.x, a0[0]); a0[1] = fmaf(x0, t.y, a0[1]);
-        a0[2] = fmaf(x0, t.z, a0[2]); a0[3] = fmaf(x0, t.w, a0[3]);
-        a1[0] = fmaf(x1, t.x, a1[0]); a1[1] = fmaf(x1, t.y, a1[1]);
-        a1[2] = fmaf(x1, t.z, a1[2]); a1[3] = fmaf(x1, t.w, a1[3]);
-      }
-      *reinterpret_cast<float4 *>(Tm + (32 + rp) * LDT + 4 * q) =
-          make_float4(-a0[0], -a0[1], -a0[2], -a0[3]);
-      *reinterpret_cast<float4 *>(Tm + (48 + rp) * LDT + 4 * q) =
-          make_float4(-a1[0], -a1[1], -a1[2], -a1[3]);
-    }
-  }
-}
-
 // rla: RLA's records (no delta rule: T_beta = T_gamma = I, written as such
 // for the tensor-core backward; Ap, Mq, M2 and the vectors are RDN's)
 __global__ void __launch_bounds__(NTH, 2) prep_tc_kernel(FwdParams p, bool rla) {
@@ -427,7 +340,7 @@ __global__ void __launch_bounds__(NTH, 2) prep_tc_kernel(FwdParams p, bool rla) 
 #pragma unroll 1
       for (int stage = 0; stage < 5; ++stage) {
         if (stage) __syncthreads();
-        inv64_stage(stage, A, Tm, W, g);
+        inv64_stage<LDA, LDT, LDW>(stage, A, Tm, W, g);
       }
     }
     __syncthreads();
