@@ -74,8 +74,7 @@ typedef enum { RDN_F32 = 0, RDN_BF16 = 1 } rdn_dtype_t;
  * and the clip mask of every chunk (the intermediates of the residual pass);
  * ask *_fwd_workspace_size with the flag set.  rla_bwd / rdn_bwd given that
  * workspace (fwd.workspace) and the same flag in fwd.flags reads them instead
- * of recomputing them.  On the bf16, Dk = 128 path this removes a pass of the
- * backward; on the others the flag only reserves the space. */
+ * of recomputing them, which removes a pass of the backward. */
 #define RDN_FLAG_SAVE_FOR_BWD 0x1u
 
 /* RDN_FLAG_TIED_GAMMA (all four entry points): the residual rate is tied to

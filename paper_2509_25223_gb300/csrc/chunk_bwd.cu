@@ -1,6 +1,5 @@
 // chunk_bwd.cu -- backward of the chunkwise RLA / RDN forward (fp32 SIMT:
-// fp32 inputs, d = 64, the tanh residual and the stateless correction), and
-// the dispatcher of both backward paths.
+// fp32 inputs and d = 64), and the dispatcher of both backward paths.
 //
 // Reverse mode of the chunk algebra in chunk_fwd.cu (the paper gives no
 // backward; this is the adjoint of the forward as computed).  Per chunk,
@@ -11,482 +10,378 @@
 //                   RDN: dX2 = Tg^T dE2, dAg = -strict(dX2 E2^T), dRv = dX2,
 //                        dKR = -diag(Gam) dX2;   RLA: dRv = dE2
 //                   dR0 = Gam_C dR + K^T dKR + Q^T diag(Gam) dOa
-//   clip            dV = dRv * [|v - P| <= c],  dP = -dV
+//   clip            dVr = dRv * [|v - P| <= c],  dP = -dVr
 //   base pass       dMq = strict(dO E^T);  dAp = strict(dP E^T)
 //                   dE = Mq^T dO + Ap^T dP + diag(wS) K dS
-//                   RDN: dX = Tb^T dE, dAb = -strict(dX E^T), dV += dX,
-//                        dKS = diag(Gprev) dP - diag(Gam) dX;   RLA: dV += dE
+//                   RDN: dX = Tb^T dE, dAb = -strict(dX E^T), dV = dVr + dX,
+//                        dKS = diag(Gprev) dP - diag(Gam) dX;   RLA: dV = dVr + dE
 //                   dS0 = Gam_C dS + K^T dKS + Q^T diag(Gam) dO
 //   dK, dQ collect the state products (E dS^T, dKS S0^T, ...); the C x C
 //   gradients dAp, dMq, dM2, dAb, dAg and the per-row factors then give
 //   d(KK^T), d(QK^T), dbeta, dgamma and the gradient of the in-chunk
 //   cumulative log-decay, whose reverse cumulative sum is dg.
 //
-// Kernel bwd_scan: one CTA per (b, h, 16-column slice of d_v), chunks in
-// reverse, recomputing the chunk's forward pieces from the chunk-start
-// states.  Value columns are independent in the forward, so each slice owns
-// its dv, dS, dR columns; its contributions to dK, dQ and to the C x C and
-// per-row gradients (sums over d_v) are added into a per-chunk accumulator.
-// Kernel bwd_finish: one CTA per chunk, folds the accumulator into dq, dk,
-// dg, dbeta, dgamma.
+// Kernel bwd_chain: one CTA per (sequence, head, slice of value columns),
+// chunks in reverse: only what the carried dS, dR need, from the forward's
+// residual mask (E, E2 and the mask are kept by the forward, or remade by
+// chunk_recompute); it keeps dX2, dX, dVr and the chunk-end dS, dR of every
+// chunk in the workspace.
+// Kernel bwd_post: one CTA per chunk, every product over the value columns
+// that no other chunk waits for, and the fold into dq, dk, dg, dbeta, dgamma.
+// Its sums over the value columns stay inside one CTA, so nothing is added
+// atomically and equal calls give equal bits.
 #include "chunk_common.cuh"
+#include "simt.cuh"
 #include "status.cuh"
 
 namespace rdn {
 namespace {
 
-constexpr int kBDVS = 16;       // value columns per backward scan CTA
-constexpr int kScanThreads = 512;  // threads of a backward scan CTA (latency bound: 16 warps)
-constexpr int LDV = kBDVS + 1;  // padded row stride of the [C][kBDVS] tiles
-
-template <int DK>
-struct Acc {  // per-chunk accumulator record (floats)
-  static constexpr int DKo = 0, DQo = C * DK;
-  static constexpr int DAP = 2 * C * DK, DMQ = DAP + kCC, DM2 = DMQ + kCC, DAB = DM2 + kCC,
-                       DAG = DAB + kCC, VEC = DAG + kCC;
-  // per-row vectors: d(gamma) from the read-out, dGam, dGprev, dwS, dwR; then dGamC
-  static constexpr int V_DGAM_OUT = 0, V_DGAM = C, V_DGPREV = 2 * C, V_DWS = 3 * C, V_DWR = 4 * C,
-                       V_DGAMC = 5 * C;
-  static constexpr int FLOATS = VEC + 6 * C;
-};
-
 struct BwdParams {
-  FwdParams f;  // forward inputs; f.ws = prep records
+  FwdParams f;  // forward inputs; f.ws = prep records; f.sv_* = E, E2, mask
   const void *dO;
   const float *dST, *dRT;
-  const float *Sc, *Rc;  // chunk-start states [B,H,NC,DK,DV]
+  const float *Sc, *Rc;  // chunk-start states [record][DK][DV]
   void *dq, *dk, *dv;
   float *dg, *dbeta, *dgamma, *dS0, *dR0;
-  float *acc;  // [B*H*NC] accumulator records
+  // per chunk, bwd_chain to bwd_post: dX2, dVr, dX [record][t][DV] (dX2 with
+  // the auxiliary delta rule, dX with the base one) and the gradients w.r.t.
+  // the chunk-end states [record][DK][DV]
+  float *dX2, *dVr, *dX, *gS, *gR;
   // RDN_FLAG_QK_NORM with bf16 inputs: dq, dk (w.r.t. the normalised q, k)
   // stored here in fp32 for the normalisation's backward; else NULL
   float *gq32, *gk32;
 };
 
-// ---------------------------------------------------------------- kernel 1
-template <int DK, bool RDNV, typename InT>
-__global__ void __launch_bounds__(kScanThreads, 1) bwd_scan_kernel(BwdParams p) {
-  constexpr int DV = DK;
-  constexpr int LDK = DK + 1;
-  using L = Acc<DK>;
-  extern __shared__ float sm[];
-  float *Ks = sm;                // [C][LDK]
-  float *Qs = Ks + C * LDK;      // [C][LDK] (scaled q)
-  float *S0 = Qs + C * LDK;      // [DK][LDV] chunk-start states (slice)
-  float *R0 = S0 + DK * LDV;
-  float *dS = R0 + DK * LDV;     // carried gradients w.r.t. the chunk-end states
-  float *dR = dS + DK * LDV;
-  float *CC = dR + DK * LDV;     // [C][C] staging of one chunk matrix
-  float *Vs = CC + C * C;        // [C][LDV] tiles
-  float *dOs = Vs + C * LDV;
-  float *KS = dOs + C * LDV;
-  float *QS = KS + C * LDV;
-  float *KR = QS + C * LDV;
-  float *QR = KR + C * LDV;
-  float *Es = QR + C * LDV;
-  float *E2 = Es + C * LDV;
-  float *XR = E2 + C * LDV;      // v - P, the residual before the clip
-  float *T1 = XR + C * LDV;
-  float *T2 = T1 + C * LDV;
-  float *T3 = T2 + C * LDV;
-  float *vec = T3 + C * LDV;     // [6*C] Gam, Gprev, alpha, wS, wR, GamC
-  float *gmv = vec + 6 * C;      // [C] gamma per token
-  float *red = gmv + C;          // [6*C] per-row sums of this slice
+// N consecutive elements of a token row as fp32 / from fp32
+template <typename InT, int N>
+__device__ __forceinline__ void ld_row(const InT *p, float (&v)[N]) {
+  if constexpr (sizeof(InT) == 4) {
+    simt::ldv<N>((const float *)p, v);
+  } else {
+#pragma unroll
+    for (int j = 0; j < N; j += 2) {
+      const uint32_t w = *reinterpret_cast<const uint32_t *>(p + j);
+      v[j] = __uint_as_float(w << 16);
+      v[j + 1] = __uint_as_float(w & 0xFFFF0000u);
+    }
+  }
+}
+template <typename InT, int N>
+__device__ __forceinline__ void st_row(InT *p, const float (&v)[N]) {
+  if constexpr (sizeof(InT) == 4) {
+    simt::stv<N>((float *)p, v);
+  } else {
+#pragma unroll
+    for (int j = 0; j < N; j += 2)
+      *reinterpret_cast<__nv_bfloat162 *>(p + j) = __floats2bfloat162_rn(v[j], v[j + 1]);
+  }
+}
 
-  const int bh = blockIdx.x;
-  const int H = p.f.H, h = bh % H;
-  const SeqSpan sp = seq_span(p.f, bh / H, h);  // this (sequence, head)'s tokens and records
-  const long long tok0 = sp.tok0;
-  const int NC = sp.nc, T = sp.len;
-  const int j0 = blockIdx.y * kBDVS;
-  const int tid = threadIdx.x;
-  const InT *q = (const InT *)p.f.q;
-  const InT *k = (const InT *)p.f.k;
-  const InT *v = (const InT *)p.f.v;
-  const InT *dO = (const InT *)p.dO;
-  InT *dv = (InT *)p.dv;
-  const float clip = p.f.clip;
-  const size_t sbase = (size_t)bh * DK * DV;
+// ---------------------------------------------------------------- kernel 1
+// Thread (warp w, lane (lm, ln)) owns rows 2 r0, 2 r0 + 1 (r0 = LM w + lm) and
+// columns TN ln .. + TN of every 64-row product: the transposed chunk
+// matrices are then read with contiguous rows (M^T's column pair is one
+// 8-byte load).  Five phases a chunk: K dS, K dR, M2^T dOa, Mq^T dO | dX2 |
+// Ap^T dVr and dR's update | dX | dS's update.  A transposed triangular
+// product starts at its warp's first row.  Bound by the FMA pipe and the
+// phases' latencies: B = 4, H = 16, T = 2048,
+// d = 64 in 0.50 ms, B = 2, H = 8, T = 1000, d = 128 fp32 in 0.32 ms.
+template <int DK, int DVS, int NT>
+struct ChainSm {  // float offsets
+  static constexpr int LDK = DK + 4;
+  static constexpr int K = 0, Q = K + C * LDK, MAT = Q + C * LDK;  // MAT: 3 slots [C][C]
+  static constexpr int S = MAT + 3 * C * C, R = S + DK * DVS, DO = R + DK * DVS;
+  static constexpr int DOA = DO + C * DVS, T1 = DOA + C * DVS, T2 = T1 + C * DVS, T3 = T2 + C * DVS;
+  static constexpr int VEC = T3 + C * DVS, FLOATS = VEC + 6 * C;
+};
+
+template <int DK, bool RDNV, typename InT, int DVS, int NT>
+__global__ void __launch_bounds__(NT, NT == 128 ? 2 : 1) bwd_chain_kernel(BwdParams p) {
+  using namespace simt;
+  using SM = ChainSm<DK, DVS, NT>;
+  constexpr int DV = DK, LDK = SM::LDK;
+  constexpr int TN = 32 * DVS / NT, LN = DVS / TN, LM = 32 / LN, TMU = DK / 32;
+  static_assert(LM * (NT / 32) == 32, "row pairs of 32");
+  extern __shared__ __align__(16) float sm[];
+  float *Ks = sm + SM::K, *Qs = sm + SM::Q, *Ss = sm + SM::S, *Rs = sm + SM::R;
+  float *DO = sm + SM::DO, *DOA = sm + SM::DOA, *T1 = sm + SM::T1, *T2 = sm + SM::T2;
+  float *T3 = sm + SM::T3, *vec = sm + SM::VEC;
+  float *mat[3] = {sm + SM::MAT, sm + SM::MAT + C * C, sm + SM::MAT + 2 * C * C};
+
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int ln = lane % LN, r0 = LM * warp + lane / LN, n0 = TN * ln;
+  const int kw = 2 * LM * warp;  // the warp's first row
+  const int H = p.f.H, sq = blockIdx.x / H, h = blockIdx.x % H;
+  const SeqSpan sp = seq_span(p.f, sq, h);
+  const int j0 = blockIdx.y * DVS;
   const bool dec_res = p.f.mods & RDN_FLAG_DECAYED_RESIDUAL;
   const bool plain = p.f.mods & RDN_FLAG_PLAIN_COMBINE;
   const bool tnh = p.f.mods & RDN_FLAG_TANH_RESIDUAL;
   const bool stl = p.f.mods & RDN_FLAG_STATELESS_AUX;
   const bool rdn_aux = RDNV && !stl;  // the auxiliary pass runs the delta rule
 
-  using MMk = BlockMM<C, kBDVS, DK, kScanThreads>;   // [C x DK] @ [DK x DVS]
-  using MMc = BlockMM<C, kBDVS, C, kScanThreads>;    // [C x C] @ [C x DVS]
-  using MMg = BlockMM<C, C, kBDVS, kScanThreads>;    // [C x DVS] @ [DVS x C]
-  using MMd = BlockMM<C, DK, kBDVS, kScanThreads>;   // [C x DVS] @ [DVS x DK]
-  using MMu = BlockMM<DK, kBDVS, C, kScanThreads>;   // [DK x C] @ [C x DVS]
-  const int col = MMk::col();
-
-  for (int e = tid; e < DK * kBDVS; e += kScanThreads) {
-    const int i = e / kBDVS, jj = e % kBDVS;
-    dS[i * LDV + jj] = p.dST ? p.dST[sbase + (size_t)i * DV + j0 + jj] : 0.f;
-    dR[i * LDV + jj] = p.dRT ? p.dRT[sbase + (size_t)i * DV + j0 + jj] : 0.f;
+  const size_t sbase = (size_t)blockIdx.x * DK * DV;
+  for (int e = tid; e < DK * DVS / 4; e += NT) {
+    const size_t off = sbase + (size_t)(e / (DVS / 4)) * DV + j0 + 4 * (e % (DVS / 4));
+    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+    *reinterpret_cast<float4 *>(Ss + 4 * e) = p.dST ? *reinterpret_cast<const float4 *>(p.dST + off) : z;
+    *reinterpret_cast<float4 *>(Rs + 4 * e) = p.dRT ? *reinterpret_cast<const float4 *>(p.dRT + off) : z;
   }
 
-  for (int c = NC - 1; c >= 0; --c) {
-    const int t0 = c * C;
-    const int n = min(C, T - t0);
-    const size_t chunk = (size_t)(sp.rbase + c);
-    const float *rec = p.f.ws + chunk * kRecFloats;
-    float *acc = p.acc + chunk * L::FLOATS;
-    __syncthreads();
-    for (int e = tid; e < C * DK; e += kScanThreads) {
-      const int t = e / DK, d = e % DK;
-      float kv = 0.f, qv = 0.f;
+  RowTile<InT, DK, NT> kt, qt;
+  constexpr int VU = 6 * C / NT + (6 * C % NT != 0);
+  float vr[VU], dor[2][TN], gmr[2], mkr[2][TN];  // mkr: the residual map's derivative
+  auto fetch = [&](int c) {  // chunk c's K, Q, dO, gates and mask
+    const int n = min(C, sp.len - c * C);
+    const size_t row = (size_t)(sp.tok0 + c * C) * H + h;
+    kt.fetch((const InT *)p.f.k + row * DK, (size_t)H * DK, n);
+    qt.fetch((const InT *)p.f.q + row * DK, (size_t)H * DK, n);
+    const float *rec = p.f.ws + (size_t)(sp.rbase + c) * kRecFloats;
+#pragma unroll
+    for (int u = 0; u < VU; ++u) {
+      const int e = tid + u * NT;
+      vr[u] = e <= V_GAMC ? rec[OFF_VEC + e] : 0.f;
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int t = 2 * r0 + i;
+#pragma unroll
+      for (int j = 0; j < TN; ++j) dor[i][j] = 0.f;
+      gmr[i] = 0.f;
       if (t < n) {
-        const size_t off = ((size_t)(tok0 + t0 + t) * H + h) * DK + d;
-        kv = to_f32(k[off]);
-        qv = p.f.scale * to_f32(q[off]);
+        ld_row<InT, TN>((const InT *)p.dO + (row + (size_t)t * H) * DV + j0 + n0, dor[i]);
+        gmr[i] = plain ? 1.f : p.f.gamma[row + (size_t)t * H];
       }
-      Ks[t * LDK + d] = kv;
-      Qs[t * LDK + d] = qv;
-    }
-    for (int e = tid; e < C * kBDVS; e += kScanThreads) {
-      const int t = e / kBDVS, jj = e % kBDVS;
-      float vv = 0.f, dd = 0.f;
-      if (t < n) {
-        const size_t off = ((size_t)(tok0 + t0 + t) * H + h) * DV + j0 + jj;
-        vv = to_f32(v[off]);
-        dd = to_f32(dO[off]);
+      const size_t m = ((size_t)(sp.rbase + c) * C + t) * DV + j0 + n0;
+      if (tnh) {
+        ldv<TN>((const float *)p.f.sv_mask + m, mkr[i]);
+      } else {
+        const uint32_t b = ((const uint8_t *)p.f.sv_mask)[m >> 3] >> (n0 & 7);
+#pragma unroll
+        for (int j = 0; j < TN; ++j) mkr[i][j] = (b >> j) & 1 ? 1.f : 0.f;
       }
-      Vs[t * LDV + jj] = vv;
-      dOs[t * LDV + jj] = dd;
     }
-    for (int e = tid; e < DK * kBDVS; e += kScanThreads) {
-      const int i = e / kBDVS, jj = e % kBDVS;
-      const size_t off = chunk * DK * DV + (size_t)i * DV + j0 + jj;
-      S0[i * LDV + jj] = p.Sc[off];
-      R0[i * LDV + jj] = p.Rc[off];
+  };
+  auto mats = [&](int c) { return p.f.ws + (size_t)(sp.rbase + c) * kRecFloats; };
+  const int last = sp.nc - 1;
+  if (last >= 0) {
+    fetch(last);
+    cp_mat<NT>(mat[0], C, mats(last) + OFF_M2);
+    cp_mat<NT>(mat[1], C, mats(last) + OFF_MQ);
+    if (rdn_aux) cp_mat<NT>(mat[2], C, mats(last) + OFF_TG);
+    cp_commit();
+  }
+
+  for (int c = last; c >= 0; --c) {
+    const int n = min(C, sp.len - c * C);
+    const size_t rec = (size_t)(sp.rbase + c);
+    kt.put(Ks, LDK, 1.f);
+    qt.put(Qs, LDK, p.f.scale);
+#pragma unroll
+    for (int u = 0; u < VU; ++u)
+      if (tid + u * NT < 6 * C) vec[tid + u * NT] = vr[u];
+    float dO[2][TN], mk[2][TN], gm[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      float d[TN];
+      gm[i] = gmr[i];
+#pragma unroll
+      for (int j = 0; j < TN; ++j) {
+        dO[i][j] = dor[i][j];
+        mk[i][j] = mkr[i][j];
+        d[j] = gm[i] * dO[i][j];
+      }
+      stv<TN>(DO + (2 * r0 + i) * DVS + n0, dO[i]);
+      stv<TN>(DOA + (2 * r0 + i) * DVS + n0, d);
     }
-    for (int e = tid; e < 6 * C; e += kScanThreads) {
-      vec[e] = rec[OFF_VEC + e];
-      red[e] = 0.f;
-    }
-    if (tid < C) gmv[tid] = tid < n ? p.f.gamma[(size_t)(tok0 + t0 + tid) * H + h] : 0.f;
+    wait_groups<0>();  // M2, Mq, T_gamma
     __syncthreads();
     const float *Gam = vec + V_GAM, *Gprev = vec + V_GPREV, *wS = vec + V_WS, *wR = vec + V_WR;
     const float GamC = vec[V_GAMC];
-
-    // ---- recompute the chunk's forward pieces
-    {
-      float a1[MMk::RPT], a2[MMk::RPT], a3[MMk::RPT], a4[MMk::RPT];
-      MMk::run(Ks, LDK, 1, S0, LDV, 1, a1);
-      MMk::run(Qs, LDK, 1, S0, LDV, 1, a2);
-      MMk::run(Ks, LDK, 1, R0, LDV, 1, a3);
-      MMk::run(Qs, LDK, 1, R0, LDV, 1, a4);
-#pragma unroll
-      for (int i = 0; i < MMk::RPT; ++i) {
-        const int t = MMk::row(i);
-        KS[t * LDV + col] = a1[i];
-        QS[t * LDV + col] = a2[i];
-        KR[t * LDV + col] = stl ? 0.f : a3[i];  // (the stateless R carries nothing)
-        QR[t * LDV + col] = stl ? 0.f : a4[i];
-        if (RDNV) T1[t * LDV + col] = Vs[t * LDV + col] - Gam[t] * a1[i];
+    {  // the chunk-end gradients
+      float *gs = p.gS + rec * DK * DV + j0, *gr = p.gR + rec * DK * DV + j0;
+      for (int e = tid; e < DK * DVS / 4; e += NT) {
+        const size_t off = (size_t)(e / (DVS / 4)) * DV + 4 * (e % (DVS / 4));
+        *reinterpret_cast<float4 *>(gs + off) = *reinterpret_cast<const float4 *>(Ss + 4 * e);
+        *reinterpret_cast<float4 *>(gr + off) = *reinterpret_cast<const float4 *>(Rs + 4 * e);
       }
     }
-    const float *E = Vs;
-    if (RDNV) {
-      for (int e = tid; e < C * C; e += kScanThreads) CC[e] = rec[OFF_TB + e];
-      __syncthreads();
-      float a1[MMc::RPT];
-      MMc::run(CC, C, 1, T1, LDV, 1, a1);
-#pragma unroll
-      for (int i = 0; i < MMc::RPT; ++i) Es[MMc::row(i) * LDV + col] = a1[i];
-      E = Es;
-    }
-    __syncthreads();
-    for (int e = tid; e < C * C; e += kScanThreads) CC[e] = rec[OFF_AP + e];
-    __syncthreads();
+    // ---- K dS, K dR, M2^T dOa, Mq^T dO; dE2
+    float kd[2][TN], x[2][TN], de[2][TN];
     {
-      float a1[MMc::RPT];
-      MMc::run(CC, C, 1, E, LDV, 1, a1);
+      float kr[2][TN];
+      zero(kd);
+      zero(kr);
+      zero(x);
+      zero(de);
+      mm_ak2<2, TN, 3, 3>(Ks + 2 * r0 * LDK, LDK, Ss + n0, Rs + n0, DVS, DK, kd, kr);
+      mm_am<2, TN>(mat[0] + kw * C + 2 * r0, C, DOA + kw * DVS + n0, DVS, C - kw, x);
+      mm_am<2, TN>(mat[1] + kw * C + 2 * r0, C, DO + kw * DVS + n0, DVS, C - kw, de);
 #pragma unroll
-      for (int i = 0; i < MMc::RPT; ++i) {
-        const int t = MMc::row(i);
-        const float x =
-            Vs[t * LDV + col] - ((dec_res ? Gam[t] : Gprev[t]) * KS[t * LDV + col] + a1[i]);
-        XR[t * LDV + col] = x;
-        if (rdn_aux) T1[t * LDV + col] = resid_map(x, clip, tnh) - Gam[t] * KR[t * LDV + col];
-        else E2[t * LDV + col] = resid_map(x, clip, tnh);
+      for (int i = 0; i < 2; ++i) {
+        const int t = 2 * r0 + i;
+#pragma unroll
+        for (int j = 0; j < TN; ++j) x[i][j] += wR[t] * kr[i][j];
+        if (rdn_aux) stv<TN>(T1 + t * DVS + n0, x[i]);
       }
     }
     __syncthreads();
+    cp_mat<NT>(mat[0], C, mats(c) + OFF_AP);
+    cp_commit();
+    if (RDNV) cp_mat<NT>(mat[1], C, mats(c) + OFF_TB);
+    cp_commit();
+    // ---- dX2 = T_gamma^T dE2; dVr; dKR = -Gam dX2; dQR = Gam dOa
     if (rdn_aux) {
-      for (int e = tid; e < C * C; e += kScanThreads) CC[e] = rec[OFF_TG + e];
-      __syncthreads();
-      float a1[MMc::RPT];
-      MMc::run(CC, C, 1, T1, LDV, 1, a1);
-#pragma unroll
-      for (int i = 0; i < MMc::RPT; ++i) E2[MMc::row(i) * LDV + col] = a1[i];
-      __syncthreads();
+      zero(x);
+      mm_am<2, TN>(mat[2] + kw * C + 2 * r0, C, T1 + kw * DVS + n0, DVS, C - kw, x);
     }
-    for (int e = tid; e < C * C; e += kScanThreads) CC[e] = rec[OFF_M2 + e];
-    __syncthreads();
-    {  // Oa -> T2, dOa -> T3, row sums d(gamma)_out and dGam
-      float a1[MMc::RPT];
-      MMc::run(CC, C, 1, E2, LDV, 1, a1);
+    float dvr[2][TN];
 #pragma unroll
-      for (int i = 0; i < MMc::RPT; ++i) {
-        const int t = MMc::row(i);
-        const float oa = Gam[t] * QR[t * LDV + col] + a1[i];
-        const float dOv = dOs[t * LDV + col];
-        const float doa = plain ? dOv : gmv[t] * dOv;
-        T3[t * LDV + col] = doa;
-        if (!plain) atomicAdd(&red[L::V_DGAM_OUT + t], dOv * oa);
-        atomicAdd(&red[L::V_DGAM + t], doa * QR[t * LDV + col]);
+    for (int i = 0; i < 2; ++i) {
+      const int t = 2 * r0 + i;
+      const size_t off = (rec * C + t) * DV + j0 + n0;
+      float a[TN], b[TN];
+#pragma unroll
+      for (int j = 0; j < TN; ++j) {
+        dvr[i][j] = x[i][j] * mk[i][j];
+        a[j] = -Gam[t] * x[i][j];
+        b[j] = Gam[t] * (gm[i] * dO[i][j]);
       }
-    }
-    __syncthreads();
-
-    // ---- adjoint of the auxiliary pass
-    {
-      float kd[MMk::RPT], a1[MMc::RPT];
-      MMk::run(Ks, LDK, 1, dR, LDV, 1, kd);
-      MMc::run(CC, 1, C, T3, LDV, 1, a1);  // M2^T dOa
-#pragma unroll
-      for (int i = 0; i < MMc::RPT; ++i) {
-        const int t = MMc::row(i);
-        T1[t * LDV + col] = a1[i] + wR[t] * kd[i];  // dE2
-        if (!stl) {  // (stateless: wR is a constant and R0 does not enter)
-          atomicAdd(&red[L::V_DWR + t], kd[i] * E2[t * LDV + col]);
-          QR[t * LDV + col] = Gam[t] * T3[t * LDV + col];  // dQR
-        }
-      }
-      float g1[MMg::RPT];
-      MMg::run(T3, LDV, 1, E2, 1, LDV, g1);  // dM2 = dOa E2^T (inclusive)
-#pragma unroll
-      for (int i = 0; i < MMg::RPT; ++i) {
-        const int t = MMg::row(i), ii = MMg::col();
-        if (ii <= t) atomicAdd(&acc[L::DM2 + t * C + ii], g1[i]);
-      }
-    }
-    __syncthreads();
-    const float *dRv = T1;
-    if (rdn_aux) {
-      for (int e = tid; e < C * C; e += kScanThreads) CC[e] = rec[OFF_TG + e];
-      __syncthreads();
-      float a1[MMc::RPT];
-      MMc::run(CC, 1, C, T1, LDV, 1, a1);  // dX2 = Tg^T dE2
-#pragma unroll
-      for (int i = 0; i < MMc::RPT; ++i) T2[MMc::row(i) * LDV + col] = a1[i];
-      __syncthreads();
-      float g1[MMg::RPT];
-      MMg::run(T2, LDV, 1, E2, 1, LDV, g1);  // dAg = -strict(dX2 E2^T)
-#pragma unroll
-      for (int i = 0; i < MMg::RPT; ++i) {
-        const int t = MMg::row(i), ii = MMg::col();
-        if (ii < t) atomicAdd(&acc[L::DAG + t * C + ii], -g1[i]);
-      }
-#pragma unroll
-      for (int i = 0; i < MMc::RPT; ++i) {
-        const int t = MMc::row(i);
-        T1[t * LDV + col] = -Gam[t] * a1[i];  // dKR
-        atomicAdd(&red[L::V_DGAM + t], -a1[i] * KR[t * LDV + col]);
-      }
-      dRv = T2;
-    }
-    // T3 <- diag(wR) E2 for dK += diag(wR) E2 dR^T
-    for (int e = tid; e < C * kBDVS; e += kScanThreads) {
-      const int t = e / kBDVS, jj = e % kBDVS;
-      T3[t * LDV + jj] = wR[t] * E2[t * LDV + jj];
-    }
-    __syncthreads();
-    float dKacc[MMd::RPT], dQacc[MMd::RPT];
-    {
-      float g1[MMd::RPT];
-      MMd::run(T3, LDV, 1, dR, 1, LDV, dKacc);
       if (rdn_aux) {
-        MMd::run(T1, LDV, 1, R0, 1, LDV, g1);
-#pragma unroll
-        for (int i = 0; i < MMd::RPT; ++i) dKacc[i] += g1[i];
+        stv<TN>(p.dX2 + off, x[i]);
+        stv<TN>(T2 + t * DVS + n0, a);
       }
-      MMd::run(QR, LDV, 1, R0, 1, LDV, dQacc);
-      float s = 0.f;
-      if (!stl)
-        for (int e = tid; e < DK * kBDVS; e += kScanThreads) {
-          const int i = e / kBDVS, jj = e % kBDVS;
-          s += dR[i * LDV + jj] * R0[i * LDV + jj];
-        }
-      atomicAdd(&red[L::V_DGAMC], s);
+      stv<TN>(p.dVr + off, dvr[i]);
+      stv<TN>(T3 + t * DVS + n0, dvr[i]);
+      stv<TN>(DOA + t * DVS + n0, b);
     }
+    wait_groups<1>();  // Ap
     __syncthreads();
-    {  // dR0 = Gam_C dR + K^T dKR + Q^T dQR (stateless: 0)
-      float u1[MMu::RPT], u2[MMu::RPT];
-      MMu::run(Qs, 1, LDK, QR, LDV, 1, u2);
-      if (rdn_aux) MMu::run(Ks, 1, LDK, T1, LDV, 1, u1);
-#pragma unroll
-      for (int i = 0; i < MMu::RPT; ++i) {
-        const int r = MMu::row(i);
-        dR[r * LDV + col] =
-            stl ? 0.f : GamC * dR[r * LDV + col] + u2[i] + (rdn_aux ? u1[i] : 0.f);
-      }
-    }
-    // clip: dV = dRv * [|x| <= c] into T3 (dP = -dV; tanh: times 1 - (r/c)^2)
-    for (int e = tid; e < C * kBDVS; e += kScanThreads) {
-      const int t = e / kBDVS, jj = e % kBDVS;
-      T3[t * LDV + jj] = dRv[t * LDV + jj] * resid_grad(XR[t * LDV + jj], clip, tnh);
-    }
-    __syncthreads();
-
-    // ---- adjoint of the base pass
+    if (c > 0 && rdn_aux) cp_mat<NT>(mat[2], C, mats(c - 1) + OFF_TG);
+    cp_commit();
+    // ---- dE = Mq^T dO - Ap^T dVr + wS K dS; dR = Gam_C dR + Q^T dQR + K^T dKR
     {
-      float g1[MMg::RPT], g2[MMg::RPT];
-      MMg::run(dOs, LDV, 1, E, 1, LDV, g1);  // dMq = strict(dO E^T)
-      MMg::run(T3, LDV, 1, E, 1, LDV, g2);   // dAp = strict(dP E^T) = -strict(dV E^T)
+      zero(x);
+      mm_am<2, TN>(mat[0] + kw * C + 2 * r0, C, T3 + kw * DVS + n0, DVS, C - kw, x);
 #pragma unroll
-      for (int i = 0; i < MMg::RPT; ++i) {
-        const int t = MMg::row(i), ii = MMg::col();
-        if (ii < t) {
-          atomicAdd(&acc[L::DMQ + t * C + ii], g1[i]);
-          atomicAdd(&acc[L::DAP + t * C + ii], -g2[i]);
-        }
+      for (int i = 0; i < 2; ++i) {
+        const int t = 2 * r0 + i;
+#pragma unroll
+        for (int j = 0; j < TN; ++j) x[i][j] = de[i][j] - x[i][j] + wS[t] * kd[i][j];
+        if (RDNV) stv<TN>(T1 + t * DVS + n0, x[i]);
+      }
+      const int m0 = TMU * r0;
+      float u[TMU][TN];
+      zero(u);
+      mm_am<TMU, TN>(Qs + m0, LDK, DOA + n0, DVS, C, u);
+      if (rdn_aux) mm_am<TMU, TN>(Ks + m0, LDK, T2 + n0, DVS, C, u);
+#pragma unroll
+      for (int i = 0; i < TMU; ++i) {
+        float s[TN];
+        ldv<TN>(Rs + (m0 + i) * DVS + n0, s);
+#pragma unroll
+        for (int j = 0; j < TN; ++j) s[j] = stl ? 0.f : GamC * s[j] + u[i][j];
+        stv<TN>(Rs + (m0 + i) * DVS + n0, s);
       }
     }
-    for (int e = tid; e < C * C; e += kScanThreads) CC[e] = rec[OFF_MQ + e];
+    wait_groups<1>();  // T_beta
     __syncthreads();
-    float de[MMc::RPT];
-    MMc::run(CC, 1, C, dOs, LDV, 1, de);  // Mq^T dO
-    __syncthreads();
-    for (int e = tid; e < C * C; e += kScanThreads) CC[e] = rec[OFF_AP + e];
-    __syncthreads();
-    {
-      float a1[MMc::RPT], kd[MMk::RPT];
-      MMc::run(CC, 1, C, T3, LDV, 1, a1);  // Ap^T dV  (= -Ap^T dP)
-      MMk::run(Ks, LDK, 1, dS, LDV, 1, kd);
-#pragma unroll
-      for (int i = 0; i < MMc::RPT; ++i) {
-        const int t = MMc::row(i);
-        const float dv_ = T3[t * LDV + col];
-        T1[t * LDV + col] = de[i] - a1[i] + wS[t] * kd[i];  // dE
-        atomicAdd(&red[L::V_DWS + t], kd[i] * E[t * LDV + col]);
-        // the prediction's state term: Gprev KS (decayed residual: Gam KS)
-        atomicAdd(&red[(dec_res ? L::V_DGAM : L::V_DGPREV) + t], -dv_ * KS[t * LDV + col]);
-        T2[t * LDV + col] = -(dec_res ? Gam[t] : Gprev[t]) * dv_;  // dKS (base part)
-        const float dOv = dOs[t * LDV + col];
-        // the base read-out Gam QS (plain combine: Gprev QS)
-        atomicAdd(&red[(plain ? L::V_DGPREV : L::V_DGAM) + t], dOv * QS[t * LDV + col]);
-        QS[t * LDV + col] = (plain ? Gprev[t] : Gam[t]) * dOv;  // dQS
-      }
-    }
-    __syncthreads();
+    if (c > 0) cp_mat<NT>(mat[0], C, mats(c - 1) + OFF_M2);
+    cp_commit();
+    // ---- dX = T_beta^T dE; dV = dVr + dX; dKS = -Gprev dVr - Gam dX; dQS = Gam dO
     if (RDNV) {
-      for (int e = tid; e < C * C; e += kScanThreads) CC[e] = rec[OFF_TB + e];
-      __syncthreads();
-      float a1[MMc::RPT];
-      MMc::run(CC, 1, C, T1, LDV, 1, a1);  // dX = Tb^T dE
-      __syncthreads();
-#pragma unroll
-      for (int i = 0; i < MMc::RPT; ++i) {
-        const int t = MMc::row(i);
-        T1[t * LDV + col] = a1[i];
-        T3[t * LDV + col] += a1[i];                  // dV += dX
-        T2[t * LDV + col] -= Gam[t] * a1[i];         // dKS -= Gam dX
-        atomicAdd(&red[L::V_DGAM + t], -a1[i] * KS[t * LDV + col]);
-      }
-      __syncthreads();
-      float g1[MMg::RPT];
-      MMg::run(T1, LDV, 1, E, 1, LDV, g1);  // dAb = -strict(dX E^T)
-#pragma unroll
-      for (int i = 0; i < MMg::RPT; ++i) {
-        const int t = MMg::row(i), ii = MMg::col();
-        if (ii < t) atomicAdd(&acc[L::DAB + t * C + ii], -g1[i]);
-      }
-    } else {
-      for (int e = tid; e < C * kBDVS; e += kScanThreads) {
-        const int t = e / kBDVS, jj = e % kBDVS;
-        T3[t * LDV + jj] += T1[t * LDV + jj];  // dV += dE
-      }
+      zero(x);
+      mm_am<2, TN>(mat[1] + kw * C + 2 * r0, C, T1 + kw * DVS + n0, DVS, C - kw, x);
     }
-    // XR <- diag(wS) E for dK += diag(wS) E dS^T
-    for (int e = tid; e < C * kBDVS; e += kScanThreads) {
-      const int t = e / kBDVS, jj = e % kBDVS;
-      XR[t * LDV + jj] = wS[t] * E[t * LDV + jj];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int t = 2 * r0 + i;
+      const float gp = dec_res ? Gam[t] : Gprev[t], gq = plain ? Gprev[t] : Gam[t];
+      float a[TN], b[TN], v[TN];
+#pragma unroll
+      for (int j = 0; j < TN; ++j) {
+        v[j] = dvr[i][j] + x[i][j];
+        a[j] = -gp * dvr[i][j] - (RDNV ? Gam[t] * x[i][j] : 0.f);
+        b[j] = gq * dO[i][j];
+      }
+      if (RDNV) stv<TN>(p.dX + (rec * C + t) * DV + j0 + n0, x[i]);
+      if (t < n)
+        st_row<InT, TN>((InT *)p.dv + ((size_t)(sp.tok0 + c * C + t) * H + h) * DV + j0 + n0, v);
+      stv<TN>(T2 + t * DVS + n0, a);
+      stv<TN>(DO + t * DVS + n0, b);
     }
     __syncthreads();
-    {
-      float g1[MMd::RPT];
-      MMd::run(XR, LDV, 1, dS, 1, LDV, g1);
-#pragma unroll
-      for (int i = 0; i < MMd::RPT; ++i) dKacc[i] += g1[i];
-      MMd::run(T2, LDV, 1, S0, 1, LDV, g1);
-#pragma unroll
-      for (int i = 0; i < MMd::RPT; ++i) dKacc[i] += g1[i];
-      MMd::run(QS, LDV, 1, S0, 1, LDV, g1);
-#pragma unroll
-      for (int i = 0; i < MMd::RPT; ++i) dQacc[i] += g1[i];
-      float s = 0.f;
-      for (int e = tid; e < DK * kBDVS; e += kScanThreads) {
-        const int i = e / kBDVS, jj = e % kBDVS;
-        s += dS[i * LDV + jj] * S0[i * LDV + jj];
-      }
-      atomicAdd(&red[L::V_DGAMC], s);
+    if (c > 0) {
+      cp_mat<NT>(mat[1], C, mats(c - 1) + OFF_MQ);
+      fetch(c - 1);
     }
-    __syncthreads();
-    {  // dS0 = Gam_C dS + K^T dKS + Q^T dQS
-      float u1[MMu::RPT], u2[MMu::RPT];
-      MMu::run(Ks, 1, LDK, T2, LDV, 1, u1);
-      MMu::run(Qs, 1, LDK, QS, LDV, 1, u2);
+    cp_commit();
+    {  // ---- dS = Gam_C dS + K^T dKS + Q^T dQS
+      const int m0 = TMU * r0;
+      float u[TMU][TN];
+      zero(u);
+      mm_am<TMU, TN>(Ks + m0, LDK, T2 + n0, DVS, C, u);
+      mm_am<TMU, TN>(Qs + m0, LDK, DO + n0, DVS, C, u);
 #pragma unroll
-      for (int i = 0; i < MMu::RPT; ++i) {
-        const int r = MMu::row(i);
-        dS[r * LDV + col] = GamC * dS[r * LDV + col] + u1[i] + u2[i];
+      for (int i = 0; i < TMU; ++i) {
+        float s[TN];
+        ldv<TN>(Ss + (m0 + i) * DVS + n0, s);
+#pragma unroll
+        for (int j = 0; j < TN; ++j) s[j] = GamC * s[j] + u[i][j];
+        stv<TN>(Ss + (m0 + i) * DVS + n0, s);
       }
     }
-    // ---- outputs of this slice
-#pragma unroll
-    for (int i = 0; i < MMd::RPT; ++i) {
-      const int t = MMd::row(i), d = MMd::col();
-      atomicAdd(&acc[L::DKo + t * DK + d], dKacc[i]);
-      atomicAdd(&acc[L::DQo + t * DK + d], dQacc[i]);
-    }
-    for (int e = tid; e < C * kBDVS; e += kScanThreads) {
-      const int t = e / kBDVS, jj = e % kBDVS;
-      if (t < n) dv[((size_t)(tok0 + t0 + t) * H + h) * DV + j0 + jj] = from_f32<InT>(T3[t * LDV + jj]);
-    }
     __syncthreads();
-    for (int e = tid; e < 5 * C + 1; e += kScanThreads) atomicAdd(&acc[L::VEC + e], red[e]);
   }
   __syncthreads();
-  for (int e = tid; e < DK * kBDVS; e += kScanThreads) {
-    const int i = e / kBDVS, jj = e % kBDVS;
-    if (p.dS0) p.dS0[sbase + (size_t)i * DV + j0 + jj] = dS[i * LDV + jj];
-    if (p.dR0) p.dR0[sbase + (size_t)i * DV + j0 + jj] = dR[i * LDV + jj];
+  for (int e = tid; e < DK * DVS / 4; e += NT) {
+    const size_t off = sbase + (size_t)(e / (DVS / 4)) * DV + j0 + 4 * (e % (DVS / 4));
+    if (p.dS0) *reinterpret_cast<float4 *>(p.dS0 + off) = *reinterpret_cast<const float4 *>(Ss + 4 * e);
+    if (p.dR0) *reinterpret_cast<float4 *>(p.dR0 + off) = *reinterpret_cast<const float4 *>(Rs + 4 * e);
   }
 }
 
 // ---------------------------------------------------------------- kernel 2
-// One CTA per chunk.  Each warp owns 4 rows t of the C x C gradients; lane l
-// handles columns l and l + 32.  Row sums (d cum_t, d cprev_t) are reduced
-// with shuffles; column sums (d cum_i, dbeta_i, dgamma_i) go through
-// shared-memory tiles and a column pass, so no shared-memory atomics are
-// contended.
+// One CTA of 256 threads per chunk.  Thread (ty, tx) owns rows 4 ty .. 4 ty + 3
+// and columns tx + 16 j of every product, so a row's sums are shuffles among
+// the 16 lanes of a half warp.  Every value-dimension product is A B^T with
+// both operands' rows contiguous (mm_nt); the value dimension is walked in
+// slices of JS columns, the next slice's tiles arriving by cp.async while the
+// current one is used: first the auxiliary pass (dO, E2, dX2 against R0, dR and
+// E2), then the base pass (dO, E, dVr, dX against S0, dS and E).
+// The per-row gate sums need no read-outs K S0, Q R0, ...: a row's
+// sum_j dKS KS is its k's product with the row of dKS S0^T, which dK takes
+// anyway.  kk, qk and the C x C gradients stay in shared memory at the
+// positions their thread owns.  Bound by the FMA pipe (two FMAs an
+// instruction): the same calls in 0.60 and 0.28 ms.  One kernel that walked
+// the chunks with every product, adding its column slices' shares atomically,
+// and a finishing pass took 6.19 and 1.85 ms for what the chain and this do in
+// 1.10 and 0.60.
+constexpr int kPostThreads = 256;
+template <int DK>
+struct PostSm {  // float offsets
+  static constexpr int JS = 2048 / DK, LDJ = JS + 4, LDK = DK + 4, LDC = C + 4;
+  static constexpr int STG = (4 * C + 2 * DK) * LDJ;  // a slice's tiles
+  static constexpr int K = 0, Q = K + C * LDK, KK = Q + C * LDK, QK = KK + C * LDC;
+  static constexpr int DKK = QK + C * LDC, DQK = DKK + C * LDC, ST = DQK + C * LDC;
+  static constexpr int VEC = ST + 2 * STG, FLOATS = VEC + 15 * C;
+  static_assert(FLOATS * 4 <= 232448, "one CTA's shared memory");
+};
+
 template <int DK, bool RDNV, typename InT>
-__global__ void __launch_bounds__(kScanThreads, 1) bwd_finish_kernel(BwdParams p) {
-  constexpr int LDK = DK + 1;
-  constexpr int LDC = C + 1;
-  using L = Acc<DK>;
-  extern __shared__ float sm[];
-  float *Ks = sm;               // [C][LDK]
-  float *Qs = Ks + C * LDK;     // [C][LDK]
-  float *KK = Qs + C * LDK;     // [C][LDC]
-  float *QK = KK + C * LDC;     // [C][LDC]
-  float *dKK = QK + C * LDC;    // [C][LDC] symmetrised before use
-  float *dQK = dKK + C * LDC;   // [C][LDC]
-  float *colG = dQK + C * LDC;  // [C][LDC] column contributions to d cum
-  float *colB = colG + C * LDC; // [C][LDC] ... to dbeta
-  float *colM = colB + C * LDC; // [C][LDC] ... to dgamma
-  float *cum = colM + C * LDC;  // [C]
-  float *cprev = cum + C;
-  float *bet = cprev + C;
-  float *gam = bet + C;
-  float *gg = gam + C;
-  float *dcum = gg + C;
-  float *dcprev = dcum + C;
-  float *dbet = dcprev + C;
-  float *dgam = dbet + C;
+__global__ void __launch_bounds__(kPostThreads, 1) bwd_post_kernel(BwdParams p) {
+  using namespace simt;
+  using SM = PostSm<DK>;
+  constexpr int DV = DK, JS = SM::JS, LDJ = SM::LDJ, LDK = SM::LDK, LDC = SM::LDC;
+  constexpr int NH = DK / 64, NSL = DV / JS, NT = kPostThreads;
+  extern __shared__ __align__(16) float sm[];
+  float *Ks = sm + SM::K, *Qs = sm + SM::Q, *KK = sm + SM::KK, *QK = sm + SM::QK;
+  float *DKK = sm + SM::DKK, *DQK = sm + SM::DQK;
+  Cum &cum = *reinterpret_cast<Cum *>(sm + SM::VEC);
+  float *bet = sm + SM::VEC + 4 * C, *gam = bet + C, *Gam = gam + C, *Gprev = Gam + C;
+  float *wS = Gprev + C, *wR = wS + C, *dcum = wR + C, *dcprev = dcum + C, *dout = dcprev + C;
+  float *dwS = dout + C, *dwR = dwS + C;
 
   const long long chunk = blockIdx.x;
   if (chunk >= total_records(p.f)) return;  // (packed sequences: the grid is a bound)
@@ -494,269 +389,455 @@ __global__ void __launch_bounds__(kScanThreads, 1) bwd_finish_kernel(BwdParams p
   int sq, h, c;
   rec_decode(p.f, chunk, sq, h, c);
   const SeqSpan sp = seq_span(p.f, sq, h);
-  const long long tok0 = sp.tok0;
-  const int t0 = c * C;
-  const int n = min(C, sp.len - t0);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const InT *q = (const InT *)p.f.q;
-  const InT *k = (const InT *)p.f.k;
-  const float *acc = p.acc + (size_t)chunk * L::FLOATS;
+  const int n = min(C, sp.len - c * C);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, tx = tid & 15, ty = tid >> 4;
   const bool dec_res = p.f.mods & RDN_FLAG_DECAYED_RESIDUAL;
   const bool plain = p.f.mods & RDN_FLAG_PLAIN_COMBINE;
   const bool stl = p.f.mods & RDN_FLAG_STATELESS_AUX;
+  const bool rdn_aux = RDNV && !stl;
+  const size_t row0 = (size_t)(sp.tok0 + c * C) * H + h;
+  const size_t toff = (size_t)chunk * C * DV, soff = (size_t)chunk * DK * DV;
 
-  for (int e = tid; e < C * DK; e += kScanThreads) {
-    const int t = e / DK, d = e % DK;
-    float kv = 0.f, qv = 0.f;
-    if (t < n) {
-      const size_t off = ((size_t)(tok0 + t0 + t) * H + h) * DK + d;
-      kv = to_f32(k[off]);
-      qv = p.f.scale * to_f32(q[off]);
-    }
-    Ks[t * LDK + d] = kv;
-    Qs[t * LDK + d] = qv;
-  }
-  if (tid < C) {
-    const int t = tid;
-    float gv = 0.f, bv = 0.f, mv = 0.f;
-    if (t < n) {
-      const size_t off = (size_t)(tok0 + t0 + t) * H + h;
-      gv = p.f.g[off];
-      bv = p.f.beta[off];
-      mv = p.f.gamma[off];
-    }
-    gg[t] = gv;
-    bet[t] = bv;
-    gam[t] = mv;
-  }
-  __syncthreads();
-  if (warp == 0) {  // in-chunk cumulative log-decay (two 32-wide shuffle scans)
-    float a = gg[lane], b2 = gg[32 + lane];
+  // tiles of a slice: dO, then three [C] tiles and two [DK] tiles
+  auto tile = [&](int s, int i) {
+    return sm + SM::ST + (s & 1) * SM::STG + (i < 4 ? i * C : 4 * C + (i - 4) * DK) * LDJ;
+  };
+  RowTile<InT, JS, NT> dot;
+  auto issue = [&](int s) {
+    const bool base = s >= NSL;
+    const int j = (s % NSL) * JS;
+    dot.fetch((const InT *)p.dO + row0 * DV + j, (size_t)H * DV, n);
+    const float *src[3] = {base ? (const float *)p.f.sv_E : (const float *)p.f.sv_E2,
+                           base ? (RDNV ? p.dX : nullptr) : (rdn_aux ? p.dX2 : nullptr),
+                           base ? p.dVr : nullptr};
 #pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const float ua = __shfl_up_sync(0xffffffffu, a, off);
-      const float ub = __shfl_up_sync(0xffffffffu, b2, off);
-      if (lane >= off) {
-        a += ua;
-        b2 += ub;
-      }
+    for (int i = 0; i < 3; ++i) {
+      if (!src[i]) continue;
+      float *d = tile(s, 1 + i);
+      for (int e = tid; e < C * JS / 4; e += NT)
+        cp16(d + (e / (JS / 4)) * LDJ + 4 * (e % (JS / 4)),
+             src[i] + toff + (size_t)(e / (JS / 4)) * DV + j + 4 * (e % (JS / 4)));
     }
-    b2 += __shfl_sync(0xffffffffu, a, 31);
-    cum[lane] = a;
-    cum[32 + lane] = b2;
-    cprev[lane] = a - gg[lane];
-    cprev[32 + lane] = b2 - gg[32 + lane];
-  }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const float *g = base ? (i ? p.gS : p.Sc) : (i ? p.gR : p.Rc);
+      float *d = tile(s, 4 + i);
+      for (int e = tid; e < DK * JS / 4; e += NT)
+        cp16(d + (e / (JS / 4)) * LDJ + 4 * (e % (JS / 4)),
+             g + soff + (size_t)(e / (JS / 4)) * DV + j + 4 * (e % (JS / 4)));
+    }
+    cp_commit();
+  };
+
+  issue(0);
   {
-    using MM = BlockMM<C, C, DK, kScanThreads>;
-    float a[MM::RPT];
-    MM::run(Ks, LDK, 1, Ks, 1, LDK, a);
+    RowTile<InT, DK, NT> kt, qt;
+    kt.fetch((const InT *)p.f.k + row0 * DK, (size_t)H * DK, n);
+    qt.fetch((const InT *)p.f.q + row0 * DK, (size_t)H * DK, n);
+    if (warp == 0) {
+      float g2[2];
 #pragma unroll
-    for (int i = 0; i < MM::RPT; ++i) KK[MM::row(i) * LDC + MM::col()] = a[i];
-    MM::run(Qs, LDK, 1, Ks, 1, LDK, a);
-#pragma unroll
-    for (int i = 0; i < MM::RPT; ++i) QK[MM::row(i) * LDC + MM::col()] = a[i];
-  }
-  __syncthreads();
-  // ---- row pass over the C x C gradients
-  constexpr int kRowsPerWarp = C / (kScanThreads / 32);
-  for (int rr = 0; rr < kRowsPerWarp; ++rr) {
-    const int t = warp * kRowsPerWarp + rr;
-    float rowc = 0.f, rowp = 0.f;
-#pragma unroll
-    for (int half = 0; half < 2; ++half) {
-      const int i = lane + 32 * half;
-      const int e = t * C + i;
-      float dkk = 0.f, dqk = 0.f, cg = 0.f, cb = 0.f, cm = 0.f;
-      if (i <= t) {
-        const float dec = expf(cum[t] - cum[i]);
-        const float kk = KK[t * LDC + i], qk = QK[t * LDC + i];
-        const float bi = bet[i], gi = gam[i];
-        if (stl) {  // M2 = diag(QK): no decay, no rate
-          if (i == t) dqk += acc[L::DM2 + e];
-        } else {  // M2: inclusive, gamma, QK
-          const float dm = acc[L::DM2 + e];
-          const float G = dm * dec * gi * qk;
-          rowc += G;
-          cg += G;
-          cm += dm * dec * qk;
-          dqk += dm * dec * gi;
-        }
-        if (i < t) {
-          const float decp = expf(cprev[t] - cum[i]);
-          {  // Ap: strict, beta, KK, previous-token decay (decayed residual: to t)
-            const float dA = dec_res ? dec : decp;
-            const float dm = acc[L::DAP + e];
-            const float G = dm * dA * bi * kk;
-            if (dec_res) rowc += G; else rowp += G;
-            cg += G;
-            cb += dm * dA * kk;
-            dkk += dm * dA * bi;
-          }
-          {  // Mq: strict, beta, QK (plain combine: decay to t-1)
-            const float dA = plain ? decp : dec;
-            const float dm = acc[L::DMQ + e];
-            const float G = dm * dA * bi * qk;
-            if (plain) rowp += G; else rowc += G;
-            cg += G;
-            cb += dm * dA * qk;
-            dqk += dm * dA * bi;
-          }
-          if (RDNV) {
-            const float da = acc[L::DAB + e], dg2 = acc[L::DAG + e];
-            const float Gb = da * dec * bi * kk, Gg = dg2 * dec * gi * kk;
-            rowc += Gb + Gg;
-            cg += Gb + Gg;
-            cb += da * dec * kk;
-            cm += dg2 * dec * kk;
-            dkk += da * dec * bi + dg2 * dec * gi;
-          }
-        }
+      for (int u = 0; u < 2; ++u) {
+        const int t = lane + 32 * u;
+        const bool ok = t < n;
+        const size_t go = row0 + (size_t)(ok ? t : 0) * H;
+        g2[u] = ok ? p.f.g[go] : 0.f;
+        bet[t] = ok ? p.f.beta[go] : 0.f;
+        gam[t] = ok ? p.f.gamma[go] : 0.f;
       }
-      dKK[t * LDC + i] = dkk;
-      dQK[t * LDC + i] = dqk;
-      colG[t * LDC + i] = cg;
-      colB[t * LDC + i] = cb;
-      colM[t * LDC + i] = cm;
+      cum64(g2[0], g2[1], cum);
+    } else if (warp < 3) {
+      const float *rec = p.f.ws + (size_t)chunk * kRecFloats + OFF_VEC;
+      const int t = tid - 32;
+      Gam[t] = rec[V_GAM + t];
+      Gprev[t] = rec[V_GPREV + t];
+      wS[t] = rec[V_WS + t];
+      wR[t] = rec[V_WR + t];
     }
-#pragma unroll
-    for (int off = 16; off; off >>= 1) {
-      rowc += __shfl_xor_sync(0xffffffffu, rowc, off);
-      rowp += __shfl_xor_sync(0xffffffffu, rowp, off);
-    }
-    if (lane == 0) {
-      dcum[t] = rowc;
-      dcprev[t] = rowp;
-    }
+    kt.put(Ks, LDK, 1.f);
+    qt.put(Qs, LDK, p.f.scale);
+    dot.put(tile(0, 0), LDJ, 1.f);
   }
-  __syncthreads();
-  // ---- column pass and per-row factors
-  if (tid < C) {
-    const int i = tid;
-    float sg = 0.f, sb = 0.f, sm2 = 0.f;
-    for (int t = i; t < C; ++t) {
-      sg += colG[t * LDC + i];
-      sb += colB[t * LDC + i];
-      sm2 += colM[t * LDC + i];
-    }
-    const float cC = cum[C - 1];
-    const float eC = expf(cC - cum[i]);
-    const float dwS = acc[L::VEC + L::V_DWS + i], dwR = acc[L::VEC + L::V_DWR + i];
-    dbet[i] = sb + dwS * eC;
-    dgam[i] = sm2 + acc[L::VEC + L::V_DGAM_OUT + i] + dwR * eC;
-    // d cum_i: - column sums - (dwS wS + dwR wR) + dGam * Gam
-    dcum[i] += -sg - (dwS * bet[i] + dwR * gam[i]) * eC + acc[L::VEC + L::V_DGAM + i] * expf(cum[i]);
-    dcprev[i] += acc[L::VEC + L::V_DGPREV + i] * expf(cprev[i]);
-  }
-  __syncthreads();
-  if (warp == 0) {  // chunk-end terms land on cum_C = cum[C-1] (padding has g = 0)
-    const float cC = cum[C - 1];
-    float s = 0.f;
-    for (int t = lane; t < C; t += 32)
-      s += (acc[L::VEC + L::V_DWS + t] * bet[t] + acc[L::VEC + L::V_DWR + t] * gam[t]) *
-           expf(cC - cum[t]);
-#pragma unroll
-    for (int off = 16; off; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    if (lane == 0) dcum[C - 1] += s + acc[L::VEC + L::V_DGAMC] * expf(cC);
-  }
-  // symmetrise: dK gets (dKK + dKK^T) K
-  for (int e = tid; e < C * C; e += kScanThreads) {
-    const int t = e / C, i = e % C;
-    if (i < t) {
-      const float s2 = dKK[t * LDC + i] + dKK[i * LDC + t];
-      dKK[t * LDC + i] = s2;
-      dKK[i * LDC + t] = s2;
-    } else if (i == t) {
-      dKK[t * LDC + i] *= 2.f;
-    }
-  }
+  wait_groups<0>();
   __syncthreads();
   {
-    using MM = BlockMM<C, DK, C, kScanThreads>;
-    float a1[MM::RPT], a2[MM::RPT], a3[MM::RPT];
-    MM::run(dKK, LDC, 1, Ks, LDK, 1, a1);   // (dKK + dKK^T) K
-    MM::run(dQK, 1, LDC, Qs, LDK, 1, a2);   // dQK^T Q
-    MM::run(dQK, LDC, 1, Ks, LDK, 1, a3);   // dQK K
-    InT *dk = (InT *)p.dk;
-    InT *dq = (InT *)p.dq;
+    float a[4][4];
+    mm_nt<4, 4, DK>(Ks + 4 * ty * LDK, LDK, Ks + tx * LDK, 16 * LDK, a);
 #pragma unroll
-    for (int i = 0; i < MM::RPT; ++i) {
-      const int t = MM::row(i), d = MM::col();
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) KK[(4 * ty + i) * LDC + tx + 16 * j] = a[i][j];
+    mm_nt<4, 4, DK>(Qs + 4 * ty * LDK, LDK, Ks + tx * LDK, 16 * LDK, a);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) QK[(4 * ty + i) * LDC + tx + 16 * j] = a[i][j];
+  }
+
+  float dk[4][4 * NH], dq[4][4 * NH];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4 * NH; ++j) dk[i][j] = dq[i][j] = 0.f;
+  // per-row partial sums over this thread's columns: gradients w.r.t. the
+  // cumulative decay to t and to t - 1, dgamma of the read-out, dwS, dwR;
+  // per-column sums over its rows: decay, dbeta, dgamma; <dS, S0> + <dR, R0>
+  float pc[4] = {0.f, 0.f, 0.f, 0.f}, pp[4] = {0.f, 0.f, 0.f, 0.f}, po[4] = {0.f, 0.f, 0.f, 0.f};
+  float ps[4] = {0.f, 0.f, 0.f, 0.f}, pr[4] = {0.f, 0.f, 0.f, 0.f};
+  float cg[4] = {0.f, 0.f, 0.f, 0.f}, cb[4] = {0.f, 0.f, 0.f, 0.f}, cm[4] = {0.f, 0.f, 0.f, 0.f};
+  float dgc = 0.f;
+
+  // acc_t += f_t (X St^T)_t over the slice, and s_t += (rows_t . (X St^T)_t)
+  auto state_mm = [&](const float *X, const float *St, const float *rows, const float (&f)[4],
+                      float (&acc)[4][4 * NH], float (&s)[4]) {
+#pragma unroll
+    for (int hb = 0; hb < NH; ++hb) {
+      float a[4][4];
+      mm_nt<4, 4, JS>(X + 4 * ty * LDJ, LDJ, St + (64 * hb + tx) * LDJ, 16 * LDJ, a);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          s[i] = fmaf(rows[(4 * ty + i) * LDK + 64 * hb + tx + 16 * j], a[i][j], s[i]);
+          acc[i][4 * hb + j] = fmaf(f[i], a[i][j], acc[i][4 * hb + j]);
+        }
+    }
+  };
+  auto add_nt = [&](const float *X, const float *Y, float (&g)[4][4]) {
+    float a[4][4];
+    mm_nt<4, 4, JS>(X + 4 * ty * LDJ, LDJ, Y + tx * LDJ, 16 * LDJ, a);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) g[i][j] += a[i][j];
+  };
+  auto state_dot = [&](const float *A, const float *B) {
+    for (int e = tid; e < DK * JS / 4; e += NT) {
+      const int o = (e / (JS / 4)) * LDJ + 4 * (e % (JS / 4));
+      float a[4], b[4];
+      ldv<4>(A + o, a);
+      ldv<4>(B + o, b);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) dgc = fmaf(a[i], b[i], dgc);
+    }
+  };
+
+  {  // ---- the auxiliary pass
+    float g1[4][4], g2[4][4], s1[4] = {0.f, 0.f, 0.f, 0.f}, s2[4] = {0.f, 0.f, 0.f, 0.f};
+    zero(g1);
+    zero(g2);
+    float fq[4], fk[4], fr[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int t = 4 * ty + i;
+      fq[i] = plain ? Gam[t] : gam[t] * Gam[t];
+      fk[i] = -Gam[t];
+      fr[i] = wR[t];
+    }
+    for (int s = 0; s < NSL; ++s) {
+      issue(s + 1);
+      const float *dO = tile(s, 0), *e2 = tile(s, 1), *x2 = tile(s, 2), *r0 = tile(s, 4), *dr = tile(s, 5);
+      if (!stl) {
+        state_mm(dO, r0, Qs, fq, dq, s1);
+        state_dot(dr, r0);
+      }
+      state_mm(e2, dr, Ks, fr, dk, pr);
+      add_nt(dO, e2, g1);
+      if (rdn_aux) {
+        state_mm(x2, r0, Ks, fk, dk, s2);
+        add_nt(x2, e2, g2);
+      }
+      dot.put(tile(s + 1, 0), LDJ, 1.f);
+      wait_groups<0>();
+      __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int t = 4 * ty + i;
+      pc[i] = fq[i] * s1[i] - Gam[t] * s2[i];
+      if (!plain) po[i] = Gam[t] * s1[i];
+      if (stl) pr[i] = 0.f;  // (wR is then a constant)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int u = tx + 16 * j;
+        float dkk = 0.f, dqk = 0.f;
+        if (u <= t) {
+          const float dec = expf(cum.to(t, u));
+          const float kk = KK[t * LDC + u], qk = QK[t * LDC + u], gu = gam[u];
+          const float dm = plain ? g1[i][j] : gam[t] * g1[i][j];  // dM2
+          if (stl) {  // M2 = diag(QK): no decay, no rate
+            if (u == t) {
+              dqk = dm;
+              if (!plain) po[i] = fmaf(qk, g1[i][j], po[i]);
+            }
+          } else {
+            const float m = dec * qk;
+            if (!plain) po[i] = fmaf(m * gu, g1[i][j], po[i]);
+            const float G = dm * m * gu;
+            pc[i] += G;
+            cg[j] += G;
+            cm[j] = fmaf(dm, m, cm[j]);
+            dqk = dm * dec * gu;
+            if (rdn_aux && u < t) {  // A_gamma
+              const float da = -g2[i][j], Gg = da * dec * gu * kk;
+              pc[i] += Gg;
+              cg[j] += Gg;
+              cm[j] = fmaf(da * dec, kk, cm[j]);
+              dkk = da * dec * gu;
+            }
+          }
+        }
+        DKK[t * LDC + u] = dkk;
+        DQK[t * LDC + u] = dqk;
+      }
+    }
+  }
+  {  // ---- the base pass
+    float g3[4][4], g4[4][4], g5[4][4];
+    float s4[4] = {0.f, 0.f, 0.f, 0.f}, s5[4] = {0.f, 0.f, 0.f, 0.f}, s6[4] = {0.f, 0.f, 0.f, 0.f};
+    zero(g3);
+    zero(g4);
+    zero(g5);
+    float fq[4], fp[4], fk[4], fs[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int t = 4 * ty + i;
+      fq[i] = plain ? Gprev[t] : Gam[t];
+      fp[i] = dec_res ? -Gam[t] : -Gprev[t];
+      fk[i] = -Gam[t];
+      fs[i] = wS[t];
+    }
+    for (int s = NSL; s < 2 * NSL; ++s) {
+      if (s + 1 < 2 * NSL) issue(s + 1);
+      const float *dO = tile(s, 0), *e = tile(s, 1), *dx = tile(s, 2), *dvr = tile(s, 3);
+      const float *s0 = tile(s, 4), *ds = tile(s, 5);
+      state_mm(dO, s0, Qs, fq, dq, s4);
+      state_mm(dvr, s0, Ks, fp, dk, s5);
+      if (RDNV) state_mm(dx, s0, Ks, fk, dk, s6);
+      state_mm(e, ds, Ks, fs, dk, ps);
+      state_dot(ds, s0);
+      add_nt(dO, e, g3);
+      add_nt(dvr, e, g4);
+      if (RDNV) add_nt(dx, e, g5);
+      if (s + 1 < 2 * NSL) {
+        dot.put(tile(s + 1, 0), LDJ, 1.f);
+        wait_groups<0>();
+      }
+      __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int t = 4 * ty + i;
+      (plain ? pp : pc)[i] += fq[i] * s4[i];
+      (dec_res ? pc : pp)[i] += fp[i] * s5[i];
+      if (RDNV) pc[i] += fk[i] * s6[i];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int u = tx + 16 * j;
+        if (u < t) {
+          const float dec = expf(cum.to(t, u)), decp = expf(cum.before(t, u));
+          const float kk = KK[t * LDC + u], qk = QK[t * LDC + u], bu = bet[u];
+          float dkk = DKK[t * LDC + u];
+          {  // Ap: previous-token decay (decayed residual: to t)
+            const float dA = dec_res ? dec : decp, dm = -g4[i][j], G = dm * dA * bu * kk;
+            (dec_res ? pc : pp)[i] += G;
+            cg[j] += G;
+            cb[j] = fmaf(dm * dA, kk, cb[j]);
+            dkk = fmaf(dm * dA, bu, dkk);
+          }
+          {  // Mq (plain combine: decay to t - 1)
+            const float dA = plain ? decp : dec, dm = g3[i][j], G = dm * dA * bu * qk;
+            (plain ? pp : pc)[i] += G;
+            cg[j] += G;
+            cb[j] = fmaf(dm * dA, qk, cb[j]);
+            DQK[t * LDC + u] += dm * dA * bu;
+          }
+          if (RDNV) {  // A_beta
+            const float da = -g5[i][j], Gb = da * dec * bu * kk;
+            pc[i] += Gb;
+            cg[j] += Gb;
+            cb[j] = fmaf(da * dec, kk, cb[j]);
+            dkk = fmaf(da * dec, bu, dkk);
+          }
+          // both halves of the symmetric d(KK^T) (its diagonal is zero)
+          DKK[t * LDC + u] = dkk;
+          DKK[u * LDC + t] = dkk;
+        }
+      }
+    }
+  }
+  // ---- row sums over the 16 lanes, column sums over the block
+  float *colp = sm + SM::ST;  // [8 warps][3][C], then the warps' dgc
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+#pragma unroll
+    for (int o = 8; o; o >>= 1) {
+      pc[i] += __shfl_xor_sync(0xffffffffu, pc[i], o);
+      pp[i] += __shfl_xor_sync(0xffffffffu, pp[i], o);
+      po[i] += __shfl_xor_sync(0xffffffffu, po[i], o);
+      ps[i] += __shfl_xor_sync(0xffffffffu, ps[i], o);
+      pr[i] += __shfl_xor_sync(0xffffffffu, pr[i], o);
+    }
+    if (tx == 0) {
+      const int t = 4 * ty + i;
+      dcum[t] = pc[i];
+      dcprev[t] = pp[i];
+      dout[t] = po[i];
+      dwS[t] = ps[i];
+      dwR[t] = pr[i];
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    cg[j] += __shfl_xor_sync(0xffffffffu, cg[j], 16);
+    cb[j] += __shfl_xor_sync(0xffffffffu, cb[j], 16);
+    cm[j] += __shfl_xor_sync(0xffffffffu, cm[j], 16);
+    if (lane < 16) {
+      colp[(warp * 3 + 0) * C + tx + 16 * j] = cg[j];
+      colp[(warp * 3 + 1) * C + tx + 16 * j] = cb[j];
+      colp[(warp * 3 + 2) * C + tx + 16 * j] = cm[j];
+    }
+  }
+#pragma unroll
+  for (int o = 16; o; o >>= 1) dgc += __shfl_xor_sync(0xffffffffu, dgc, o);
+  if (lane == 0) colp[24 * C + warp] = dgc;
+  __syncthreads();
+  if (warp == 0) {  // the gates' gradients, lane l for tokens l and 32 + l
+    float a[2], b[2], dg2 = 0.f, ends = 0.f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) dg2 += colp[24 * C + w];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int t = lane + 32 * u;
+      float sg = 0.f, sb = 0.f, sg2 = 0.f;
+#pragma unroll
+      for (int w = 0; w < 8; ++w) {
+        sg += colp[(w * 3 + 0) * C + t];
+        sb += colp[(w * 3 + 1) * C + t];
+        sg2 += colp[(w * 3 + 2) * C + t];
+      }
+      const float eC = expf(cum.to(C - 1, t));
+      const float we = (dwS[t] * bet[t] + dwR[t] * gam[t]) * eC;
+      ends += we;
+      a[u] = dcum[t] - sg - we;
+      b[u] = dcprev[t];
       if (t < n) {
-        const size_t off = ((size_t)(tok0 + t0 + t) * H + h) * DK + d;
-        const float gk = acc[L::DKo + t * DK + d] + a1[i] + a2[i];
-        const float gq = p.f.scale * (acc[L::DQo + t * DK + d] + a3[i]);
+        const size_t off = row0 + (size_t)t * H;
+        p.dbeta[off] = sb + dwS[t] * eC;
+        p.dgamma[off] = sg2 + dout[t] + dwR[t] * eC;
+      }
+    }
+    // the chunk-end terms land on the last token (padding has g = 0)
+#pragma unroll
+    for (int o = 16; o; o >>= 1) ends += __shfl_xor_sync(0xffffffffu, ends, o);
+    if (lane == 31) a[1] += ends + dg2 * expf(cum.hi[C - 1]);
+    // dg_s = sum_{t >= s} dcum_t + sum_{t > s} dcprev_t: suffix sums
+    float x0 = a[0] + b[0], x1 = a[1] + b[1];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const float y0 = __shfl_down_sync(0xffffffffu, x0, o), y1 = __shfl_down_sync(0xffffffffu, x1, o);
+      if (lane + o < 32) {
+        x0 += y0;
+        x1 += y1;
+      }
+    }
+    x0 += __shfl_sync(0xffffffffu, x1, 0);
+    if (lane < n) p.dg[row0 + (size_t)lane * H] = x0 - b[0];
+    if (lane + 32 < n) p.dg[row0 + (size_t)(lane + 32) * H] = x1 - b[1];
+  }
+  // ---- dk += (dKK + dKK^T) K + dQK^T Q;  dq += dQK K
+#pragma unroll 1
+  for (int hb = 0; hb < NH; ++hb) {
+    float ak[4][4], aq[4][4];
+    zero(ak);
+    zero(aq);
+#pragma unroll 1
+    for (int k = 0; k < C; k += 4) {
+      float s[4][4], q4[4][4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        ldv<4>(DKK + (4 * ty + i) * LDC + k, s[i]);
+        ldv<4>(DQK + (4 * ty + i) * LDC + k, q4[i]);
+      }
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk) {
+        float m[4];  // row k of dQK: dQK^T's column
+        ldv<4>(DQK + (k + kk) * LDC + 4 * ty, m);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int o = (k + kk) * LDK + 64 * hb + tx + 16 * j;
+          const float kv = Ks[o], qv = Qs[o];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            ak[i][j] = fmaf(s[i][kk], kv, ak[i][j]);
+            ak[i][j] = fmaf(m[i], qv, ak[i][j]);
+            aq[i][j] = fmaf(q4[i][kk], kv, aq[i][j]);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int t = 4 * ty + i;
+      if (t >= n) continue;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const size_t off = (row0 + (size_t)t * H) * DK + 64 * hb + tx + 16 * j;
+        const float gk = (NH == 1 || hb == 0 ? dk[i][j] : dk[i][4 * (NH - 1) + j]) + ak[i][j];
+        const float gq = p.f.scale * ((NH == 1 || hb == 0 ? dq[i][j] : dq[i][4 * (NH - 1) + j]) + aq[i][j]);
         if (p.gq32) {
           p.gk32[off] = gk;
           p.gq32[off] = gq;
         } else {
-          dk[off] = from_f32<InT>(gk);
-          dq[off] = from_f32<InT>(gq);
+          ((InT *)p.dk)[off] = from_f32<InT>(gk);
+          ((InT *)p.dq)[off] = from_f32<InT>(gq);
         }
       }
     }
   }
-  if (warp == 0) {  // dg_s = sum_{t>=s} dcum_t + sum_{t>s} dcprev_t (reverse scans)
-    float a = dcum[C - 1 - lane], b2 = dcum[31 - lane];
-    float pa = dcprev[C - 1 - lane], pb = dcprev[31 - lane];
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const float ua = __shfl_up_sync(0xffffffffu, a, off), ub = __shfl_up_sync(0xffffffffu, b2, off);
-      const float upa = __shfl_up_sync(0xffffffffu, pa, off), upb = __shfl_up_sync(0xffffffffu, pb, off);
-      if (lane >= off) {
-        a += ua;
-        b2 += ub;
-        pa += upa;
-        pb += upb;
-      }
-    }
-    // a: suffix sums over t in [C-1-lane, C) ; b2 over [31-lane, 32) plus the upper half
-    const float topc = __shfl_sync(0xffffffffu, a, 31), topp = __shfl_sync(0xffffffffu, pa, 31);
-    b2 += topc;
-    pb += topp;
-    // sum_{t>s} dcprev_t = (suffix including s) - dcprev_s
-    gg[C - 1 - lane] = a + (pa - dcprev[C - 1 - lane]);
-    gg[31 - lane] = b2 + (pb - dcprev[31 - lane]);
-  }
-  __syncthreads();
-  if (tid < n) {
-    const size_t off = (size_t)(tok0 + t0 + tid) * H + h;
-    p.dg[off] = gg[tid];
-    p.dbeta[off] = dbet[tid];
-    p.dgamma[off] = dgam[tid];
-  }
 }
 
-template <int DK>
-constexpr size_t scan_smem() {
-  return sizeof(float) * (2 * C * (DK + 1) + 4 * DK * LDV + C * C + 13 * C * LDV + 6 * C + C + 6 * C);
-}
-template <int DK>
-constexpr size_t finish_smem() {
-  return sizeof(float) * (2 * C * (DK + 1) + 7 * C * (C + 1) + 9 * C);
-}
-
-template <int DK, bool RDNV, typename InT>
-cudaError_t launch_t(const BwdParams &p, cudaStream_t s) {
-  auto scan = bwd_scan_kernel<DK, RDNV, InT>;
-  auto fin = bwd_finish_kernel<DK, RDNV, InT>;
-  cudaError_t e;
-  if ((e = cudaFuncSetAttribute(scan, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)scan_smem<DK>())) != cudaSuccess)
-    return e;
-  if ((e = cudaFuncSetAttribute(fin, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)finish_smem<DK>())) != cudaSuccess)
-    return e;
-  RDN_LAUNCH("bwd_scan", s, scan<<<dim3(p.f.nseq * p.f.H, DK / kBDVS), kScanThreads, scan_smem<DK>(), s>>>(p));
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  RDN_LAUNCH("bwd_finish", s, fin<<<(unsigned)p.f.nrec, kScanThreads, finish_smem<DK>(), s>>>(p));
+template <int DK, bool RDNV, typename InT, int DVS, int NT>
+cudaError_t launch_chain_t(const BwdParams &p, cudaStream_t s) {
+  auto chain = bwd_chain_kernel<DK, RDNV, InT, DVS, NT>;
+  constexpr int smem = (int)sizeof(float) * ChainSm<DK, DVS, NT>::FLOATS;
+  const cudaError_t e = cudaFuncSetAttribute(chain, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  RDN_LAUNCH("bwd_chain_f32", s, chain<<<dim3(p.f.nseq * p.f.H, DK / DVS), NT, smem, s>>>(p));
   return cudaGetLastError();
 }
+
+struct RunBwd {
+  const BwdParams &p;
+  cudaStream_t s;
+  template <int DK, bool RDNV, typename InT>
+  cudaError_t run() const {
+    int nsm = 0;
+    cudaError_t e = sm_count(&nsm);
+    if (e != cudaSuccess) return e;
+    const int dvs = scan_columns(DK, (long long)p.f.nseq * p.f.H, nsm);
+    if constexpr (DK == 64) {
+      e = dvs == 16 ? launch_chain_t<64, RDNV, InT, 16, 128>(p, s)
+                    : launch_chain_t<64, RDNV, InT, 8, 128>(p, s);
+    } else {
+      e = dvs == 32   ? launch_chain_t<128, RDNV, InT, 32, 256>(p, s)
+          : dvs == 16 ? launch_chain_t<128, RDNV, InT, 16, 256>(p, s)
+                      : launch_chain_t<128, RDNV, InT, 8, 256>(p, s);
+    }
+    if (e != cudaSuccess) return e;
+    auto post = bwd_post_kernel<DK, RDNV, InT>;
+    constexpr int smem = (int)sizeof(float) * PostSm<DK>::FLOATS;
+    if ((e = cudaFuncSetAttribute(post, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
+      return e;
+    RDN_LAUNCH("bwd_post_f32", s, post<<<(unsigned)p.f.nrec, kPostThreads, smem, s>>>(p));
+    return cudaGetLastError();
+  }
+};
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct BwdLayout {
-  size_t prep, acc, states, o, tc, qk, g32, tied, seq, total;
+  size_t prep, chain, saved, states, o, tc, qk, g32, tied, seq, total;
 };
 
 // bf16 inputs with d = 128 take the tensor-core backward (RDN, and RLA with
@@ -771,16 +852,22 @@ bool use_tc_bwd(const rdn_fwd_args &f, int variant) {
 // the format this backward reads: both choose their kernels by fwd_uses_tc).
 bool reuse_fwd_records(const rdn_fwd_args &f) { return f.workspace && f.S_chunks; }
 
+// ... and E, E2 and the mask (RDN_FLAG_SAVE_FOR_BWD) with them
+bool fwd_saved(const rdn_fwd_args &f) {
+  return reuse_fwd_records(f) && (f.flags & RDN_FLAG_SAVE_FOR_BWD);
+}
+
 BwdLayout layout(const rdn_bwd_args &a, int variant) {
   const rdn_fwd_args &f = a.fwd;
   const bool tc = use_tc_bwd(f, variant);
   const long long nrec = call_records(f);  // record slots
-  const size_t accf = f.Dk == 128 ? Acc<128>::FLOATS : Acc<64>::FLOATS;
   BwdLayout l;
   // the forward's records are read from its workspace when it is passed
   l.prep = reuse_fwd_records(f) ? 0 : align256(sizeof(float) * nrec * kRecFloats);
-  // (the tensor-core kernels keep their per-chunk sums in shared memory)
-  l.acc = tc ? 0 : align256(sizeof(float) * nrec * accf);
+  // what the fp32 chain keeps of each chunk (the tensor-core kernels': l.tc)
+  l.chain = tc ? 0 : align256(sizeof(float) * nrec * (3 * C * f.Dv + 2 * f.Dk * f.Dv));
+  // E, E2 and the residual's mask, unless the forward kept them
+  l.saved = tc || fwd_saved(f) ? 0 : align256(saved_layout(f).bytes);
   const bool need_states = f.S_chunks == nullptr;
   l.states = need_states ? align256(sizeof(float) * nrec * f.Dk * f.Dv) : 0;  // each of S, R
   const size_t esz = f.dtype == RDN_BF16 ? 2 : 4;
@@ -800,7 +887,7 @@ BwdLayout layout(const rdn_bwd_args &a, int variant) {
                ? align256(sizeof(float) * (size_t)f.B * f.T * f.H)
                : 0;
   // + the packed-sequence table and a 256-byte tail
-  l.total = l.prep + l.acc + 2 * l.states + l.o + l.tc + l.qk + l.g32 + l.tied + l.seq + 256;
+  l.total = l.prep + l.chain + l.saved + 2 * l.states + l.o + l.tc + l.qk + l.g32 + l.tied + l.seq + 256;
   return l;
 }
 
@@ -868,12 +955,14 @@ static cudaError_t launch_bwd_impl(const rdn_bwd_args &a, int variant, cudaStrea
   }
   if (p.f.qk_norm)  // the normalised q, k: the forward's, or made with this call's records
     set_qk_norm_copies(p.f, f, reuse ? (char *)f.workspace + qk_norm_offset(f)
-                                     : ws + l.prep + l.acc + 2 * l.states + l.o + l.tc);
-  if (reuse && (f.flags & RDN_FLAG_SAVE_FOR_BWD)) {  // E, E2 and the mask kept by the forward
+                                     : ws + l.prep + l.chain + l.saved + 2 * l.states + l.o + l.tc);
+  const bool saved = fwd_saved(f);
+  if (saved || l.saved) {  // E, E2 and the mask: kept by the forward, or made here
     const SavedLayout sl = saved_layout(f);
-    p.f.sv_E = (uint8_t *)f.workspace + sl.e;
-    p.f.sv_E2 = (uint8_t *)f.workspace + sl.e2;
-    p.f.sv_mask = (unsigned long long *)((char *)f.workspace + sl.mask);
+    char *base = saved ? (char *)f.workspace : ws + l.prep + l.chain - sl.e;
+    p.f.sv_E = (uint8_t *)base + sl.e;
+    p.f.sv_E2 = (uint8_t *)base + sl.e2;
+    p.f.sv_mask = (unsigned long long *)(base + sl.mask);
   }
   p.f.ST = p.f.RT = nullptr;
   const bool bf = f.dtype == RDN_BF16;
@@ -881,17 +970,24 @@ static cudaError_t launch_bwd_impl(const rdn_bwd_args &a, int variant, cudaStrea
   const bool tc = use_tc_bwd(f, variant);
   cudaError_t e = cudaSuccess;  // (nothing to launch first when both the states and records are reused)
   if (f.S_chunks == nullptr) {  // recompute the chunk-start states
-    p.f.S_chunks = (float *)(ws + l.prep + l.acc);
-    p.f.R_chunks = (float *)(ws + l.prep + l.acc + l.states);
-    p.f.o = ws + l.prep + l.acc + 2 * l.states;
+    p.f.S_chunks = (float *)(ws + l.prep + l.chain + l.saved);
+    p.f.R_chunks = (float *)(ws + l.prep + l.chain + l.saved + l.states);
+    p.f.o = ws + l.prep + l.chain + l.saved + 2 * l.states;
     e = launch_fwd_parts(p.f, f.Dk, rdnv, bf, s);
   } else if (!reuse) {
     e = launch_prep(p.f, f.Dk, rdnv, bf, s);
   }
+  // chunk-start states without the forward's intermediates: remake them chunk
+  // by chunk (a forward run above wrote them as it went)
+  if (e == cudaSuccess && !tc && f.S_chunks && !saved) e = launch_recompute(p.f, f.Dk, rdnv, bf, s);
   if (e != cudaSuccess) return e;
   p.Sc = p.f.S_chunks;
   p.Rc = p.f.R_chunks;
-  p.acc = (float *)(ws + l.prep);
+  p.dX2 = (float *)(ws + l.prep);
+  p.dVr = p.dX2 + (size_t)p.f.nrec * C * f.Dv;
+  p.dX = p.dVr + (size_t)p.f.nrec * C * f.Dv;
+  p.gS = p.dX + (size_t)p.f.nrec * C * f.Dv;
+  p.gR = p.gS + (size_t)p.f.nrec * f.Dk * f.Dv;
   p.dO = a.dO;
   p.dST = a.dST;
   p.dRT = a.dRT;
@@ -905,23 +1001,16 @@ static cudaError_t launch_bwd_impl(const rdn_bwd_args &a, int variant, cudaStrea
   p.dR0 = a.dR0;
   p.gq32 = p.gk32 = nullptr;
   if (l.g32) {
-    p.gq32 = (float *)(ws + l.prep + l.acc + 2 * l.states + l.o + l.tc + l.qk);
+    p.gq32 = (float *)(ws + l.prep + l.chain + l.saved + 2 * l.states + l.o + l.tc + l.qk);
     p.gk32 = p.gq32 + (size_t)f.B * f.T * f.H * f.Dk;
   }
   if (tc) {  // (with the normalisation: dq, dk into the fp32 copies, as fp32 results)
     e = launch_bwd_tc(p.f, a.dO, a.dST, a.dRT, p.Sc, p.Rc, p.gq32 ? p.gq32 : a.dq,
                       p.gk32 ? p.gk32 : a.dk, a.dv, a.dg, a.dbeta, a.dgamma, a.dS0, a.dR0,
-                      ws + l.prep + l.acc + 2 * l.states + l.o, !rdnv, grad_f32,
+                      ws + l.prep + l.chain + l.saved + 2 * l.states + l.o, !rdnv, grad_f32,
                       p.gq32 != nullptr, s);
   } else {
-    if ((e = cudaMemsetAsync(p.acc, 0, l.acc, s)) != cudaSuccess) return e;
-    if (rdnv) {
-      if (f.Dk == 128) e = bf ? launch_t<128, true, __nv_bfloat16>(p, s) : launch_t<128, true, float>(p, s);
-      else e = bf ? launch_t<64, true, __nv_bfloat16>(p, s) : launch_t<64, true, float>(p, s);
-    } else {
-      if (f.Dk == 128) e = bf ? launch_t<128, false, __nv_bfloat16>(p, s) : launch_t<128, false, float>(p, s);
-      else e = bf ? launch_t<64, false, __nv_bfloat16>(p, s) : launch_t<64, false, float>(p, s);
-    }
+    e = simt_dispatch(f.Dk, rdnv, bf, RunBwd{p, s});
   }
   if (e != cudaSuccess || !p.f.qk_norm) return e;
   // dq, dk w.r.t. the caller's x: the normalisation's transposed Jacobian, in place

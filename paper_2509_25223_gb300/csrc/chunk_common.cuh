@@ -27,31 +27,6 @@ constexpr int kRecFloats = OFF_VEC + 6 * C;
 constexpr int IMG_TB = 0, IMG_APMQ = 16384, IMG_TG = 49152, IMG_M2 = 65536;
 static_assert(IMG_M2 + 16384 == OFF_VEC * 4, "image fills the matrix part of the record");
 
-// Block-level fp32 product over shared memory (NT threads): the calling thread
-// gets acc[i] = sum_k A(m_i, k) B(k, n) for n = tid % N and m_i = tid / N + i * (NT / N).
-// A(m,k) = A[m*a_m + k*a_k], B(k,n) = B[k*b_k + n*b_n].  With N >= 32 the lanes
-// of a warp share m, so A reads are broadcasts.
-template <int M, int N, int K, int NT = kThreads>
-struct BlockMM {
-  static constexpr int RG = NT / N;
-  static constexpr int RPT = M / RG;
-  static_assert(NT % N == 0 && M % RG == 0, "tile");
-  __device__ static __forceinline__ void run(const float *A, int a_m, int a_k, const float *B,
-                                             int b_k, int b_n, float (&acc)[RPT]) {
-    const int n = threadIdx.x % N, rg = threadIdx.x / N;
-#pragma unroll
-    for (int i = 0; i < RPT; ++i) acc[i] = 0.f;
-#pragma unroll 4
-    for (int k = 0; k < K; ++k) {
-      const float bv = B[k * b_k + n * b_n];
-#pragma unroll
-      for (int i = 0; i < RPT; ++i) acc[i] = fmaf(A[(rg + i * RG) * a_m + k * a_k], bv, acc[i]);
-    }
-  }
-  __device__ static __forceinline__ int row(int i) { return threadIdx.x / N + i * RG; }
-  __device__ static __forceinline__ int col() { return threadIdx.x % N; }
-};
-
 // T = (I + A)^-1 for a strictly lower 64 x 64 A, by 128 threads (g = thread
 // index in the group); W is 32 x 32 scratch (row stride LDW; the block of Tm
 // at rows 0..31, columns 32..63 will do, which no stage touches).  The caller synchronises the
