@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(NTC, 1) bwd_pair_kernel(const __grid_constant_
       // (a phase that has not completed takes no further arrival)
       if (got && tid == 0 && c > 0) mbar_expect_tx(barX, 32768);
       __syncwarp();
-      if (got && (tid & 31) == 0) mbar_arrive_remote(peer_bar);
+      if (got && (tid & 31) == 0) mbar_arrive_remote_relaxed(peer_bar);
 #pragma unroll
       for (int i = 0; i < 16; ++i) {
         if (tnh) {  // the derivative of c tanh(x / c) instead of the mask

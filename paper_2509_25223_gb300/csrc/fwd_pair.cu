@@ -7,23 +7,32 @@
 // reads the auxiliary one: CTA 0 carries S, forms E, the clipped residual r
 // and the base output Ob, and sends r and Ob (32 fp32 values a thread, the
 // same thread mapping on both sides) into CTA 1's shared memory; CTA 1 carries
-// R and finishes the output, one chunk behind.  Each has three phases a chunk
-// where the one-CTA scan has six:
+// R and finishes the output, one chunk behind.  Products and arithmetic are
+// those of fwd_tc.cu, in the same order: the results are the same bits.
 //
-//   CTA 0:  MMA1 [KS | QS]  |  MMA2 E  |  MMA3 [P | Ob], MMA4 S        -> r, Ob
-//   CTA 1:  MMA5 [KR | QR]  |  MMA6 E2 |  MMA7 Ob += .., MMA8 R        -> o
+// Within a CTA only the carried state is a chain (operand names as there):
 //
-// (phases, operands and arithmetic as in fwd_tc.cu, in the same order: the
-// results are the same bits).  The hand-over is one 64 KB buffer in CTA 1,
-// filled by two bulk copies from CTA 0's shared memory, with a pair of
-// mbarriers: `full` in CTA 1 (the copies' bytes), `empty` in CTA 0 (one arrival
-// per warp of CTA 1 once it holds the values in registers; CTA 0 then also
-// reuses what it copied from).  Both waits are bounded like every other; a CTA
-// that gave up stops, its partner's waits then run out too, and the two meet
-// at the cluster's barrier before either releases its shared memory.
+//   CTA 0:  K S  ->  X  ->  MMA2 E   ->  wS E   ->  MMA4 S  ->  S's copies
+//   CTA 1:  K R  ->  X2 ->  MMA6 E2  ->  wR E2  ->  MMA8 R  ->  R's copy
 //
-// Measured: B = 2, H = 16, T = 16384 with states, 2.24 ms in one CTA per head,
-// 1.59 ms in pairs; B = 1, T = 777, 0.123 and 0.095 ms.
+// and what hangs off it is issued behind it on the tensor pipe and finished
+// under a later phase: MMA3 [P | Ob] and MMA7 behind MMA4 and MMA8 on a barrier
+// of their own, their read-outs (r and Ob handed over; o stored) under the next
+// chunk's first product, whose accumulators are a second set of TMEM columns.
+// The products are issued by a warp of their own and the copies by another: an
+// issuing thread is held for most of its products' time (54 cycles a 128 x 64 x
+// 16 product, 70 a 128 x 128 x 16 one, which the operands' shared-memory reads
+// set); as one of the 16 element-wise warps it held up all the others, and
+// issuing the copies as well it delayed the next chunk's K and Q by 800 cycles.
+//
+// The hand-over is one 64 KB buffer in CTA 1, filled by bulk copies of each
+// warp's part from CTA 0's shared memory, with a pair of mbarriers: `full` in
+// CTA 1 (the copies' bytes), `empty` in CTA 0 (one arrival per warp of CTA 1
+// once it holds the values in registers; CTA 0 then also reuses what it copied
+// from).  Every wait is bounded: a thread whose wait gave up sets the CTA's
+// flag, which all read after the next chunk's first barrier; a CTA that gave up
+// stops, its partner's waits then run out too, and the two meet at the
+// cluster's barrier before either releases its shared memory.
 #include "fwd_tc.cuh"
 
 namespace rdn {
@@ -34,29 +43,39 @@ using namespace fwdtc;
 // shared memory (bytes from the 1024-aligned base); both CTAs:
 constexpr uint32_t SM_ST = 0;        // the carried state's bf16 copy, two 64-column blocks
 constexpr uint32_t SM_KQ = 32768;    // [K ; Q], 128 rows x 128
-constexpr uint32_t SM_XE = 65536;    // X^T then E^T (X2^T then E2^T), hi | lo; CTA 0: from a
-constexpr uint32_t SM_XE_LO = 81920; // chunk's end to the next MMA1 the state's lo part
-constexpr uint32_t SM_W = 98304;     // (wS E)^T / (wR E2)^T, hi | lo; then CTA 0: Ob, fp32, to
-constexpr uint32_t SM_W_LO = 114688; // be handed over; CTA 1: the o tile
+constexpr uint32_t SM_XE = 65536;    // X^T then E^T (X2^T then E2^T), hi | lo
+constexpr uint32_t SM_XE_LO = 81920;
+constexpr uint32_t SM_OUT = 98304;   // CTA 0: Ob, fp32, being handed over; CTA 1: o's rows
 constexpr uint32_t SM_SLOTA = 131072;  // T_beta / T_gamma image (hi | lo)
-constexpr uint32_t SM_SLOTB = 147456;  // CTA 0: [Ap ; Mq] image, 32 KB; CTA 1: M2 image, 16 KB
-// CTA 0: r, fp32, to be handed over (32 KB), V;  CTA 1: the hand-over buffer (r | Ob)
+constexpr uint32_t SM_SLOTB = 147456;  // [Ap ; Mq] image, 32 KB / M2 image, 16 KB
+// CTA 0: r, fp32, being handed over (32 KB), V;  CTA 1: the hand-over buffer (r | Ob)
 constexpr uint32_t SM_RES = 180224, SM_V = 212992;
 constexpr uint32_t SM_X = 163840;
-constexpr uint32_t SM_VEC = 229376;  // 5 x 64 fp32: Gam Gprev wS wR gamma
-constexpr uint32_t SM_BAR = SM_VEC + 5 * 64 * 4;  // MMA, slot A, slot B, drain, tiles, hand-over
-constexpr uint32_t SM_SLOT = SM_BAR + 48;
+// two chunks' gates, fp32: Gam, Gprev / gamma, wS / wR (64 each), GamC
+constexpr uint32_t SM_VEC = 229376;
+constexpr int kVec = 196;
+constexpr uint32_t SM_BAR = SM_VEC + 2 * kVec * 4;
+// mbarriers: chain, slot A, slot B, drain, tiles, hand-over, side, MMA2 / 6, MMA4 / 8
+constexpr uint32_t SM_SLOT = SM_BAR + 72;
 constexpr uint32_t SM_FLAG = SM_SLOT + 4;
 constexpr size_t kPairSmem = SM_FLAG + 4;
 static_assert(SM_X + 65536 == SM_VEC && SM_V + 16384 == SM_VEC, "carve-up");
 static_assert(kPairSmem <= 232448, "shared memory");
 
-// TMEM columns: the state, the read-outs D1 (CTA 0: KS | QS, ..; CTA 1: E2 |
-// Ob) and CTA 1's KR | QR
-constexpr uint32_t T_ST = 0, T_D1 = 128, T_X = 256;
+constexpr int kPairThreads = kTcThreads + 64;  // and the issuing and the copying warp
+constexpr int kHandThreads = kTcThreads + 32;  // the element-wise warps and one of the two
+// named barriers on which the element-wise warps hand operands to the issuing
+// warp (X, E) and results to the copying warp (O), and one among themselves
+constexpr int kBarX = 1, kBarE = 2, kBarO = 3, kBarW = 4;
+
+// TMEM columns: the state; CTA 0: KS | QS, then E | Ob, then P | Ob, two sets by
+// the chunk's parity, then as A operands S's lo part and (wS E)^T (hi | lo), so
+// that their shared memory can hold what is being handed over; CTA 1: KR | QR,
+// two sets, where (wR E2)^T takes KR's place, and E2 | Ob
+constexpr uint32_t T_ST = 0, T_PAR = 128, T_D1 = 384, T_SLO = 384, T_W = 448;
 
 template <bool RDNV, bool kGeneric>
-__global__ void __launch_bounds__(kTcThreads, 1)
+__global__ void __launch_bounds__(kPairThreads, 1)
     fwd_pair_kernel(FwdParams p, const __grid_constant__ FwdMaps maps) {
   extern __shared__ __align__(1024) uint8_t sm[];
   const uint32_t sbase = smem_u32(sm);
@@ -64,11 +83,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     if (threadIdx.x == 0 && p.err) atomicExch(p.err, RDN_ERR_CUDA);
     return;
   }
-  float *vec = reinterpret_cast<float *>(sm + SM_VEC);
-  float *Gam = vec, *Gprev = vec + 64, *wS = vec + 128, *wR = vec + 192, *gamv = vec + 256;
   uint64_t *bar = reinterpret_cast<uint64_t *>(sm + SM_BAR);
   uint64_t *barA = bar + 1, *barB = bar + 2, *barD = bar + 3, *barE = bar + 4;
   uint64_t *barX = bar + 5;  // CTA 1: full; CTA 0: empty
+  uint64_t *barN = bar + 6;  // the products issued behind the chain's
+  uint64_t *barM2 = bar + 7, *barM4 = bar + 8;  // MMA2 / 6 and MMA4 / 8, for the copying warp
   uint32_t *slot = reinterpret_cast<uint32_t *>(sm + SM_SLOT);
   volatile int *flag = reinterpret_cast<volatile int *>(sm + SM_FLAG);
 
@@ -85,7 +104,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   const __nv_bfloat16 *q = (const __nv_bfloat16 *)p.q;
   const __nv_bfloat16 *k = (const __nv_bfloat16 *)p.k;
   const __nv_bfloat16 *v = (const __nv_bfloat16 *)p.v;
-  __nv_bfloat16 *o = (__nv_bfloat16 *)p.o;
   const float clip = p.clip;
   // (the variants: fwd_tc.cu)
   const bool dec_res = kGeneric && (p.mods & RDN_FLAG_DECAYED_RESIDUAL);
@@ -97,6 +115,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   if (tid == 0) {
     for (int b = 0; b < 5; ++b) mbar_init(bar + b, 1);
     mbar_init(barX, base ? kTcThreads / 32 : 1);
+    mbar_init(barN, 1);
+    mbar_init(barM2, 1);
+    mbar_init(barM4, 1);
     fence_mbar_init();
     if (!base) mbar_expect_tx(barX, 65536);
     *flag = 0;
@@ -108,43 +129,21 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   fence_after_sync();
   const uint32_t tm = *slot;
   const uint32_t lane = (uint32_t)((warp & 3) * 32) << 16;
-  uint32_t phase = 0, phA = 0, phB = 0;  // phA/phB: tracked by thread 0 only
-  bool pendA = false, pendB = false;     // (thread 0) a slot copy armed and not yet waited for
   const long long limit = p.inject == 1 ? 10000000ll : 2000000000ll;
-  bool skip_commit = p.inject == 1 && base;
   const uint32_t peer_bar = map_rank(barX, rank ^ 1u);
   const uint32_t peer_x = map_rank(sm + SM_X, 1u);
-
-  auto rec_of = [&](int c) {
-    return reinterpret_cast<const uint8_t *>(p.ws + (size_t)(sp.rbase + c) * kRecFloats);
+  uint32_t phase = 0;  // chain phases waited for (parity)
+  // a warp's wait: one lane polls (512 polling threads take shared-memory
+  // bandwidth from the products' operands)
+  auto warp_wait = [&](uint64_t *b, uint32_t parity) {
+    if ((tid & 31) == 0 && !mbar_wait(b, parity, limit)) *flag = 1;
+    __syncwarp();
   };
-  auto load_a = [&](int c) {  // (thread 0) T_beta / T_gamma
-    mbar_expect_tx(barA, 16384);
-    bulk_g2s(sm + SM_SLOTA, rec_of(c) + (base ? IMG_TB : IMG_TG), 16384, barA);
-    pendA = true;
+  auto wait_chain = [&] {
+    warp_wait(bar, phase);
+    phase ^= 1u;
+    fence_after_sync();
   };
-  auto load_b = [&](int c) {  // (thread 0) [Ap ; Mq] / M2
-    const uint32_t bytes = base ? 32768u : 16384u;
-    mbar_expect_tx(barB, bytes);
-    bulk_g2s(sm + SM_SLOTB, rec_of(c) + (base ? IMG_APMQ : IMG_M2), bytes, barB);
-    pendB = true;
-  };
-  auto wait_a = [&]() {
-    if (!mbar_wait(barA, phA)) return false;
-    phA ^= 1u;
-    pendA = false;
-    return true;
-  };
-  auto wait_b = [&]() {
-    if (!mbar_wait(barB, phB)) return false;
-    phB ^= 1u;
-    pendB = false;
-    return true;
-  };
-  if (tid == 0 && NC > 0) {
-    if (RDNV) load_a(0);
-    load_b(0);
-  }
   // a chunk's tiles: by tensor-map copies on barrier E where the chunk is whole
   // (not the first, not the last), by cp.async with zero fill otherwise
   auto fetch_v = [&](int c) {
@@ -167,50 +166,304 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       cp_async16(sm + SM_KQ + blk * 16384 + sw128(64 + t, cc), q + off, vld);
     }
   };
+  // (CTA 1) whether chunk c's o leaves as two tensor-map tiles (whole chunks of
+  // bf16 results; a row-by-row copy of 64 rows holds its source for 4k cycles)
+  auto o_tiles = [&](int c) { return maps.o_ok && T - c * 64 >= 64; };
   auto by_tma = [&](int cc) { return maps.ok && cc > 0 && cc < NC - 1; };
-  uint32_t phE = 0;    // phases of barrier E waited for
-  bool pendE = false;  // (thread 0) a phase armed and not yet waited for
-  // V is free a phase earlier than K, Q: CTA 0 arms barrier E with V's copy,
-  // CTA 1, which reads no V, with K's and Q's
-  auto next_v = [&](int cc) {
-    if (!by_tma(cc)) {
-      fetch_v(cc);
-    } else if (tid == 0) {
-      const int row = (int)(tok0 + (long long)cc * 64);
-      mbar_expect_tx(barE, 49152);
-      pendE = true;
-      for (int kb = 0; kb < 2; ++kb) tma_load_3d(sm + SM_V + kb * 8192, maps.v, 64 * kb, h, row, barE);
-    }
-  };
-  auto next_kq = [&](int cc) {
-    if (!by_tma(cc)) {
-      fetch_kq(cc);
-    } else if (tid == 0) {
-      const int row = (int)(tok0 + (long long)cc * 64);
-      if (!base) {
-        mbar_expect_tx(barE, 32768);
-        pendE = true;
+  if (warp == kTcThreads / 32) {
+    // =============================================== the issuing warp (lane 0)
+    const bool one = (tid & 31) == 0;
+    bool skip_commit = p.inject == 1 && base;
+    const uint32_t i64 = idesc_bf16(128, 64), i128 = idesc_bf16(128, 128);
+    // wait for a copy by the copying warp
+    auto wait_copy = [&](uint64_t *b, uint32_t ph) {
+      if (!mbar_wait(b, ph)) *flag = 1;
+    };
+    bool alive = true;
+    for (int c = 0; c < NC; ++c) {
+      const uint32_t d1 = T_PAR + 128u * (c & 1), tw = base ? T_W : d1;
+      __syncthreads();
+      fence_after_sync();
+      if (*flag) {
+        alive = false;
+        break;
       }
+      if (one) {  // the state's read-outs [K ; Q] S (S as hi + lo) / [K ; Q] R (RLA: Q R)
+        if (base) {
+          mma_tile(tm + d1, sbase + SM_ST, 16384, sbase + SM_KQ, 16384, 8, i128, false);
+#pragma unroll
+          for (int kk = 0; kk < 8; ++kk)
+            mma_bf16_ta(tm + d1, tm + T_SLO + 8 * kk,
+                        sdesc_sw128(sbase + SM_KQ + (kk >> 2) * 16384 + (kk & 3) * 32), i128, 1u);
+        } else if (RDNV) {
+          mma_tile(tm + d1, sbase + SM_ST, 16384, sbase + SM_KQ, 16384, 8, i128, false);
+        } else {
+          mma_tile(tm + d1 + 64, sbase + SM_ST, 16384, sbase + SM_KQ + 8192, 16384, 8, i64, false);
+        }
+        if (RDNV || base) {
+          if (!skip_commit) mma_commit(bar);
+          skip_commit = false;
+        }
+      }
+      __syncwarp();
+      if (RDNV) {  // MMA2: E^T = X^T T_beta^T / MMA6: E2^T = X2^T T_gamma^T
+        bar_sync(kBarX, kHandThreads);
+        fence_after_sync();
+        if (one) {
+          wait_copy(barA, (uint32_t)c & 1u);
+          mma_split3(tm + (base ? d1 : T_D1), sbase + SM_XE, sbase + SM_XE_LO, sbase + SM_SLOTA,
+                     sbase + SM_SLOTA + 8192, i64, false);
+          mma_commit(bar);
+          mma_commit(barM2);
+        }
+        __syncwarp();
+      }
+      bar_sync(kBarE, kHandThreads);
+      fence_after_sync();
+      if (one) {
+        // MMA4: S += (wS E)^T K / MMA8: R += (wR E2)^T K (hi, then lo); behind it
+        // MMA3: D1 += E^T [Ap;Mq]^T / MMA7: Ob += E2^T (gamma M2)^T
+#pragma unroll
+        for (int kk = 0; kk < 8; ++kk)
+          mma_bf16_ta(tm + T_ST, tm + tw + 8 * kk, sdesc_sw128_mn(sbase + SM_KQ + (kk & 3) * 2048, 16384),
+                      i128 | kBMajorMN, 1u);
+        mma_commit(bar);
+        mma_commit(barM4);
+        wait_copy(barB, (uint32_t)c & 1u);
+        if (base)
+          mma_split3(tm + d1, sbase + SM_XE, sbase + SM_XE_LO, sbase + SM_SLOTB,
+                     sbase + SM_SLOTB + 16384, i128, true);
+        else
+          mma_split3(tm + T_D1 + 64, sbase + SM_XE, sbase + SM_XE_LO, sbase + SM_SLOTB,
+                     sbase + SM_SLOTB + 8192, i64, true);
+        mma_commit(barN);
+      }
+      __syncwarp();
+    }
+    __syncthreads();
+    if ((!alive || *flag) && one) {  // a bounded wait gave up: drain the products, bounded
+      if (p.err) atomicExch(p.err, RDN_ERR_TIMEOUT);
+      mma_commit(barD);
+      mbar_wait(barD, 0);
+    }
+    __syncwarp();
+    fence_before_sync();
+    __syncthreads();
+    cluster_sync();
+    return;
+  }
+  if (warp == kTcThreads / 32 + 1) {
+    // =============================================== the copying warp
+    const bool one = (tid & 31) == 0;
+    const int ln = tid & 31;
+    uint32_t armA = 0, armB = 0, armE = 0;  // copies armed on the slots' and the tiles' barriers
+    auto rec_of = [&](int c) {
+      return reinterpret_cast<const uint8_t *>(p.ws + (size_t)(sp.rbase + c) * kRecFloats);
+    };
+    auto load_a = [&](int c) {  // T_beta / T_gamma
+      ++armA;
+      mbar_expect_tx(barA, 16384);
+      bulk_g2s(sm + SM_SLOTA, rec_of(c) + (base ? IMG_TB : IMG_TG), 16384, barA);
+    };
+    auto load_b = [&](int c) {  // [Ap ; Mq] / M2
+      const uint32_t bytes = base ? 32768u : 16384u;
+      ++armB;
+      mbar_expect_tx(barB, bytes);
+      bulk_g2s(sm + SM_SLOTB, rec_of(c) + (base ? IMG_APMQ : IMG_M2), bytes, barB);
+    };
+    auto arm_tiles = [&] {
+      ++armE;
+      mbar_expect_tx(barE, base ? 49152u : 32768u);
+    };
+    auto load_v = [&](int c) {
+      const int row = (int)(tok0 + (long long)c * 64);
+      for (int kb = 0; kb < 2; ++kb) tma_load_3d(sm + SM_V + kb * 8192, maps.v, 64 * kb, h, row, barE);
+    };
+    auto load_kq = [&](int c) {
+      const int row = (int)(tok0 + (long long)c * 64);
       for (int kb = 0; kb < 2; ++kb) {
         tma_load_3d(sm + SM_KQ + kb * 16384, maps.k, 64 * kb, h, row, barE);
         tma_load_3d(sm + SM_KQ + kb * 16384 + 8192, maps.q, 64 * kb, h, row, barE);
       }
+    };
+    // a chunk's gates, lane l those of tokens l and l + 32: loaded a chunk ahead,
+    // written to their set once nothing reads it any more
+    float g0[2], g1[2], g2[2], gc = 0.f;
+    auto load_gates = [&](int c) {
+      const float *rc = p.ws + (size_t)(sp.rbase + c) * kRecFloats + OFF_VEC;
+      const int t0 = c * 64, n = min(64, T - t0);
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int t = ln + 32 * u;
+        g0[u] = rc[V_GAM + t];
+        g1[u] = base ? rc[V_GPREV + t] : t < n ? p.gamma[(size_t)(tok0 + t0 + t) * H + h] : 0.f;
+        g2[u] = rc[(base ? V_WS : V_WR) + t];
+      }
+      gc = rc[V_GAMC];
+    };
+    auto put_gates = [&](int c) {
+      float *v = reinterpret_cast<float *>(sm + SM_VEC) + kVec * (c & 1);
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int t = ln + 32 * u;
+        v[t] = g0[u];
+        v[64 + t] = g1[u];
+        v[128 + t] = g2[u];
+      }
+      if (ln == 0) v[192] = gc;
+    };
+    // L2 prefetch of what this CTA reads of a chunk
+    auto prefetch_chunk = [&](int c) {
+      const uint8_t *r = rec_of(c);
+      prefetch_l2_bulk(r + (base ? IMG_TB : IMG_TG), base ? 49152 : 32768);
+      static_assert(IMG_APMQ == IMG_TB + 16384 && IMG_M2 == IMG_TG + 16384, "contiguous images");
+      prefetch_l2_bulk(r + OFF_VEC * 4, (kRecFloats - OFF_VEC) * 4);
+      if (!maps.ok) return;
+      const int row = (int)(tok0 + (long long)c * 64);
+      for (int kb = 0; kb < 2; ++kb) {
+        tma_prefetch_3d(maps.k, 64 * kb, h, row);
+        tma_prefetch_3d(maps.q, 64 * kb, h, row);
+        if (base) tma_prefetch_3d(maps.v, 64 * kb, h, row);
+      }
+    };
+    // CTA 0: chunk c's r and Ob, staged by the element-wise warps -> CTA 1;
+    // CTA 1: chunk c's o rows -> global memory
+    uint32_t handed = 0;
+    auto send = [&](int c) {
+      bar_sync(kBarO, kHandThreads);
+      if (base) {
+        if (one) {
+          bulk_s2s(peer_x, sm + SM_RES, 32768, peer_bar);
+          bulk_s2s(peer_x + 32768, sm + SM_OUT, 32768, peer_bar);
+        }
+        ++handed;
+        return;
+      }
+      const int t0 = c * 64, n = min(64, T - t0);
+      if (o_tiles(c)) {
+        if (one) {
+          for (int kb = 0; kb < 2; ++kb)
+            tma_store_3d(maps.o, 64 * kb, h, (int)(tok0 + t0), sm + SM_OUT + 8192 * kb);
+          bulk_commit();
+        }
+        return;
+      }
+      const uint32_t bytes = p.f32out ? 512u : 256u;
+      for (int t = ln; t < n; t += 32)
+        bulk_s2g((uint8_t *)p.o + ((size_t)(tok0 + t0 + t) * H + h) * bytes, sm + SM_OUT + t * bytes, bytes);
+      bulk_commit();
+    };
+    if (NC > 0) {
+      if (one) {
+        if (RDNV) load_a(0);
+        load_b(0);
+      }
+      load_gates(0);
+      put_gates(0);
     }
-  };
+    uint8_t *keep = base ? p.sv_E : p.sv_E2;  // E's images (hi | lo) for the backward
+    bool alive = true, good = true;  // good: (lane 0) no wait of this warp gave up
+    // (a wait that gave up leaves its phase incomplete, which takes no further
+    // arrival: nothing is armed after it)
+    auto await = [&](bool done) {
+      if (!done) {
+        good = false;
+        *flag = 1;
+      }
+    };
+    for (int c = 0; c < NC; ++c) {
+      const bool more = c + 1 < NC;
+      const bool tma_next = more && by_tma(c + 1);
+      if (by_tma(c) && one) await(mbar_wait(barE, (armE - 1) & 1u));
+      bulk_wait_read();  // o's rows and E's image of the chunk before
+      __syncwarp();
+      __syncthreads();
+      if (*flag) {
+        alive = false;
+        break;
+      }
+      if (more) load_gates(c + 1);
+      if (one) {
+        if (more) prefetch_chunk(c + 1);
+        if (c > 0) {  // slot B: free once chunk c - 1's product with it is complete
+          await(mbar_wait(barN, (uint32_t)(c - 1) & 1u, limit));
+          if (good) load_b(c);
+        }
+      }
+      __syncwarp();
+      if (c > 0) send(c - 1);
+      if (RDNV) {
+        if (one) {
+          await(mbar_wait(barM2, (uint32_t)c & 1u, limit));
+          if (good && more) load_a(c + 1);
+          if (good && base && tma_next) {  // (every V of this chunk has been read)
+            arm_tiles();
+            load_v(c + 1);
+          }
+        }
+        __syncwarp();
+        if (more) put_gates(c + 1);  // (CTA 1: chunk c - 1's are read before MMA6)
+      }
+      if (one) {
+        await(mbar_wait(barM4, (uint32_t)c & 1u, limit));
+        if (good && tma_next) {  // K, Q are done with
+          if (!RDNV || !base) arm_tiles();
+          if (!RDNV && base) load_v(c + 1);
+          load_kq(c + 1);
+        }
+        if (keep) {
+          static_assert(SM_XE_LO == SM_XE + 16384, "contiguous");
+          bulk_s2g(keep + (size_t)(sp.rbase + c) * 32768, sm + SM_XE, 32768);
+          bulk_commit();
+        }
+        // the copies of chunk c - 1 have left what chunk c's are staged in next
+        if (base && c > 0) await(mbar_wait_cluster(barX, (uint32_t)(c - 1) & 1u, limit));
+      }
+      __syncwarp();
+      if (!RDNV && more) put_gates(c + 1);
+    }
+    if (alive && NC > 0) {
+      bulk_wait_read();  // (what the last chunk's results are staged in is free)
+      __syncwarp();
+      bar_sync(kBarO, kHandThreads);
+      send(NC - 1);
+    }
+    bulk_wait_all();
+    __syncthreads();
+    if ((!alive || *flag) && one) {  // every copy armed has landed, bounded
+      if (armA) mbar_wait(barA, (armA - 1) & 1u);
+      if (armB) mbar_wait(barB, (armB - 1) & 1u);
+      if (armE) mbar_wait(barE, (armE - 1) & 1u);
+      if (handed) mbar_wait_cluster(barX, (handed - 1) & 1u, limit);  // (those into CTA 1)
+    }
+    __syncwarp();
+    fence_before_sync();
+    __syncthreads();
+    cluster_sync();
+    return;
+  }
+
+  // ================================================= the 16 element-wise warps
   if (NC > 0) {
     if (base) fetch_v(0);
     fetch_kq(0);
   }
 
-  // a state's bf16 copy, and CTA 0's also its lo part, 16 columns
+  // a state's bf16 copy, and CTA 0's also its lo part (s - bf16(s)), 16 columns
   auto put_state = [&](int c0, const float (&s)[16]) {
-    st_row16(sm + SM_ST, 16384, j, c0, s);
-    if (base) {
-      float lo[16];
+    uint32_t hi[8], lo[8];
 #pragma unroll
-      for (int i = 0; i < 16; ++i) lo[i] = s[i] - __bfloat162float(__float2bfloat16_rn(s[i]));
-      st_row16(sm + SM_XE, SM_XE_LO - SM_XE, j, c0, lo);
+    for (int i = 0; i < 8; ++i) {
+      hi[i] = pack_bf16(s[2 * i], s[2 * i + 1]);
+      lo[i] = pack_bf16(s[2 * i] - __uint_as_float(hi[i] << 16),
+                        s[2 * i + 1] - __uint_as_float(hi[i] & 0xFFFF0000u));
     }
+    const uint32_t blk = (uint32_t)(c0 >> 6) * 16384u;
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+      *reinterpret_cast<uint4 *>(sm + SM_ST + blk + sw128(j, (c0 & 63) + 8 * u)) =
+          make_uint4(hi[4 * u], hi[4 * u + 1], hi[4 * u + 2], hi[4 * u + 3]);
+    if (base) tmem_st8(tm + lane + T_SLO + c0 / 2, lo);
   };
   const float *init = base ? p.S0 : p.R0;
   float *chunks = base ? p.S_chunks : p.R_chunks;
@@ -226,43 +479,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         chunks[(size_t)sp.rbase * D * D + (size_t)(c0 + i) * D + j] = s[i];
   }
 
-  auto run_phase = [&](auto issue, auto during) -> bool {
+  // hand this warp's shared-memory writes and TMEM accesses to the issuing or
+  // the copying warp
+  auto publish = [&](int id) {
     fence_async_smem();
     fence_before_sync();
-    __syncthreads();
-    if (tid == 0) {
-      fence_after_sync();
-      if (!issue()) *flag = 1;
-      if (!skip_commit) mma_commit(bar);
-      skip_commit = false;
-    }
-    during();
-    const bool ok = mbar_wait(bar, phase, limit);
-    phase ^= 1u;
-    if (!ok) *flag = 1;
-    __syncthreads();
-    fence_after_sync();
-    return *flag == 0;
-  };
-  auto nothing = [] {};
-  // L2 prefetch of what this CTA reads of a chunk's record and rows
-  auto prefetch_chunk = [&](int c) {
-    const int t0_ = c * 64, n_ = min(64, T - t0_);
-    if (tid == 0) {
-      const uint8_t *r = rec_of(c);
-      prefetch_l2_bulk(r + (base ? IMG_TB : IMG_TG), base ? 49152 : 32768);
-      static_assert(IMG_APMQ == IMG_TB + 16384 && IMG_M2 == IMG_TG + 16384, "contiguous images");
-      prefetch_l2_bulk(r + OFF_VEC * 4, (kRecFloats - OFF_VEC) * 4);
-    }
-    if (tid < 384) {
-      const int rr = tid >> 1, t = rr & 63, w = rr >> 6;
-      const __nv_bfloat16 *src = w == 0 ? k : (w == 1 ? q : v);
-      if (t < n_ && (base || w < 2))
-        prefetch_l2_line(src + ((size_t)(tok0 + t0_ + t) * H + h) * D + (tid & 1) * 64);
-    } else if (!base && tid < 416) {
-      const int t = 2 * (tid - 384);
-      if (t < n_) prefetch_l2_line(p.gamma + (size_t)(tok0 + t0_ + t) * H + h);
-    }
+    bar_arrive(id, kHandThreads);
   };
   // the state's TMEM copy times the chunk's total decay, in place, its values
   // before that to the chunk-start states (fwd_tc.cu's scale_state)
@@ -284,236 +506,192 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     tmem_st16(tm + lane + T_ST + g16, x);
     tmem_st16(tm + lane + T_ST + g16 + 64, y);
   };
-  struct Pre {  // a chunk's gate values (threads 0..63) and its total decay
-    float gm, gp, w, g, gc;
-  };
-  auto fetch_pre = [&](int c) {
-    const float *rc = p.ws + (size_t)(sp.rbase + c) * kRecFloats;
-    const int t0_ = c * 64, n_ = min(64, T - t0_);
-    Pre x;
-    x.gm = x.gp = x.w = x.g = 0.f;
-    if (tid < 64) {
-      x.gm = rc[OFF_VEC + V_GAM + tid];
-      x.w = rc[OFF_VEC + (base ? V_WS : V_WR) + tid];
-      if (base) x.gp = rc[OFF_VEC + V_GPREV + tid];
-      else x.g = tid < n_ ? p.gamma[(size_t)(tok0 + t0_ + tid) * H + h] : 0.f;
+  float vv[16];         // CTA 0: this thread's V entries of the last chunk begun
+  // CTA 0: chunk c's P | Ob are complete: r = clip(V - P); r and Ob -> CTA 1.
+  // (The copies of chunk c - 1 have left their places: the issuing warp saw
+  // `empty` before this chunk's first barrier.)
+  auto hand_over = [&](int c) {
+    const size_t ci = (size_t)(sp.rbase + c);
+    const uint32_t d1 = T_PAR + 128u * (c & 1);
+    warp_wait(barN, (uint32_t)c & 1u);
+    fence_after_sync();
+    float pp[16], ob[16];
+    tmem_ld16x2(tm + lane + d1 + g16, pp, tm + lane + d1 + 64 + g16, ob);
+    if (!tnh && !p.sv_mask) {
+#pragma unroll
+      for (int i = 0; i < 16; ++i) pp[i] = clampf(vv[i] - pp[i], clip);
+    } else if (!tnh) {
+      unsigned msk = 0u;  // bit i: |x| <= c at t = g16 + i
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const float x = vv[i] - pp[i];
+        if (fabsf(x) <= clip) msk |= 1u << i;
+        pp[i] = clampf(x, clip);
+      }
+      reinterpret_cast<uint16_t *>(p.sv_mask + ci * D + j)[g16 >> 4] = (uint16_t)msk;
+    } else {
+      uint32_t dg[8];
+#pragma unroll
+      for (int i = 0; i < 16; i += 2) {
+        const float x0 = vv[i] - pp[i], x1 = vv[i + 1] - pp[i + 1];
+        pp[i] = resid_map(x0, clip, true);
+        pp[i + 1] = resid_map(x1, clip, true);
+        dg[i / 2] = grad_q16(resid_grad(x0, clip, true)) |
+                    (grad_q16(resid_grad(x1, clip, true)) << 16);
+      }
+      if (p.sv_mask) {
+        uint4 *dst = reinterpret_cast<uint4 *>(reinterpret_cast<uint16_t *>(p.sv_mask) +
+                                               (ci * D + j) * 64 + g16);
+        dst[0] = make_uint4(dg[0], dg[1], dg[2], dg[3]);
+        dst[1] = make_uint4(dg[4], dg[5], dg[6], dg[7]);
+      }
     }
-    x.gc = rc[OFF_VEC + V_GAMC];
-    return x;
+    float4 *xr = reinterpret_cast<float4 *>(sm + SM_RES + 2048 * warp) + (tid & 31);
+    float4 *xo = reinterpret_cast<float4 *>(sm + SM_OUT + 2048 * warp) + (tid & 31);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      xr[32 * i] = make_float4(pp[4 * i], pp[4 * i + 1], pp[4 * i + 2], pp[4 * i + 3]);
+      xo[32 * i] = make_float4(ob[4 * i], ob[4 * i + 1], ob[4 * i + 2], ob[4 * i + 3]);
+    }
+    publish(kBarO);
   };
-  Pre pre{};
-  if (NC > 0) pre = fetch_pre(0);
-
-  // CTA 0, thread 0 (after a barrier that published them): r and Ob -> CTA 1
-  uint32_t handed = 0;
-  auto hand_over = [&] {
-    ++handed;
-    bulk_s2s(peer_x, sm + SM_RES, 32768, peer_bar);
-    bulk_s2s(peer_x + 32768, sm + SM_W, 32768, peer_bar);
+  // CTA 1: chunk c's Ob + gamma M2 E2 is complete: o = that + gamma Gam QR,
+  // staged as tiles or rows [t][j] (2-byte stores of them straight to
+  // global memory took 2.9k cycles a chunk)
+  auto finish_o = [&](int c) {
+    const float *Gam = reinterpret_cast<const float *>(sm + SM_VEC) + kVec * (c & 1), *gamv = Gam + 64;
+    warp_wait(barN, (uint32_t)c & 1u);
+    fence_after_sync();
+    float ob[16], oa[16], gm[16], gv[16];
+    tmem_ld16x2(tm + lane + T_D1 + 64 + g16, ob, tm + lane + T_PAR + 128u * (c & 1) + 64 + g16, oa);
+    lds16(Gam + g16, gm);
+    lds16(gamv + g16, gv);
+    const bool tiles = o_tiles(c);
+    __nv_bfloat16 *stg = reinterpret_cast<__nv_bfloat16 *>(sm + SM_OUT) + g16 * D + j;
+    float *stg32 = reinterpret_cast<float *>(sm + SM_OUT) + g16 * D + j;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const float gg = plain ? 1.f : gv[i];
+      const float ov = stl ? ob[i] : fmaf(gg * gm[i] * p.scale, oa[i], ob[i]);
+      if (tiles)
+        *reinterpret_cast<__nv_bfloat16 *>(sm + SM_OUT + (j >> 6) * 8192 + sw128(g16 + i, j & 63)) =
+            __float2bfloat16_rn(ov);
+      else if (p.f32out) stg32[i * D] = ov;
+      else stg[i * D] = __float2bfloat16_rn(ov);
+    }
+    publish(kBarO);
+  };
+  // (wS E)^T / (wR E2)^T as an A operand in TMEM
+  auto put_w = [&](uint32_t col, const float (&w)[16]) {
+    uint32_t hi[8], lo[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) split_pack_bf16(w[2 * i], w[2 * i + 1], hi[i], lo[i]);
+    tmem_st8x2(tm + lane + col + g16 / 2, hi, tm + lane + col + 32 + g16 / 2, lo);
+  };
+  // CTA 1: this warp has used what it read of the hand-over buffer
+  auto taken = [&](bool got) {
+    __syncwarp();
+    if (got && (tid & 31) == 0) mbar_arrive_remote_relaxed(peer_bar);
   };
 
   bool alive = true;
   for (int c = 0; c < NC && alive; ++c) {
-    const int t0 = c * 64;
-    const int n = min(64, T - t0);
     const size_t ci = (size_t)(sp.rbase + c);  // chunk index of the saved intermediates
-    if (c + 1 < NC) prefetch_chunk(c + 1);
-    if (by_tma(c)) {
-      if (!mbar_wait(barE, phE & 1u)) *flag = 1;
-      ++phE;
-      if (tid == 0) pendE = false;
-    } else {
-      cp_async_wait_all();
-    }
+    const bool more = c + 1 < NC;
+    if (!by_tma(c)) cp_async_wait_all();
     float *start = (chunks && c > 0) ? chunks + ci * D * D : nullptr;
-    if (tid < 64) {  // (last read before the previous chunk's last barrier)
-      Gam[tid] = pre.gm;
-      if (base) {
-        Gprev[tid] = pre.gp;
-        wS[tid] = pre.w;
-      } else {
-        wR[tid] = pre.w;
-        gamv[tid] = pre.g;
-      }
-    }
-    const float GamC = pre.gc;
-    if (c + 1 < NC) pre = fetch_pre(c + 1);  // in flight during this chunk
-    if (base) fence_async_smem();            // r and Ob of the previous chunk
-    __syncthreads();
+    fence_async_smem();
+    fence_before_sync();
+    __syncthreads();  // (with the issuing warp, which has waited for the tiles)
+    fence_after_sync();
     if (*flag) {
       alive = false;
       break;
     }
+    const float *Gam = reinterpret_cast<const float *>(sm + SM_VEC) + kVec * (c & 1);
+    const float *Gp = Gam + 64, *ww = Gam + 128;
+    const float GamC = Gam[192];
+    const uint32_t d1 = T_PAR + 128u * (c & 1);
     if (base) {
-      if (tid == 0 && c > 0) hand_over();
-      // ---- MMA1: D1 = S^T [K ; Q]^T (S as hi + lo)
-      alive = run_phase([&] {
-        mma_tile(tm + T_D1, sbase + SM_ST, 16384, sbase + SM_KQ, 16384, 8, idesc_bf16(128, 128), false);
-        mma_tile(tm + T_D1, sbase + SM_XE, SM_XE_LO - SM_XE, sbase + SM_KQ, 16384, 8, idesc_bf16(128, 128), true);
-        return true;
-      }, [&] { scale_state(GamC, start); });
-      if (!alive) break;
-      float gks[16], vv[16];
+      if (c > 0) hand_over(c - 1);
+      if (!RDNV) scale_state(GamC, start);
+      wait_chain();
+      float gks[16];
       {
-        float x[16], gm[16], gp[16];
-        tmem_ld16x2(tm + lane + T_D1 + 64 + g16, x, tm + lane + T_D1 + g16, gks);
-        lds16(plain ? Gprev + g16 : Gam + g16, gm);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) x[i] *= gm[i] * p.scale;  // Ob accumulates onto Gam scale QS
-        tmem_st16(tm + lane + T_D1 + 64 + g16, x);
+        float x[16], gm[16];
+        tmem_ld16(tm + lane + d1 + g16, gks);
         lds16(Gam + g16, gm);
-        lds16(Gprev + g16, gp);
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
           vv[i] = __bfloat162float(*reinterpret_cast<const __nv_bfloat16 *>(
               sm + SM_V + (j >> 6) * 8192 + sw128(g16 + i, j & 63)));
           x[i] = vv[i] - gm[i] * gks[i];
-          gks[i] *= dec_res ? gm[i] : gp[i];
         }
-        if (RDNV) {
-          st_row16_split(sm + SM_XE, sm + SM_XE_LO, j, g16, x);
-        } else {
-          tmem_st16(tm + lane + T_D1 + g16, gks);
-        }
-      }
-      if (RDNV) {  // ---- MMA2: E^T = X^T T_beta^T
-        alive = run_phase([&] {
-          if (!wait_a()) return false;
-          mma_split3(tm + T_D1, sbase + SM_XE, sbase + SM_XE_LO, sbase + SM_SLOTA,
-                     sbase + SM_SLOTA + 8192, idesc_bf16(128, 64), false);
-          return true;
-        }, nothing);
-        if (!alive) break;
-        if (tid == 0 && c + 1 < NC) load_a(c + 1);
-      } else {
-        __syncthreads();  // (every thread has read its V)
-      }
-      if (c + 1 < NC) next_v(c + 1);
-      {
-        float e[16], w[16];
-        if (RDNV) {
-          tmem_ld16(tm + lane + T_D1 + g16, e);
-          tmem_st16(tm + lane + T_D1 + g16, gks);
-        } else {
+        if (RDNV) st_row16_split(sm + SM_XE, sm + SM_XE_LO, j, g16, x);
+        lds16(dec_res ? Gam + g16 : Gp + g16, gm);
 #pragma unroll
-          for (int i = 0; i < 16; ++i) e[i] = vv[i];
+        for (int i = 0; i < 16; ++i) gks[i] *= gm[i];
+      }
+      if (RDNV) {
+        publish(kBarX);
+        scale_state(GamC, start);  // (the read-outs use the state's bf16 copies)
+        wait_chain();
+      }
+      {  // E, wS E; P and Ob accumulate onto Gprev KS and Gam scale QS
+        float e[16], w[16], x[16];
+        tmem_ld16x2(tm + lane + d1 + g16, e, tm + lane + d1 + 64 + g16, x);
+        lds16(plain ? Gp + g16 : Gam + g16, w);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          x[i] *= w[i] * p.scale;
+          if (!RDNV) e[i] = vv[i];
         }
-        lds16(wS + g16, w);
+        tmem_st16x2(tm + lane + d1 + g16, gks, tm + lane + d1 + 64 + g16, x);
+        lds16(ww + g16, w);
 #pragma unroll
         for (int i = 0; i < 16; ++i) w[i] *= e[i];
+        put_w(T_W, w);
         st_row16_split(sm + SM_XE, sm + SM_XE_LO, j, g16, e);
-        // (the previous chunk's hand-over has left W and the r staging)
-        if (c > 0 && !mbar_wait_cluster(barX, (uint32_t)(c - 1) & 1u, limit)) *flag = 1;
-        st_row16_split(sm + SM_W, sm + SM_W_LO, j, g16, w);
-      }
-      // ---- MMA3: D1 += E^T [Ap;Mq]^T;  MMA4: S += (wS E)^T K
-      alive = run_phase([&] {
-        if (!wait_b()) return false;
-        mma_split3(tm + T_D1, sbase + SM_XE, sbase + SM_XE_LO, sbase + SM_SLOTB,
-                   sbase + SM_SLOTB + 16384, idesc_bf16(128, 128), true);
-        if (p.sv_E) {  // keep the E^T image (hi | lo) for the backward
-          static_assert(SM_XE_LO == SM_XE + 16384, "contiguous");
-          bulk_s2g(p.sv_E + ci * 32768, sm + SM_XE, 32768);
-          bulk_commit();
-        }
-        mma_tile_kmn(tm + T_ST, sbase + SM_W, 0, sbase + SM_KQ, 16384, 4, idesc_bf16(128, 128), true);
-        mma_tile_kmn(tm + T_ST, sbase + SM_W_LO, 0, sbase + SM_KQ, 16384, 4, idesc_bf16(128, 128), true);
-        return true;
-      }, [&] {
-        if (tid == 0 && p.sv_E) bulk_wait_read();  // the E^T tiles are rewritten next
-      });
-      if (!alive) break;
-      if (c + 1 < NC) {
-        if (tid == 0) load_b(c + 1);
-        next_kq(c + 1);
-      }
-      // ---- S (= Gam_C S + U) -> its bf16 copies; r = clip(V - P); r, Ob -> CTA 1
-      {
-        float s0[16], s1[16];
-        tmem_ld16x2(tm + lane + T_ST + g16, s0, tm + lane + T_ST + g16 + 64, s1);
-        put_state(g16, s0);
-        put_state(g16 + 64, s1);
-      }
-      {
-        float pp[16], ob[16], r[16];
-        tmem_ld16x2(tm + lane + T_D1 + g16, pp, tm + lane + T_D1 + 64 + g16, ob);
-        if (!tnh) {
-          unsigned msk = 0u;  // bit i: |x| <= c at t = g16 + i
-#pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const float x = vv[i] - pp[i];
-            if (fabsf(x) <= clip) msk |= 1u << i;
-            r[i] = clampf(x, clip);
-          }
-          if (p.sv_mask) reinterpret_cast<uint16_t *>(p.sv_mask + ci * D + j)[g16 >> 4] = (uint16_t)msk;
-        } else {
-          uint32_t dg[8];
-#pragma unroll
-          for (int i = 0; i < 16; i += 2) {
-            const float x0 = vv[i] - pp[i], x1 = vv[i + 1] - pp[i + 1];
-            r[i] = resid_map(x0, clip, true);
-            r[i + 1] = resid_map(x1, clip, true);
-            dg[i / 2] = grad_q16(resid_grad(x0, clip, true)) |
-                        (grad_q16(resid_grad(x1, clip, true)) << 16);
-          }
-          if (p.sv_mask) {
-            uint4 *dst = reinterpret_cast<uint4 *>(reinterpret_cast<uint16_t *>(p.sv_mask) +
-                                                   (ci * D + j) * 64 + g16);
-            dst[0] = make_uint4(dg[0], dg[1], dg[2], dg[3]);
-            dst[1] = make_uint4(dg[4], dg[5], dg[6], dg[7]);
-          }
-        }
-        float4 *xr = reinterpret_cast<float4 *>(sm + SM_RES) + tid;
-        float4 *xo = reinterpret_cast<float4 *>(sm + SM_W) + tid;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          xr[512 * i] = make_float4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
-          xo[512 * i] = make_float4(ob[4 * i], ob[4 * i + 1], ob[4 * i + 2], ob[4 * i + 3]);
-        }
       }
     } else {
-      // ---- MMA5: X = R^T [K ; Q]^T
-      alive = run_phase([&] {
-        if (p.sv_E2) bulk_wait_read();  // the E2^T tiles of the previous chunk are rewritten next
-        mma_tile(tm + T_X, sbase + SM_ST, 16384, sbase + SM_KQ, 16384, 8, idesc_bf16(128, 128), false);
-        return true;
-      }, [&] { scale_state(stl ? 0.f : GamC, start); });
-      if (!alive) break;
-      float r[16];
-      const bool got = mbar_wait_cluster(barX, (uint32_t)c & 1u, limit);
-      if (!got) *flag = 1;
+      if (c > 0) finish_o(c - 1);
+      if (RDNV) wait_chain();
+      else scale_state(stl ? 0.f : GamC, start);
+      bool got = true;  // (lane 0)
+      if ((tid & 31) == 0 && !mbar_wait_cluster(barX, (uint32_t)c & 1u, limit)) {
+        got = false;
+        *flag = 1;
+      }
+      __syncwarp();
+      float r[16], ob[16];
       {
-        float ob[16];
-        const float4 *x = reinterpret_cast<const float4 *>(sm + SM_X) + tid;
+        const float4 *x = reinterpret_cast<const float4 *>(sm + SM_X + 2048 * warp) + (tid & 31);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          const float4 a = x[512 * i], b = x[512 * (4 + i)];
+          const float4 a = x[32 * i], b = x[2048 + 32 * i];
           r[4 * i] = a.x; r[4 * i + 1] = a.y; r[4 * i + 2] = a.z; r[4 * i + 3] = a.w;
           ob[4 * i] = b.x; ob[4 * i + 1] = b.y; ob[4 * i + 2] = b.z; ob[4 * i + 3] = b.w;
         }
         // (a phase that has not completed takes no further arrival)
-        if (got && tid == 0 && c + 1 < NC) mbar_expect_tx(barX, 65536);
-        __syncwarp();
-        if (got && (tid & 31) == 0) mbar_arrive_remote(peer_bar);
-        tmem_st16(tm + lane + T_D1 + 64 + g16, ob);
+        if (got && tid == 0 && more) mbar_expect_tx(barX, 65536);
       }
       if (RDNV) {  // ---- X2 = r - Gam KR;  MMA6: E2^T = X2^T T_gamma^T
         {
           float x[16], gm[16];
-          tmem_ld16(tm + lane + T_X + g16, x);
+          tmem_ld16(tm + lane + d1 + g16, x);
           lds16(Gam + g16, gm);
 #pragma unroll
           for (int i = 0; i < 16; ++i) x[i] = stl ? r[i] : r[i] - gm[i] * x[i];
           st_row16_split(sm + SM_XE, sm + SM_XE_LO, j, g16, x);
         }
-        alive = run_phase([&] {
-          if (!wait_a()) return false;
-          mma_split3(tm + T_D1, sbase + SM_XE, sbase + SM_XE_LO, sbase + SM_SLOTA,
-                     sbase + SM_SLOTA + 8192, idesc_bf16(128, 64), false);
-          return true;
-        }, nothing);
-        if (!alive) break;
-        if (tid == 0 && c + 1 < NC) load_a(c + 1);
+        publish(kBarX);
+        tmem_st16(tm + lane + T_D1 + 64 + g16, ob);
+        taken(got);
+        scale_state(stl ? 0.f : GamC, start);
+        wait_chain();
+      } else {
+        tmem_st16(tm + lane + T_D1 + 64 + g16, ob);
+        taken(got);
       }
       {
         float e[16], w[16];
@@ -523,85 +701,41 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 #pragma unroll
           for (int i = 0; i < 16; ++i) e[i] = r[i];
         }
-        lds16(wR + g16, w);
+        lds16(ww + g16, w);
 #pragma unroll
         for (int i = 0; i < 16; ++i) w[i] *= e[i];
+        put_w(d1, w);
         st_row16_split(sm + SM_XE, sm + SM_XE_LO, j, g16, e);
-        st_row16_split(sm + SM_W, sm + SM_W_LO, j, g16, w);
       }
-      // ---- MMA7: Ob += E2^T (gamma M2)^T;  MMA8: R += (wR E2)^T K
-      alive = run_phase([&] {
-        if (!wait_b()) return false;
-        mma_split3(tm + T_D1 + 64, sbase + SM_XE, sbase + SM_XE_LO, sbase + SM_SLOTB,
-                   sbase + SM_SLOTB + 8192, idesc_bf16(128, 64), true);
-        if (p.sv_E2) {
-          bulk_s2g(p.sv_E2 + ci * 32768, sm + SM_XE, 32768);
-          bulk_commit();
-        }
-        mma_tile_kmn(tm + T_ST, sbase + SM_W, 0, sbase + SM_KQ, 16384, 4, idesc_bf16(128, 128), true);
-        mma_tile_kmn(tm + T_ST, sbase + SM_W_LO, 0, sbase + SM_KQ, 16384, 4, idesc_bf16(128, 128), true);
-        return true;
-      }, nothing);
-      if (!alive) break;
-      if (c + 1 < NC) {
-        if (tid == 0) load_b(c + 1);
-        next_kq(c + 1);
-      }
-      // ---- R -> its bf16 copy; o = Ob + gamma Gam QR, staged in W's place
-      {
-        float r0[16], r1[16];
-        tmem_ld16x2(tm + lane + T_ST + g16, r0, tm + lane + T_ST + g16 + 64, r1);
-        put_state(g16, r0);
-        put_state(g16 + 64, r1);
-      }
-      {
-        __nv_bfloat16 *ostg = reinterpret_cast<__nv_bfloat16 *>(sm + SM_W);
-        float *ostg32 = reinterpret_cast<float *>(sm + SM_W);
-        static_assert(SM_W_LO == SM_W + 16384, "fp32 o staging spans W and its lo part");
-        float ob[16], oa[16], gm[16], gv[16];
-        tmem_ld16x2(tm + lane + T_D1 + 64 + g16, ob, tm + lane + T_X + 64 + g16, oa);
-        lds16(Gam + g16, gm);
-        lds16(gamv + g16, gv);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const int t = g16 + i;
-          const float gg = plain ? 1.f : gv[i];
-          const float ov = stl ? ob[i] : fmaf(gg * gm[i] * p.scale, oa[i], ob[i]);
-          if (p.f32out)
-            ostg32[t * D + j] = ov;
-          else
-            ostg[t * D + j] = __float2bfloat16_rn(ov);
-        }
-      }
-      __syncthreads();  // the o tile
-      if (p.f32out) {
-        float *of = (float *)p.o;
-        for (int e = tid; e < 64 * 32; e += kTcThreads) {
-          const int t = e >> 5, ch = e & 31;
-          if (t < n)
-            *reinterpret_cast<uint4 *>(of + ((size_t)(tok0 + t0 + t) * H + h) * D + ch * 4) =
-                *reinterpret_cast<const uint4 *>(sm + SM_W + t * 512 + ch * 16);
-        }
-      } else {
-        for (int e = tid; e < 64 * 16; e += kTcThreads) {
-          const int t = e >> 4, ch = e & 15;
-          if (t < n)
-            *reinterpret_cast<uint4 *>(o + ((size_t)(tok0 + t0 + t) * H + h) * D + ch * 8) =
-                *reinterpret_cast<const uint4 *>(sm + SM_W + t * 256 + ch * 16);
-        }
-      }
+    }
+    publish(kBarE);
+    // the updated state -> its bf16 copies; K, Q are done with
+    wait_chain();
+    if (more && !by_tma(c + 1)) {  // (every thread is past its reads of V)
+      bar_sync(kBarW, kTcThreads);
+      if (base) fetch_v(c + 1);
+      fetch_kq(c + 1);
+    }
+    {
+      float s0[16], s1[16];
+      tmem_ld16x2(tm + lane + T_ST + g16, s0, tm + lane + T_ST + g16 + 64, s1);
+      put_state(g16, s0);
+      put_state(g16 + 64, s1);
     }
   }
 
-  if (tid == 0 && p.sv_E) bulk_wait_all();
-  if (base) fence_async_smem();
-  __syncthreads();
-  if (*flag) alive = false;  // (a wait of the last chunk)
-  if (base && alive && NC > 0) {  // the last chunk's r and Ob, until CTA 1 holds them
-    if (tid == 0) hand_over();
-    if (!mbar_wait_cluster(barX, (uint32_t)(NC - 1) & 1u, limit) && tid == 0 && p.err)
-      atomicExch(p.err, RDN_ERR_TIMEOUT);
+  if (alive && NC > 0) {  // the last chunk's read-outs
+    bar_sync(kBarO, kHandThreads);  // (the chunk before's have left)
+    if (base) {
+      hand_over(NC - 1);
+      // until CTA 1 holds them
+      if (tid == 0 && !mbar_wait_cluster(barX, (uint32_t)(NC - 1) & 1u, limit)) *flag = 1;
+    } else {
+      finish_o(NC - 1);
+    }
   }
+  __syncthreads();
+  if (*flag) alive = false;
   if (alive) {  // final state
     float *fin = base ? p.ST : p.RT;
     for (int c0 = g16; c0 < D && fin; c0 += 64) {
@@ -610,20 +744,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 #pragma unroll
       for (int i = 0; i < 16; ++i) fin[st_base + (size_t)(c0 + i) * D + j] = s[i];
     }
-  } else {
-    // a bounded wait gave up: drain what is in flight (fwd_tc.cu), bounded
-    if (tid == 0) {
-      if (p.err) atomicExch(p.err, RDN_ERR_TIMEOUT);
-      mma_commit(barD);
-      mbar_wait(barD, 0);
-      if (pendA) mbar_wait(barA, phA);
-      if (pendB) mbar_wait(barB, phB);
-      if (pendE) mbar_wait(barE, phE & 1u);
-      if (handed) mbar_wait_cluster(barX, (handed - 1) & 1u, limit);
-      bulk_wait_all();
-    }
-    cp_async_wait_all();
   }
+  cp_async_wait_all();
   fence_before_sync();
   __syncthreads();
   cluster_sync();  // the partner may still write here, or arrive on a barrier
@@ -641,7 +763,7 @@ cudaError_t launch_fwd_pair(const FwdParams &p, const fwdtc::FwdMaps &maps, bool
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(2 * p.nseq * p.H);
-  cfg.blockDim = dim3(kTcThreads);
+  cfg.blockDim = dim3(kPairThreads);
   cfg.dynamicSmemBytes = kPairSmem;
   cfg.stream = s;
   cudaLaunchAttribute at{};

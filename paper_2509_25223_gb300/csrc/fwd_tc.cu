@@ -719,7 +719,10 @@ cudaError_t launch_fwd_tc(const FwdParams &p, bool rdnv, cudaStream_t s) {
   int nsm = 0;
   cudaError_t e = sm_count(&nsm);
   if (e != cudaSuccess) return e;
-  if (use_pairs(p, nsm)) return launch_fwd_pair(p, maps, rdnv, s);
+  if (use_pairs(p, nsm)) {
+    maps.o_ok = !p.f32out && make_tile_map(maps.o, p.o, D, p.H, rows);
+    return launch_fwd_pair(p, maps, rdnv, s);
+  }
   const bool generic = p.mods != 0;
   auto kern = rdnv ? (generic ? fwd_tc_kernel<true, true> : fwd_tc_kernel<true, false>)
                    : (generic ? fwd_tc_kernel<false, true> : fwd_tc_kernel<false, false>);

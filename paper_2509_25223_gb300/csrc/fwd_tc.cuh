@@ -68,6 +68,8 @@ struct FwdMaps {
   alignas(64) unsigned char k[128];
   alignas(64) unsigned char q[128];
   bool ok;
+  alignas(64) unsigned char o[128];  // (fwd_pair.cu: bf16 results)
+  bool o_ok;
 };
 
 }  // namespace fwdtc

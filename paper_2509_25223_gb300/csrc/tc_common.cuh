@@ -85,6 +85,20 @@ __device__ __forceinline__ void tma_load_3d(void *dst_smem, const void *map, int
       : "memory");
 }
 
+// A box of shared memory (same layouts) stored to global memory, tracked by this
+// thread's bulk groups (bulk_commit, bulk_wait_*).
+__device__ __forceinline__ void tma_store_3d(const void *map, int c0, int c1, int c2, const void *src_smem) {
+  asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"(map),
+               "r"(c0), "r"(c1), "r"(c2), "r"(smem_u32(src_smem))
+               : "memory");
+}
+// The same box brought into L2 ahead of its copy.
+__device__ __forceinline__ void tma_prefetch_3d(const void *map, int c0, int c1, int c2) {
+  asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(map),
+               "r"(c0), "r"(c1), "r"(c2)
+               : "memory");
+}
+
 // Hints that bring global memory closer ahead of its use (no completion to
 // wait for; the later loads find the lines cached): into L2, a contiguous
 // range (16-byte aligned address and size) or the 128-byte line of one address.
@@ -162,6 +176,15 @@ __device__ __forceinline__ void bulk_wait_all() {
   asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
+// Named barrier `id` of `count` threads (whole warps): arrive without waiting,
+// or arrive and wait.
+__device__ __forceinline__ void bar_arrive(int id, int count) {
+  asm volatile("barrier.cta.arrive %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
+__device__ __forceinline__ void bar_sync(int id, int count) {
+  asm volatile("barrier.cta.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
+
 // ----------------------------------------------------------------- clusters
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
@@ -191,10 +214,11 @@ __device__ __forceinline__ void bulk_s2s(uint32_t dst, const void *src, uint32_t
       "r"(smem_u32(src)), "r"(bytes), "r"(bar)
       : "memory");
 }
-// One arrival on a barrier of another CTA, releasing this thread's earlier
-// accesses (and, after a __syncwarp, its warp's) at cluster scope.
-__device__ __forceinline__ void mbar_arrive_remote(uint32_t addr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+// One arrival on a barrier of another CTA, without releasing this thread's
+// earlier writes (a release would wait until its global stores are performed):
+// for signals that something has been read, sent once the values are used.
+__device__ __forceinline__ void mbar_arrive_remote_relaxed(uint32_t addr) {
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
 // mbar_wait for a barrier that another CTA of the cluster arrives on.
 __device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t *bar, uint32_t parity) {
@@ -308,6 +332,44 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&v)[16]) 
       : "memory");
 }
 
+// 8 32-bit columns (16 packed bf16 of an A operand) hi at ta and lo at tb, one
+// wait for both.
+__device__ __forceinline__ void tmem_st8x2(uint32_t ta, const uint32_t (&a)[8], uint32_t tb,
+                                           const uint32_t (&b)[8]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%2,%3,%4,%5,%6,%7,%8,%9};\n"
+      "tcgen05.st.sync.aligned.32x32b.x8.b32 [%1], {%10,%11,%12,%13,%14,%15,%16,%17};\n"
+      "tcgen05.wait::st.sync.aligned;\n" ::"r"(ta),
+      "r"(tb), "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(a[4]), "r"(a[5]), "r"(a[6]),
+      "r"(a[7]), "r"(b[0]), "r"(b[1]), "r"(b[2]), "r"(b[3]), "r"(b[4]), "r"(b[5]), "r"(b[6]),
+      "r"(b[7])
+      : "memory");
+}
+// ... and of one such operand
+__device__ __forceinline__ void tmem_st8(uint32_t ta, const uint32_t (&a)[8]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};\n"
+      "tcgen05.wait::st.sync.aligned;\n" ::"r"(ta),
+      "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(a[4]), "r"(a[5]), "r"(a[6]), "r"(a[7])
+      : "memory");
+}
+// Two such stores with one wait for both.
+__device__ __forceinline__ void tmem_st16x2(uint32_t ta, const float (&a)[16], uint32_t tb,
+                                            const float (&b)[16]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+      "{%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17};\n"
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%1], "
+      "{%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32,%33};\n"
+      "tcgen05.wait::st.sync.aligned;\n" ::"r"(ta),
+      "r"(tb), "f"(a[0]), "f"(a[1]), "f"(a[2]), "f"(a[3]), "f"(a[4]), "f"(a[5]), "f"(a[6]),
+      "f"(a[7]), "f"(a[8]), "f"(a[9]), "f"(a[10]), "f"(a[11]), "f"(a[12]), "f"(a[13]), "f"(a[14]),
+      "f"(a[15]), "f"(b[0]), "f"(b[1]), "f"(b[2]), "f"(b[3]), "f"(b[4]), "f"(b[5]), "f"(b[6]),
+      "f"(b[7]), "f"(b[8]), "f"(b[9]), "f"(b[10]), "f"(b[11]), "f"(b[12]), "f"(b[13]), "f"(b[14]),
+      "f"(b[15])
+      : "memory");
+}
+
 // --------------------------------------------------------------------- MMA
 // Instruction descriptor, kind::f16: D fp32, A and B bf16, both K-major,
 // shape M x N (M in {64, 128}; N a multiple of 16 up to 256).
@@ -362,6 +424,20 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n"
       "}\n" ::"r"(d_tmem),
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+
+// The same with A in TMEM: lane = row of A, two bf16 of K a 32-bit column (8
+// columns for K = 16).
+__device__ __forceinline__ void mma_bf16_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc,
+                                            uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n"
+      ".reg .pred p;\n"
+      "setp.ne.b32 p, %4, 0;\n"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n"
+      "}\n" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 
