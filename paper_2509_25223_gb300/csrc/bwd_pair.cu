@@ -52,6 +52,7 @@ __global__ void __launch_bounds__(NTC, 1) bwd_pair_kernel(const __grid_constant_
   const FwdParams &p = P.f;
   const bool rla = kGeneric && P.rla;
   const unsigned mods = kGeneric ? p.mods : 0u;
+  if (!picked(p)) return;
   if (sb & 1023u) {  // (the same in both CTAs)
     if (threadIdx.x == 0 && p.err) atomicExch(p.err, RDN_ERR_CUDA);
     return;
@@ -64,15 +65,14 @@ __global__ void __launch_bounds__(NTC, 1) bwd_pair_kernel(const __grid_constant_
   const uint32_t rank = cluster_rank();
   const bool base = rank == 0;  // CTA 0: dS; CTA 1: dR
   const int g16 = (warp >> 2) * 16;  // this thread's token (and key) columns start
-  const int bh = blockIdx.x >> 1;
-  const int H = p.H, h = bh % H;
-  const SeqSpan sp = seq_span(p, bh / H, h);
+  const int H = p.H, sq = seq_at(p, (blockIdx.x >> 1) / H), h = (blockIdx.x >> 1) % H;
+  const SeqSpan sp = seq_span(p, sq, h);
   const long long tok0 = sp.tok0;
   const int NC = sp.nc, T = sp.len;
   const __nv_bfloat16 *q = (const __nv_bfloat16 *)p.q, *k = (const __nv_bfloat16 *)p.k,
                       *dOp = (const __nv_bfloat16 *)P.dO;
   __nv_bfloat16 *dv = (__nv_bfloat16 *)P.dv;
-  const size_t st_base = (size_t)bh * D * D;
+  const size_t st_base = ((size_t)sq * H + h) * D * D;
   const bool tnh = kGeneric && (mods & RDN_FLAG_TANH_RESIDUAL);
   const bool stl = kGeneric && (mods & RDN_FLAG_STATELESS_AUX);
   const bool plain = mods & RDN_FLAG_PLAIN_COMBINE;

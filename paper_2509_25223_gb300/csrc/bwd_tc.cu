@@ -271,6 +271,7 @@ __global__ void __launch_bounds__(NTC, 1) bwd_chain_kernel(const __grid_constant
   const FwdParams &p = P.f;
   const bool rla = kGeneric && P.rla;
   const unsigned mods = kGeneric ? p.mods : 0u;
+  if (!picked(p)) return;
   if (sb & 1023u) {
     if (threadIdx.x == 0 && p.err) atomicExch(p.err, RDN_ERR_CUDA);
     return;
@@ -280,15 +281,14 @@ __global__ void __launch_bounds__(NTC, 1) bwd_chain_kernel(const __grid_constant
   uint32_t *slot = reinterpret_cast<uint32_t *>(sm + SLOT);
   const int tid = threadIdx.x, warp = tid >> 5, j = tid & 127;
   const int g16 = (warp >> 2) * 16;  // this thread's token (and key) columns start
-  const int bh = blockIdx.x;
-  const int H = p.H, h = bh % H;
-  const SeqSpan sp = seq_span(p, bh / H, h);  // this (sequence, head)'s tokens and records
+  const int H = p.H, sq = seq_at(p, blockIdx.x / H), h = blockIdx.x % H;
+  const SeqSpan sp = seq_span(p, sq, h);  // this (sequence, head)'s tokens and records
   const long long tok0 = sp.tok0;
   const int NC = sp.nc, T = sp.len;
   const __nv_bfloat16 *q = (const __nv_bfloat16 *)p.q, *k = (const __nv_bfloat16 *)p.k,
                       *dOp = (const __nv_bfloat16 *)P.dO;
   __nv_bfloat16 *dv = (__nv_bfloat16 *)P.dv;
-  const size_t st_base = (size_t)bh * D * D;
+  const size_t st_base = ((size_t)sq * H + h) * D * D;
 
   Ctl K;
   ctl_init(K, sm + CTL, tid);
@@ -1574,9 +1574,13 @@ cudaError_t launch_bwd_tc(const FwdParams &f, const void *dO, const float *dST, 
   }
   int nsm = 0;
   if ((e = sm_count(&nsm)) != cudaSuccess) return e;
-  if (use_pairs(f, nsm)) {
+  const bool both = pick_on_device(f, nsm);
+  if (both || use_pairs(f, nsm)) {
+    P.f.pick = both ? 2 : 0;
     if ((e = launch_bwd_pair(P, s)) != cudaSuccess) return e;
-  } else {
+    P.f.pick = 1;
+  }
+  if (both || !use_pairs(f, nsm)) {
     RDN_LAUNCH("bwd_chain", s, chain<<<f.nseq * f.H, NTC, ch::SMEM, s>>>(P));
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }

@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 2 : 1) bwd_chain_kernel(BwdPar
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int ln = lane % LN, r0 = LM * warp + lane / LN, n0 = TN * ln;
   const int kw = 2 * LM * warp;  // the warp's first row
-  const int H = p.f.H, sq = blockIdx.x / H, h = blockIdx.x % H;
+  const int H = p.f.H, sq = seq_at(p.f, blockIdx.x / H), h = blockIdx.x % H;
   const SeqSpan sp = seq_span(p.f, sq, h);
   const int j0 = blockIdx.y * DVS;
   const bool dec_res = p.f.mods & RDN_FLAG_DECAYED_RESIDUAL;
@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 2 : 1) bwd_chain_kernel(BwdPar
   const bool stl = p.f.mods & RDN_FLAG_STATELESS_AUX;
   const bool rdn_aux = RDNV && !stl;  // the auxiliary pass runs the delta rule
 
-  const size_t sbase = (size_t)blockIdx.x * DK * DV;
+  const size_t sbase = ((size_t)sq * H + h) * DK * DV;
   for (int e = tid; e < DK * DVS / 4; e += NT) {
     const size_t off = sbase + (size_t)(e / (DVS / 4)) * DV + j0 + 4 * (e % (DVS / 4));
     const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);

@@ -134,8 +134,13 @@ struct FwdParams {
   unsigned long long *sv_mask;
   // Packed variable-length sequences (rdn_fwd_args.cu_seqlens), or NULL for B
   // sequences of T tokens each: for s = 0 .. nseq, {first token, first chunk}
-  // of sequence s (entry nseq closes the list: {T, total chunks}).
+  // of sequence s (entry nseq closes the list: {T, total chunks}).  The upper
+  // halves of the chunk numbers hold the sequences from the longest to the
+  // shortest and, in entry nseq, whether the sequential tensor-core kernels run
+  // on CTA pairs (launch_seq_table).
   const long long *seq;
+  int pick;        // of two kernels launched for a packed call, this is the one for single
+                   // CTAs (1) or for pairs (2), and the table says which runs; 0: the only one
   int nseq;        // sequences: B, or the number of packed sequences
   long long nrec;  // record slots: B * H * NC, or a bound on H * (total chunks)
   unsigned mods;   // the variant flags (RDN_FLAG_VARIANTS bits of rdn_fwd_args.flags)
@@ -159,13 +164,16 @@ struct SeqSpan {
   long long tok0, rbase;
   int len, nc;
 };
+__host__ __device__ __forceinline__ long long first_chunk(const FwdParams &p, int s) {
+  return p.seq[2 * s + 1] & 0xffffffffll;
+}
 __host__ __device__ __forceinline__ SeqSpan seq_span(const FwdParams &p, int s, int h) {
   SeqSpan q;
   if (p.seq) {
     q.tok0 = p.seq[2 * s];
     q.len = (int)(p.seq[2 * s + 2] - q.tok0);
     q.nc = (q.len + C - 1) / C;
-    q.rbase = p.seq[2 * s + 1] * p.H + (long long)h * q.nc;
+    q.rbase = first_chunk(p, s) * p.H + (long long)h * q.nc;
   } else {
     q.tok0 = (long long)s * p.T;
     q.len = p.T;
@@ -174,9 +182,19 @@ __host__ __device__ __forceinline__ SeqSpan seq_span(const FwdParams &p, int s, 
   }
   return q;
 }
+// The k-th sequence to start on: packed sequences from the longest to the
+// shortest, since the sequential kernels end with the last chunk of the one
+// that ends last.
+__device__ __forceinline__ int seq_at(const FwdParams &p, int k) {
+  return p.seq ? (int)(p.seq[2 * k + 1] >> 32) : k;
+}
+// Whether this kernel is the one of a packed call's two that runs.
+__device__ __forceinline__ bool picked(const FwdParams &p) {
+  return p.pick == 0 || (p.seq[2 * p.nseq + 1] >> 32 != 0) == (p.pick == 2);
+}
 // chunk records in use (at most nseq * H * NC slots)
 __device__ __forceinline__ long long total_records(const FwdParams &p) {
-  return p.seq ? p.seq[2 * p.nseq + 1] * p.H : (long long)p.nseq * p.H * p.NC;
+  return p.seq ? first_chunk(p, p.nseq) * p.H : (long long)p.nseq * p.H * p.NC;
 }
 // record r -> (sequence s, head h, chunk c); r < total_records(p)
 __device__ __forceinline__ void rec_decode(const FwdParams &p, long long r, int &s, int &h, int &c) {
@@ -198,11 +216,11 @@ __device__ __forceinline__ void rec_decode(const FwdParams &p, long long r, int 
   int lo = 0, hi = p.nseq - 1;  // the last sequence whose records start at or before r
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
-    if (p.seq[2 * mid + 1] * p.H <= r) lo = mid; else hi = mid - 1;
+    if (first_chunk(p, mid) * p.H <= r) lo = mid; else hi = mid - 1;
   }
   s = lo;
   const int nc = (int)((p.seq[2 * s + 2] - p.seq[2 * s] + C - 1) / C);
-  const long long off = r - p.seq[2 * s + 1] * p.H;  // < H * nc
+  const long long off = r - first_chunk(p, s) * p.H;  // < H * nc
   h = (int)((unsigned)off / (unsigned)nc);
   c = (int)(off - (long long)h * nc);
 }
@@ -250,6 +268,7 @@ inline FwdParams make_fwd_params(const rdn_fwd_args &a) {
   p.sv_E = p.sv_E2 = nullptr;
   p.sv_mask = nullptr;
   p.seq = nullptr;  // set by the launcher once the table is in its workspace
+  p.pick = 0;
   p.nseq = call_seqs(a);
   p.nrec = call_records(a);
   p.mods = a.flags & RDN_FLAG_VARIANTS;
@@ -314,15 +333,26 @@ inline cudaError_t sm_count(int *n) {
   return e != cudaSuccess ? e : cudaDeviceGetAttribute(n, cudaDevAttrMultiProcessorCount, dev);
 }
 
-// Whether a sequential tensor-core kernel gives each (sequence, head) a pair
-// of CTAs (fwd_pair.cu, bwd_pair.cu) or one: whichever ends first, in waves of
-// one CTA per SM, a chunk costing a pair about 0.7 of what it costs one CTA
-// (forward 6.2 us against 8.8, saving 7.6 against 8.8; backward 9.0 against
-// 12.0; 32 heads, T = 16384 and 2000).
+// Whether a sequential tensor-core kernel gives each (sequence, head) a pair of
+// CTAs (fwd_pair.cu, bwd_pair.cu) or one: whichever ends first.  A chunk costs
+// a pair about 0.6 of what it costs one CTA (forward 4.4 us against 8.8, saving
+// 6.1 against 8.8; backward 8.1 against 12.0; 32 heads, T = 16384 and 2000).
+// Equal sequences run in waves of one CTA per SM:
 inline bool use_pairs(const FwdParams &p, int nsm) {
   const long long n = (long long)p.nseq * p.H;
   const long long waves1 = (n + nsm - 1) / nsm, waves2 = (2 * n + nsm - 1) / nsm;
-  return 10 * waves1 > 7 * waves2;
+  return 10 * waves1 > 6 * waves2;
+}
+// Packed sequences differ in length: the longest one's chain of chunks or the
+// chip's throughput sets the time.  The lengths are on the device, so that
+// where pairs do not all fit at once both kernels are launched and the table
+// says which one runs (the other's CTAs return at once).
+__host__ __device__ inline bool pairs_for(long long longest, long long chunks, int H, int nsm) {
+  const long long t1 = chunks * H / nsm, t2 = 2 * chunks * H / nsm;
+  return 10 * (longest > t1 ? longest : t1) > 6 * (longest > t2 ? longest : t2);
+}
+inline bool pick_on_device(const FwdParams &p, int nsm) {
+  return p.seq && 2ll * p.nseq * p.H > nsm;
 }
 
 }  // namespace rdn

@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 2 : 1) chunk_scan_kernel(FwdPa
     rec_decode(p, blockIdx.x, sq, h, c0);
     c1 = c0 + 1;
   } else {
-    sq = blockIdx.x / p.H;
+    sq = seq_at(p, blockIdx.x / p.H);
     h = blockIdx.x % p.H;
   }
   const SeqSpan sp = seq_span(p, sq, h);
@@ -602,14 +602,17 @@ __device__ long long block_incl_scan(long long x, Op op, long long *wsum) {
   return x;
 }
 
+constexpr int kOrdered = 1024;  // packed sequences that are put in order of length
 // The packed-sequence table FwdParams::seq from cu_seqlens[0 .. N]: first
 // tokens are the running maximum of the entries clamped into [0, T] (with
 // entry 0 read as 0 and entry N as T, so the table always covers [0, T) in
 // order), first chunks the exclusive prefix sum of ceil(len_s / 64).  One CTA.
 __global__ void __launch_bounds__(1024) seq_table_kernel(const int *__restrict__ cu, int N, int T,
+                                                         int H, int nsm,
                                                          long long *__restrict__ seq) {
   __shared__ long long wsum[32];
   __shared__ long long carry;
+  __shared__ int ncs[kOrdered];  // the sequences' chunks
   const int tid = threadIdx.x;
   if (tid == 0) carry = 0;
   __syncthreads();
@@ -631,13 +634,30 @@ __global__ void __launch_bounds__(1024) seq_table_kernel(const int *__restrict__
     const long long nc = s < N ? (seq[2 * s + 2] - seq[2 * s] + C - 1) / C : 0;
     const long long incl = block_incl_scan(nc, add, wsum) + carry;
     if (s <= N) seq[2 * s + 1] = incl - nc;  // entry N: the total
+    if (s < min(N, kOrdered)) ncs[s] = (int)nc;
     if (tid == 1023) carry = incl;
     __syncthreads();
+  }
+  // longest first (more than kOrdered sequences: as they come)
+  int *upper = reinterpret_cast<int *>(seq) + 3;  // of the k-th chunk number: upper[4 k]
+  if (N > kOrdered) {
+    for (int s = tid; s < N; s += 1024) upper[4 * s] = s;
+  } else if (tid < N) {
+    const int mine = ncs[tid];
+    int rank = 0;
+    for (int u = 0; u < N; ++u) rank += ncs[u] > mine || (ncs[u] == mine && u < tid);
+    upper[4 * rank] = tid;
+    // (entry N's stays 0, no pairs, for more than kOrdered sequences)
+    if (rank == 0) upper[4 * N] = pairs_for(mine, carry, H, nsm);
   }
 }
 
 cudaError_t launch_seq_table(const rdn_fwd_args &a, long long *seq, cudaStream_t s) {
-  RDN_LAUNCH("seq_table", s, seq_table_kernel<<<1, 1024, 0, s>>>(a.cu_seqlens, a.num_seqs, a.T, seq));
+  int nsm = 0;
+  const cudaError_t e = sm_count(&nsm);
+  if (e != cudaSuccess) return e;
+  RDN_LAUNCH("seq_table", s,
+             seq_table_kernel<<<1, 1024, 0, s>>>(a.cu_seqlens, a.num_seqs, a.T, a.H, nsm, seq));
   return cudaGetLastError();
 }
 

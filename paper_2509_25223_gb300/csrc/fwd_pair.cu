@@ -79,6 +79,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     fwd_pair_kernel(FwdParams p, const __grid_constant__ FwdMaps maps) {
   extern __shared__ __align__(1024) uint8_t sm[];
   const uint32_t sbase = smem_u32(sm);
+  if (!picked(p)) return;
   if (sbase & 1023u) {  // (the same in both CTAs)
     if (threadIdx.x == 0 && p.err) atomicExch(p.err, RDN_ERR_CUDA);
     return;
@@ -96,9 +97,8 @@ __global__ void __launch_bounds__(kPairThreads, 1)
   const bool base = rank == 0;     // CTA 0: S; CTA 1: R
   const int j = tid & 127;         // value column == TMEM lane
   const int g16 = (warp >> 2) * 16;  // this thread's token (and state) columns start
-  const int bh = blockIdx.x >> 1;
-  const int h = bh % p.H;
-  const SeqSpan sp = seq_span(p, bh / p.H, h);
+  const int sq = seq_at(p, (blockIdx.x >> 1) / p.H), h = (blockIdx.x >> 1) % p.H;
+  const SeqSpan sp = seq_span(p, sq, h);
   const long long tok0 = sp.tok0;
   const int T = sp.len, H = p.H, NC = sp.nc;
   const __nv_bfloat16 *q = (const __nv_bfloat16 *)p.q;
@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
   const bool plain = kGeneric && (p.mods & RDN_FLAG_PLAIN_COMBINE);
   const bool tnh = kGeneric && (p.mods & RDN_FLAG_TANH_RESIDUAL);
   const bool stl = kGeneric && (p.mods & RDN_FLAG_STATELESS_AUX);
-  const size_t st_base = (size_t)bh * D * D;
+  const size_t st_base = ((size_t)sq * p.H + h) * D * D;
 
   if (tid == 0) {
     for (int b = 0; b < 5; ++b) mbar_init(bar + b, 1);

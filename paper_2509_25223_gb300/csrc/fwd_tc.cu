@@ -83,6 +83,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     fwd_tc_kernel(FwdParams p, const __grid_constant__ FwdMaps maps) {
   extern __shared__ __align__(1024) uint8_t sm[];
   const uint32_t sbase = smem_u32(sm);
+  if (!picked(p)) return;
   if (sbase & 1023u) {  // the swizzled tiles need a 1024-byte aligned base
     if (threadIdx.x == 0 && p.err) atomicExch(p.err, RDN_ERR_CUDA);
     return;
@@ -100,9 +101,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   const int tid = threadIdx.x, warp = tid >> 5;
   const int j = tid & 127;       // value column == TMEM lane
   const int g16 = (warp >> 2) * 16;  // this thread's token (and state) columns start
-  const int bh = blockIdx.x;
-  const int h = bh % p.H;
-  const SeqSpan sp = seq_span(p, bh / p.H, h);  // this (sequence, head)'s tokens and records
+  const int sq = seq_at(p, blockIdx.x / p.H), h = blockIdx.x % p.H;
+  const SeqSpan sp = seq_span(p, sq, h);  // this (sequence, head)'s tokens and records
   const long long tok0 = sp.tok0;
   const int T = sp.len, H = p.H, NC = sp.nc;
   const __nv_bfloat16 *q = (const __nv_bfloat16 *)p.q;
@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   // by 0); the records hold the identity T_gamma, diag(gamma qk) and the
   // one-hot wR that make the rest of the pass compute it
   const bool stl = kGeneric && (p.mods & RDN_FLAG_STATELESS_AUX);
-  const size_t st_base = (size_t)bh * D * D;
+  const size_t st_base = ((size_t)sq * p.H + h) * D * D;
 
   if (tid == 0) {
     mbar_init(bar, 1);
@@ -719,16 +719,21 @@ cudaError_t launch_fwd_tc(const FwdParams &p, bool rdnv, cudaStream_t s) {
   int nsm = 0;
   cudaError_t e = sm_count(&nsm);
   if (e != cudaSuccess) return e;
-  if (use_pairs(p, nsm)) {
+  FwdParams one = p;
+  const bool both = pick_on_device(p, nsm);
+  if (both || use_pairs(p, nsm)) {
     maps.o_ok = !p.f32out && make_tile_map(maps.o, p.o, D, p.H, rows);
-    return launch_fwd_pair(p, maps, rdnv, s);
+    FwdParams two = p;
+    two.pick = both ? 2 : 0;
+    if ((e = launch_fwd_pair(two, maps, rdnv, s)) != cudaSuccess || !both) return e;
+    one.pick = 1;
   }
   const bool generic = p.mods != 0;
   auto kern = rdnv ? (generic ? fwd_tc_kernel<true, true> : fwd_tc_kernel<true, false>)
                    : (generic ? fwd_tc_kernel<false, true> : fwd_tc_kernel<false, false>);
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmem);
   if (e != cudaSuccess) return e;
-  RDN_LAUNCH("fwd_tc_scan", s, kern<<<p.nseq * p.H, kTcThreads, kTcSmem, s>>>(p, maps));
+  RDN_LAUNCH("fwd_tc_scan", s, kern<<<p.nseq * p.H, kTcThreads, kTcSmem, s>>>(one, maps));
   return cudaGetLastError();
 }
 

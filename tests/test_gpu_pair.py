@@ -40,3 +40,29 @@ def test_pair_equals_one_cta(variant, T, saved, flags):
     for n, t in few.items():
         assert torch.equal(t, many[n][7:8]), n
     assert rdn.device_status() == 0
+
+
+@pytest.mark.parametrize("lens,H", [
+    ([64] * 80, 2),              # equal lengths in more heads than pairs fit: one CTA each
+    ([1, 5] + [3] * 80 + [700], 2),  # one long sequence among many, last: pairs, it first
+    ([2, 0, 1] * 400, 1),        # more sequences than are put in order
+])
+def test_packed_order_and_kernel_choice(lens, H):
+    """Packed calls start on the longest sequences and let the table choose the
+    kernel: every sequence as in a call of its own, bit for bit."""
+    T = sum(lens)
+    x = make_inputs(1, T, H, 128, dtype="bf16", device="cuda")
+    cu = torch.tensor([0] + lens, dtype=torch.int32).cumsum(0).to(torch.int32).cuda()
+    st = 0.1 * torch.randn(2, len(lens), H, 128, 128, generator=torch.Generator().manual_seed(3)).cuda()
+    o, ST, RT = rdn.rdn_fwd(*(x[n] for n in NAMES), clip=0.7, S0=st[0], R0=st[1], cu_seqlens=cu)
+    first = 0
+    for s, n in enumerate(lens):
+        if n and (s < 4 or n > 10 or s % 97 == 0):
+            sl = {m: x[m][:, first:first + n].clone() for m in NAMES}  # (aligned)
+            o1, S1, R1 = rdn.rdn_fwd(*(sl[m] for m in NAMES), clip=0.7,
+                                     S0=st[0, s:s + 1].contiguous(), R0=st[1, s:s + 1].contiguous())
+            assert torch.equal(o[:, first:first + n], o1), s
+            assert torch.equal(ST[s], S1[0]) and torch.equal(RT[s], R1[0]), s
+        elif not n:
+            assert torch.equal(ST[s], st[0, s]) and torch.equal(RT[s], st[1, s]), s
+        first += n
