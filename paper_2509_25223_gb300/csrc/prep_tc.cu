@@ -17,6 +17,10 @@
 //      T_ij = -T_ii A_ij T_jj for the 16-row blocks (1,0), (3,2) and the
 //      32-row block (1,0), the products register-tiled;
 //   4. their image rows and the gate vectors.
+// Images are staged in shared memory that is free by then and leave by bulk
+// copies: a lane's 16 bytes of a row straight to global memory touch 32 lines a
+// warp, and those stores took two fifths of the kernel (8192 chunks 0.395 ->
+// 0.337 ms; three CTAs of 80 registers per SM without it 0.369 ms).
 #include "chunk_common.cuh"
 #include "tc_common.cuh"
 
@@ -29,7 +33,6 @@ constexpr int D = 128;
 constexpr int NTH = 256;
 constexpr int LDA = C + 1;  // A_beta, A_gamma: rows written by the row pass, read as scalars
 constexpr int LDT = C + 4;  // T_beta, T_gamma: rows read as 16-byte vectors
-constexpr int LDW = 36;     // product scratch W, 32 x 32
 
 namespace pp {
 constexpr uint32_t KQ = 0;                   // K rows 0..63, Q rows 64..127, 2 x 16 KB
@@ -37,19 +40,24 @@ constexpr uint32_t AB = 32768;               // fp32 A_beta, A_gamma [64][LDA]
 constexpr uint32_t AG = AB + 64 * LDA * 4;
 constexpr uint32_t TB = AG + 64 * LDA * 4;   // fp32 T_beta, T_gamma [64][LDT]
 constexpr uint32_t TG = TB + 64 * LDT * 4;
-constexpr uint32_t WS = TG + 64 * LDT * 4;   // product scratch, 2 x [32][LDW]
+                                             // (product scratch: rows 0..31, columns 32..63)
 // cum, cprev, beta, gamma, g, and cum, cprev times log2(e) (7 x 64)
-constexpr uint32_t VEC = WS + 2 * 32 * LDW * 4;
-static_assert(TB % 16 == 0 && TG % 16 == 0 && WS % 16 == 0 && VEC % 16 == 0, "16-byte rows");
-constexpr uint32_t CTL = VEC + 7 * 64 * 4;   // mbarrier, flag, drain mbarrier
+constexpr uint32_t VEC = TG + 64 * LDT * 4;
+constexpr uint32_t M2H = VEC + 7 * 64 * 4;   // the hi part of M2's image, 8 KB
+constexpr uint32_t CTL = M2H + 8192;         // mbarrier, flag, drain mbarrier
 constexpr uint32_t SLOT = CTL + 24;          // TMEM base
 constexpr size_t SMEM = SLOT + 16;
+static_assert(TB % 16 == 0 && TG % 16 == 0 && VEC % 16 == 0 && M2H % 16 == 0, "16-byte rows");
+// the images leave by bulk copies: [Ap ; Mq]'s from the place of K and Q, those
+// of T from the place of A
+constexpr uint32_t APMQ = KQ, TIMG = AB;
+static_assert(AB % 16 == 0 && TB - AB >= 32768, "T's images fit over A_beta, A_gamma");
 static_assert(2 * (SMEM + 1024) <= 233472, "two CTAs per SM");
 }  // namespace pp
 
 // Row r, columns c0 .. c0+15 (c0 a multiple of 16 below 64) of a 64-column
-// image in global memory: bf16 hi part at `hi`, lo part `lo_off` bytes later.
-__device__ __forceinline__ void img_row16(uint8_t *hi, uint32_t lo_off, int r, int c0,
+// image: bf16 hi part at `hi`, lo part at `lo`.
+__device__ __forceinline__ void img_row16(uint8_t *hi, uint8_t *lo, int r, int c0,
                                           const float (&v)[16]) {
   uint32_t h[8], l[8];
 #pragma unroll
@@ -59,7 +67,7 @@ __device__ __forceinline__ void img_row16(uint8_t *hi, uint32_t lo_off, int r, i
     const uint32_t off = sw128(r, c0 + 8 * half);
     *reinterpret_cast<uint4 *>(hi + off) =
         make_uint4(h[4 * half], h[4 * half + 1], h[4 * half + 2], h[4 * half + 3]);
-    *reinterpret_cast<uint4 *>(hi + lo_off + off) =
+    *reinterpret_cast<uint4 *>(lo + off) =
         make_uint4(l[4 * half], l[4 * half + 1], l[4 * half + 2], l[4 * half + 3]);
   }
 }
@@ -78,7 +86,6 @@ __global__ void __launch_bounds__(NTH, 2) prep_tc_kernel(FwdParams p, bool rla) 
         *gam = cum + 192, *gg = cum + 256, *cum2 = cum + 320, *cprev2 = cum + 384;
   float *Ab = reinterpret_cast<float *>(sm + AB), *Ag = reinterpret_cast<float *>(sm + AG);
   float *Tb = reinterpret_cast<float *>(sm + TB), *Tg = reinterpret_cast<float *>(sm + TG);
-  float *Wsc = reinterpret_cast<float *>(sm + WS);
   uint64_t *bar = reinterpret_cast<uint64_t *>(sm + CTL);
   volatile int *flag = reinterpret_cast<volatile int *>(sm + CTL + 8);
   uint64_t *barD = reinterpret_cast<uint64_t *>(sm + CTL + 16);  // the drain after a wait gave up
@@ -257,14 +264,12 @@ __global__ void __launch_bounds__(NTH, 2) prep_tc_kernel(FwdParams p, bool rla) 
       cprev2[32 + lane] = p2 * kLog2e;
     }
     if (!mbar_wait(bar, it & 1u)) *flag = 1;
+    if (tid == 0) bulk_wait_read();  // (the previous chunk's images of T have left A's place)
     __syncthreads();
     fence_after_sync();
     ok = *flag == 0;
     if (!ok) break;
-    if (next < nct) {  // K, Q are done with: the next chunk's, during this one
-      fetch_kq(next);
-      gt = fetch_gates(next);
-    }
+    if (next < nct) gt = fetch_gates(next);
     uint8_t *img = reinterpret_cast<uint8_t *>(p.ws + chunk * kRecFloats);
     {  // thread (row r, half hf) of the Gram read-out: columns i in [32 hf, 32 hf + 32)
       const int r = tid & 127, hf = tid >> 7;
@@ -304,7 +309,7 @@ __global__ void __launch_bounds__(NTH, 2) prep_tc_kernel(FwdParams p, bool rla) 
             Ab[t * LDA + i] = a_b;
             Ag[t * LDA + i] = a_g;
           }
-          img_row16(img + IMG_APMQ, 16384, t, i0, ap);
+          img_row16(sm + APMQ, sm + APMQ + 16384, t, i0, ap);
         }
       } else {  // Q K^T row t: Mq (strict), diag(gamma) M2 (inclusive)
         const int t = r - 64;
@@ -326,39 +331,55 @@ __global__ void __launch_bounds__(NTH, 2) prep_tc_kernel(FwdParams p, bool rla) 
             mq[u] = i < t ? (plain ? exp2f(cq2 - c2[u]) * qk : dec) * bt[u] : 0.f;
             m2[u] = stl ? (i == t ? gtt * qk : 0.f) : gtt * dec * gm[u];
           }
-          img_row16(img + IMG_APMQ, 16384, 64 + t, i0, mq);
-          img_row16(img + IMG_M2, 8192, t, i0, m2);
+          img_row16(sm + APMQ, sm + APMQ + 16384, 64 + t, i0, mq);
+          img_row16(sm + M2H, img + IMG_M2 + 8192, t, i0, m2);
         }
       }
     }
+    fence_async_smem();
     __syncthreads();
+    if (tid == 0) {
+      bulk_s2g(img + IMG_APMQ, sm + APMQ, 32768);
+      bulk_s2g(img + IMG_M2, sm + M2H, 8192);
+      bulk_commit();
+    }
     if (!rla) {  // T_beta (threads 0..127) and T_gamma (128..255)
       const int g = tid & 127;
       const float *A = tid < 128 ? Ab : Ag;
       float *Tm = tid < 128 ? Tb : Tg;
-      float *W = Wsc + (tid < 128 ? 0 : 32 * LDW);
 #pragma unroll 1
       for (int stage = 0; stage < 5; ++stage) {
         if (stage) __syncthreads();
-        inv64_stage<LDA, LDT, LDW>(stage, A, Tm, W, g);
+        if (stage == 3 && next < nct) fetch_kq(next);  // (the [Ap ; Mq] image has left)
+        inv64_stage<LDA, LDT, LDT>(stage, A, Tm, Tm + 32, g);
+        if (stage == 2 && tid == 0) bulk_wait_read();
       }
+      __syncthreads();
+    } else {
+      if (tid == 0) bulk_wait_read();
+      __syncthreads();
+      if (next < nct) fetch_kq(next);
     }
-    __syncthreads();
-    {  // image rows of T: thread (row r, matrix m, half hf)
+    {  // image rows of T: thread (row r, matrix m, half hf); the block above the
+       // diagonal at rows 0..31 was the products' scratch
       const int r = tid & 63, m = (tid >> 6) & 1, hf = tid >> 7;
       const float *Tm = m ? Tg : Tb;
-      uint8_t *dst = img + (m ? IMG_TG : IMG_TB);
+      uint8_t *dst = sm + TIMG + 16384 * m;
 #pragma unroll
       for (int c0 = 0; c0 < 32; c0 += 16) {
         float v[16];
         if (rla || (m && stl)) {
 #pragma unroll
           for (int u = 0; u < 16; ++u) v[u] = r == 32 * hf + c0 + u ? 1.f : 0.f;
+        } else if (hf == 1 && r < 32) {
+#pragma unroll
+          for (int u = 0; u < 16; ++u) v[u] = 0.f;
         } else {
           lds16(Tm + r * LDT + 32 * hf + c0, v);
         }
-        img_row16(dst, 8192, r, 32 * hf + c0, v);
+        img_row16(dst, dst + 8192, r, 32 * hf + c0, v);
       }
+      fence_async_smem();
     }
     if (tid < C) {
       float *rec = p.ws + chunk * kRecFloats;
@@ -374,12 +395,19 @@ __global__ void __launch_bounds__(NTH, 2) prep_tc_kernel(FwdParams p, bool rla) 
       rec[OFF_VEC + V_WR + t] = stl ? (t == n_ - 1 ? 1.f : 0.f) : gam[t] * __expf(cC - cum[t]);
       if (t == 0) rec[OFF_VEC + V_GAMC] = __expf(cC);
     }
+    __syncthreads();  // T's images
+    if (tid == 0) {
+      bulk_s2g(img + IMG_TB, sm + TIMG, 16384);
+      bulk_s2g(img + IMG_TG, sm + TIMG + 16384, 16384);
+      bulk_commit();
+    }
   }
   if (!ok && tid == 0) {
     if (p.err) atomicExch(p.err, RDN_ERR_TIMEOUT);
     mma_commit(barD);  // the Gram product still in flight, before TMEM is freed
     mbar_wait(barD, 0);
   }
+  if (tid == 0) bulk_wait_all();
   cp_async_wait_all();  // no copy of this CTA outlives it (a fetch for a chunk not reached)
   fence_before_sync();
   __syncthreads();
