@@ -21,7 +21,7 @@ import math
 import torch
 
 from . import _abi
-from ._abi import BwdArgs, DecodeArgs, FwdArgs
+from ._abi import BwdArgs, FwdArgs
 # variant flags (variant_flags= of the forward and backward calls): residual
 # against a_t S_{t-1} k_t; ungated combine S_{t-1} q + R_t q; c tanh(x / c)
 # residual; stateless correction R_t = r_t k_t^T
@@ -59,7 +59,7 @@ def _ptr(t):
         raise ValueError("rdn: tensors must be on a CUDA device")
     if not t.is_contiguous():
         raise ValueError("rdn: tensors must be contiguous")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _dtype_code(t):
@@ -70,14 +70,25 @@ def _dtype_code(t):
     raise ValueError(f"rdn: unsupported dtype {t.dtype}")
 
 
+def _addr(t):
+    """_ptr as a number: 0 = NULL."""
+    return _ptr(t) or 0
+
+
 def _stream(t):
-    return ctypes.c_void_p(torch.cuda.current_stream(t.device).cuda_stream)
+    # the current stream's handle without the Python stream object around it
+    return torch._C._cuda_getCurrentRawStream(t.device.index)
 
 
 def _alloc_ws(nbytes, device):
     if nbytes == 0:
         return None
     return torch.empty(nbytes, dtype=torch.uint8, device=device)
+
+
+def _f32(x):
+    """x as the nearest C float (out of range: infinite), as a Python float."""
+    return ctypes.c_float(x).value
 
 
 def _check_variant_flags(f):
@@ -309,23 +320,21 @@ def rdn_decode_step(q, k, v, g, beta, gamma, S, R, clip=1.0, scale=1.0, variant=
     """One recurrent step for N sequences; S, R [N,H,Dk,Dv] fp32 are updated
     in place.  q, k [N,H,Dk]; v [N,H,Dv]; gates [N,H].  Returns o [N,H,Dv].
     tied_gamma / variant_flags / qk_norm, qk_eps: as for the forward."""
-    lib = _abi.load()
-    _check_variant_flags(variant_flags)
+    if variant_flags:
+        _check_variant_flags(variant_flags)
     N, H, Dk = q.shape
     Dv = v.shape[-1]
     o = out if out is not None else torch.empty(N, H, Dv, dtype=q.dtype, device=q.device)
-    a = DecodeArgs()
-    a.N, a.H, a.Dk, a.Dv = N, H, Dk, Dv
-    a.dtype = _dtype_code(q)
-    a.variant = 1 if variant == "rdn" else 0
-    a.q, a.k, a.v = _ptr(q), _ptr(k), _ptr(v)
-    a.g, a.beta, a.gamma = _ptr(g), _ptr(beta), _ptr(gamma)
-    a.clip, a.scale = float(clip), float(scale)
-    a.S, a.R, a.o = _ptr(S), _ptr(R), _ptr(o)
-    a.flags = (_abi.RDN_FLAG_TIED_GAMMA if tied_gamma else 0) | variant_flags \
+    flags = (_abi.RDN_FLAG_TIED_GAMMA if tied_gamma else 0) | variant_flags \
         | (_abi.RDN_FLAG_QK_NORM if qk_norm else 0)
-    a.qk_eps = float(qk_eps)
-    _check("rdn_decode_step", lib.rdn_decode_step(ctypes.byref(a), _stream(q)))
+    # one token is a few microseconds of device time: the argument struct is
+    # packed in one call instead of field by field (17.7 -> 9.7 us a step at
+    # N = 1, H = 16, D = 128, back to back)
+    args = _abi.DECODE_PACK(N, H, Dk, Dv, _dtype_code(q), 1 if variant == "rdn" else 0,
+                            _addr(q), _addr(k), _addr(v), _addr(g), _addr(beta), _addr(gamma),
+                            _f32(clip), _f32(scale), _addr(S), _addr(R), _addr(o), flags,
+                            _f32(qk_eps))
+    _check("rdn_decode_step", _abi.decode_step()(args, _stream(q)))
     return o
 
 

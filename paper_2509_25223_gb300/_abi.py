@@ -3,6 +3,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 
 from . import build as _build
 
@@ -61,6 +62,12 @@ class DecodeArgs(ctypes.Structure):
                 ("qk_eps", ctypes.c_float)]
 
 
+# rdn_decode_args as bytes, every field in one call (pointers as addresses, 0 = NULL)
+_DECODE_LAYOUT = struct.Struct("@6i6P2f3PIf")
+DECODE_PACK = _DECODE_LAYOUT.pack
+assert _DECODE_LAYOUT.size == ctypes.sizeof(DecodeArgs)
+
+
 class PrologueArgs(ctypes.Structure):
     _fields_ = [("rows", ctypes.c_longlong), ("D", ctypes.c_int), ("dtype", ctypes.c_int),
                 ("eps", ctypes.c_float), ("x", P * 2), ("y", P * 2), ("dy", P * 2),
@@ -68,6 +75,18 @@ class PrologueArgs(ctypes.Structure):
 
 
 _lib = None
+_decode_step = None
+
+
+def decode_step():
+    """rdn_decode_step taking its arguments as packed bytes (DECODE_PACK)."""
+    global _decode_step
+    if _decode_step is None:
+        fn = load()["rdn_decode_step"]  # (a function object of its own)
+        fn.argtypes = [ctypes.c_char_p, P]
+        fn.restype = ctypes.c_int
+        _decode_step = fn
+    return _decode_step
 
 
 def lib_path() -> str:
