@@ -86,7 +86,7 @@ __device__ __forceinline__ void st_row(InT *p, const float (&v)[N]) {
 // Ap^T dVr and dR's update | dX | dS's update.  A transposed triangular
 // product starts at its warp's first row.  Bound by the FMA pipe and the
 // phases' latencies: B = 4, H = 16, T = 2048,
-// d = 64 in 0.50 ms, B = 2, H = 8, T = 1000, d = 128 fp32 in 0.32 ms.
+// d = 64 in 0.42 ms, B = 2, H = 8, T = 1000, d = 128 fp32 in 0.19 ms.
 template <int DK, int DVS, int NT>
 struct ChainSm {  // float offsets
   static constexpr int LDK = DK + 4;
@@ -110,7 +110,9 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 2 : 1) bwd_chain_kernel(BwdPar
   float *mat[3] = {sm + SM::MAT, sm + SM::MAT + C * C, sm + SM::MAT + 2 * C * C};
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int ln = lane % LN, r0 = LM * warp + lane / LN, n0 = TN * ln;
+  int lm, ln;
+  lane_mn<LN>(lane, lm, ln);
+  const int r0 = LM * warp + lm, n0 = TN * ln;
   const int kw = 2 * LM * warp;  // the warp's first row
   const int H = p.f.H, sq = seq_at(p.f, blockIdx.x / H), h = blockIdx.x % H;
   const SeqSpan sp = seq_span(p.f, sq, h);
@@ -345,7 +347,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 2 : 1) bwd_chain_kernel(BwdPar
 // ---------------------------------------------------------------- kernel 2
 // One CTA of 256 threads per chunk.  Thread (ty, tx) owns rows 4 ty .. 4 ty + 3
 // and columns tx + 16 j of every product, so a row's sums are shuffles among
-// the 16 lanes of a half warp.  Every value-dimension product is A B^T with
+// 16 lanes of a warp.  Every value-dimension product is A B^T with
 // both operands' rows contiguous (mm_nt); the value dimension is walked in
 // slices of JS columns, the next slice's tiles arriving by cp.async while the
 // current one is used: first the auxiliary pass (dO, E2, dX2 against R0, dR and
@@ -354,10 +356,10 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 2 : 1) bwd_chain_kernel(BwdPar
 // sum_j dKS KS is its k's product with the row of dKS S0^T, which dK takes
 // anyway.  kk, qk and the C x C gradients stay in shared memory at the
 // positions their thread owns.  Bound by the FMA pipe (two FMAs an
-// instruction): the same calls in 0.60 and 0.28 ms.  One kernel that walked
+// instruction): the same calls in 0.57 and 0.27 ms.  One kernel that walked
 // the chunks with every product, adding its column slices' shares atomically,
 // and a finishing pass took 6.19 and 1.85 ms for what the chain and this do in
-// 1.10 and 0.60.
+// 0.99 and 0.46.
 constexpr int kPostThreads = 256;
 template <int DK>
 struct PostSm {  // float offsets
@@ -390,7 +392,8 @@ __global__ void __launch_bounds__(kPostThreads, 1) bwd_post_kernel(BwdParams p) 
   rec_decode(p.f, chunk, sq, h, c);
   const SeqSpan sp = seq_span(p.f, sq, h);
   const int n = min(C, sp.len - c * C);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, tx = tid & 15, ty = tid >> 4;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tx = lane >> 1, ty = 2 * warp + (lane & 1);
   const bool dec_res = p.f.mods & RDN_FLAG_DECAYED_RESIDUAL;
   const bool plain = p.f.mods & RDN_FLAG_PLAIN_COMBINE;
   const bool stl = p.f.mods & RDN_FLAG_STATELESS_AUX;
@@ -666,12 +669,12 @@ __global__ void __launch_bounds__(kPostThreads, 1) bwd_post_kernel(BwdParams p) 
       }
     }
   }
-  // ---- row sums over the 16 lanes, column sums over the block
+  // ---- row sums over a row's 16 lanes, column sums over the block
   float *colp = sm + SM::ST;  // [8 warps][3][C], then the warps' dgc
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
 #pragma unroll
-    for (int o = 8; o; o >>= 1) {
+    for (int o = 16; o > 1; o >>= 1) {
       pc[i] += __shfl_xor_sync(0xffffffffu, pc[i], o);
       pp[i] += __shfl_xor_sync(0xffffffffu, pp[i], o);
       po[i] += __shfl_xor_sync(0xffffffffu, po[i], o);
@@ -689,10 +692,10 @@ __global__ void __launch_bounds__(kPostThreads, 1) bwd_post_kernel(BwdParams p) 
   }
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    cg[j] += __shfl_xor_sync(0xffffffffu, cg[j], 16);
-    cb[j] += __shfl_xor_sync(0xffffffffu, cb[j], 16);
-    cm[j] += __shfl_xor_sync(0xffffffffu, cm[j], 16);
-    if (lane < 16) {
+    cg[j] += __shfl_xor_sync(0xffffffffu, cg[j], 1);
+    cb[j] += __shfl_xor_sync(0xffffffffu, cb[j], 1);
+    cm[j] += __shfl_xor_sync(0xffffffffu, cm[j], 1);
+    if ((lane & 1) == 0) {
       colp[(warp * 3 + 0) * C + tx + 16 * j] = cg[j];
       colp[(warp * 3 + 1) * C + tx + 16 * j] = cb[j];
       colp[(warp * 3 + 2) * C + tx + 16 * j] = cm[j];

@@ -43,7 +43,7 @@ namespace {
 // from its accumulators to the decayed matrices without a pass through shared
 // memory, and only A_beta, A_gamma stay there for the inverses; T_beta,
 // T_gamma take the place of K and Q.  Bound by shared-memory loads and the
-// inverses' chain: 2048 chunks of d = 64 in 0.129 ms (0.402 ms with scalar
+// inverses' chain: 2048 chunks of d = 64 in 0.124 ms (0.402 ms with scalar
 // operand loads, every matrix in shared memory and one CTA per SM).
 template <int DK>
 struct PrepSm {  // float offsets
@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(kThreads, 2) chunk_prep_kernel(FwdParams p) {
   const SeqSpan sp = seq_span(p, sq, h);
   const int t0 = c * C;
   const int n = min(C, sp.len - t0);
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int tid = threadIdx.x, tx = (tid & 31) >> 1, ty = 2 * (tid >> 5) + (tid & 1);
 
   {
     simt::RowTile<InT, DK, kThreads> kt, qt;
@@ -181,9 +181,9 @@ __global__ void __launch_bounds__(kThreads, 2) chunk_prep_kernel(FwdParams p) {
 // matrices arrive by cp.async a phase or more ahead, in three slots; the next
 // chunk's K, Q, V and gate vectors wait in registers over the last phase.
 // Bound by the FMA pipe and the phases' latencies: B = 4, H = 16, T = 2048,
-// d = 64 in 0.458 ms (1.079 ms with scalar operand loads), B = 2, H = 8,
-// T = 1000, d = 128 fp32 in 0.293 ms (0.718), B = 1, H = 2, T = 256, d = 64 in
-// 0.024 ms (0.085, on 4 CTAs).
+// d = 64 in 0.396 ms (1.079 ms with scalar operand loads), B = 2, H = 8,
+// T = 1000, d = 128 fp32 in 0.181 ms (0.718), B = 1, H = 2, T = 256, d = 64 in
+// 0.023 ms (0.085, on 4 CTAs).
 // REC: one chunk per CTA from the chunk-start states p.S_chunks, p.R_chunks,
 // writing only what the backward reads (E, E2 and the residual's mask).
 template <int DK, int DVS, int NT>
@@ -209,7 +209,9 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 2 : 1) chunk_scan_kernel(FwdPa
   float *mat[3] = {sm + SM::MAT, sm + SM::MAT + C * LDM, sm + SM::MAT + 2 * C * LDM};
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int ln = lane % LN, r0 = LM * warp + lane / LN, n0 = TN * ln;
+  int lm, ln;
+  lane_mn<LN>(lane, lm, ln);
+  const int r0 = LM * warp + lm, n0 = TN * ln;
   int sq, h, c0 = 0, c1;
   if (REC) {
     if ((long long)blockIdx.x >= total_records(p)) return;
@@ -375,7 +377,8 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 2 : 1) chunk_scan_kernel(FwdPa
           } else {  // the row's DVS bits: one byte per 8 columns
             in <<= n0 & 7;
 #pragma unroll
-            for (int d = 1; d < 8 / TN; d <<= 1) in |= __shfl_xor_sync(0xffffffffu, in, d);
+            for (int b = 0; 1 << b < 8 / TN; ++b)  // (bit b of ln is lane bit 2 b)
+              in |= __shfl_xor_sync(0xffffffffu, in, 1 << 2 * b);
             if (n0 % 8 == 0)
               ((uint8_t *)p.sv_mask)[((rec * C + t) * DV + j0 + n0) >> 3] = (uint8_t)in;
           }

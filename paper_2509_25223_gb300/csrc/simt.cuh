@@ -7,12 +7,32 @@
 // pipe sets the pace.  Row strides are odd multiples of 4 floats: rows that
 // differ by one then start 4 banks apart and the 16-byte loads of 8 lanes fall
 // on all 32 banks.
+//
+// A 16-byte shared load takes 2.25 cycles of the SM where lanes differing in
+// lane bit 0, or those differing in bit 1, read the same address, and 4.04
+// otherwise, however few addresses there are (measured; 8-byte ones 1.42 and
+// 2.07).  So the lanes of a tile are laid out over its rows and columns with
+// bit 0 in the one and bit 1 in the other (lane_mn, or a column per lane pair),
+// which keeps both operands' loads at the lower cost.
 #pragma once
 #include "chunk_common.cuh"
 
 namespace rdn {
 namespace simt {
 
+// Row lm and column ln of a lane in a warp's 32 / LN x LN lanes (LN 4 or 8):
+// columns on lane bits 0, 2 (, 4), rows on the others.
+template <int LN>
+__device__ __forceinline__ void lane_mn(int lane, int &lm, int &ln) {
+  static_assert(LN == 4 || LN == 8, "lanes across");
+  ln = (lane & 1) | ((lane >> 1) & 2);
+  if (LN == 8) {
+    ln |= (lane >> 2) & 4;
+    lm = ((lane >> 1) & 1) | ((lane >> 2) & 2);
+  } else {
+    lm = ((lane >> 1) & 1) | ((lane >> 2) & 6);
+  }
+}
 // v = p[0 .. N), N in {1, 2, 4}, p aligned to N floats
 template <int N>
 __device__ __forceinline__ void ldv(const float *p, float (&v)[N]) {
@@ -272,9 +292,29 @@ cudaError_t simt_dispatch(int DK, bool rdnv, bool bf16, const F &fn) {
 }
 // Value columns per CTA of the sequential kernels (forward scan, backward
 // chain): fewer columns make a chunk shorter but repeat the reads of K, Q and
-// the chunk matrices, so the widest slice that still gives every SM a CTA.
+// the chunk matrices, and more CTAs may need another wave.  A chunk's cost in us
+// by the forward's measurements: d = 128 (one CTA per SM) 16.7, 11.2 and 9.2 for
+// 32, 16 and 8 columns; d = 64 with two CTAs on every SM 12.5 and 9.0 for 16 and
+// 8, with one 8.3 and 6.1.
 inline int scan_columns(int DK, long long heads, int nsm) {
-  if (DK == 64) return heads * 4 > nsm ? 16 : 8;
-  return heads * 4 > nsm ? 32 : heads * 8 > nsm ? 16 : 8;
+  static const int cols[3] = {32, 16, 8}, cost128[3] = {167, 112, 92}, two64[3] = {0, 125, 90},
+                   one64[3] = {0, 83, 61};
+  int best = 0;
+  long long least = 0;
+  for (int i = DK == 64; i < 3; ++i) {
+    const long long ctas = heads * (DK / cols[i]);
+    long long t;
+    if (DK == 64) {
+      const long long rest = ctas % (2 * nsm);
+      t = ctas / (2 * nsm) * two64[i] + (rest > nsm ? two64[i] : rest ? one64[i] : 0);
+    } else {
+      t = (ctas + nsm - 1) / nsm * cost128[i];
+    }
+    if (!best || t < least) {
+      best = cols[i];
+      least = t;
+    }
+  }
+  return best;
 }
 }  // namespace rdn
