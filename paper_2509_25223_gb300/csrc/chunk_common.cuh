@@ -1,5 +1,6 @@
-// chunk_common.cuh -- layout of the per-chunk records shared by the
-// chunkwise forward and backward, and a block-level fp32 product helper.
+// chunk_common.cuh -- what the chunkwise forward and backward share: the layout
+// of the per-chunk records, their parameters, packed sequences, and the rules
+// that choose a kernel.
 #pragma once
 #include "common.cuh"
 
@@ -333,10 +334,10 @@ inline cudaError_t sm_count(int *n) {
   return e != cudaSuccess ? e : cudaDeviceGetAttribute(n, cudaDevAttrMultiProcessorCount, dev);
 }
 
-// Whether a sequential tensor-core kernel gives each (sequence, head) a pair of
-// CTAs (fwd_pair.cu, bwd_pair.cu) or one: whichever ends first.  A chunk costs
-// a pair about 0.6 of what it costs one CTA (forward 4.4 us against 8.8, saving
-// 6.1 against 8.8; backward 8.1 against 12.0; 32 heads, T = 16384 and 2000).
+// Whether the forward tensor-core scan gives each (sequence, head) a pair of
+// CTAs (fwd_pair.cu) or one: whichever ends first.  A chunk costs a pair about
+// 0.6 of what it costs one CTA (4.4 us against 7.5, saving for the backward 6.1
+// against 9.7; 32 heads, T = 16384 and 2000, against 128 heads).
 // Equal sequences run in waves of one CTA per SM:
 inline bool use_pairs(const FwdParams &p, int nsm) {
   const long long n = (long long)p.nseq * p.H;

@@ -172,12 +172,15 @@ __global__ void __launch_bounds__(kPairThreads, 1)
   auto by_tma = [&](int cc) { return maps.ok && cc > 0 && cc < NC - 1; };
   if (warp == kTcThreads / 32) {
     // =============================================== the issuing warp (lane 0)
-    const bool one = (tid & 31) == 0;
+    bool one = (tid & 31) == 0;
     bool skip_commit = p.inject == 1 && base;
     const uint32_t i64 = idesc_bf16(128, 64), i128 = idesc_bf16(128, 128);
-    // wait for a copy by the copying warp
+    // wait for a copy by the copying warp; when it gave up, nothing more is issued
+    // or completed (no barrier is armed again before its phase is complete)
     auto wait_copy = [&](uint64_t *b, uint32_t ph) {
-      if (!mbar_wait(b, ph)) *flag = 1;
+      if (mbar_wait(b, ph)) return true;
+      *flag = 1;
+      return one = false;
     };
     bool alive = true;
     for (int c = 0; c < NC; ++c) {
@@ -209,8 +212,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
       if (RDNV) {  // MMA2: E^T = X^T T_beta^T / MMA6: E2^T = X2^T T_gamma^T
         bar_sync(kBarX, kHandThreads);
         fence_after_sync();
-        if (one) {
-          wait_copy(barA, (uint32_t)c & 1u);
+        if (one && wait_copy(barA, (uint32_t)c & 1u)) {
           mma_split3(tm + (base ? d1 : T_D1), sbase + SM_XE, sbase + SM_XE_LO, sbase + SM_SLOTA,
                      sbase + SM_SLOTA + 8192, i64, false);
           mma_commit(bar);
@@ -229,19 +231,20 @@ __global__ void __launch_bounds__(kPairThreads, 1)
                       i128 | kBMajorMN, 1u);
         mma_commit(bar);
         mma_commit(barM4);
-        wait_copy(barB, (uint32_t)c & 1u);
-        if (base)
-          mma_split3(tm + d1, sbase + SM_XE, sbase + SM_XE_LO, sbase + SM_SLOTB,
-                     sbase + SM_SLOTB + 16384, i128, true);
-        else
-          mma_split3(tm + T_D1 + 64, sbase + SM_XE, sbase + SM_XE_LO, sbase + SM_SLOTB,
-                     sbase + SM_SLOTB + 8192, i64, true);
-        mma_commit(barN);
+        if (wait_copy(barB, (uint32_t)c & 1u)) {
+          if (base)
+            mma_split3(tm + d1, sbase + SM_XE, sbase + SM_XE_LO, sbase + SM_SLOTB,
+                       sbase + SM_SLOTB + 16384, i128, true);
+          else
+            mma_split3(tm + T_D1 + 64, sbase + SM_XE, sbase + SM_XE_LO, sbase + SM_SLOTB,
+                       sbase + SM_SLOTB + 8192, i64, true);
+          mma_commit(barN);
+        }
       }
       __syncwarp();
     }
     __syncthreads();
-    if ((!alive || *flag) && one) {  // a bounded wait gave up: drain the products, bounded
+    if ((!alive || *flag) && (tid & 31) == 0) {  // a wait gave up: drain the products, bounded
       if (p.err) atomicExch(p.err, RDN_ERR_TIMEOUT);
       mma_commit(barD);
       mbar_wait(barD, 0);

@@ -52,6 +52,11 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity,
   return true;
 }
 
+// One arrival on a barrier of this CTA, after this thread's earlier accesses.
+__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
 // Arm `bar` for `bytes` of asynchronous copies (counts as this thread's arrival).
 __device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
