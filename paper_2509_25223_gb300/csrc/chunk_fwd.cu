@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 2 : 1) chunk_scan_kernel(FwdPa
       float x[TN];
 #pragma unroll
       for (int j = 0; j < TN; ++j)  // RDN: X = V - Gam K S; RLA (E = V): wS E
-        x[j] = RDNV ? vv[i][j] - Gam[t] * a1[i][j] : wS[t] * vv[i][j];
+        x[j] = RDNV ? fmaf(-Gam[t], a1[i][j], vv[i][j]) : wS[t] * vv[i][j];
       stv<TN>((RDNV ? Xs : Ws) + t * DVS + n0, x);
     }
     const float *E = Vs;
@@ -363,10 +363,10 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 2 : 1) chunk_scan_kernel(FwdPa
 #pragma unroll
         for (int j = 0; j < TN; ++j) {
           // P_t = S_{t-1}^T k_t (decayed residual: a_t S_{t-1}^T k_t)
-          const float x = vv[i][j] - (gp * a1[i][j] + pm[i][j]);
+          const float x = vv[i][j] - fmaf(gp, a1[i][j], pm[i][j]);
           r[i][j] = resid_map(x, clip, tnh);  // Section 3.3
-          ob[i][j] = gq * a1[2 + i][j] + pm[2 + i][j];
-          x2[j] = r[i][j] - Gam[t] * a2[i][j];
+          ob[i][j] = fmaf(gq, a1[2 + i][j], pm[2 + i][j]);
+          x2[j] = fmaf(-Gam[t], a2[i][j], r[i][j]);
           in |= (fabsf(x) <= clip ? 1u : 0u) << j;
           if (tnh) dr[j] = resid_grad(x, clip, true);
         }
@@ -394,7 +394,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 2 : 1) chunk_scan_kernel(FwdPa
           float s[TN];
           ldv<TN>(Ss + (m0 + i) * DVS + n0, s);
 #pragma unroll
-          for (int j = 0; j < TN; ++j) s[j] = GamC * s[j] + u[i][j];
+          for (int j = 0; j < TN; ++j) s[j] = fmaf(GamC, s[j], u[i][j]);
           stv<TN>(Ss + (m0 + i) * DVS + n0, s);
         }
       }
@@ -449,7 +449,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 2 : 1) chunk_scan_kernel(FwdPa
           float y[TN];
 #pragma unroll
           for (int j = 0; j < TN; ++j)
-            y[j] = ob[i][j] + gm * (Gam[t] * a2[2 + i][j] + oa[i][j]);
+            y[j] = fmaf(gm, fmaf(Gam[t], a2[2 + i][j], oa[i][j]), ob[i][j]);
           if constexpr (sizeof(InT) == 4) {
             stv<TN>((float *)o + off, y);
           } else {
@@ -473,7 +473,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 2 : 1) chunk_scan_kernel(FwdPa
         float s[TN];
         ldv<TN>(Rs + (m0 + i) * DVS + n0, s);
 #pragma unroll
-        for (int j = 0; j < TN; ++j) s[j] = (stl ? 0.f : GamC) * s[j] + u[i][j];
+        for (int j = 0; j < TN; ++j) s[j] = fmaf(stl ? 0.f : GamC, s[j], u[i][j]);
         stv<TN>(Rs + (m0 + i) * DVS + n0, s);
       }
     }

@@ -28,7 +28,7 @@ def _step(x, variant, saved, flags):
 
 
 @pytest.mark.parametrize("variant", ["rdn", "rla"])
-@pytest.mark.parametrize("d,dtype", [(128, "fp32"), (64, "fp32"), (64, "bf16")])
+@pytest.mark.parametrize("d,dtype", [(128, "f32"), (64, "f32"), (64, "bf16")])
 @pytest.mark.parametrize("T,saved,flags", [
     (1, True, 0), (65, False, 0), (200, True, 0),
     (130, False, rdn.TANH_RESIDUAL), (130, True, rdn.STATELESS_AUX),
