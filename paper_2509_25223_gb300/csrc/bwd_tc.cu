@@ -2,33 +2,22 @@
 // forward, bf16 inputs, d_k = d_v = 128; RLA (TcBwdParams::rla) and two of
 // the variant flags are runtime modes of separate kernel instances.
 //
-// Reverse mode of the chunk algebra of chunk_fwd.cu (the same steps as
-// chunk_bwd.cu, whose header lists them), split by what depends on the
-// gradients carried between chunks:
+// Reverse mode of the chunk algebra of chunk_fwd.cu, split by what depends on
+// the gradients carried between chunks:
 //
 //  1. bwd_recompute (parallel, one CTA per chunk): from the chunk-start
 //     states rebuild E, E2 and the clip mask (the forward's pieces for one
 //     chunk).  It does not run when the forward saved them.
-//  2. bwd_chain (sequential over chunks, one CTA per (b,h)): the carried
-//     gradients.  With dR, dS the gradients w.r.t. a chunk's end states,
-//        dE2 = M2^T dOa + diag(wR) K dR        dX2 = T_gamma^T dE2
-//        dP  = -mask * dX2                     dKR = -diag(Gam) dX2
-//        dR_prev = Gam_C dR + K^T dKR + Q^T diag(Gam gamma) dO
-//        dE  = Mq^T dO + Ap^T dP + diag(wS) K dS     dX = T_beta^T dE
-//        dKS = diag(Gprev) dP - diag(Gam) dX
-//        dS_prev = Gam_C dS + K^T dKS + Q^T diag(Gam) dO
-//        dv  = -dP + dX
-//     No forward quantity other than the clip mask enters this chain.
+//  2. bwd_chain (sequential over chunks, one CTA per (b,h); bwd_chain.cu): the
+//     gradients carried between chunks, dX2, dX and dv.  No forward quantity
+//     other than the clip mask enters this chain.
 //  3. bwd_post (parallel, one CTA per chunk): every product that reduces over
 //     the value dimension -- the state terms of dK, dQ, the five C x C
 //     gradients, the per-row gate terms -- and then the gradients of the chunk
-//     matrices' entries turned into dq, dk, dg, dbeta, dgamma (the work that
-//     bwd_finish of chunk_bwd.cu does on the SIMT path).
+//     matrices' entries turned into dq, dk, dg, dbeta, dgamma.
 //
 // Orientation: value column j = TMEM lane j, owned by thread j of a group of
-// 128 threads (bwd_chain: 4 groups, group g taking the token and key columns
-// [16g, 16g + 16) and [64 + 16g, 80 + 16g); bwd_post: 2 groups), for every
-// column quantity (X, E, dO, dX2, ...), which is kept as a bf16 hi + lo tile
+// 128 threads, for every column quantity (X, E, dO, dX2, ...), which is kept as a bf16 hi + lo tile
 // [j][t] (K-major for products over t).  Products over j use the same tiles
 // as MN-major operands.  The chunk matrices come from chunk_prep's images
 // (bf16 hi + lo); products with them are three MMAs (hi*hi + hi*lo + lo*hi).
@@ -239,503 +228,10 @@ __global__ void __launch_bounds__(NT, 1) bwd_recompute_kernel(TcBwdParams P) {
   if (warp == 0) tmem_dealloc(tm, 512);
 }
 
-// ======================================================================== 2
-// bwd_chain: the gradients carried between chunks, chunks in reverse.
-namespace ch {
-// K, Q | carried gradients dS, dR as bf16 hi + lo A operands (phase A) | slots
-// | dO.  After phase A the 128 KB of gradient tiles serve as scratch for the
-// split column tiles; the gradient tiles are rewritten at the chunk end.
-constexpr uint32_t KQ = 0;
-constexpr uint32_t DSH = 32768, DRH = 65536, DSL = 98304, DRL = 131072;
-constexpr uint32_t SLOTA = 163840;   // diag(gamma) M2 -> T_gamma -> T_beta (16 KB)
-constexpr uint32_t SLOTB = 180224;   // Mq -> Ap (hi 8 KB | lo 8 KB)
-constexpr uint32_t DOT = 196608;     // dO, exact bf16, rows t (two 8 KB column blocks)
-// scratch column tiles (hi, lo) inside the gradient-tile region
-constexpr uint32_t S0H = 32768, S0L = 49152, S1H = 65536, S1L = 81920;
-constexpr uint32_t S2H = 98304, S2L = 114688, S3H = 131072, S3L = 147456;
-constexpr uint32_t VEC = 212992;                 // Gam Gprev wS wR gamma (5 x 64)
-constexpr uint32_t CTL = VEC + 5 * 64 * 4;
-constexpr uint32_t SLOT = CTL + 48;
-constexpr size_t SMEM = SLOT + 16;
-static_assert(SMEM <= 232448, "shared memory");
-constexpr uint32_t T_DS = 0, T_DR = 128, T_R1 = 256, T_R2 = 320, T_R3 = 384, T_R4 = 448;
-}  // namespace ch
-
-// kGeneric: the RLA mode and the variant flags (TcBwdParams::rla, FwdParams::mods)
-// are read; the RDN method's instance has them folded away
-template <bool kGeneric>
-__global__ void __launch_bounds__(NTC, 1) bwd_chain_kernel(const __grid_constant__ TcBwdParams P) {
-  using namespace ch;
-  extern __shared__ __align__(1024) uint8_t sm[];
-  const uint32_t sb = smem_u32(sm);
-  const FwdParams &p = P.f;
-  const bool rla = kGeneric && P.rla;
-  const unsigned mods = kGeneric ? p.mods : 0u;
-  if (!picked(p)) return;
-  if (sb & 1023u) {
-    if (threadIdx.x == 0 && p.err) atomicExch(p.err, RDN_ERR_CUDA);
-    return;
-  }
-  float *vec = reinterpret_cast<float *>(sm + VEC);
-  float *Gam = vec, *Gprev = vec + 64, *wS = vec + 128, *wR = vec + 192, *gamv = vec + 256;
-  uint32_t *slot = reinterpret_cast<uint32_t *>(sm + SLOT);
-  const int tid = threadIdx.x, warp = tid >> 5, j = tid & 127;
-  const int g16 = (warp >> 2) * 16;  // this thread's token (and key) columns start
-  const int H = p.H, sq = seq_at(p, blockIdx.x / H), h = blockIdx.x % H;
-  const SeqSpan sp = seq_span(p, sq, h);  // this (sequence, head)'s tokens and records
-  const long long tok0 = sp.tok0;
-  const int NC = sp.nc, T = sp.len;
-  const __nv_bfloat16 *q = (const __nv_bfloat16 *)p.q, *k = (const __nv_bfloat16 *)p.k,
-                      *dOp = (const __nv_bfloat16 *)P.dO;
-  __nv_bfloat16 *dv = (__nv_bfloat16 *)P.dv;
-  const size_t st_base = ((size_t)sq * H + h) * D * D;
-
-  Ctl K;
-  ctl_init(K, sm + CTL, tid);
-  if (p.inject == 2) {  // (a test: the first phase's signal is skipped, the wait gives up)
-    K.limit = 10000000ll;
-    K.skip = true;
-  }
-  if (warp == 0) tmem_alloc(slot, 512);
-  // slot loads: A holds diag(gamma) M2, then T_gamma, then T_beta; B holds
-  // Mq (hi | lo), then Ap (hi | lo) -- each 8 KB half copied from the
-  // [Ap ; Mq] image
-  auto load_mq = [&](size_t ck) {
-    const uint8_t *r = rec_bytes(p, ck);
-    ctl_arm<1>(K, 16384);
-    bulk_g2s(sm + SLOTB, r + IMG_APMQ + 8192, 8192, K.barB);
-    bulk_g2s(sm + SLOTB + 8192, r + IMG_APMQ + 16384 + 8192, 8192, K.barB);
-  };
-  auto load_ap = [&](size_t ck) {
-    const uint8_t *r = rec_bytes(p, ck);
-    ctl_arm<1>(K, 16384);
-    bulk_g2s(sm + SLOTB, r + IMG_APMQ, 8192, K.barB);
-    bulk_g2s(sm + SLOTB + 8192, r + IMG_APMQ + 16384, 8192, K.barB);
-  };
-  if (tid == 0 && NC > 0) {  // (a packed sequence may be empty)
-    const size_t last = (size_t)(sp.rbase + NC - 1);
-    load_slot<0>(K, sm + SLOTA, rec_bytes(p, last) + IMG_M2, 16384);
-    load_mq(last);
-  }
-  fence_before_sync();
-  __syncthreads();
-  fence_after_sync();
-  const uint32_t tm = *slot;
-  const uint32_t lane = (uint32_t)((warp & 3) * 32) << 16;
-  // a carried gradient's bf16 hi + lo tiles (rows j), 16 of its key rows
-  auto put_grad16 = [&](uint32_t hi, uint32_t lo, int c0, const float (&g)[16]) {
-    put16s(sm + hi + (c0 >> 6) * 16384, sm + lo + (c0 >> 6) * 16384, j, c0, g);
-  };
-  // both carried gradients' tiles from their fp32 TMEM copies
-  auto write_grad_tiles = [&]() {
-#pragma unroll 1
-    for (int c0 = g16; c0 < D; c0 += 64) {
-      float s[16], r[16];
-      tmem_ld16x2(tm + lane + T_DS + c0, s, tm + lane + T_DR + c0, r);
-      put_grad16(DSH, DSL, c0, s);
-      put_grad16(DRH, DRL, c0, r);
-    }
-    fence_async_smem();  // the tiles are read by the MMAs and by a bulk copy
-  };
-  // a carried gradient's TMEM copy times the chunk's total decay, in place
-  // (this chunk's products accumulate onto it); this thread's columns
-  auto scale_grad = [&](uint32_t col, float f) {
-    float x[16], y[16];
-    tmem_ld16x2(tm + lane + col + g16, x, tm + lane + col + g16 + 64, y);
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      x[i] *= f;
-      y[i] *= f;
-    }
-    tmem_st16(tm + lane + col + g16, x);
-    tmem_st16(tm + lane + col + g16 + 64, y);
-  };
-  for (int c0 = g16; c0 < D; c0 += 64) {  // upstream gradients of the final states
-    float s[16], r[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      s[i] = P.dST ? P.dST[st_base + (size_t)(c0 + i) * D + j] : 0.f;
-      r[i] = P.dRT ? P.dRT[st_base + (size_t)(c0 + i) * D + j] : 0.f;
-    }
-    tmem_st16(tm + lane + T_DS + c0, s);
-    tmem_st16(tm + lane + T_DR + c0, r);
-  }
-  write_grad_tiles();
-
-  // a chunk's K, Q, dO tiles (rows t, exact bf16, zero past the end), asynchronous
-  auto fetch_kq = [&](int c) {
-    const int t0 = c * 64, n = min(64, T - t0);
-    for (int e = tid; e < 64 * 16; e += NTC) {
-      const int t = e >> 4, chn = e & 15;
-      const bool vld = t < n;
-      const size_t off = ((size_t)(tok0 + t0 + (vld ? t : 0)) * H + h) * D + chn * 8;
-      const int blk = chn >> 3, cc = (chn & 7) * 8;
-      cp_async16(sm + KQ + blk * 16384 + sw128(t, cc), k + off, vld);
-      cp_async16(sm + KQ + blk * 16384 + sw128(64 + t, cc), q + off, vld);
-    }
-  };
-  auto fetch_do = [&](int c) {
-    const int t0 = c * 64, n = min(64, T - t0);
-    for (int e = tid; e < 64 * 16; e += NTC) {
-      const int t = e >> 4, chn = e & 15;
-      const bool vld = t < n;
-      const size_t off = ((size_t)(tok0 + t0 + (vld ? t : 0)) * H + h) * D + chn * 8;
-      cp_async16(sm + DOT + (chn >> 3) * 8192 + sw128(t, (chn & 7) * 8), dOp + off, vld);
-    }
-  };
-  // a chunk's gate vectors (threads 0..63, one token each) and this thread's
-  // 16 bits of the clip-mask word, into registers
-  struct Pre {
-    float gam_, gprev, ws_, wr_, g_, gamc;
-    unsigned m;
-    uint4 d0, d1;  // the tanh residual's derivative at this thread's 16 tokens (grad_q16)
-  };
-  const bool tnh = kGeneric && (mods & RDN_FLAG_TANH_RESIDUAL);
-  // the stateless correction: the chunk-end R is not carried into the next
-  // chunk nor read out there, so the gradient carried back to it is zero
-  // (dR_prev = 0; a chunk's own dR is the upstream dRT for the last chunk)
-  const bool stl = kGeneric && (mods & RDN_FLAG_STATELESS_AUX);
-  auto fetch_pre = [&](int c) {
-    const size_t ck = (size_t)(sp.rbase + c);
-    const int t0 = c * 64, n = min(64, T - t0);
-    const float *rf = p.ws + ck * kRecFloats;
-    Pre x;
-    x.gam_ = x.gprev = x.ws_ = x.wr_ = x.g_ = 0.f;
-    if (tid < 64) {
-      const int t = tid;
-      x.gam_ = rf[OFF_VEC + V_GAM + t];
-      x.gprev = rf[OFF_VEC + V_GPREV + t];
-      x.ws_ = rf[OFF_VEC + V_WS + t];
-      x.wr_ = rf[OFF_VEC + V_WR + t];
-      x.g_ = t < n ? p.gamma[(size_t)(tok0 + t0 + t) * H + h] : 0.f;
-    }
-    x.gamc = rf[OFF_VEC + V_GAMC];
-    // bits [g16, g16 + 16) of the column's 64-bit word (little-endian)
-    if (!tnh) {
-      x.m = reinterpret_cast<const uint16_t *>(P.mask + ck * D + j)[g16 >> 4];
-    } else {
-      const uint4 *dp_ = reinterpret_cast<const uint4 *>(
-          reinterpret_cast<const uint16_t *>(P.mask) + (ck * D + j) * 64 + g16);
-      x.d0 = dp_[0];
-      x.d1 = dp_[1];
-    }
-    return x;
-  };
-  Pre pre{};
-  if (NC > 0) {
-    fetch_kq(NC - 1);
-    fetch_do(NC - 1);
-    pre = fetch_pre(NC - 1);
-  }
-  // Chunks before the last are whole 64-token chunks: with tensor maps, thread 0
-  // brings their dO (after phase D) and K, Q (after phase E) tiles by tiled bulk
-  // copies, all on one phase of barrier C; the last chunk, which may be ragged,
-  // is fetched above by cp.async with zero fill.
-  const bool tma = P.tma;
-  uint32_t tma_ph = 0;    // phases of barrier C waited for
-  uint32_t tma_arms = 0;  // (thread 0) phases armed, and of those seen complete
-  uint32_t tma_seen = 0;
-  auto tma_do = [&](int cc) {  // (thread 0) arms barrier C for the whole chunk
-    const int row = (int)(tok0 + (long long)cc * 64);
-    ++tma_arms;
-    mbar_expect_tx(K.barC, 49152);
-    for (int kb = 0; kb < 2; ++kb) tma_load_3d(sm + DOT + kb * 8192, P.map_do, 64 * kb, h, row, K.barC);
-  };
-  auto tma_kq = [&](int cc) {
-    const int row = (int)(tok0 + (long long)cc * 64);
-    for (int kb = 0; kb < 2; ++kb) {
-      tma_load_3d(sm + KQ + kb * 16384, P.map_k, 64 * kb, h, row, K.barC);
-      tma_load_3d(sm + KQ + kb * 16384 + 8192, P.map_q, 64 * kb, h, row, K.barC);
-    }
-  };
-
-  bool ok = true;
-  for (int c = NC - 1; c >= 0 && ok; --c) {
-    const size_t chunk = (size_t)(sp.rbase + c);
-    const int t0 = c * 64, n = min(64, T - t0);
-    __syncthreads();
-    if (tid == 0) {  // gradients w.r.t. this chunk's end states, for bwd_post: the tile
-      // images, as two groups: the hi tiles (rewritten after phase A), then the
-      // lo tiles (rewritten after phase B)
-      static_assert(DRH == DSH + 32768 && DSL == DRH + 32768 && DRL == DSL + 32768, "contiguous");
-      bulk_s2g(P.gimg + chunk * 131072, sm + DSH, 65536);
-      bulk_commit();
-      bulk_s2g(P.gimg + chunk * 131072 + 65536, sm + DSL, 65536);
-      bulk_commit();
-    }
-    if (tid < 64) {
-      Gam[tid] = pre.gam_;
-      Gprev[tid] = pre.gprev;
-      wS[tid] = pre.ws_;
-      wR[tid] = pre.wr_;
-      gamv[tid] = pre.g_;
-    }
-    const float GamC = pre.gamc;
-    const unsigned m = pre.m;  // bit i: clip inactive at t = g16 + i
-    const uint4 dd0 = pre.d0, dd1 = pre.d1;  // (tanh residual)
-    // this chunk's tiles: by cp.async (waited for here) only for the first, ragged
-    // chunk or without tensor maps -- a cp.async wait with none in flight still
-    // cost about 3.6k cycles a chunk (clock64 marks)
-    if (!tma || c == NC - 1) cp_async_wait_all();
-    if (tma && c < NC - 1) {  // (by tiled bulk copies)
-      if (mbar_wait(K.barC, tma_ph & 1u))
-        tma_seen = tma_ph + 1;
-      else
-        *K.flag = 1;
-      ++tma_ph;
-    }
-    __syncthreads();
-    if (*K.flag) {
-      ok = false;
-      break;
-    }
-    auto dO = [&](int t) {  // dO[t, j] from the tile
-      return __bfloat162float(*reinterpret_cast<const __nv_bfloat16 *>(
-          sm + DOT + (j >> 6) * 8192 + sw128(t, j & 63)));
-    };
-    // ---- phase A: K dR, K dS (gradients hi + lo), M2^T (gamma dO), Mq^T dO; meanwhile
-    // dR, dS (TMEM) times Gam_C, onto which the products of phases B .. E accumulate
-    // (the MMAs read their shared-memory tiles)
-    ok = phase_run_with(K, tid, [&] {
-      if (!slot_wait<0>(K, K.phA)) return false;
-      if (!slot_wait<1>(K, K.phB)) return false;
-      const uint32_t i64 = idesc_bf16(128, 64);
-      mma_tile(tm + T_R1, sb + DRH, 16384, sb + KQ, 16384, 8, i64, false);
-      mma_tile(tm + T_R1, sb + DRL, 16384, sb + KQ, 16384, 8, i64, true);
-      mma_tile(tm + T_R2, sb + DSH, 16384, sb + KQ, 16384, 8, i64, false);
-      mma_tile(tm + T_R2, sb + DSL, 16384, sb + KQ, 16384, 8, i64, true);
-      // dO enters as the MN-major A operand (rows t, value-column atoms 8 KB apart)
-      mma_tile_mnmn(tm + T_R3, sb + DOT, 8192, sb + SLOTA, 16384, 4, i64, false);
-      mma_tile_mnmn(tm + T_R3, sb + DOT, 8192, sb + SLOTA + 8192, 16384, 4, i64, true);
-      mma_tile_mnmn(tm + T_R4, sb + DOT, 8192, sb + SLOTB, 16384, 4, i64, false);
-      mma_tile_mnmn(tm + T_R4, sb + DOT, 8192, sb + SLOTB + 8192, 16384, 4, i64, true);
-      bulk_wait_read_all_but_last();  // the hi tiles become scratch after this phase
-      return true;
-    }, [&] {
-      scale_grad(T_DR, stl ? 0.f : GamC);
-      scale_grad(T_DS, GamC);
-    });
-    if (!ok) break;
-    if (tid == 0) {
-      load_slot<0>(K, sm + SLOTA, rec_bytes(p, chunk) + IMG_TG, 16384);
-      load_ap(chunk);
-    }
-    // dE2 = M2^T dOa + wR K dR ; dE (partial) = Mq^T dO + wS K dS ; dQR = Gam gamma dO
-    {
-      const int c0 = g16;
-      float x[16], y[16], w[16];
-      tmem_ld16x2(tm + lane + T_R1 + c0, x, tm + lane + T_R3 + c0, y);
-      lds16(wR + c0, w);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) y[i] += w[i] * x[i];
-      put16s(sm + S0H, sm + S0L, j, c0, y);
-      tmem_ld16x2(tm + lane + T_R2 + c0, x, tm + lane + T_R4 + c0, y);
-      lds16(wS + c0, w);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) y[i] += w[i] * x[i];
-      tmem_st16(tm + lane + T_R4 + c0, y);
-      lds16(Gam + c0, x);
-      lds16(gamv + c0, w);
-      const bool plain = mods & RDN_FLAG_PLAIN_COMBINE;  // (no gamma_t in the output)
-#pragma unroll
-      for (int i = 0; i < 16; ++i)  // dQR (Q unscaled)
-        x[i] = stl ? 0.f : p.scale * x[i] * (plain ? 1.f : w[i]) * dO(c0 + i);
-      put16s(sm + S1H, sm + S1L, j, c0, x);
-    }
-    // ---- phase B: dX2 = T_gamma^T dE2 ; U_R = Q^T dQR
-    ok = phase_run(K, tid, [&] {
-      if (!slot_wait<0>(K, K.phA)) return false;
-      mma_s3_kmn(tm + T_R3, sb + S0H, sb + S0L, sb + SLOTA, sb + SLOTA + 8192, 16384,
-                 idesc_bf16(128, 64), false);
-      const uint32_t i128 = idesc_bf16(128, 128);
-      mma_tile_kmn(tm + T_DR, sb + S1H, 0, sb + KQ + 8192, 16384, 4, i128, true);
-      mma_tile_kmn(tm + T_DR, sb + S1L, 0, sb + KQ + 8192, 16384, 4, i128, true);
-      bulk_wait_read();  // and the lo tiles after this one
-      return true;
-    });
-    if (!ok) break;
-    if (tid == 0) load_slot<0>(K, sm + SLOTA, rec_bytes(p, chunk) + IMG_TB, 16384);
-    float dP[16];  // t in [g16, g16 + 16)
-    {  // dX2 -> dP = -mask dX2, dKR = -Gam dX2; dX2 itself (fp32 [t][j]) for bwd_post,
-       // staged in the free scratch tiles and bulk-copied
-      float *stg = reinterpret_cast<float *>(sm + S0H);
-      {
-        const int c0 = g16;
-        float x[16], dkr[16], dp[16];
-        tmem_ld16(tm + lane + T_R3 + c0, x);
-        lds16(Gam + c0, dkr);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const int t = c0 + i;
-          stg[t * D + j] = x[i];
-          if (tnh) {  // the derivative of c tanh(x / c) instead of the mask
-            const uint32_t w = (i < 8 ? reinterpret_cast<const uint32_t *>(&dd0)
-                                      : reinterpret_cast<const uint32_t *>(&dd1))[(i & 7) >> 1];
-            dp[i] = -grad_uq16((i & 1) ? w >> 16 : w & 0xffffu) * x[i];
-          } else {
-            dp[i] = ((m >> i) & 1u) ? -x[i] : 0.f;
-          }
-          dP[i] = dp[i];
-          dkr[i] = (rla || stl) ? 0.f : -dkr[i] * x[i];
-        }
-        put16s(sm + S2H, sm + S2L, j, c0, dkr);
-        put16s(sm + S3H, sm + S3L, j, c0, dp);
-      }
-    }
-    // ---- phase C: U_R += K^T dKR ; Ap^T dP
-    ok = phase_run(K, tid, [&] {
-      static_assert(S0L == S0H + 16384, "contiguous");
-      bulk_s2g(P.dX2buf + chunk * 64 * D, sm + S0H, 32768);  // (published by this barrier)
-      bulk_commit();
-      if (!slot_wait<1>(K, K.phB)) return false;
-      const uint32_t i128 = idesc_bf16(128, 128);
-      mma_tile_kmn(tm + T_DR, sb + S2H, 0, sb + KQ, 16384, 4, i128, true);
-      mma_tile_kmn(tm + T_DR, sb + S2L, 0, sb + KQ, 16384, 4, i128, true);
-      mma_s3_kmn(tm + T_R3, sb + S3H, sb + S3L, sb + SLOTB, sb + SLOTB + 8192, 16384,
-                 idesc_bf16(128, 64), false);
-      bulk_wait_read();  // the staging is rewritten next
-      return true;
-    });
-    if (!ok) break;
-    if (tid == 0 && c > 0) load_mq(chunk - 1);
-    {  // dE = dE_partial + Ap^T dP; dQS = Gam dO (dR is complete in TMEM)
-      {
-        const int c0 = g16;
-        float a[16], e[16], dqs[16];
-        tmem_ld16x2(tm + lane + T_R4 + c0, a, tm + lane + T_R3 + c0, e);
-        // the base read-out Gam Q S0 (plain combine: Gprev Q S0)
-        lds16((mods & RDN_FLAG_PLAIN_COMBINE) ? Gprev + c0 : Gam + c0, dqs);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          a[i] += e[i];
-          dqs[i] = p.scale * dqs[i] * dO(c0 + i);
-        }
-        put16s(sm + S0H, sm + S0L, j, c0, a);
-        put16s(sm + S1H, sm + S1L, j, c0, dqs);
-      }
-    }
-    // ---- phase D: dX = T_beta^T dE ; U_S = Q^T dQS
-    ok = phase_run(K, tid, [&] {
-      if (!slot_wait<0>(K, K.phA)) return false;
-      mma_s3_kmn(tm + T_R3, sb + S0H, sb + S0L, sb + SLOTA, sb + SLOTA + 8192, 16384,
-                 idesc_bf16(128, 64), false);
-      const uint32_t i128 = idesc_bf16(128, 128);
-      mma_tile_kmn(tm + T_DS, sb + S1H, 0, sb + KQ + 8192, 16384, 4, i128, true);
-      mma_tile_kmn(tm + T_DS, sb + S1L, 0, sb + KQ + 8192, 16384, 4, i128, true);
-      return true;
-    });
-    if (!ok) break;
-    if (tid == 0 && c > 0) load_slot<0>(K, sm + SLOTA, rec_bytes(p, chunk - 1) + IMG_M2, 16384);
-    if (c > 0) {  // every thread is past its last read of this chunk's dO
-      if (!tma)
-        fetch_do(c - 1);
-      else if (tid == 0)
-        tma_do(c - 1);
-    }
-    {  // dX -> dv = -dP + dX ; dKS = Gprev dP - Gam dX; dX (fp32 [t][j]) and dv
-       // (bf16 [t][j]) staged in the free scratch tiles
-      float *stg = reinterpret_cast<float *>(sm + S0H);
-      __nv_bfloat16 *dvs = reinterpret_cast<__nv_bfloat16 *>(sm + S1H);
-      float *dvs32 = reinterpret_cast<float *>(sm + S1H);  // (fp32 dv: over S1H and S1L)
-      static_assert(S1L == S1H + 16384, "fp32 dv staging spans the pair");
-      {
-        const int c0 = g16;
-        float x[16], dks[16], gm[16];
-        tmem_ld16(tm + lane + T_R3 + c0, x);
-        // the prediction's state term: Gprev K S0 (decayed residual: Gam K S0)
-        lds16((mods & RDN_FLAG_DECAYED_RESIDUAL) ? Gam + c0 : Gprev + c0, dks);
-        lds16(Gam + c0, gm);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const int t = c0 + i;
-          stg[t * D + j] = x[i];
-          if (P.f32g)
-            dvs32[t * D + j] = x[i] - dP[i];
-          else
-            dvs[t * D + j] = __float2bfloat16_rn(x[i] - dP[i]);
-          dks[i] = dks[i] * dP[i] - (rla ? 0.f : gm[i] * x[i]);
-        }
-        put16s(sm + S2H, sm + S2L, j, c0, dks);
-      }
-      fence_async_smem();
-      __syncthreads();
-      if (tid == 0) {
-        bulk_s2g(P.dXbuf + chunk * 64 * D, sm + S0H, 32768);
-        bulk_commit();
-      }
-      if (P.f32g) {  // dv rows, 16 bytes at a time
-        float *dvf = (float *)P.dv;
-        for (int e = tid; e < 64 * 32; e += NTC) {
-          const int t = e >> 5, chn = e & 31;
-          if (t < n)
-            *reinterpret_cast<uint4 *>(dvf + ((size_t)(tok0 + t0 + t) * H + h) * D + chn * 4) =
-                *reinterpret_cast<const uint4 *>(sm + S1H + t * 512 + chn * 16);
-        }
-      } else {
-        for (int e = tid; e < 64 * 16; e += NTC) {
-          const int t = e >> 4, chn = e & 15;
-          if (t < n)
-            *reinterpret_cast<uint4 *>(dv + ((size_t)(tok0 + t0 + t) * H + h) * D + chn * 8) =
-                *reinterpret_cast<const uint4 *>(sm + S1H + t * 256 + chn * 16);
-        }
-      }
-    }
-    // ---- phase E: U_S += K^T dKS
-    ok = phase_run(K, tid, [&] {
-      const uint32_t i128 = idesc_bf16(128, 128);
-      mma_tile_kmn(tm + T_DS, sb + S2H, 0, sb + KQ, 16384, 4, i128, true);
-      mma_tile_kmn(tm + T_DS, sb + S2L, 0, sb + KQ, 16384, 4, i128, true);
-      bulk_wait_read();  // the staging is rewritten next (the gradient tiles)
-      return true;
-    });
-    if (!ok) break;
-    if (c > 0) {  // the next chunk's inputs, while this one finishes
-      if (!tma)
-        fetch_kq(c - 1);
-      else if (tid == 0)
-        tma_kq(c - 1);
-      pre = fetch_pre(c - 1);
-    }
-    // the carried gradients' tiles (dS, dR complete in TMEM): the A operands of
-    // the next chunk's phase A (the scratch tiles in their place are done with)
-#pragma unroll 1
-    for (int c0 = g16; c0 < D; c0 += 64) {
-      float s[16], r[16];
-      tmem_ld16x2(tm + lane + T_DS + c0, s, tm + lane + T_DR + c0, r);
-      put_grad16(DSH, DSL, c0, s);
-      put_grad16(DRH, DRL, c0, r);
-    }
-    fence_async_smem();  // the tiles are read by the MMAs and by a bulk copy
-  }
-  if (ok) {
-    for (int c0 = g16; c0 < D; c0 += 64) {
-      float s[16], r[16];
-      tmem_ld16(tm + lane + T_DS + c0, s);
-      tmem_ld16(tm + lane + T_DR + c0, r);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        if (P.dS0) P.dS0[st_base + (size_t)(c0 + i) * D + j] = s[i];
-        if (P.dR0) P.dR0[st_base + (size_t)(c0 + i) * D + j] = r[i];
-      }
-    }
-  } else if (tid == 0) {
-    if (p.err) atomicExch(p.err, RDN_ERR_TIMEOUT);
-    // no copy into this CTA's shared memory or MMA outlives it (bounded waits)
-    ctl_drain(K);
-    for (; tma_seen < tma_arms; ++tma_seen) mbar_wait(K.barC, tma_seen & 1u);
-  }
-  cp_async_wait_all();
-  if (tid == 0) bulk_wait_all();
-  fence_before_sync();
-  __syncthreads();
-  if (warp == 0) tmem_dealloc(tm, 512);
-}
-
 // ======================================================================== 3
 // bwd_post: everything that reduces over the value dimension, followed by the
-// chunk-matrix part of the gradients (the work bwd_finish of chunk_bwd.cu does
-// for the SIMT path), one persistent CTA of 512 threads per SM walking the
-// chunks.  Thread (j, qd) owns value column j = TMEM lane j and quarter qd of
+// chunk-matrix part of the gradients, one persistent CTA of 512 threads per SM
+// walking the chunks.  Thread (j, qd) owns value column j = TMEM lane j and quarter qd of
 // the chunk's tokens (or of the key rows of a state).
 //
 // dK and dQ are accumulated transposed in TMEM (lane = key dimension d,
@@ -789,7 +285,9 @@ __device__ __forceinline__ float row_total(const float *part, int t) {
          part[(4 * g + 3) * 16 + i];
 }
 
-template <bool kGeneric>  // (as bwd_chain_kernel's)
+// kGeneric: the RLA mode and the variant flags (TcBwdParams::rla, FwdParams::mods)
+// are read; the RDN method's instance has them folded away
+template <bool kGeneric>
 __global__ void __launch_bounds__(po::NTP, 1) bwd_post_kernel(TcBwdParams P) {
   using namespace po;
   extern __shared__ __align__(1024) uint8_t sm[];
@@ -1549,6 +1047,7 @@ cudaError_t launch_bwd_tc(const FwdParams &f, const void *dO, const float *dST, 
   const long long rows = (long long)f.B * f.T;
   P.tma = make_tile_map(P.map_k, f.k, D, f.H, rows) && make_tile_map(P.map_q, f.q, D, f.H, rows) &&
           make_tile_map(P.map_do, dO, D, f.H, rows);
+  P.dv_ok = !grad_f32 && make_tile_map(P.map_dv, dv, D, f.H, rows);
   const bool saved = f.sv_E && f.sv_E2 && f.sv_mask;  // E, E2, mask kept by the forward
   if (saved) {
     P.Ebuf = f.sv_E;
@@ -1560,11 +1059,7 @@ cudaError_t launch_bwd_tc(const FwdParams &f, const void *dO, const float *dST, 
                                 (int)rc::SMEM)) != cudaSuccess)
     return e;
   const bool generic = rla || f.mods != 0;
-  auto chain = generic ? bwd_chain_kernel<true> : bwd_chain_kernel<false>;
   auto post = generic ? bwd_post_kernel<true> : bwd_post_kernel<false>;
-  if ((e = cudaFuncSetAttribute(chain, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)ch::SMEM)) != cudaSuccess)
-    return e;
   if ((e = cudaFuncSetAttribute(post, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)po::SMEM)) != cudaSuccess)
     return e;
@@ -1572,18 +1067,9 @@ cudaError_t launch_bwd_tc(const FwdParams &f, const void *dO, const float *dST, 
     RDN_LAUNCH("bwd_recompute", s, bwd_recompute_kernel<<<(unsigned)nct, NT, rc::SMEM, s>>>(P));
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
+  if ((e = launch_bwd_chain(P, s)) != cudaSuccess) return e;
   int nsm = 0;
   if ((e = sm_count(&nsm)) != cudaSuccess) return e;
-  const bool both = pick_on_device(f, nsm);
-  if (both || use_pairs(f, nsm)) {
-    P.f.pick = both ? 2 : 0;
-    if ((e = launch_bwd_pair(P, s)) != cudaSuccess) return e;
-    P.f.pick = 1;
-  }
-  if (both || !use_pairs(f, nsm)) {
-    RDN_LAUNCH("bwd_chain", s, chain<<<f.nseq * f.H, NTC, ch::SMEM, s>>>(P));
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
   const unsigned post_grid = (unsigned)(nct < (size_t)nsm ? nct : (size_t)nsm);  // one CTA per SM
   RDN_LAUNCH("bwd_post", s, post<<<post_grid, po::NTP, po::SMEM, s>>>(P));
   return cudaGetLastError();

@@ -1,4 +1,4 @@
-// bwd_tc.cuh -- what the tensor-core backward kernels (bwd_tc.cu, bwd_pair.cu)
+// bwd_tc.cuh -- what the tensor-core backward kernels (bwd_tc.cu, bwd_chain.cu)
 // share: their parameters, operand-tile writers, and the barriers and phases of
 // a CTA.
 #pragma once
@@ -11,7 +11,7 @@ namespace bwdtc {
 using namespace tc;
 
 constexpr int D = 128;
-constexpr int NTC = 512;  // threads per CTA of bwd_chain (4 warps per TMEM lane quadrant)
+constexpr int NTC = 512;  // bwd_chain's element-wise threads (4 warps per TMEM lane quadrant)
 
 struct TcBwdParams {
   FwdParams f;          // inputs; f.ws = prep records (shared-memory images)
@@ -40,6 +40,8 @@ struct TcBwdParams {
   alignas(64) unsigned char map_q[128];
   alignas(64) unsigned char map_do[128];
   bool tma;
+  alignas(64) unsigned char map_dv[128];  // and over dv (bf16); dv_ok: it is valid
+  bool dv_ok;
 };
 
 __device__ __forceinline__ uint32_t pack2(float a, float b) {
@@ -78,14 +80,6 @@ __device__ __forceinline__ void put8s(uint8_t *hi, uint8_t *lo, int r, int c0,
   for (int i = 0; i < 4; ++i) split_pack_bf16(v[2 * i], v[2 * i + 1], h[i], l[i]);
   *reinterpret_cast<uint4 *>(hi + sw128(r, c0)) = make_uint4(h[0], h[1], h[2], h[3]);
   *reinterpret_cast<uint4 *>(lo + sw128(r, c0)) = make_uint4(l[0], l[1], l[2], l[3]);
-}
-// K-major A (single block, K = 64) times MN-major B, split both: 3 products
-__device__ __forceinline__ void mma_s3_kmn(uint32_t d, uint32_t a_hi, uint32_t a_lo,
-                                           uint32_t b_hi, uint32_t b_lo, uint32_t b_lbo,
-                                           uint32_t idesc, bool acc_first) {
-  mma_tile_kmn(d, a_hi, 0, b_hi, b_lbo, 4, idesc, acc_first);
-  mma_tile_kmn(d, a_hi, 0, b_lo, b_lbo, 4, idesc, true);
-  mma_tile_kmn(d, a_lo, 0, b_hi, b_lbo, 4, idesc, true);
 }
 // K-major A and B (single block, K = 64), split both
 __device__ __forceinline__ void mma_s3_kk(uint32_t d, uint32_t a_hi, uint32_t a_lo, uint32_t b_hi,
@@ -211,6 +205,7 @@ __device__ __forceinline__ bool phase_run_with(Ctl &k, int tid, F issue, G durin
     if (!k.skip) mma_commit(k.bar);
     k.skip = false;
   }
+  __syncwarp();  // (TMEM accesses take whole warps)
   during();
   const bool ok = mbar_wait(k.bar, k.phase, k.limit);
   k.phase ^= 1u;
@@ -233,6 +228,7 @@ __device__ __forceinline__ void phase_issue(Ctl &k, int tid, F issue) {
     if (!k.skip) mma_commit(k.bar);
     k.skip = false;
   }
+  __syncwarp();  // (TMEM accesses take whole warps)
 }
 // ... then wait for them (every thread).
 __device__ __forceinline__ bool phase_wait(Ctl &k) {
@@ -258,7 +254,7 @@ __device__ __forceinline__ const uint8_t *rec_bytes(const FwdParams &p, size_t c
 
 }  // namespace bwdtc
 
-// The chain over a CTA pair per (sequence, head) (bwd_pair.cu).
-cudaError_t launch_bwd_pair(const bwdtc::TcBwdParams &P, cudaStream_t s);
+// The gradients carried between chunks (bwd_chain.cu).
+cudaError_t launch_bwd_chain(const bwdtc::TcBwdParams &P, cudaStream_t s);
 
 }  // namespace rdn
