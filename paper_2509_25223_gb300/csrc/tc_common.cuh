@@ -104,20 +104,11 @@ __device__ __forceinline__ void tma_prefetch_3d(const void *map, int c0, int c1,
                : "memory");
 }
 
-// Hints that bring global memory closer ahead of its use (no completion to
-// wait for; the later loads find the lines cached): into L2, a contiguous
-// range (16-byte aligned address and size) or the 128-byte line of one address.
+// A hint that brings a contiguous range of global memory (16-byte aligned address
+// and size) into L2 ahead of its use (no completion to wait for).
 __device__ __forceinline__ void prefetch_l2_bulk(const void *src_gmem, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src_gmem), "r"(bytes)
                : "memory");
-}
-__device__ __forceinline__ void prefetch_l2_line(const void *src_gmem) {
-  asm volatile("prefetch.global.L2 [%0];" ::"l"(src_gmem));
-}
-// ... and the line of one address into this SM's L1, for loads a few
-// thousand cycles later
-__device__ __forceinline__ void prefetch_l1_line(const void *src_gmem) {
-  asm volatile("prefetch.global.L1 [%0];" ::"l"(src_gmem));
 }
 
 // 16 consecutive floats of shared memory at a 16-byte aligned address, by
@@ -273,11 +264,6 @@ __device__ __forceinline__ void tmem_alloc(uint32_t *slot, uint32_t ncols) {
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols)
                : "memory");
-}
-
-// TMEM address of (lane, column): lane in the upper 16 bits.
-__device__ __forceinline__ uint32_t tmem_addr(uint32_t base, uint32_t lane, uint32_t col) {
-  return base + (lane << 16) + col;
 }
 
 // One warp reads 32 lanes x 16 consecutive 32-bit columns: thread i of the
@@ -535,92 +521,8 @@ __device__ __forceinline__ void mma_tile_mnmn(uint32_t d_tmem, uint32_t a_base, 
   }
 }
 
-// Sum a per-thread vector v[64] over the 32 lanes of a warp by halving
-// exchanges: afterwards lane l holds the warp sums for tokens
-// t = tbase(l) and tbase(l) + 1 in out[0..1], with
-// tbase(l) = 32 b4 + 16 b3 + 8 b2 + 4 b1 + 2 b0 for the bits b of l.
-__device__ __forceinline__ void warp_transpose_reduce64(const float (&v)[64], float (&out)[2]) {
-  const int lane = threadIdx.x & 31;
-  float a[32];
-  {
-    const bool hi = lane & 16;
-#pragma unroll
-    for (int k = 0; k < 32; ++k) {
-      const float send = hi ? v[k] : v[32 + k];
-      const float keep = hi ? v[32 + k] : v[k];
-      a[k] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-    }
-  }
-  float b[16];
-  {
-    const bool hi = lane & 8;
-#pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      const float send = hi ? a[k] : a[16 + k];
-      const float keep = hi ? a[16 + k] : a[k];
-      b[k] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-    }
-  }
-  float c[8];
-  {
-    const bool hi = lane & 4;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const float send = hi ? b[k] : b[8 + k];
-      const float keep = hi ? b[8 + k] : b[k];
-      c[k] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-    }
-  }
-  float d[4];
-  {
-    const bool hi = lane & 2;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const float send = hi ? c[k] : c[4 + k];
-      const float keep = hi ? c[4 + k] : c[k];
-      d[k] = keep + __shfl_xor_sync(0xffffffffu, send, 2);
-    }
-  }
-  {
-    const bool hi = lane & 1;
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const float send = hi ? d[k] : d[2 + k];
-      const float keep = hi ? d[2 + k] : d[k];
-      out[k] = keep + __shfl_xor_sync(0xffffffffu, send, 1);
-    }
-  }
-}
-// Sum a per-thread vector v[32] over the 32 lanes of a warp by halving
-// exchanges: afterwards lane l holds the warp sum of v[l].
-__device__ __forceinline__ float warp_transpose_reduce32(const float (&v)[32]) {
-  const int lane = threadIdx.x & 31;
-  float a[16], b[8], c[4], d[2];
-#pragma unroll
-  for (int k = 0; k < 16; ++k) {
-    const bool hi = lane & 16;
-    a[k] = (hi ? v[16 + k] : v[k]) + __shfl_xor_sync(0xffffffffu, hi ? v[k] : v[16 + k], 16);
-  }
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const bool hi = lane & 8;
-    b[k] = (hi ? a[8 + k] : a[k]) + __shfl_xor_sync(0xffffffffu, hi ? a[k] : a[8 + k], 8);
-  }
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const bool hi = lane & 4;
-    c[k] = (hi ? b[4 + k] : b[k]) + __shfl_xor_sync(0xffffffffu, hi ? b[k] : b[4 + k], 4);
-  }
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    const bool hi = lane & 2;
-    d[k] = (hi ? c[2 + k] : c[k]) + __shfl_xor_sync(0xffffffffu, hi ? c[k] : c[2 + k], 2);
-  }
-  const bool hi = lane & 1;
-  return (hi ? d[1] : d[0]) + __shfl_xor_sync(0xffffffffu, hi ? d[0] : d[1], 1);
-}
-
-// The same for v[16]: afterwards lanes 2 i and 2 i + 1 hold the warp sum of v[i].
+// Sum a per-thread vector v[16] over the 32 lanes of a warp by halving
+// exchanges: afterwards lanes 2 i and 2 i + 1 hold the warp sum of v[i].
 __device__ __forceinline__ float warp_transpose_reduce16(const float (&v)[16]) {
   const int lane = threadIdx.x & 31;
   float a[8], b[4], c[2];
@@ -642,11 +544,6 @@ __device__ __forceinline__ float warp_transpose_reduce16(const float (&v)[16]) {
   const bool hi = lane & 2;
   const float d = (hi ? c[1] : c[0]) + __shfl_xor_sync(0xffffffffu, hi ? c[0] : c[1], 2);
   return d + __shfl_xor_sync(0xffffffffu, d, 1);
-}
-
-__device__ __forceinline__ int transpose_reduce_tbase(int lane) {
-  return ((lane >> 4) & 1) * 32 + ((lane >> 3) & 1) * 16 + ((lane >> 2) & 1) * 8 +
-         ((lane >> 1) & 1) * 4 + (lane & 1) * 2;
 }
 
 // Byte offset of element (r, c), c in [0, 64), in a K-major 128B-swizzled tile
