@@ -337,7 +337,7 @@ inline cudaError_t sm_count(int *n) {
 // Whether the forward tensor-core scan gives each (sequence, head) a pair of
 // CTAs (fwd_pair.cu) or one: whichever ends first.  A chunk costs a pair about
 // 0.6 of what it costs one CTA (4.4 us against 7.5, saving for the backward 6.1
-// against 9.7; 32 heads, T = 16384 and 2000, against 128 heads).
+// against 9.2; 32 heads, T = 16384 and 2000, against 128 heads).
 // Equal sequences run in waves of one CTA per SM:
 inline bool use_pairs(const FwdParams &p, int nsm) {
   const long long n = (long long)p.nseq * p.H;

@@ -55,8 +55,8 @@ constexpr uint32_t SM_X = 163840;
 constexpr uint32_t SM_VEC = 229376;
 constexpr int kVec = 196;
 constexpr uint32_t SM_BAR = SM_VEC + 2 * kVec * 4;
-// mbarriers: chain, slot A, slot B, drain, tiles, hand-over, side, MMA2 / 6, MMA4 / 8
-constexpr uint32_t SM_SLOT = SM_BAR + 72;
+// mbarriers: chain, slot A, slot B, drain, tiles, hand-over, side, MMA2 / 6, MMA4 / 8, image
+constexpr uint32_t SM_SLOT = SM_BAR + 80;
 constexpr uint32_t SM_FLAG = SM_SLOT + 4;
 constexpr size_t kPairSmem = SM_FLAG + 4;
 static_assert(SM_X + 65536 == SM_VEC && SM_V + 16384 == SM_VEC, "carve-up");
@@ -89,6 +89,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
   uint64_t *barX = bar + 5;  // CTA 1: full; CTA 0: empty
   uint64_t *barN = bar + 6;  // the products issued behind the chain's
   uint64_t *barM2 = bar + 7, *barM4 = bar + 8;  // MMA2 / 6 and MMA4 / 8, for the copying warp
+  uint64_t *barJ = bar + 9;  // E's image has left
   uint32_t *slot = reinterpret_cast<uint32_t *>(sm + SM_SLOT);
   volatile int *flag = reinterpret_cast<volatile int *>(sm + SM_FLAG);
 
@@ -111,6 +112,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
   const bool tnh = kGeneric && (p.mods & RDN_FLAG_TANH_RESIDUAL);
   const bool stl = kGeneric && (p.mods & RDN_FLAG_STATELESS_AUX);
   const size_t st_base = ((size_t)sq * p.H + h) * D * D;
+  uint8_t *keep = base ? p.sv_E : p.sv_E2;  // E's images (hi | lo) for the backward
 
   if (tid == 0) {
     for (int b = 0; b < 5; ++b) mbar_init(bar + b, 1);
@@ -118,6 +120,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     mbar_init(barN, 1);
     mbar_init(barM2, 1);
     mbar_init(barM4, 1);
+    mbar_init(barJ, 1);
     fence_mbar_init();
     if (!base) mbar_expect_tx(barX, 65536);
     *flag = 0;
@@ -364,7 +367,6 @@ __global__ void __launch_bounds__(kPairThreads, 1)
       load_gates(0);
       put_gates(0);
     }
-    uint8_t *keep = base ? p.sv_E : p.sv_E2;  // E's images (hi | lo) for the backward
     bool alive = true, good = true;  // good: (lane 0) no wait of this warp gave up
     // (a wait that gave up leaves its phase incomplete, which takes no further
     // arrival: nothing is armed after it)
@@ -378,7 +380,10 @@ __global__ void __launch_bounds__(kPairThreads, 1)
       const bool more = c + 1 < NC;
       const bool tma_next = more && by_tma(c + 1);
       if (by_tma(c) && one) await(mbar_wait(barE, (armE - 1) & 1u));
-      bulk_wait_read();  // o's rows and E's image of the chunk before
+      // o of the chunk before has left its staging; E's image, which went out
+      // behind it (lane 0), is waited for past the barrier
+      if (one && keep && c > 0) bulk_wait_read_all_but_last();
+      else bulk_wait_read();
       __syncwarp();
       __syncthreads();
       if (*flag) {
@@ -387,6 +392,10 @@ __global__ void __launch_bounds__(kPairThreads, 1)
       }
       if (more) load_gates(c + 1);
       if (one) {
+        if (keep && c > 0) {
+          bulk_wait_read();
+          mbar_arrive(barJ);
+        }
         if (more) prefetch_chunk(c + 1);
         if (c > 0) {  // slot B: free once chunk c - 1's product with it is complete
           await(mbar_wait(barN, (uint32_t)(c - 1) & 1u, limit));
@@ -619,6 +628,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
       if (c > 0) hand_over(c - 1);
       if (!RDNV) scale_state(GamC, start);
       wait_chain();
+      if (keep && c > 0) warp_wait(barJ, (uint32_t)(c - 1) & 1u);  // (E's image has left XE)
       float gks[16];
       {
         float x[16], gm[16];
@@ -666,6 +676,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
         *flag = 1;
       }
       __syncwarp();
+      if (keep && c > 0) warp_wait(barJ, (uint32_t)(c - 1) & 1u);  // (E2's image has left XE)
       float r[16], ob[16];
       {
         const float4 *x = reinterpret_cast<const float4 *>(sm + SM_X + 2048 * warp) + (tid & 31);

@@ -49,8 +49,8 @@
 //
 // Measured (128 heads; before, with every product and copy issued by an
 // element-wise thread): T = 2048 240 us (293), 7.5 us a chunk; T = 4096 saving
-// for the backward 618 us (685), 9.7 us a chunk, of which a CTA moves 390 KB from
-// and to HBM (5.2 TB/s of the 6.9 a copy reaches).
+// for the backward 592 us (685), 9.2 us a chunk, of which a CTA moves 390 KB from
+// and to HBM (5.4 TB/s of the 6.9 a copy reaches).
 //
 // TMEM (512 columns): [0,128) S   [128,256) R   [256,384) D1   [384,512) D3
 // (D1 holds KS|QS, then E | Ob, Gprev KS + Ap E = P | Ob, then E2 | Ob + gamma
@@ -83,9 +83,9 @@ constexpr uint32_t SM_W_LO = 212992;
 constexpr uint32_t SM_VEC = 229376;
 constexpr int kVec = 324;
 // mbarriers: chain, slot A, slot B, drain, tiles, then one phase a chunk: MMA2,
-// MMA3, MMA4, MMA6, MMA7, MMA8, E's image copied
+// MMA3, MMA4, MMA6, MMA7, MMA8, E's image copied, E2's
 constexpr uint32_t SM_BAR = SM_VEC + 2 * kVec * 4;
-constexpr int kBars = 12;
+constexpr int kBars = 13;
 constexpr uint32_t SM_SLOT = SM_BAR + 8 * kBars;
 constexpr uint32_t SM_FLAG = SM_SLOT + 4;
 constexpr size_t kTcSmem = SM_FLAG + 4;
@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(kScanThreads, 1)
   uint64_t *barD = bar + 3;  // the drain after a wait that gave up
   uint64_t *barE = bar + 4;  // a whole chunk's V, K, Q tiles by tensor-map copies
   uint64_t *barM2 = bar + 5, *barM3 = bar + 6, *barM4 = bar + 7, *barM6 = bar + 8, *barM7 = bar + 9,
-           *barM8 = bar + 10, *barI = bar + 11;
+           *barM8 = bar + 10, *barI = bar + 11, *barJ = bar + 12;
   uint32_t *slot = reinterpret_cast<uint32_t *>(sm + SM_SLOT);
   volatile int *flag = reinterpret_cast<volatile int *>(sm + SM_FLAG);
 
@@ -349,7 +349,6 @@ __global__ void __launch_bounds__(kScanThreads, 1)
       const bool tma_next = more && by_tma(c + 1);
       const uint32_t ph = (uint32_t)c & 1u;
       if (by_tma(c) && one) await(barE, (armE - 1) & 1u);
-      if (one) bulk_wait_read();  // E2's image of the chunk before
       __syncwarp();
       __syncthreads();
       if (*flag) {
@@ -358,6 +357,10 @@ __global__ void __launch_bounds__(kScanThreads, 1)
       }
       if (more) load_gates(c + 1);
       if (one) {
+        if (p.sv_E2 && c > 0) {
+          bulk_wait_read();
+          mbar_arrive(barJ);  // X may come over the chunk before's E2
+        }
         if (more) prefetch_chunk(c + 1);
         if (RDNV) {
           await(barM2, ph);
@@ -397,7 +400,6 @@ __global__ void __launch_bounds__(kScanThreads, 1)
       __syncwarp();
       bar_sync(kBarE2, kScanThreads);
       if (one) {
-        if (p.sv_E2) image(p.sv_E2, c);
         await(barM8, ph);
         if (good && tma_next) {  // K, Q are done with
           const int row = (int)(tok0 + (long long)(c + 1) * 64);
@@ -406,6 +408,7 @@ __global__ void __launch_bounds__(kScanThreads, 1)
             tma_load_3d(sm + SM_KQ + kb * 16384 + 8192, maps.q, 64 * kb, h, row, barE);
           }
         }
+        if (p.sv_E2) image(p.sv_E2, c);  // (behind what the next chunk waits for)
         if (more) {
           await(barM7, ph);
           if (good) load_b(rec_of(c + 1) + IMG_APMQ, 32768);
@@ -577,6 +580,7 @@ __global__ void __launch_bounds__(kScanThreads, 1)
       scale_state(T_R, stl ? 0.f : GamC, p.S_chunks && c > 0 ? p.R_chunks + ci * D * D : nullptr);
     }
     wait_chain();
+    if (p.sv_E2 && c > 0) warp_wait(barJ, (uint32_t)(c - 1) & 1u);  // (its image has left XE)
     // ---- X = V - Gam KS (= V - alpha Gprev KS); P accumulates onto Gprev KS (kept in
     // registers while MMA2 overwrites it), Ob onto Gam scale QS
     float gks[16], vv[16];
