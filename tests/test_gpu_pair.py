@@ -1,7 +1,8 @@
-"""The tensor-core scan and chain over a pair of CTAs per (sequence, head),
-which calls with few heads take, against the one-CTA kernels, which calls with
-more take: the same operands in the same order, so every result is the same
-bits.  (On a chip of 152 SMs 4 heads run in pairs, 80 one CTA each.)"""
+"""The tensor-core scan over a pair of CTAs per (sequence, head), which calls with
+few heads take, against the one-CTA kernel, which calls with more take: the same
+operands in the same order, so every result, and every gradient from what it
+saved, is the same bits.  (On a chip of 152 SMs 4 heads run in pairs, 80 one CTA
+each.)"""
 import pytest
 import torch
 
