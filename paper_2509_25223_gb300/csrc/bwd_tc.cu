@@ -157,6 +157,7 @@ __global__ void __launch_bounds__(NT, 1) bwd_recompute_kernel(TcBwdParams P) {
   }
   if (ok) {
     if (tid == 0) load_slot<0>(K, sm + SLOTA, rec + IMG_TG, 16384);
+    __syncwarp();  // (TMEM accesses take whole warps)
 #pragma unroll
     for (int c0 = 0; c0 < 64; c0 += 16) {
       float e[16];

@@ -604,6 +604,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
   auto taken = [&](bool got) {
     __syncwarp();
     if (got && (tid & 31) == 0) mbar_arrive_remote_relaxed(peer_bar);
+    __syncwarp();  // (TMEM accesses follow, which take whole warps)
   };
 
   bool alive = true;
@@ -688,6 +689,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
         }
         // (a phase that has not completed takes no further arrival)
         if (got && tid == 0 && more) mbar_expect_tx(barX, 65536);
+        __syncwarp();
       }
       if (RDNV) {  // ---- X2 = r - Gam KR;  MMA6: E2^T = X2^T T_gamma^T
         {
@@ -744,6 +746,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
       hand_over(NC - 1);
       // until CTA 1 holds them
       if (tid == 0 && !mbar_wait_cluster(barX, (uint32_t)(NC - 1) & 1u, limit)) *flag = 1;
+      __syncwarp();
     } else {
       finish_o(NC - 1);
     }

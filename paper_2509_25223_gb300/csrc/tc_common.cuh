@@ -255,6 +255,7 @@ __device__ __forceinline__ void fence_async_smem() {
 // Called by one full warp.  The allocated column base (lane 0) is written to
 // *slot in shared memory.
 __device__ __forceinline__ void tmem_alloc(uint32_t *slot, uint32_t ncols) {
+  __syncwarp();  // (its callers initialise barriers by one thread first)
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                    smem_u32(slot)),
                "r"(ncols)
