@@ -65,8 +65,13 @@ static_assert(kPairSmem <= 232448, "shared memory");
 constexpr int kPairThreads = kTcThreads + 64;  // and the issuing and the copying warp
 constexpr int kHandThreads = kTcThreads + 32;  // the element-wise warps and one of the two
 // named barriers on which the element-wise warps hand operands to the issuing
-// warp (X, E) and results to the copying warp (O), and one among themselves
-constexpr int kBarX = 1, kBarE = 2, kBarO = 3, kBarW = 4;
+// warp (X, E) and results to the copying warp (O), one among themselves, and one
+// on which both wait before the last chunk's results (Z).  No barrier may be
+// arrived at again before all its threads have joined the time before: within the
+// loop the chunk's first barrier, which every warp joins, keeps two uses apart;
+// behind it nothing does, so that the last use of O waits on Z, which the copying
+// warp joins once it has left O.
+constexpr int kBarX = 1, kBarE = 2, kBarO = 3, kBarW = 4, kBarZ = 5;
 
 // TMEM columns: the state; CTA 0: KS | QS, then E | Ob, then P | Ob, two sets by
 // the chunk's parity, then as A operands S's lo part and (wS E)^T (hi | lo), so
@@ -437,7 +442,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     if (alive && NC > 0) {
       bulk_wait_read();  // (what the last chunk's results are staged in is free)
       __syncwarp();
-      bar_sync(kBarO, kHandThreads);
+      bar_sync(kBarZ, kHandThreads);
       send(NC - 1);
     }
     bulk_wait_all();
@@ -741,7 +746,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
   }
 
   if (alive && NC > 0) {  // the last chunk's read-outs
-    bar_sync(kBarO, kHandThreads);  // (the chunk before's have left)
+    bar_sync(kBarZ, kHandThreads);  // (the chunk before's have left)
     if (base) {
       hand_over(NC - 1);
       // until CTA 1 holds them
