@@ -605,7 +605,8 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     for (int i = 0; i < 8; ++i) split_pack_bf16(w[2 * i], w[2 * i + 1], hi[i], lo[i]);
     tmem_st8x2(tm + lane + col + g16 / 2, hi, tm + lane + col + 32 + g16 / 2, lo);
   };
-  // CTA 1: this warp has used what it read of the hand-over buffer
+  // CTA 1: this warp has used what it read of the hand-over buffer (r and ob: the
+  // arrival orders nothing, the uses before it do)
   auto taken = [&](bool got) {
     __syncwarp();
     if (got && (tid & 31) == 0) mbar_arrive_remote_relaxed(peer_bar);
@@ -712,7 +713,6 @@ __global__ void __launch_bounds__(kPairThreads, 1)
         wait_chain();
       } else {
         tmem_st16(tm + lane + T_D1 + 64 + g16, ob);
-        taken(got);
       }
       {
         float e[16], w[16];
@@ -727,6 +727,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
         for (int i = 0; i < 16; ++i) w[i] *= e[i];
         put_w(d1, w);
         st_row16_split(sm + SM_XE, sm + SM_XE_LO, j, g16, e);
+        if (!RDNV) taken(got);  // (r was used only here)
       }
     }
     publish(kBarE);

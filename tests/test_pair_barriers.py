@@ -100,3 +100,16 @@ def test_no_barrier_is_arrived_at_again_before_it_completes(NC, rdn):
     for b in {tail_copy, tail_elem, O}:
         members[b] = [1, 2, 3]
     _explore(_programs(NC, rdn, tail_copy, tail_elem, O), members)
+
+
+def test_the_hand_over_is_taken_after_its_values_are_used():
+    """CTA 1 tells CTA 0 that the hand-over buffer may be written again by an
+    arrival that orders no earlier load: it has to stand behind the use of
+    everything read from there, r as well as ob, in either method."""
+    text = open(SRC).read()
+    part = text[text.index("float r[16], ob[16];"):text.index("publish(kBarE);", text.index("float r[16], ob[16];"))]
+    taken = [m.start() for m in re.finditer(r"taken\(got\);", part)]
+    assert len(taken) == 2
+    rdn_use, rla_use = part.index("r[i] - gm[i] * x[i]"), part.index("e[i] = r[i]")
+    puts = [m.start() for m in re.finditer(r"tmem_st16\(tm \+ lane \+ T_D1 \+ 64 \+ g16, ob\)", part)]
+    assert rdn_use < puts[0] < taken[0] and max(rla_use, puts[1]) < taken[1]
