@@ -235,27 +235,27 @@ __global__ void __launch_bounds__(NT, 1) bwd_recompute_kernel(TcBwdParams P) {
 // walking the chunks.  Thread (j, qd) owns value column j = TMEM lane j and quarter qd of
 // the chunk's tokens (or of the key rows of a state).
 //
-// Products (lane = key dimension i, column = token):
-//   A   R0 [dX2 ; dO]^T, S0 dO^T       B   S0 [dX ; dP]^T
-//   P4  dR E2^T, dS E^T
+// dK and dQ are accumulated transposed in TMEM (lane = key dimension d,
+// column t for dK_t, 64 + t for dQ_t):
+//   P2  R0 [dKR ; dQR]^T        P3  S0 [dKS ; dQS]^T
+//   P4  dR (diag(wR) E2)^T + dS (diag(wS) E)^T        (dK columns only)
 //   P7  K^T [dKK + dKK^T ; dQK]^T, and Q^T dQK kept apart (scaled at read-out)
-// dK and dQ are the sums of A, B and P4, each times its token's gate, onto which
-// P7 accumulates in TMEM.  The per-token gate terms are the same products again,
-// summed over the lanes against K or Q (dO . (Q R0) = Q . (R0 dO^T)), so that
-// the states' and gradients' read-outs (K S0, Q S0, K R0, Q R0, K dR, K dS: 64 of
-// the 226 products a chunk took before) are not formed.  The C x C gradients (P5)
-// and the Gram matrices K K^T, Q K^T go through shared memory for the
-// element-wise pass over (t, i) of Eqs. for T, M2, Mq, Ap.
+// The per-token gate terms are sums over the value columns of the read-outs K S0,
+// Q S0, K R0, Q R0 (P1) and K dR, K dS (P4) against the gradients in fp32.  They
+// cancel: summed over the key index of P2's and P3's products instead (Q . (R0 dO^T)
+// for dO . (Q R0)), which saves 64 of a chunk's 226 products and 4 % of the time,
+// the gradients enter as bf16 hi + lo pairs, and dbeta was 4.7 % further from 64
+// bits on the training pass, 51 to 81 % with upstream state gradients of unit size.
+// The C x C gradients (P5) and the Gram matrices K K^T, Q K^T go through
+// shared memory for the element-wise pass over (t, i) of Eqs. for T, M2, Mq, Ap.
 // Q enters the tensor-core products unscaled; the scale is applied to the
 // fp32 results.
 //
-// What bounds it: latencies.  A chunk takes about 48k cycles of an SM, in which
-// the products take 12k, the issue slots are 35 % busy and HBM is at 2.7 TB/s;
-// shared memory (227 KB) holds one chunk at a time, so that its phases follow one
-// another.  Hence the loads ahead: 32 of a state at once for <dR, R0> and
-// <dS, S0> (16 at a time cost 16 %), the next chunk's dO ahead of its bulk copies
-// (behind them 11 %).  Measured against the kernel that formed the read-outs:
-// 8192 chunks 1341 us (1397), packed 1384 (1471), RLA, 1024 chunks 198 (245).
+// What bounds it: latencies.  A chunk takes about 50k cycles of an SM, in which
+// the products take 14k and HBM is at 2.6 TB/s; shared memory (227 KB) holds one
+// chunk at a time, so that its phases follow one another.  8192 chunks 1399 us,
+// packed (32,768 tokens, 16 heads) 1480, RLA, 1024 chunks 207 (245 without an
+// instance of its own).
 namespace po {
 constexpr int NTP = 512;
 constexpr uint32_t SA = 0, SB = 65536;  // state images: hi 2 x 16 KB | lo 2 x 16 KB, rows j
@@ -274,10 +274,10 @@ constexpr int F_DM2 = 0, F_DMQ = TILE, F_DAB = 2 * TILE, F_KK = 3 * TILE, F_DAG 
               F_DAP = 5 * TILE, F_QK = 6 * TILE, F_VEC = 7 * TILE;
 static_assert((F_VEC + 9 * 64 + 6 * 8 * 64) * 4 <= (int)XH, "finish scratch");
 // TMEM columns
-constexpr uint32_t T_W2 = 0, T_W3O = 128, T_DKQ = 256, T_D2 = 384;  // A
-constexpr uint32_t T_W3 = 0, T_U1 = 128, T_U2 = 192;                 // B (over R0's), P4
-// P5 (after those): two 128-column products and the Gram one (past the dK, dQ
-// accumulators)
+constexpr uint32_t T_KS = 0, T_KR = 128, T_DKQ = 256, T_D2 = 384;
+constexpr uint32_t T_KDR = 0, T_KDS = 64, T_U1 = 128, T_U2 = 192;  // P4, after the read-outs
+// P5 (after the read-outs and P4): two 128-column products and the Gram one
+// (past the dK, dQ accumulators)
 constexpr uint32_t T_P5A = 0, T_P5B = 128, T_GR = 448;
 }  // namespace po
 
@@ -344,8 +344,8 @@ __global__ void __launch_bounds__(po::NTP, 1) bwd_post_kernel(TcBwdParams P) {
   const uint32_t tm = *slot;
   // A chunk's inputs are fetched in two parts, each during the previous chunk
   // (this CTA loops over chunks): the chunk-start states, fp32, staged where
-  // their images go; then dX2, dX (fp32 [t][j], staged in the operand pair's
-  // place) and the K, Q tile.
+  // their images go; then dX2, dX (fp32 [t][j], staged in the pair's place
+  // until P2) and the K, Q tile.
   auto fetch_states = [&](size_t ck) {
     if (tid == 0) {
       ctl_arm<0>(K, 131072);
@@ -353,106 +353,71 @@ __global__ void __launch_bounds__(po::NTP, 1) bwd_post_kernel(TcBwdParams P) {
       bulk_g2s(sm + SB, P.Rc + ck * D * D, 65536, K.barA);
     }
   };
-  // a chunk's first row (token * H + head) and its valid tokens
-  struct Span {
-    long long row;
-    int n;
-  };
-  auto span_of = [&](size_t ck) {
-    int s, h, c;
-    rec_decode(p, (long long)ck, s, h, c);
-    const SeqSpan sp = seq_span(p, s, h);
-    return Span{(sp.tok0 + c * 64) * H + h, min(64, sp.len - c * 64)};
-  };
-  auto fetch_rest = [&](size_t ck, const Span &to) {
+  auto fetch_rest = [&](size_t ck) {
     if (tid == 0) {
       ctl_arm<2>(K, 65536);
       bulk_g2s(sm + XH, P.dX2buf + ck * 64 * D, 32768, K.barC);
       bulk_g2s(sm + YH, P.dXbuf + ck * 64 * D, 32768, K.barC);
     }
+    int s_, h_, cc_;
+    rec_decode(p, (long long)ck, s_, h_, cc_);
+    const SeqSpan sp_ = seq_span(p, s_, h_);
+    const long long tok0_ = sp_.tok0;
+    const int t0_ = cc_ * 64, n_ = min(64, sp_.len - t0_);
     for (int e = tid; e < 64 * 16; e += NTP) {  // K, Q (exact bf16), asynchronous
       const int t = e >> 4, chn = e & 15;
-      const bool vld = t < to.n;
-      const size_t off = (size_t)(to.row + (vld ? t : 0) * H) * D + chn * 8;
+      const bool vld = t < n_;
+      const size_t off = ((size_t)(tok0_ + t0_ + (vld ? t : 0)) * H + h_) * D + chn * 8;
       const int blk = chn >> 3, cc = (chn & 7) * 8;
       cp_async16(sm + KQ + blk * 16384 + sw128(t, cc), k + off, vld);
       cp_async16(sm + KQ + blk * 16384 + sw128(64 + t, cc), q + off, vld);
     }
   };
-  // ... and this thread's dO (pairs of tokens), mask and gates, into registers
-  // ahead of those copies: behind them the loads took 5k cycles
-  uint32_t dob[8];
-  unsigned long long m = 0ull;
-  float gvv[5];
-  auto fetch_own = [&](size_t ck, const Span &to) {
-    if (!tnh) m = P.mask[ck * D + j] >> tb;
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      const unsigned short *src = reinterpret_cast<const unsigned short *>(dOp) +
-                                  (size_t)(to.row + (long long)(tb + i) * H) * D + j;
-      const uint32_t v = tb + i < to.n ? *src : 0;
-      dob[i >> 1] = i & 1 ? dob[i >> 1] | v << 16 : v;
-    }
-    if (tid < 64) {
-      const float *rec = p.ws + ck * kRecFloats + OFF_VEC;
-      gvv[0] = rec[V_GAM + tid];
-      gvv[1] = rec[V_GPREV + tid];
-      gvv[2] = rec[V_WS + tid];
-      gvv[3] = rec[V_WR + tid];
-      gvv[4] = tid < to.n ? p.gamma[to.row + (long long)tid * H] : 0.f;
-    }
-  };
-  auto put_gates = [&] {
-    if (tid < 64) {
-      Gam[tid] = gvv[0];
-      Gprev[tid] = gvv[1];
-      wS[tid] = gvv[2];
-      wR[tid] = gvv[3];
-      gamv[tid] = gvv[4];
-    }
-  };
-  Span cur{0, 0}, nxt{0, 0};
   if (blockIdx.x < nct) {
-    cur = span_of(blockIdx.x);
-    fetch_own(blockIdx.x, cur);
-    put_gates();
     fetch_states(blockIdx.x);
-    fetch_rest(blockIdx.x, cur);
+    fetch_rest(blockIdx.x);
   }
   // the previous chunk's dq, dk from TMEM to HBM (row = its first token row *
   // H + h; n = its valid tokens, -1 = none pending)
   long long dkq_row = 0;
   int dkq_n = -1;
-  auto store_dkq = [&](int tb) {  // tokens [tb, tb + 16)
+  auto store_dkq = [&]() {
+    __nv_bfloat16 *dk = (__nv_bfloat16 *)P.dk, *dq = (__nv_bfloat16 *)P.dq;
     const uint32_t tl = (uint32_t)((warp & 3) * 32) << 16;
-    const size_t at = (size_t)(dkq_row + (long long)tb * H) * D + j;
-    auto store = [&](void *out, const float (&v)[16]) {
+    float a[16], d2[16], qv[16];
+    tmem_ld16x2(tm + tl + T_DKQ + tb, a, tm + tl + T_D2 + tb, d2);
+    tmem_ld16(tm + tl + T_DKQ + 64 + tb, qv);
 #pragma unroll
-      for (int i = 0; i < 16; ++i)
-        if (tb + i < dkq_n) {
-          if (P.f32qk) ((float *)out)[at + (size_t)i * H * D] = v[i];
-          else ((__nv_bfloat16 *)out)[at + (size_t)i * H * D] = __float2bfloat16_rn(v[i]);
+    for (int i = 0; i < 16; ++i) {
+      const int t = tb + i;
+      if (t < dkq_n) {
+        const size_t off = (size_t)(dkq_row + (long long)t * H) * D + j;
+        if (P.f32qk) {
+          ((float *)P.dk)[off] = a[i] + scale * d2[i];
+          ((float *)P.dq)[off] = scale * qv[i];
+        } else {
+          dk[off] = __float2bfloat16_rn(a[i] + scale * d2[i]);
+          dq[off] = __float2bfloat16_rn(scale * qv[i]);
         }
-    };
-    float a[16], b[16];
-    tmem_ld16x2(tm + tl + T_DKQ + tb, a, tm + tl + T_D2 + tb, b);
-#pragma unroll
-    for (int i = 0; i < 16; ++i) a[i] += scale * b[i];
-    store(P.dk, a);
-    tmem_ld16(tm + tl + T_DKQ + 64 + tb, a);
-#pragma unroll
-    for (int i = 0; i < 16; ++i) a[i] *= scale;
-    store(P.dq, a);
+      }
+    }
+    dkq_n = -1;
   };
   bool ok = true;
   uint32_t it = 0;  // chunks done by this CTA: the parity of barrier B
   for (size_t chunk = blockIdx.x; chunk < nct && ok; chunk += gridDim.x, ++it) {
   const size_t next = chunk + gridDim.x;
-  const long long row0 = cur.row;
-  const int n = cur.n;
+  int sq, h, c;
+  rec_decode(p, (long long)chunk, sq, h, c);
+  const SeqSpan sp = seq_span(p, sq, h);
+  const long long tok0 = sp.tok0;
+  const int t0 = c * 64, n = min(64, sp.len - t0);
+  const float *recf = p.ws + chunk * kRecFloats;
   const float *S0 = P.Sc + chunk * D * D, *R0 = P.Rc + chunk * D * D;
   const uint8_t *gimg = P.gimg + chunk * 131072;  // dS hi | dR hi | dS lo | dR lo
-  float x2v[16], xv[16];  // this thread's tokens of dX2, dX
+  // this thread's tokens of dX2, dX (from the staging) and dO: read after P1 is
+  // issued, so that the MMA issue does not wait behind them
+  float x2v[16], xv[16], dov[16];
   // this thread's key rows of a state: [32 qd, 32 qd + 32), the columns
   // [32 (qd & 1), +32) of 64-row block qd >> 1 of the image
   const uint32_t kblk = (uint32_t)(qd >> 1) * 16384u;
@@ -473,16 +438,13 @@ __global__ void __launch_bounds__(po::NTP, 1) bwd_post_kernel(TcBwdParams P) {
       put16s(sm + base + kblk, sm + base + 32768 + kblk, j, kc0 + c0, w);
     }
   };
-  // sum over column j's entries of key rows [32 quarter, + 32) of (image at base,
-  // hi + lo) * st[i][j]
-  auto dot_image = [&](uint32_t base, const float *st, int quarter) {
-    float s = 0.f, x[32];
-#pragma unroll
-    for (int i = 0; i < 32; ++i) x[i] = __ldcg(st + (size_t)(32 * quarter + i) * D + j);
+  // sum over this thread's entries of (image at base, hi + lo) * x[i][j]
+  auto dot_image = [&](uint32_t base, const float (&x)[32]) {
+    float s = 0.f;
 #pragma unroll
     for (int k8 = 0; k8 < 4; ++k8) {
-      const int c8 = 4 * (quarter & 1) + k8;
-      const uint32_t o = base + (quarter >> 1) * 16384 + j * 128 + (((c8 ^ (j & 7)) & 7) << 4);
+      const int c8 = (kc0 >> 3) + k8;
+      const uint32_t o = base + kblk + j * 128 + (((c8 ^ (j & 7)) & 7) << 4);
       const uint4 hv = *reinterpret_cast<const uint4 *>(sm + o);
       const uint4 lv = *reinterpret_cast<const uint4 *>(sm + o + 32768);
       const __nv_bfloat16 *hb = reinterpret_cast<const __nv_bfloat16 *>(&hv);
@@ -500,22 +462,49 @@ __global__ void __launch_bounds__(po::NTP, 1) bwd_post_kernel(TcBwdParams P) {
   const uint32_t tm_lane = (uint32_t)((warp & 3) * 32) << 16;
   const uint32_t i128 = idesc_bf16(128, 128), i64 = idesc_bf16(128, 64);
 
-  // K (r0 = 0) or Q (64) of this thread's token tb + i at key index j
-  // (sw128; the offset hidden from the compiler, which would keep the 16 addresses
-  // over all chunks and spill them)
-  uint32_t koff = KQ + (j >> 6) * 16384 + tb * 128 + (j & 63) * 2;
-  asm volatile("" : "+r"(koff));
-  auto key = [&](int r0, int i) {
-    return __bfloat162float(*reinterpret_cast<const __nv_bfloat16 *>(
-        sm + (koff ^ ((i & 7) << 4)) + (r0 + i) * 128));
-  };
-
   cp_async_wait_all();  // K, Q tile (published by the barriers below)
-  if (!ctl_wait<0>(K, 0, tid)) *K.flag = 1;  // phase_wait below reports it to every thread
+  if (!ctl_wait<0>(K, 0, tid)) *K.flag = 1;  // phase_run below reports it to every thread
 #pragma unroll 1
   for (int s2 = 0; s2 < 2; ++s2) stage_to_image(s2 ? SB : SA);  // images of S0, R0
+  // ---- P1: read-outs [K S0 | Q S0] and [K R0 | Q R0] (lanes j, columns t')
+  phase_issue(K, tid, [&] {
+    const uint32_t t_ = *slot;
+    mma_tile<true>(t_ + T_KS, sb + SA, 16384, sb + KQ, 16384, 8, i128, false);
+    mma_tile<true>(t_ + T_KS, sb + SA + 32768, 16384, sb + KQ, 16384, 8, i128, true);
+    mma_tile<true>(t_ + T_KR, sb + SB, 16384, sb + KQ, 16384, 8, i128, false);
+    mma_tile<true>(t_ + T_KR, sb + SB + 32768, 16384, sb + KQ, 16384, 8, i128, true);
+    return true;
+  });
+  // while P1 runs: this thread's dO and the gate vectors (loads first, their
+  // latency under the stores), the previous chunk's dq, dk, then dX2 and dX
+  // from their staging
+  const unsigned long long m = tnh ? 0ull : P.mask[chunk * D + j] >> tb;
   const uint16_t *drow = reinterpret_cast<const uint16_t *>(P.mask) + (chunk * D + j) * 64 + tb;
-  auto dov = [&](int i) { return __uint_as_float(i & 1 ? dob[i >> 1] & 0xFFFF0000u : dob[i >> 1] << 16); };
+  __nv_bfloat16 dob[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const int t = tb + i;
+    dob[i] = t < n ? dOp[((size_t)(tok0 + t0 + t) * H + h) * D + j] : __float2bfloat16(0.f);
+  }
+  float gvv[5];
+  if (tid < 64) {
+    gvv[0] = recf[OFF_VEC + V_GAM + tid];
+    gvv[1] = recf[OFF_VEC + V_GPREV + tid];
+    gvv[2] = recf[OFF_VEC + V_WS + tid];
+    gvv[3] = recf[OFF_VEC + V_WR + tid];
+    gvv[4] = tid < n ? p.gamma[(size_t)(tok0 + t0 + tid) * H + h] : 0.f;
+  }
+  __syncwarp();  // (TMEM accesses take whole warps)
+  if (dkq_n >= 0) store_dkq();
+#pragma unroll
+  for (int i = 0; i < 16; ++i) dov[i] = __bfloat162float(dob[i]);
+  if (tid < 64) {
+    Gam[tid] = gvv[0];
+    Gprev[tid] = gvv[1];
+    wS[tid] = gvv[2];
+    wR[tid] = gvv[3];
+    gamv[tid] = gvv[4];
+  }
   if (!ctl_wait<2>(K, 0, tid)) *K.flag = 1;
   {
     const float *x2s = reinterpret_cast<const float *>(sm + XH);
@@ -526,104 +515,125 @@ __global__ void __launch_bounds__(po::NTP, 1) bwd_post_kernel(TcBwdParams P) {
       xv[i] = xs[(tb + i) * D + j];
     }
   }
-  __syncthreads();  // (the operands go where dX2, dX were staged)
-  put_tok(x2v, XH, XL);
-  {  // dO is exact in bf16: no lo part
-    uint8_t *row = sm + YH;
-    *reinterpret_cast<uint4 *>(row + sw128(j, tb)) = make_uint4(dob[0], dob[1], dob[2], dob[3]);
-    *reinterpret_cast<uint4 *>(row + sw128(j, tb + 8)) = make_uint4(dob[4], dob[5], dob[6], dob[7]);
-  }
-  // ---- A: R0 [dX2 ; dO]^T, S0 dO^T
-  phase_issue(K, tid, [&] {
-    mma_tile_mnmn<true>(tm + T_W2, sb + SB, 16384, sb + XH, 32768, 8, i128, false);
-    mma_tile_mnmn<true>(tm + T_W2, sb + SB, 16384, sb + XL, 16384, 8, i64, true);
-    mma_tile_mnmn<true>(tm + T_W2, sb + SB + 32768, 16384, sb + XH, 32768, 8, i128, true);
-    mma_tile_mnmn<true>(tm + T_W3O, sb + SA, 16384, sb + YH, 16384, 8, i64, false);
-    mma_tile_mnmn<true>(tm + T_W3O, sb + SA + 32768, 16384, sb + YH, 16384, 8, i64, true);
-    return true;
-  });
-  if (dkq_n >= 0) store_dkq(tb);  // the previous chunk's dq, dk
-  dkq_n = -1;
-  ok = phase_wait(K);
+  ok = phase_wait(K);  // (its barrier also publishes the gate vectors)
   auto dp_of = [&](int i) {
     if (tnh) return -grad_uq16(drow[i]) * x2v[i];
     return ((m >> i) & 1ull) ? -x2v[i] : 0.f;
   };
+  if (ok) {  // per-token gate terms: dGam, dGprev, and <dR,R0> + <dS,S0>
+    // the three sums' warp parts go where dX2 was staged (read into x2v above)
+    float *part = reinterpret_cast<float *>(sm + XH);
+    float rv[16];
+    {
+      float qs[16], qr[16];
+      tmem_ld16x2(tm + tm_lane + T_KS + 64 + tb, qs, tm + tm_lane + T_KR + 64 + tb, qr);
+      if (stl) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) qr[i] = 0.f;
+      }
+      // d gamma_t from the read-out: dO_t . (Gam_t Q R0)_t (the rest of Oa_t in P6)
+      lds16(Gam + tb, rv);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) rv[i] = plain ? 0.f : scale * rv[i] * dov[i] * qr[i];
+      warp_row_part(rv, part, tid);
+      lds16(gamv + tb, rv);
+#pragma unroll
+      for (int i = 0; i < 16; ++i)  // (plain combine: Gprev Q S0 and no gamma_t)
+        rv[i] = plain ? scale * dov[i] * qr[i] : scale * dov[i] * (qs[i] + rv[i] * qr[i]);
+    }
+    {
+      float ks[16], kr[16];
+      tmem_ld16x2(tm + tm_lane + T_KS + tb, ks, tm + tm_lane + T_KR + tb, kr);
+      if (stl) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) kr[i] = 0.f;
+      }
+      if (!rla) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) rv[i] -= x2v[i] * kr[i] + xv[i] * ks[i];
+      }
+      // the prediction's state term: Gprev K S0 (decayed residual: Gam K S0)
+      if (dec_res) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) rv[i] += dp_of(i) * ks[i];
+      }
+      warp_row_part(rv, part + 256, tid);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) rv[i] = dec_res ? 0.f : dp_of(i) * ks[i];
+      if (plain) {  // the base read-out's gate is Gprev
+        float qs[16];
+        tmem_ld16(tm + tm_lane + T_KS + 64 + tb, qs);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) rv[i] += scale * dov[i] * qs[i];
+      }
+    }
+    warp_row_part(rv, part + 512, tid);
+    __syncthreads();
+    if (tid < 192) {
+      const int w = tid >> 6, t = tid & 63;
+      const float tot = row_total(part + 256 * w, t);
+      if (w == 0)
+        park[A8::V_DGAM_OUT + t] = tot;
+      else
+        (w == 1 ? dGamS : dGprevS)[t] = tot;
+    }
+    __syncthreads();  // (P2's operands go where the parts are)
+    // ---- P2: dK, dQ += R0 [dKR ; dQR]^T, dKR = -Gam dX2, dQR = Gam gamma dO
+    float x[16], y[16];
+    lds16(Gam + tb, x);
+    lds16(gamv + tb, y);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      y[i] = stl ? 0.f : (plain ? 1.f : y[i]) * x[i] * dov[i];
+      x[i] = (rla || stl) ? 0.f : -x[i] * x2v[i];
+    }
+    put_tok(x, XH, XL);
+    put_tok(y, YH, YL);
+    ok = phase_run(K, tid, [&] {
+      mma_tile_mnmn<true>(tm + T_DKQ, sb + SB, 16384, sb + XH, 32768, 8, i128, false);
+      mma_tile_mnmn<true>(tm + T_DKQ, sb + SB, 16384, sb + XL, 32768, 8, i128, true);
+      mma_tile_mnmn<true>(tm + T_DKQ, sb + SB + 32768, 16384, sb + XH, 32768, 8, i128, true);
+      return true;
+    });
+  }
   if (ok && tid == 0) {  // R0's image is done with: dR's image into its place
     ctl_arm<1>(K, 65536);
     bulk_g2s(sm + SB, gimg + 32768, 32768, K.barB);
     bulk_g2s(sm + SB + 32768, gimg + 98304, 32768, K.barB);
   }
   __syncwarp();  // (TMEM accesses take whole warps)
-  // the per-token sums over the 128 lanes, a warp's part of each in lane 2 i for
-  // token tb + i: d gamma's read-out part (less its factor), dGam, dGprev
-  float o_gam = 0.f, o_dgam = 0.f, o_dgp = 0.f;
-  float v1[16];
-  if (ok) {
-    // dK = -Gam R0 dX2 + ..., dQ = Gam gamma R0 dO + Gam S0 dO (scaled at read-out);
-    // plain combine: no gamma, Gprev S0 dO
-    float a[16], b[16], w[16];
-    tmem_ld16(tm + tm_lane + T_W2 + 64 + tb, a);
-    if (stl) {
-#pragma unroll
-      for (int i = 0; i < 16; ++i) a[i] = 0.f;
-    }
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v1[i] = key(64, i) * a[i];
-    o_gam = warp_transpose_reduce16(v1);
-    if (!plain) {
-      lds16(gamv + tb, w);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        a[i] *= w[i];
-        v1[i] *= w[i];
-      }
-    }
-    tmem_ld16(tm + tm_lane + T_W3O + tb, b);
-    lds16(Gam + tb, w);
-#pragma unroll
-    for (int i = 0; i < 16; ++i) a[i] *= w[i];
-    if (plain) lds16(Gprev + tb, w);
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      a[i] = fmaf(w[i], b[i], a[i]);
-      b[i] *= scale * key(64, i);
-      v1[i] = plain ? scale * v1[i] : fmaf(scale, v1[i], b[i]);
-    }
-    if (plain) o_dgp = warp_transpose_reduce16(b);
-    tmem_st16(tm + tm_lane + T_DKQ + 64 + tb, a);
-    if (rla || stl) {
-#pragma unroll
-      for (int i = 0; i < 16; ++i) b[i] = 0.f;
-    } else {
-      tmem_ld16(tm + tm_lane + T_W2 + tb, b);
-      lds16(Gam + tb, w);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        v1[i] = fmaf(-key(0, i), b[i], v1[i]);
-        b[i] *= -w[i];
-      }
-    }
-    tmem_st16(tm + tm_lane + T_DKQ + tb, b);
-    // ---- B: S0 [dX ; dP]^T; meanwhile <dR, R0>
-    put_tok(xv, XH, XL);
-#pragma unroll
-    for (int i = 0; i < 16; ++i) a[i] = dp_of(i);
-    put_tok(a, YH, YL);
-  }
   // <dR, R0> + <dS, S0> into dGamC, each computed while MMAs run: the states
   // are re-read from L2 (not through L1, which holds the prefetched dO rows),
   // the gradients' images are in the states' places
   float gdot = 0.f;
-  if (ok) {
+  auto dot_state = [&](const float *st, uint32_t img) {
+    float x[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) x[i] = __ldcg(st + (size_t)(32 * qd + i) * D + j);
+    return dot_image(img, x);
+  };
+  if (ok) {  // ---- P3: dK, dQ += S0 [dKS ; dQS]^T, dKS = Gprev dP - Gam dX, dQS = Gam dO;
+             // meanwhile <dR, R0>
+    float x[16], y[16];
+    lds16(dec_res ? Gam + tb : Gprev + tb, x);
+    lds16(Gam + tb, y);
+    float gq[16];  // the base read-out's gate: Gam (plain combine: Gprev)
+    lds16(plain ? Gprev + tb : Gam + tb, gq);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      x[i] = x[i] * dp_of(i) - (rla ? 0.f : y[i] * xv[i]);
+      y[i] = gq[i] * dov[i];
+    }
+    put_tok(x, XH, XL);
+    put_tok(y, YH, YL);
     ok = phase_run_with(K, tid, [&] {
-      mma_tile_mnmn<true>(tm + T_W3, sb + SA, 16384, sb + XH, 32768, 8, i128, false);
-      mma_tile_mnmn<true>(tm + T_W3, sb + SA, 16384, sb + XL, 32768, 8, i128, true);
-      mma_tile_mnmn<true>(tm + T_W3, sb + SA + 32768, 16384, sb + XH, 32768, 8, i128, true);
+      mma_tile_mnmn<true>(tm + T_DKQ, sb + SA, 16384, sb + XH, 32768, 8, i128, true);
+      mma_tile_mnmn<true>(tm + T_DKQ, sb + SA, 16384, sb + XL, 32768, 8, i128, true);
+      mma_tile_mnmn<true>(tm + T_DKQ, sb + SA + 32768, 16384, sb + XH, 32768, 8, i128, true);
       return true;
     }, [&] {
       if (!ctl_wait<1>(K, it & 1u, tid)) *K.flag = 1;  // dR's image
-      gdot = stl ? 0.f : dot_image(SB, R0, qd);
+      gdot = stl ? 0.f : dot_state(R0, SB);
     });
   }
   if (ok && tid == 0) {  // and dS's image into S0's; the E2^T, E^T images into the pair's
@@ -634,33 +644,23 @@ __global__ void __launch_bounds__(po::NTP, 1) bwd_post_kernel(TcBwdParams P) {
     bulk_g2s(sm + XH, P.E2buf + chunk * 32768, 32768, K.barC);  // hi at XH, lo at XL
     bulk_g2s(sm + YH, P.Ebuf + chunk * 32768, 32768, K.barC);   // hi at YH, lo at YL
   }
-  __syncwarp();
-  float dkv[16];  // dK, without P7's part
-  if (ok) {  // (while the images arrive) B's part of dK and of the gate sums
-    float x[16], w[16];
-    tmem_ld16x2(tm + tm_lane + T_W3 + 64 + tb, x, tm + tm_lane + T_DKQ + tb, dkv);
-    // the prediction's state term: Gprev K S0 (decayed residual: Gam K S0)
-    lds16(dec_res ? Gam + tb : Gprev + tb, w);
+  __syncwarp();  // (TMEM accesses take whole warps)
+  // this thread's 16 tokens of row j of a (hi | lo) image of a [j][t] matrix
+  auto image_row = [&](uint32_t base, float (&out)[16]) {
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      dkv[i] = fmaf(w[i], x[i], dkv[i]);
-      x[i] *= key(0, i);
-      if (dec_res) v1[i] += x[i];
-    }
-    if (!dec_res) o_dgp += warp_transpose_reduce16(x);
-    if (!rla) {
-      tmem_ld16(tm + tm_lane + T_W3 + tb, x);
-      lds16(Gam + tb, w);
+    for (int k8 = 0; k8 < 2; ++k8) {
+      const int c8 = (tb >> 3) + k8;
+      const uint32_t o = base + j * 128 + (((c8 ^ (j & 7)) & 7) << 4);
+      const uint4 hv = *reinterpret_cast<const uint4 *>(sm + o);
+      const uint4 lv = *reinterpret_cast<const uint4 *>(sm + o + 16384);
+      const __nv_bfloat16 *hb = reinterpret_cast<const __nv_bfloat16 *>(&hv);
+      const __nv_bfloat16 *lb = reinterpret_cast<const __nv_bfloat16 *>(&lv);
 #pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        dkv[i] = fmaf(-w[i], x[i], dkv[i]);
-        v1[i] = fmaf(-key(0, i), x[i], v1[i]);
-      }
+      for (int e = 0; e < 8; ++e) out[k8 * 8 + e] = __bfloat162float(hb[e]) + __bfloat162float(lb[e]);
     }
-    o_dgam = warp_transpose_reduce16(v1);
-  }
-  if (ok) {  // ---- P4: dR E2^T, dS E^T (scaled by wR, wS per token below); meanwhile
-             // <dS, S0> and the dGamC reduction
+  };
+  if (ok) {  // ---- P4: dR E2^T, dS E^T (scaled by wR, wS per token below); K dR, K dS read-outs;
+             // meanwhile <dS, S0> and the dGamC reduction
     if (!ctl_wait<2>(K, 1, tid)) *K.flag = 1;  // the E images, for every thread
     if (!ctl_wait<0>(K, 1, tid)) *K.flag = 1;  // dS's image
     phase_issue(K, tid, [&] {
@@ -670,14 +670,17 @@ __global__ void __launch_bounds__(po::NTP, 1) bwd_post_kernel(TcBwdParams P) {
       mma_tile_mnmn<true>(tm + T_U2, sb + SA, 16384, sb + YH, 16384, 8, i64, false);
       mma_tile_mnmn<true>(tm + T_U2, sb + SA, 16384, sb + YL, 16384, 8, i64, true);
       mma_tile_mnmn<true>(tm + T_U2, sb + SA + 32768, 16384, sb + YH, 16384, 8, i64, true);
+      // (K dR)^T, (K dS)^T (lanes j, columns t; K exact)
+      mma_tile<true>(tm + T_KDR, sb + SB, 16384, sb + KQ, 16384, 8, i64, false);
+      mma_tile<true>(tm + T_KDR, sb + SB + 32768, 16384, sb + KQ, 16384, 8, i64, true);
+      mma_tile<true>(tm + T_KDS, sb + SA, 16384, sb + KQ, 16384, 8, i64, false);
+      mma_tile<true>(tm + T_KDS, sb + SA + 32768, 16384, sb + KQ, 16384, 8, i64, true);
       return true;
     });
-    if (warp != 0) gdot += dot_image(SA, S0, qd);  // (warp 0 issues; warp 4 has its columns)
-    if (warp == 4) gdot += dot_image(SA, S0, 0);
+    gdot += dot_state(S0, SA);
 #pragma unroll
     for (int off = 16; off; off >>= 1) gdot += __shfl_xor_sync(0xffffffffu, gdot, off);
     if (lane == 0) red[warp] = gdot;
-    if (next < nct) nxt = span_of(next);
     ok = phase_wait(K);  // (its barrier publishes the parts)
     if (ok && tid == 0) {
       float s = 0.f;
@@ -687,52 +690,33 @@ __global__ void __launch_bounds__(po::NTP, 1) bwd_post_kernel(TcBwdParams P) {
     __syncwarp();
   }
   if (ok) {
-    // dK += diag(wR) E2 dR^T + diag(wS) E dS^T; dwR_t = K_t . (dR E2^T)_t, dwS
-    // likewise.  The warp parts of the sums go where dS's image was.
-    float *part = reinterpret_cast<float *>(sm + SA);
+    // dK += diag(wR) E2 dR^T + diag(wS) E dS^T  (lanes i, columns t of this half)
     {
-      float u1[16], u2[16], w[16];
-      tmem_ld16x2(tm + tm_lane + T_U1 + tb, u1, tm + tm_lane + T_U2 + tb, u2);
-      lds16(wR + tb, w);
+      float a[16], u1[16], u2[16], wr[16], ws[16];
+      tmem_ld16x2(tm + tm_lane + T_DKQ + tb, a, tm + tm_lane + T_U1 + tb, u1);
+      tmem_ld16(tm + tm_lane + T_U2 + tb, u2);
+      lds16(wR + tb, wr);
+      lds16(wS + tb, ws);
 #pragma unroll
-      for (int i = 0; i < 16; ++i) dkv[i] = fmaf(w[i], u1[i], dkv[i]);
-      lds16(wS + tb, w);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) dkv[i] = fmaf(w[i], u2[i], dkv[i]);
-      tmem_st16(tm + tm_lane + T_DKQ + tb, dkv);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        const float kv = key(0, i);
-        u1[i] = stl ? 0.f : u1[i] * kv;
-        u2[i] *= kv;
-      }
-      warp_row_part(u1, part, tid);
-      warp_row_part(u2, part + 256, tid);
-      if (!(lane & 1)) {
-        part[512 + warp * 16 + (lane >> 1)] = o_gam;
-        part[768 + warp * 16 + (lane >> 1)] = o_dgam;
-        part[1024 + warp * 16 + (lane >> 1)] = o_dgp;
-      }
+      for (int i = 0; i < 16; ++i) a[i] = fmaf(wr[i], u1[i], fmaf(ws[i], u2[i], a[i]));
+      tmem_st16(tm + tm_lane + T_DKQ + tb, a);
     }
-    // this thread's dX2, dX again, for P5 (kept since A they would spill)
-    {
-      const float *x2s = P.dX2buf + chunk * 64 * D + j, *xs = P.dXbuf + chunk * 64 * D + j;
+    // dwR_t = sum_j (K dR)[t,j] E2[t,j], dwS_t = sum_j (K dS)[t,j] E[t,j]; the
+    // warp parts where dS's image was
+    float *part = reinterpret_cast<float *>(sm + SA);
+#pragma unroll 1
+    for (int w = 0; w < 2; ++w) {
+      float ev[16], rv[16];
+      image_row(w == 0 ? XH : YH, ev);
+      tmem_ld16(tm + tm_lane + (w == 0 ? T_KDR : T_KDS) + tb, rv);
 #pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        x2v[i] = __ldcg(x2s + (tb + i) * D);
-        xv[i] = __ldcg(xs + (tb + i) * D);
-      }
+      for (int i = 0; i < 16; ++i) rv[i] = (w == 0 && stl) ? 0.f : rv[i] * ev[i];
+      warp_row_part(rv, part + 256 * w, tid);
     }
     __syncthreads();
-    if (tid < 320) {  // read in the gate pass
+    if (tid < 128) {  // read in the gate pass
       const int w = tid >> 6, t = tid & 63;
-      const float tot = row_total(part + 256 * w, t);
-      if (w < 2)
-        park[(w == 0 ? A8::V_DWR : A8::V_DWS) + t] = tot;
-      else if (w == 2)
-        park[A8::V_DGAM_OUT + t] = plain ? 0.f : scale * Gam[t] * tot;
-      else
-        (w == 3 ? dGamS : dGprevS)[t] = tot;
+      park[(w == 0 ? A8::V_DWR : A8::V_DWS) + t] = row_total(part + 256 * w, t);
     }
     __syncthreads();  // (P5's operands go where the parts are)
   }
@@ -748,7 +732,7 @@ __global__ void __launch_bounds__(po::NTP, 1) bwd_post_kernel(TcBwdParams P) {
   float g_t = 0.f, beta_t = 0.f;
   if (ok) {
     if (tid < n) {
-      const size_t off = (size_t)(row0 + (long long)tid * H);
+      const size_t off = (size_t)(tok0 + t0 + tid) * H + h;
       g_t = p.g[off];
       beta_t = p.beta[off];
     }
@@ -757,9 +741,7 @@ __global__ void __launch_bounds__(po::NTP, 1) bwd_post_kernel(TcBwdParams P) {
     for (int i = 0; i < 16; ++i) y[i] = dp_of(i);
     put_tok(xv, SB, SB + 16384);
     put_tok(y, SB + 32768, SB + 49152);
-#pragma unroll
-    for (int i = 0; i < 16; ++i) y[i] = dov(i);
-    put_tok(y, SA, SA + 16384);  // gamma_t enters in the element-wise pass
+    put_tok(dov, SA, SA + 16384);  // gamma_t enters in the element-wise pass
     put_tok(x2v, SA + 32768, SA + 49152);
     static_assert(YH - XH == 32768 && YL - XL == 32768, "the [E2 ; E] atoms");
     ok = phase_run(K, tid, [&] {
@@ -780,7 +762,7 @@ __global__ void __launch_bounds__(po::NTP, 1) bwd_post_kernel(TcBwdParams P) {
     prefetch_l2_bulk(P.Sc + next * D * D, 65536);
     prefetch_l2_bulk(P.Rc + next * D * D, 65536);
   }
-  __syncwarp();
+  __syncwarp();  // (TMEM accesses take whole warps)
   // ---- element-wise pass over (t, i): the gradients of the chunk matrices'
   // entries turned into gradients of K K^T, Q K^T and of the gates
   float *F = reinterpret_cast<float *>(sm);
@@ -995,28 +977,44 @@ __global__ void __launch_bounds__(po::NTP, 1) bwd_post_kernel(TcBwdParams P) {
       o_dbeta = dbet[tid];
       o_dgamma = dgam[tid];
     }
-    if (next < nct) fetch_own(next, nxt);
     __syncthreads();
     if (next < nct) fetch_states(next);  // the state images and the fp32 tiles are done with
+    if (next < nct) {  // the next chunk's dO rows, mask words and gate vectors into L1
+      int s_, h_, cc_;
+      rec_decode(p, (long long)next, s_, h_, cc_);
+      const SeqSpan sp_ = seq_span(p, s_, h_);
+      const long long tok0_ = sp_.tok0;
+      const int t0_ = cc_ * 64, n_ = min(64, sp_.len - t0_);
+      if (tid < 128) {  // 64 rows of 256 bytes
+        const int t = tid >> 1;
+        if (t < n_) prefetch_l1_line(dOp + ((size_t)(tok0_ + t0_ + t) * H + h_) * D + (tid & 1) * 64);
+      } else if (tid < 136) {  // 128 mask words
+        if (!tnh) prefetch_l1_line(P.mask + next * D + (tid - 128) * 16);
+      } else if (tid < 148) {  // the record's 6 x 64 gate floats
+        prefetch_l1_line(p.ws + next * kRecFloats + OFF_VEC + (tid - 136) * 32);
+      } else if (tid < 180) {  // gamma, one line per two tokens
+        const int t = 2 * (tid - 148);
+        if (t < n_) prefetch_l1_line(p.gamma + (size_t)(tok0_ + t0_ + t) * H + h_);
+      }
+    }
     ok = phase_wait(K);
-    if (next < nct) put_gates();
-    if (ok && next < nct) fetch_rest(next, nxt);  // K, Q and the pair region are done with
+    if (ok && next < nct) fetch_rest(next);  // K, Q and the pair region are done with
   }
   if (ok) {
     if (tid < n) {
-      const size_t off = (size_t)(row0 + (long long)tid * H);
+      const size_t off = (size_t)(tok0 + t0 + tid) * H + h;
       P.dg[off] = o_dg;
       P.dbeta[off] = o_dbeta;
       P.dgamma[off] = o_dgamma;
     }
-    // dq, dk of this chunk: read out and stored during the next chunk's A
-    // (T_DKQ, T_D2 keep them until its end), or after the last chunk
-    dkq_row = row0;
+    // dq, dk of this chunk: read out and stored during the next chunk's P1
+    // (T_DKQ, T_D2 keep them until its P2), or after the last chunk
+    dkq_row = (tok0 + t0) * H + h;
     dkq_n = n;
   }
-  cur = nxt;
   }  // chunks
-  if (ok && dkq_n >= 0) store_dkq(tb);
+  __syncwarp();  // (TMEM accesses take whole warps)
+  if (ok && dkq_n >= 0) store_dkq();
   if (!ok && tid == 0) {
     if (p.err) atomicExch(p.err, RDN_ERR_TIMEOUT);
     ctl_drain(K);  // no bulk copy or MMA of this CTA outlives it

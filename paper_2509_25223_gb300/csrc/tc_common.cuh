@@ -110,6 +110,11 @@ __device__ __forceinline__ void prefetch_l2_bulk(const void *src_gmem, uint32_t 
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src_gmem), "r"(bytes)
                : "memory");
 }
+// ... and the line of one address into this SM's L1, for loads a few
+// thousand cycles later
+__device__ __forceinline__ void prefetch_l1_line(const void *src_gmem) {
+  asm volatile("prefetch.global.L1 [%0];" ::"l"(src_gmem));
+}
 
 // 16 consecutive floats of shared memory at a 16-byte aligned address, by
 // four 16-byte loads
