@@ -952,7 +952,7 @@ static cudaError_t launch_bwd_impl(const rdn_bwd_args &a, int variant, cudaStrea
   p.f.err = status_word();
   if (f.cu_seqlens) {  // this call's own copy of the packed-sequence table
     long long *seq = (long long *)(ws + l.total - 256 - l.seq);
-    cudaError_t e = launch_seq_table(f, seq, s);
+    cudaError_t e = launch_seq_table(f, variant, true, seq, s);
     if (e != cudaSuccess) return e;
     p.f.seq = seq;
   }

@@ -335,23 +335,41 @@ inline cudaError_t sm_count(int *n) {
 }
 
 // Whether the forward tensor-core scan gives each (sequence, head) a pair of
-// CTAs (fwd_pair.cu) or one: whichever ends first.  A chunk costs a pair about
-// 0.6 of what it costs one CTA (4.4 us against 7.5, saving for the backward 6.1
-// against 9.2; 32 heads, T = 16384 and 2000, against 128 heads).
-// Equal sequences run in waves of one CTA per SM:
-inline bool use_pairs(const FwdParams &p, int nsm) {
-  const long long n = (long long)p.nseq * p.H;
-  const long long waves1 = (n + nsm - 1) / nsm, waves2 = (2 * n + nsm - 1) / nsm;
-  return 10 * waves1 > 6 * waves2;
+// CTAs (fwd_pair.cu) or one: whichever ends first.  What a (sequence, head) costs,
+// in 0.1 us, fitted to calls of 4 to 304 heads and 1 to 64 chunks (rdnv: the delta
+// rule; states: chunk-start states kept, as for a backward): one CTA `one` and
+// `one_chunk` a chunk, a pair `two` and `two_chunk` a chunk, or `two_full` where
+// pairs fill the chip and wait for memory.  A pair's chunk is shorter and its
+// start longer, so that 16 RDN heads take 18.3 us by one CTA and 20.4 by pairs at
+// one chunk, 31.4 and 30.6 at three, 67 and 51 at eight; and pairs need twice the
+// SMs: 200 heads of eight chunks take 133 us by one CTA each and 168 by pairs.
+struct ScanCost {
+  int one, one_chunk, two, two_chunk, two_full;
+};
+__host__ __device__ inline ScanCost scan_cost(bool rdnv, bool states) {
+  if (rdnv) return states ? ScanCost{69, 90, 130, 60, 63} : ScanCost{63, 70, 120, 42, 61};
+  return states ? ScanCost{69, 65, 103, 54, 55} : ScanCost{59, 54, 95, 43, 45};
 }
-// Packed sequences differ in length: the longest one's chain of chunks or the
-// chip's throughput sets the time.  The lengths are on the device, so that
-// where pairs do not all fit at once both kernels are launched and the table
-// says which one runs (the other's CTAs return at once).
-__host__ __device__ inline bool pairs_for(long long longest, long long chunks, int H, int nsm) {
-  const long long t1 = chunks * H / nsm, t2 = 2 * chunks * H / nsm;
-  return 10 * (longest > t1 ? longest : t1) > 6 * (longest > t2 ? longest : t2);
+// The longest sequence's chain of chunks or the chip's throughput over all `seqs`
+// sequences of `chunks` chunks sets the time of either (both sides times nsm).
+__host__ __device__ inline bool pairs_for(const ScanCost &c, long long longest, long long seqs,
+                                          long long chunks, int H, int nsm) {
+  const long long l1 = (c.one + c.one_chunk * longest) * nsm, l2 = (c.two + c.two_chunk * longest) * nsm;
+  const long long f1 = (c.one * seqs + c.one_chunk * chunks) * H;
+  const long long f2 = (c.two * seqs + c.two_full * chunks) * 2 * H;
+  return (l2 > f2 ? l2 : f2) < (l1 > f1 ? l1 : f1);
 }
+// Where every pair has its two SMs at once the host decides (packed: the lengths
+// are on the device, the longest is taken for half of the tokens); where not, equal
+// sequences take one CTA each (f1 < f2, and in waves l1 never is above l2's).
+inline bool use_pairs(const FwdParams &p, bool rdnv, int nsm) {
+  if (2ll * p.nseq * p.H > nsm) return false;
+  const ScanCost c = scan_cost(rdnv, p.S_chunks != nullptr);
+  if (p.seq) return pairs_for(c, p.nseq > 1 ? (p.NC + 1) / 2 : p.NC, p.nseq, p.NC + p.nseq, p.H, nsm);
+  return pairs_for(c, p.NC, p.nseq, (long long)p.nseq * p.NC, p.H, nsm);
+}
+// ... and packed sequences, of which one may be long, have both kernels launched and
+// the table say which one runs (the other's CTAs return at once).
 inline bool pick_on_device(const FwdParams &p, int nsm) {
   return p.seq && 2ll * p.nseq * p.H > nsm;
 }

@@ -611,7 +611,7 @@ constexpr int kOrdered = 1024;  // packed sequences that are put in order of len
 // entry 0 read as 0 and entry N as T, so the table always covers [0, T) in
 // order), first chunks the exclusive prefix sum of ceil(len_s / 64).  One CTA.
 __global__ void __launch_bounds__(1024) seq_table_kernel(const int *__restrict__ cu, int N, int T,
-                                                         int H, int nsm,
+                                                         int H, ScanCost cost, int nsm,
                                                          long long *__restrict__ seq) {
   __shared__ long long wsum[32];
   __shared__ long long carry;
@@ -651,16 +651,18 @@ __global__ void __launch_bounds__(1024) seq_table_kernel(const int *__restrict__
     for (int u = 0; u < N; ++u) rank += ncs[u] > mine || (ncs[u] == mine && u < tid);
     upper[4 * rank] = tid;
     // (entry N's stays 0, no pairs, for more than kOrdered sequences)
-    if (rank == 0) upper[4 * N] = pairs_for(mine, carry, H, nsm);
+    if (rank == 0) upper[4 * N] = pairs_for(cost, mine, N, carry, H, nsm);
   }
 }
 
-cudaError_t launch_seq_table(const rdn_fwd_args &a, long long *seq, cudaStream_t s) {
+cudaError_t launch_seq_table(const rdn_fwd_args &a, int variant, bool states, long long *seq,
+                             cudaStream_t s) {
   int nsm = 0;
   const cudaError_t e = sm_count(&nsm);
   if (e != cudaSuccess) return e;
   RDN_LAUNCH("seq_table", s,
-             seq_table_kernel<<<1, 1024, 0, s>>>(a.cu_seqlens, a.num_seqs, a.T, a.H, nsm, seq));
+             seq_table_kernel<<<1, 1024, 0, s>>>(a.cu_seqlens, a.num_seqs, a.T, a.H,
+                                                 scan_cost(variant == 1, states), nsm, seq));
   return cudaGetLastError();
 }
 
@@ -696,7 +698,7 @@ cudaError_t launch_fwd(const rdn_fwd_args &a, int variant, cudaStream_t s) {
   p.inject = fault_injection() == 3 ? 1 : 0;
   if (a.cu_seqlens) {
     long long *seq = (long long *)((char *)a.workspace + total - 256 - seq_table_bytes(a));
-    const cudaError_t e = launch_seq_table(a, seq, s);
+    const cudaError_t e = launch_seq_table(a, variant, a.S_chunks != nullptr, seq, s);
     if (e != cudaSuccess) return e;
     p.seq = seq;
   }

@@ -95,8 +95,10 @@ inline size_t seq_table_bytes(const rdn_fwd_args &a) {
   return a.cu_seqlens ? ((sizeof(long long) * 2 * ((size_t)a.num_seqs + 1) + 255) & ~(size_t)255) : 0;
 }
 // Fill seq (seq_table_bytes) from the caller's cu_seqlens, clamping it into a
-// valid table; one small kernel on s.
-cudaError_t launch_seq_table(const rdn_fwd_args &a, long long *seq, cudaStream_t s);
+// valid table; one small kernel on s.  states: a forward scan that follows keeps
+// chunk-start states.
+cudaError_t launch_seq_table(const rdn_fwd_args &a, int variant, bool states, long long *seq,
+                             cudaStream_t s);
 
 struct FwdPlan {
   int NC;                // chunks per sequence

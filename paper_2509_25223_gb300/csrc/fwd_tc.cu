@@ -798,7 +798,7 @@ cudaError_t launch_fwd_tc(const FwdParams &p, bool rdnv, cudaStream_t s) {
   FwdParams one = p;
   const bool both = pick_on_device(p, nsm);
   maps.o_ok = !p.f32out && make_tile_map(maps.o, p.o, D, p.H, rows);
-  if (both || use_pairs(p, nsm)) {
+  if (both || use_pairs(p, rdnv, nsm)) {
     FwdParams two = p;
     two.pick = both ? 2 : 0;
     if ((e = launch_fwd_pair(two, maps, rdnv, s)) != cudaSuccess || !both) return e;

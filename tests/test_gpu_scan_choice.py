@@ -1,0 +1,72 @@
+"""Which forward scan a bf16, d = 128 call takes: one CTA a head (`fwd_tc_scan`) or a
+pair (`fwd_tc_pair`), whichever ends first.  Both give the same bits
+(tests/test_gpu_pair.py); here it is the choice, at sizes where one of the two took
+clearly longer, measured on a chip of 152 SMs (us, one CTA / pairs)."""
+import pytest
+import torch
+
+import paper_2509_25223_gb300 as rdn
+from rdn_synthetic import make_inputs
+
+pytestmark = pytest.mark.gpu
+
+NAMES = ("q", "k", "v", "g", "beta", "gamma")
+ONE, PAIR = "fwd_tc_scan", "fwd_tc_pair"
+
+
+@pytest.fixture(autouse=True)
+def _chip():
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("measured on 152 SMs")
+
+
+def _scans(variant, x, **kw):
+    """The scan kernels a forward launches, and its workspace."""
+    B, T, H, D = x["q"].shape
+    ws = torch.empty(rdn.workspace_bytes(variant + "_fwd", B, T, H, D, cu_seqlens=kw.get("cu_seqlens")),
+                     dtype=torch.uint8, device="cuda")
+    fwd = rdn.rdn_fwd if variant == "rdn" else rdn.rla_fwd
+    with rdn.LaunchTimer() as lt:
+        fwd(*(x[n] for n in NAMES), workspace=ws, **kw)
+    return {n for n, _ in lt.records if n in (ONE, PAIR)}, ws
+
+
+@pytest.mark.parametrize("variant,heads,T,states,want", [
+    ("rdn", 16, 64, False, ONE),      # 18.3 / 20.5
+    ("rdn", 4, 1, False, ONE),        # 18.0 / 20.9
+    ("rdn", 16, 256, False, PAIR),    # 38.8 / 34.7
+    ("rdn", 32, 128, True, ONE),      # 28.6 / 28.7
+    ("rdn", 76, 512, True, PAIR),     # 83.9 / 70.0
+    ("rla", 16, 192, False, ONE),     # 24.9 / 26.6
+    ("rla", 16, 512, False, PAIR),    # 51.5 / 47.0
+    ("rdn", 77, 512, False, ONE),     # 67.5 / 103
+    ("rdn", 200, 512, False, ONE),    # 133 / 168
+    ("rla", 160, 1024, True, ONE),    # 244 / 287
+])
+def test_equal_sequences(variant, heads, T, states, want):
+    x = make_inputs(heads, T, 1, 128, dtype="bf16", device="cuda", device_rng=True)
+    got, _ = _scans(variant, x, return_chunk_states=states)
+    assert got == {want}
+
+
+def _table_says_pairs(ws, n):
+    """The choice in the sequence table at the workspace's end: the upper half of
+    entry n's chunk number."""
+    size = (16 * (n + 1) + 255) // 256 * 256
+    table = ws[ws.numel() - 256 - size:][:16 * (n + 1)].view(torch.int64)
+    return int(table[2 * n + 1]) >> 32 != 0
+
+
+@pytest.mark.parametrize("lens,H,want", [
+    ([30] * 500 + [8000], 16, ONE),   # 887 / 1922: each pair's start costs more than the long one gains
+    ([200] * 60 + [4000], 16, ONE),   # 458 / 491
+    ([500] * 30 + [10000], 16, PAIR),  # 1114 / 780
+    ([30] * 80 + [8000], 16, PAIR),   # 886 / 564
+    ([30] * 200 + [16000], 4, PAIR),  # 1750 / 1093
+])
+def test_packed_sequences(lens, H, want):
+    x = make_inputs(1, sum(lens), H, 128, dtype="bf16", device="cuda", device_rng=True)
+    cu = torch.tensor([0] + lens, dtype=torch.int32).cumsum(0).to(torch.int32).cuda()
+    got, ws = _scans("rdn", x, cu_seqlens=cu)
+    assert got == {ONE, PAIR}  # (the lengths are on the device: both are launched)
+    assert _table_says_pairs(ws, len(lens)) == (want == PAIR)
