@@ -368,10 +368,15 @@ inline bool use_pairs(const FwdParams &p, bool rdnv, int nsm) {
   if (p.seq) return pairs_for(c, p.nseq > 1 ? (p.NC + 1) / 2 : p.NC, p.nseq, p.NC + p.nseq, p.H, nsm);
   return pairs_for(c, p.NC, p.nseq, (long long)p.nseq * p.NC, p.H, nsm);
 }
-// ... and packed sequences, of which one may be long, have both kernels launched and
-// the table say which one runs (the other's CTAs return at once).
-inline bool pick_on_device(const FwdParams &p, int nsm) {
-  return p.seq && 2ll * p.nseq * p.H > nsm;
+// ... and packed sequences have both kernels launched and the table say which one
+// runs, if pairs can be the choice at all: with one long sequence and the others as
+// short as can be, and no more sequences than the table puts in order (kOrdered).
+// The other kernel's CTAs return at once, but each takes an SM's shared memory to
+// start, 0.64 us a CTA and SM: 2000 sequences of 16 heads 262 us.
+constexpr int kOrdered = 1024;  // packed sequences that are put in order of length
+inline bool pick_on_device(const FwdParams &p, bool rdnv, int nsm) {
+  return p.seq && 2ll * p.nseq * p.H > nsm && p.nseq <= kOrdered &&
+         pairs_for(scan_cost(rdnv, p.S_chunks != nullptr), p.NC, p.nseq, p.NC, p.H, nsm);
 }
 
 }  // namespace rdn

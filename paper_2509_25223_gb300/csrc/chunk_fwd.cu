@@ -605,7 +605,6 @@ __device__ long long block_incl_scan(long long x, Op op, long long *wsum) {
   return x;
 }
 
-constexpr int kOrdered = 1024;  // packed sequences that are put in order of length
 // The packed-sequence table FwdParams::seq from cu_seqlens[0 .. N]: first
 // tokens are the running maximum of the entries clamped into [0, T] (with
 // entry 0 read as 0 and entry N as T, so the table always covers [0, T) in

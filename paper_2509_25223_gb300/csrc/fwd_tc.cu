@@ -796,7 +796,7 @@ cudaError_t launch_fwd_tc(const FwdParams &p, bool rdnv, cudaStream_t s) {
   cudaError_t e = sm_count(&nsm);
   if (e != cudaSuccess) return e;
   FwdParams one = p;
-  const bool both = pick_on_device(p, nsm);
+  const bool both = pick_on_device(p, rdnv, nsm);
   maps.o_ok = !p.f32out && make_tile_map(maps.o, p.o, D, p.H, rows);
   if (both || use_pairs(p, rdnv, nsm)) {
     FwdParams two = p;

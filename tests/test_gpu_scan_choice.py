@@ -70,3 +70,17 @@ def test_packed_sequences(lens, H, want):
     got, ws = _scans("rdn", x, cu_seqlens=cu)
     assert got == {ONE, PAIR}  # (the lengths are on the device: both are launched)
     assert _table_says_pairs(ws, len(lens)) == (want == PAIR)
+
+
+@pytest.mark.parametrize("variant,lens,H", [
+    ("rdn", [16, 64, 40, 33] * 300, 4),   # more sequences than are put in order
+    ("rdn", [2] * 900, 16),               # too few chunks for any one to be long enough
+    ("rla", [30] * 40 + [300], 40),       # too many heads for it
+])
+def test_packed_pairs_are_not_launched_where_they_cannot_run(variant, lens, H):
+    """The kernel that the table does not choose returns at once, which still takes
+    each of its CTAs an SM (0.64 us each, 262 us for 2000 sequences of 16 heads)."""
+    x = make_inputs(1, sum(lens), H, 128, dtype="bf16", device="cuda", device_rng=True)
+    cu = torch.tensor([0] + lens, dtype=torch.int32).cumsum(0).to(torch.int32).cuda()
+    got, ws = _scans(variant, x, cu_seqlens=cu)
+    assert got == {ONE} and not _table_says_pairs(ws, len(lens))
