@@ -49,12 +49,15 @@ def test_equal_sequences(variant, heads, T, states, want):
     assert got == {want}
 
 
-def _table_says_pairs(ws, n):
-    """The choice in the sequence table at the workspace's end: the upper half of
-    entry n's chunk number."""
+def _table(ws, n):
+    """The n + 1 chunk numbers of the sequence table at the workspace's end."""
     size = (16 * (n + 1) + 255) // 256 * 256
-    table = ws[ws.numel() - 256 - size:][:16 * (n + 1)].view(torch.int64)
-    return int(table[2 * n + 1]) >> 32 != 0
+    return ws[ws.numel() - 256 - size:][:16 * (n + 1)].view(torch.int64)[1::2].cpu()
+
+
+def _table_says_pairs(ws, n):
+    """The choice: the upper half of entry n's chunk number."""
+    return int(_table(ws, n)[n]) >> 32 != 0
 
 
 @pytest.mark.parametrize("lens,H,want", [
@@ -84,3 +87,17 @@ def test_packed_pairs_are_not_launched_where_they_cannot_run(variant, lens, H):
     cu = torch.tensor([0] + lens, dtype=torch.int32).cumsum(0).to(torch.int32).cuda()
     got, ws = _scans(variant, x, cu_seqlens=cu)
     assert got == {ONE} and not _table_says_pairs(ws, len(lens))
+
+
+@pytest.mark.parametrize("n", [1, 2, 15, 256, 257, 511, 600, 1023, 1024, 1025])
+def test_packed_order(n):
+    """The order in which packed sequences start: by chunks, most first, equal ones as
+    they come; above 1024 as they come."""
+    lens = torch.randint(0, 400, (n,), generator=torch.Generator().manual_seed(n)).tolist()
+    x = make_inputs(1, max(sum(lens), 1), 1, 64, dtype="bf16", device="cuda", device_rng=True)
+    lens[-1] += 1 if sum(lens) == 0 else 0
+    cu = torch.tensor([0] + lens, dtype=torch.int32).cumsum(0).to(torch.int32).cuda()
+    _, ws = _scans("rdn", x, cu_seqlens=cu)
+    order = (_table(ws, n)[:n] >> 32).tolist()
+    chunks = [(c + 63) // 64 for c in lens]
+    assert order == (sorted(range(n), key=lambda s: -chunks[s]) if n <= 1024 else list(range(n)))
