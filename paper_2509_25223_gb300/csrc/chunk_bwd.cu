@@ -48,6 +48,9 @@ struct BwdParams {
   // the auxiliary delta rule, dX with the base one) and the gradients w.r.t.
   // the chunk-end states [record][DK][DV]
   float *dX2, *dVr, *dX, *gS, *gR;
+  // dv is dO's buffer: bwd_post, which still reads dO, writes it (then dX is kept
+  // with either base pass)
+  bool dv_late;
   // RDN_FLAG_QK_NORM with bf16 inputs: dq, dk (w.r.t. the normalised q, k)
   // stored here in fp32 for the normalisation's backward; else NULL
   float *gq32, *gk32;
@@ -307,8 +310,8 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 2 : 1) bwd_chain_kernel(BwdPar
         a[j] = -gp * dvr[i][j] - (RDNV ? Gam[t] * x[i][j] : 0.f);
         b[j] = gq * dO[i][j];
       }
-      if (RDNV) stv<TN>(p.dX + (rec * C + t) * DV + j0 + n0, x[i]);
-      if (t < n)
+      if (RDNV || p.dv_late) stv<TN>(p.dX + (rec * C + t) * DV + j0 + n0, x[i]);
+      if (t < n && !p.dv_late)
         st_row<InT, TN>((InT *)p.dv + ((size_t)(sp.tok0 + c * C + t) * H + h) * DV + j0 + n0, v);
       stv<TN>(T2 + t * DVS + n0, a);
       stv<TN>(DO + t * DVS + n0, b);
@@ -669,6 +672,16 @@ __global__ void __launch_bounds__(kPostThreads, 1) bwd_post_kernel(BwdParams p) 
       }
     }
   }
+  if (p.dv_late)  // (every dO of this chunk has been read)
+    for (int e = tid; e < n * DV / 4; e += NT) {
+      const int t = e / (DV / 4), j = 4 * (e % (DV / 4));
+      float v[4], x[4];
+      ldv<4>(p.dVr + toff + t * DV + j, v);
+      ldv<4>(p.dX + toff + t * DV + j, x);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) v[i] += x[i];
+      st_row<InT, 4>((InT *)p.dv + (row0 + (size_t)t * H) * DV + j, v);
+    }
   // ---- row sums over a row's 16 lanes, column sums over the block
   float *colp = sm + SM::ST;  // [8 warps][3][C], then the warps' dgc
 #pragma unroll
@@ -997,6 +1010,7 @@ static cudaError_t launch_bwd_impl(const rdn_bwd_args &a, int variant, cudaStrea
   p.dq = a.dq;
   p.dk = a.dk;
   p.dv = a.dv;
+  p.dv_late = a.dv == a.dO;
   p.dg = a.dg;
   p.dbeta = a.dbeta;
   p.dgamma = a.dgamma;
