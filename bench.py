@@ -47,23 +47,24 @@ C = 64
 #     the products over the value dimension        12 d^2 + 5 C d
 #     (dK, dQ state terms; C x C gradients)
 #     the backward of the prep                     2 (2 C d + (4/3) C^2)
-#   (the tensor-core bwd_post does the last two; the SIMT path splits them
-#   into bwd_scan and bwd_finish).  Recomputation of forward pieces is not
-#   algorithmic work (counted 0).
+#   (bwd_chain and bwd_chain_f32 do the first, bwd_post and bwd_post_f32 the
+#   last two).  Recomputation of forward pieces is not algorithmic work
+#   (counted 0).
 #   The same work with every C x C x d product counted as a dense tile (the
 #   triangular ones at full size): forward + 7 C d per token-head.
 def flops_per_token_head(d=128, c=C):
     scan = 12 * d * d + 5 * c * d
     prep = 2 * c * d + (4.0 / 3.0) * c * c
-    return dict(fwd=scan + prep, fwd_scan=scan, fwd_prep=prep, bwd_scan=2 * scan,
-                bwd_chain=scan, bwd_post=scan + 2 * prep, bwd_finish=2 * prep, recompute=0.0,
+    return dict(fwd=scan + prep, fwd_scan=scan, fwd_prep=prep, bwd_chain=scan,
+                bwd_post=scan + 2 * prep, recompute=0.0,
                 step=3 * (scan + prep), step_dense_tiles=3 * (scan + prep + 7 * c * d))
 
 
 # kernel name (as recorded by the library) -> algorithmic flop per token-head
-KERNEL_WORK = {"chunk_scan": "fwd_scan", "fwd_tc_scan": "fwd_scan", "chunk_prep": "fwd_prep",
-               "bwd_scan": "bwd_scan", "bwd_chain": "bwd_chain", "bwd_post": "bwd_post",
-               "bwd_finish": "bwd_finish", "bwd_recompute": "recompute"}
+KERNEL_WORK = {"chunk_scan": "fwd_scan", "fwd_tc_scan": "fwd_scan", "fwd_tc_pair": "fwd_scan",
+               "chunk_prep": "fwd_prep", "bwd_chain": "bwd_chain", "bwd_post": "bwd_post",
+               "bwd_chain_f32": "bwd_chain", "bwd_post_f32": "bwd_post",
+               "bwd_recompute": "recompute", "chunk_recompute": "recompute"}
 
 # decode: read + write S and R fp32, plus q, k, v, o bf16 and three fp32 gates
 def decode_bytes_per_head(d=128):
@@ -712,7 +713,7 @@ def run_ours(args):
                           "states": "S0, R0 in, S_T, R_T out" if ret else "zero, not returned"}
             del xf, of, wsff
 
-    # ---- the paper's variants (variant_flags, fp32 chunk kernels) on the
+    # ---- the paper's variants (variant_flags) on the
     # bench workload: RDN fwd+bwd with each flag, as the RDN step above
     var = None
     if not args.no_variants:
