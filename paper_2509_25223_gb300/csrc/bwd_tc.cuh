@@ -99,8 +99,6 @@ struct Ctl {
   volatile int *flag;
   uint32_t phase, phA, phB;
   uint32_t armA, armB, armC, seenA, seenB, seenC;  // (thread 0) copy phases on A, B, C
-  long long limit;             // the MMA waits' limit in cycles
-  bool skip;                   // (thread 0) the next phase skips its completion signal (tests)
 };
 
 __device__ __forceinline__ void ctl_init(Ctl &k, uint8_t *base, int tid) {
@@ -112,8 +110,6 @@ __device__ __forceinline__ void ctl_init(Ctl &k, uint8_t *base, int tid) {
   k.barD = reinterpret_cast<uint64_t *>(base + 40);
   k.phase = k.phA = k.phB = 0;
   k.armA = k.armB = k.armC = k.seenA = k.seenB = k.seenC = 0;
-  k.limit = 2000000000ll;
-  k.skip = false;
   if (tid == 0) {
     mbar_init(k.bar, 1);
     mbar_init(k.barA, 1);
@@ -181,10 +177,9 @@ __device__ __forceinline__ bool phase_run(Ctl &k, int tid, F issue) {
   if (tid == 0) {
     fence_after_sync();
     if (!issue()) *k.flag = 1;
-    if (!k.skip) mma_commit(k.bar);
-    k.skip = false;
+    mma_commit(k.bar);
   }
-  const bool ok = mbar_wait(k.bar, k.phase, k.limit);
+  const bool ok = mbar_wait(k.bar, k.phase);
   k.phase ^= 1u;
   if (!ok) *k.flag = 1;
   __syncthreads();
@@ -202,12 +197,11 @@ __device__ __forceinline__ bool phase_run_with(Ctl &k, int tid, F issue, G durin
   if (tid == 0) {
     fence_after_sync();
     if (!issue()) *k.flag = 1;
-    if (!k.skip) mma_commit(k.bar);
-    k.skip = false;
+    mma_commit(k.bar);
   }
   __syncwarp();  // (TMEM accesses take whole warps)
   during();
-  const bool ok = mbar_wait(k.bar, k.phase, k.limit);
+  const bool ok = mbar_wait(k.bar, k.phase);
   k.phase ^= 1u;
   if (!ok) *k.flag = 1;
   __syncthreads();
@@ -225,14 +219,13 @@ __device__ __forceinline__ void phase_issue(Ctl &k, int tid, F issue) {
   if (tid == 0) {
     fence_after_sync();
     if (!issue()) *k.flag = 1;
-    if (!k.skip) mma_commit(k.bar);
-    k.skip = false;
+    mma_commit(k.bar);
   }
   __syncwarp();  // (TMEM accesses take whole warps)
 }
 // ... then wait for them (every thread).
 __device__ __forceinline__ bool phase_wait(Ctl &k) {
-  const bool ok = mbar_wait(k.bar, k.phase, k.limit);
+  const bool ok = mbar_wait(k.bar, k.phase);
   k.phase ^= 1u;
   if (!ok) *k.flag = 1;
   __syncthreads();

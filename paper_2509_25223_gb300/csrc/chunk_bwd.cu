@@ -856,8 +856,8 @@ struct BwdLayout {
   size_t prep, chain, saved, states, o, tc, qk, g32, tied, seq, total;
 };
 
-// bf16 inputs with d = 128 take the tensor-core backward (RDN, and RLA with
-// identity T matrices in its records), the variants the fp32 one
+// bf16 inputs with d = 128 take the tensor-core backward (RDN, RLA with identity T
+// matrices in its records, and every variant flag), all else the fp32 one
 bool use_tc_bwd(const rdn_fwd_args &f, int variant) {
   (void)variant;
   return fwd_uses_tc(f.Dk, f.dtype == RDN_BF16);

@@ -525,7 +525,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
   };
   float vv[16];         // CTA 0: this thread's V entries of the last chunk begun
   // CTA 0: chunk c's P | Ob are complete: r = clip(V - P); r and Ob -> CTA 1.
-  // (The copies of chunk c - 1 have left their places: the issuing warp saw
+  // (The copies of chunk c - 1 have left their places: the copying warp saw
   // `empty` before this chunk's first barrier.)
   auto hand_over = [&](int c) {
     const size_t ci = (size_t)(sp.rbase + c);
@@ -621,7 +621,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     float *start = (chunks && c > 0) ? chunks + ci * D * D : nullptr;
     fence_async_smem();
     fence_before_sync();
-    __syncthreads();  // (with the issuing warp, which has waited for the tiles)
+    __syncthreads();  // (with the copying warp, which has waited for the tiles)
     fence_after_sync();
     if (*flag) {
       alive = false;
