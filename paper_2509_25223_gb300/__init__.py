@@ -88,7 +88,10 @@ def _alloc_ws(nbytes, device):
 
 def _f32(x):
     """float(x) as the nearest C float (out of range: infinite), as a Python float."""
-    return ctypes.c_float(float(x)).value
+    try:
+        return ctypes.c_float(x).value
+    except TypeError:
+        return ctypes.c_float(float(x)).value
 
 
 def _check_variant_flags(f):

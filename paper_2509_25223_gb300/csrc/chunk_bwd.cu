@@ -880,8 +880,8 @@ BwdLayout layout(const rdn_bwd_args &a, int variant) {
   BwdLayout l;
   // the forward's records are read from its workspace when it is passed
   l.prep = reuse_fwd_records(f) ? 0 : align256(sizeof(float) * nrec * kRecFloats);
-  // what the fp32 chain keeps of each chunk (the tensor-core kernels': l.tc): dVr,
-  // dX and, with the auxiliary delta rule, dX2; the chunk-end gradients
+  // what the fp32 chain keeps of each chunk (the tensor-core kernels': l.tc): RDN's
+  // dX2, dVr, dX, the chunk-end gradients
   l.chain = tc ? 0 : align256(sizeof(float) * nrec * ((variant ? 3 : 2) * C * f.Dv + 2 * f.Dk * f.Dv));
   // E, E2 and the residual's mask, unless the forward kept them
   l.saved = tc || fwd_saved(f) ? 0 : align256(saved_layout(f).bytes);
@@ -889,7 +889,7 @@ BwdLayout layout(const rdn_bwd_args &a, int variant) {
   l.states = need_states ? align256(sizeof(float) * nrec * f.Dk * f.Dv) : 0;  // each of S, R
   const size_t esz = f.dtype == RDN_BF16 ? 2 : 4;
   // (a forward run here writes its o, which nobody reads, where the fp32 chain's
-  // dVr goes later: a record's 64 rows of Dv floats hold its tokens')
+  // first rows go later: a record's 64 rows of Dv floats hold its tokens')
   l.o = need_states && tc ? align256(esz * (size_t)f.B * f.T * f.H * f.Dv) : 0;
   l.tc = tc ? align256(bwd_tc_extra_bytes(nrec, f.flags & RDN_FLAG_TANH_RESIDUAL)) : 0;
   // normalised q, k (RDN_FLAG_QK_NORM), unless the forward's workspace has them
@@ -1002,11 +1002,11 @@ static cudaError_t launch_bwd_impl(const rdn_bwd_args &a, int variant, cudaStrea
   if (e != cudaSuccess) return e;
   p.Sc = p.f.S_chunks;
   p.Rc = p.f.R_chunks;
-  p.dVr = (float *)(ws + l.prep);
+  p.dX2 = (float *)(ws + l.prep);
+  p.dVr = p.dX2 + (rdnv ? (size_t)p.f.nrec * C * f.Dv : 0);
   p.dX = p.dVr + (size_t)p.f.nrec * C * f.Dv;
   p.gS = p.dX + (size_t)p.f.nrec * C * f.Dv;
   p.gR = p.gS + (size_t)p.f.nrec * f.Dk * f.Dv;
-  p.dX2 = rdnv ? p.gR + (size_t)p.f.nrec * f.Dk * f.Dv : nullptr;
   p.dO = a.dO;
   p.dST = a.dST;
   p.dRT = a.dRT;
