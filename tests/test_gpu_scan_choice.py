@@ -101,3 +101,44 @@ def test_packed_order(n):
     order = (_table(ws, n)[:n] >> 32).tolist()
     chunks = [(c + 63) // 64 for c in lens]
     assert order == (sorted(range(n), key=lambda s: -chunks[s]) if n <= 1024 else list(range(n)))
+
+
+@pytest.mark.parametrize("variant", ["rdn", "rla"])
+def test_short_sequences_in_pairs(variant):
+    """Sequences of one and two chunks by the pair kernel, which they take only beside
+    a long one: results, kept states and the gradients from what it saved are those of
+    a call of their own, bit for bit."""
+    lens, H = [1, 64, 65, 128, 0, 63] + [30] * 74 + [700], 2
+    T, N = sum(lens), len(lens)
+    x = make_inputs(1, T, H, 128, dtype="bf16", with_grad_out=True, device="cuda")
+    cu = torch.tensor([0] + lens, dtype=torch.int32).cumsum(0).to(torch.int32).cuda()
+    st = 0.1 * torch.randn(4, N, H, 128, 128, generator=torch.Generator().manual_seed(5)).cuda()
+    fwd, bwd = (rdn.rdn_fwd, rdn.rdn_bwd) if variant == "rdn" else (rdn.rla_fwd, rdn.rla_bwd)
+
+    def step(x, st, cu):
+        B, T = x["q"].shape[:2]
+        kw = dict(clip=0.7, S0=st[0], R0=st[1], cu_seqlens=cu)
+        ws = torch.empty(rdn.workspace_bytes(variant + "_fwd", B, T, H, 128, save_for_bwd=True,
+                                             cu_seqlens=cu), dtype=torch.uint8, device="cuda")
+        o, ST, RT, Sc, Rc = fwd(*(x[n] for n in NAMES), return_chunk_states=True, save_for_bwd=True,
+                                workspace=ws, **kw)
+        d = bwd(*(x[n] for n in NAMES), x["dO"], S_chunks=Sc, R_chunks=Rc, dST=st[2], dRT=st[3],
+                fwd_workspace=ws, fwd_saved=True, **kw)
+        return ws, dict(o=o, **{n: d[n] for n in ("dq", "dk", "dv", "dg", "dbeta", "dgamma")}), \
+            dict(ST=ST, RT=RT, dS0=d["dS0"], dR0=d["dR0"]), (Sc, Rc)
+
+    ws, tok, per, chunks = step(x, st, cu)
+    assert _table_says_pairs(ws, N)
+    first = slot = 0
+    for s, n in enumerate(lens):
+        nc = (n + 63) // 64
+        if n and (s < 8 or n > 64):
+            sl = {m: t[:, first:first + n].clone() for m, t in x.items() if t is not None}
+            _, tok1, per1, chunks1 = step(sl, st[:, s:s + 1].contiguous(), None)
+            for m, t in tok1.items():
+                assert torch.equal(tok[m][:, first:first + n], t), (s, m)
+            for m, t in per1.items():
+                assert torch.equal(per[m][s:s + 1], t), (s, m)
+            for a, b in zip(chunks, chunks1):
+                assert torch.equal(a[slot:slot + nc * H], b.reshape(-1, 128, 128)), s
+        first, slot = first + n, slot + nc * H
