@@ -361,7 +361,7 @@ __host__ __device__ inline bool pairs_for(const ScanCost &c, long long longest, 
 }
 // Where every pair has its two SMs at once the host decides (packed: the lengths
 // are on the device, the longest is taken for half of the tokens); where not, equal
-// sequences take one CTA each (f1 < f2, and in waves l1 never is above l2's).
+// sequences take one CTA each, which needs half the waves at less than twice the time.
 inline bool use_pairs(const FwdParams &p, bool rdnv, int nsm) {
   if (2ll * p.nseq * p.H > nsm) return false;
   const ScanCost c = scan_cost(rdnv, p.S_chunks != nullptr);
